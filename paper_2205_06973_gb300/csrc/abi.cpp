@@ -41,6 +41,9 @@ constexpr int kProbBlocks = 152 * 8;
 // (sv_measure_summary)
 constexpr int kSummaryAt = kProbBlocks + 1;
 constexpr int kPartialsLen = kSummaryAt + 3 * kProbBlocks + 4;
+// per-state device words: the error word of bounded waits, then the block
+// tickets of the two measurements
+constexpr int kErrWords = 3;
 }  // namespace
 
 namespace hisv {
@@ -102,8 +105,8 @@ static sv_status create_state(int n, sv_precision prec, void *dev_buf, size_t de
         s->owns = true;
     }
     cudaError_t e = dev_alloc(reinterpret_cast<void **>(&s->d_partials), sizeof(double) * kPartialsLen, s->stream);
-    if (e == cudaSuccess) e = dev_alloc(reinterpret_cast<void **>(&s->d_err), sizeof(int), s->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(s->d_err, 0, sizeof(int), s->stream);
+    if (e == cudaSuccess) e = dev_alloc(reinterpret_cast<void **>(&s->d_err), sizeof(int) * kErrWords, s->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(s->d_err, 0, sizeof(int) * kErrWords, s->stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
         if (s->owns) dev_free(s->buf, s->stream);
@@ -646,7 +649,7 @@ sv_status sv_measure_probs(sv_state *s, void *dev_out, int out_fp64, double *nor
     if (!s) return fail(SV_ERR_ARG, "state is NULL");
     double *d_norm = s->d_partials + kProbBlocks;
     CUDA_TRY(launch_probs(is_fp64(s), s->buf, s->n, dev_out, out_fp64, s->d_partials, kProbBlocks, d_norm, s->stream,
-                          is_df(s)));
+                          is_df(s), reinterpret_cast<uint32_t *>(s->d_err + 1)));
     if (norm_out) {
         CUDA_TRY(cudaMemcpyAsync(&s->h_norm, d_norm, sizeof(double), cudaMemcpyDeviceToHost, s->stream));
         CUDA_TRY(cudaStreamSynchronize(s->stream));
@@ -665,7 +668,8 @@ sv_status sv_measure_summary(sv_state *s, double *norm_out, double *p0_out, uint
                              double *pmax_out) {
     if (!s) return fail(SV_ERR_ARG, "state is NULL");
     double *scratch = s->d_partials + kSummaryAt, *d_out = scratch + 3 * kProbBlocks;
-    CUDA_TRY(launch_summary(is_fp64(s), s->buf, s->n, scratch, kProbBlocks, d_out, s->stream, is_df(s)));
+    CUDA_TRY(launch_summary(is_fp64(s), s->buf, s->n, scratch, kProbBlocks, d_out, s->stream, is_df(s),
+                            reinterpret_cast<uint32_t *>(s->d_err + 2)));
     double h[4];
     CUDA_TRY(cudaMemcpyAsync(h, d_out, sizeof(h), cudaMemcpyDeviceToHost, s->stream));
     CUDA_TRY(cudaStreamSynchronize(s->stream));

@@ -51,7 +51,8 @@ struct sv_state {
     int dev = 0;
     double *d_partials = nullptr;   // kProbBlocks + 1 doubles; the last holds the norm
     double h_norm = 0.0;            // norm read back from the device
-    int *d_err = nullptr;           // device error word of bounded waits (0 = none)
+    int *d_err = nullptr;           // device error word of bounded waits (0 = none), then the
+                                    // block tickets of the measurements
     double *d_dnorm = nullptr;      // norm accumulators of one apply's dense passes
     size_t dnorm_cap = 0;           // (1 + tensor-core passes), grown on demand
     void *d_stage = nullptr;        // double2 staging of double-float downloads (allocated on first use)

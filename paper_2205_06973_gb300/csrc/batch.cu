@@ -16,6 +16,7 @@
 
 #include "batch.hpp"
 #include "ops.cuh"
+#include "prob_split.cuh"
 
 namespace hisv {
 
@@ -170,22 +171,77 @@ __global__ void __launch_bounds__(256) k_batch(float2 *__restrict__ svbase, cons
     }
 }
 
-// p[i] = |a_i|^2 over the concatenated states; one block per circuit also
-// sums its norm in FP64.
-__global__ void __launch_bounds__(256) k_batch_probs(const float2 *__restrict__ svbase,
+// p[i] = |a_i|^2 over the concatenated states, 2^10 amplitudes per block and
+// iteration (the smallest circuit, and every circuit's offset is a multiple
+// of it), on the FP32 pipes as in k_probs_fast; partials (may be null)
+// receives each chunk's FP64 sum. One block per circuit with FP64 arithmetic
+// left a batch's largest circuits to single SMs: 2.83 ms for 160 circuits of
+// 10 to 20 qubits (28.5 M amplitudes), the time of one 20-qubit circuit;
+// 0.1 ms here.
+constexpr int BPROB_CHUNK = 1 << BATCH_MIN_QUBITS;
+static_assert(BPROB_CHUNK == 4 * 256, "two 16-byte loads per thread");
+
+__global__ void __launch_bounds__(256) k_batch_probs(const float4 *__restrict__ sv, uint64_t n_chunks,
+                                                     float *__restrict__ out, bool pairs,
+                                                     double *__restrict__ partials) {
+    __shared__ double red[8];
+    for (uint64_t c = blockIdx.x; c < n_chunks; c += gridDim.x) {
+        const uint64_t at = c * (BPROB_CHUNK / 2) + threadIdx.x;
+        float4 v[2];
+#pragma unroll
+        for (int u = 0; u < 2; u++) v[u] = __ldcs(sv + at + 256 * u);
+        float S = 0.0f, T = 0.0f;
+        double acc = 0.0;
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            float p, q;
+            if (split_range<false>(v[u])) {
+                const float2 a = split_prob(v[u].x, v[u].y), b = split_prob(v[u].z, v[u].w);
+                split_add(S, T, a);
+                split_add(S, T, b);
+                p = a.x + a.y;
+                q = b.x + b.y;
+            } else {
+                const double a = (double)v[u].x * v[u].x + (double)v[u].y * v[u].y;
+                const double b = (double)v[u].z * v[u].z + (double)v[u].w * v[u].w;
+                acc += a + b;
+                p = (float)a;
+                q = (float)b;
+            }
+            if (out) {
+                const uint64_t i = 2 * (at + 256 * u);
+                if (pairs) *reinterpret_cast<float2 *>(out + i) = make_float2(p, q);
+                else {
+                    out[i] = p;
+                    out[i + 1] = q;
+                }
+            }
+        }
+        if (!partials) continue;
+        acc += (double)S + (double)T;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double s = 0.0;
+            for (int w = 0; w < 8; w++) s += red[w];
+            partials[c] = s;
+        }
+        __syncthreads();
+    }
+}
+
+// A circuit's norm: its chunks' sums in a fixed order, one block per circuit.
+__global__ void __launch_bounds__(256) k_batch_norms(const double *__restrict__ partials,
                                                      const uint64_t *__restrict__ circ_off,
-                                                     const uint32_t *__restrict__ circ_n, float *__restrict__ out,
-                                                     double *__restrict__ norms) {
+                                                     const uint32_t *__restrict__ circ_n, double *__restrict__ norms) {
     __shared__ double red[8];
     const uint32_t c = blockIdx.x;
-    const uint64_t off = circ_off[c], N = 1ull << circ_n[c];
+    const double *const v = partials + circ_off[c] / BPROB_CHUNK;
+    const uint32_t m = 1u << (circ_n[c] - BATCH_MIN_QUBITS);
     double acc = 0.0;
-    for (uint64_t i = threadIdx.x; i < N; i += blockDim.x) {
-        const float2 v = __ldcs(svbase + off + i);
-        const double p = (double)v.x * v.x + (double)v.y * v.y;
-        if (out) out[off + i] = (float)p;
-        acc += p;
-    }
+    for (uint32_t i = threadIdx.x; i < m; i += blockDim.x) acc += v[i];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
@@ -228,9 +284,18 @@ cudaError_t launch_batch(const BatchLaunch &B, int warps_per_cta, int n_ctas, cu
     return cudaGetLastError();
 }
 
-cudaError_t launch_batch_probs(float2 *svbase, const uint64_t *circ_off, const uint32_t *circ_n, uint32_t n_circ,
-                               float *out, double *norms, cudaStream_t st) {
-    k_batch_probs<<<n_circ, 256, 0, st>>>(svbase, circ_off, circ_n, out, norms);
+cudaError_t launch_batch_probs(float2 *svbase, uint64_t total, const uint64_t *circ_off, const uint32_t *circ_n,
+                               uint32_t n_circ, float *out, double *partials, double *norms, cudaStream_t st) {
+    const uint64_t chunks = total / BPROB_CHUNK;
+    const uint64_t blocks = chunks < 152 * 8 ? chunks : 152 * 8;
+    if (out || norms) {
+        k_batch_probs<<<(unsigned)blocks, 256, 0, st>>>(reinterpret_cast<const float4 *>(svbase), chunks, out,
+                                                        (reinterpret_cast<uintptr_t>(out) & 7) == 0,
+                                                        norms ? partials : nullptr);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    if (norms) k_batch_norms<<<n_circ, 256, 0, st>>>(partials, circ_off, circ_n, norms);
     return cudaGetLastError();
 }
 

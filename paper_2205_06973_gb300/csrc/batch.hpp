@@ -41,8 +41,10 @@ constexpr int BATCH_MIN_QUBITS = 10;
 // resident on all SMs) for a CTA of warps_per_cta warps.
 cudaError_t batch_prepare(int warps_per_cta, int *n_ctas);
 cudaError_t launch_batch(const BatchLaunch &B, int warps_per_cta, int n_ctas, cudaStream_t st);
-cudaError_t launch_batch_probs(float2 *svbase, const uint64_t *circ_off, const uint32_t *circ_n, uint32_t n_circ,
-                               float *out, double *norms, cudaStream_t st);
+// Probabilities of all states (out, may be null) and, with norms, each
+// circuit's norm: partials then holds total / 2^BATCH_MIN_QUBITS doubles.
+cudaError_t launch_batch_probs(float2 *svbase, uint64_t total, const uint64_t *circ_off, const uint32_t *circ_n,
+                               uint32_t n_circ, float *out, double *partials, double *norms, cudaStream_t st);
 cudaError_t launch_batch_reset(float2 *svbase, const uint64_t *circ_off, uint32_t n_circ, uint64_t total,
                                cudaStream_t st);
 

@@ -53,6 +53,7 @@ struct sv_batch {
     uint32_t *d_done = nullptr;          // n counters + the two queue tickets (gate lists, dense)
     int *d_err = nullptr;                // error word, then the dense kernel's record of a failed wait
     double *d_norms = nullptr;
+    double *d_chunk_norms = nullptr;     // per 2^10 amplitudes (allocated when norms are first asked for)
     std::vector<double> h_norms;
     // compiled program (rebuilt when plans or the configuration change)
     bool built = false;
@@ -502,8 +503,17 @@ sv_status sv_batch_reset(sv_batch *b) {
 
 sv_status sv_batch_probs(sv_batch *b, void *dev_out, double *norms_host) {
     if (!b) return bfail(SV_ERR_ARG, "batch is NULL");
-    BCUDA(launch_batch_probs(b->sv, b->d_off, b->d_nq, b->n, reinterpret_cast<float *>(dev_out), b->d_norms,
-                             b->stream));
+    if (norms_host && !b->d_chunk_norms) {
+        cudaError_t e = dev_alloc(reinterpret_cast<void **>(&b->d_chunk_norms),
+                                  sizeof(double) * (b->total >> BATCH_MIN_QUBITS), b->stream);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            b->d_chunk_norms = nullptr;
+            return bfail(SV_ERR_OOM, std::string("batch norms: ") + cudaGetErrorString(e));
+        }
+    }
+    BCUDA(launch_batch_probs(b->sv, b->total, b->d_off, b->d_nq, b->n, reinterpret_cast<float *>(dev_out),
+                             b->d_chunk_norms, norms_host ? b->d_norms : nullptr, b->stream));
     if (norms_host) {
         BCUDA(cudaMemcpyAsync(b->h_norms.data(), b->d_norms, sizeof(double) * b->n, cudaMemcpyDeviceToHost,
                               b->stream));
@@ -567,6 +577,7 @@ sv_status sv_batch_destroy(sv_batch *b) {
     dev_free(b->d_done, b->stream);
     dev_free(b->d_err, b->stream);
     dev_free(b->d_norms, b->stream);
+    dev_free(b->d_chunk_norms, b->stream);
     if (b->own_stream) {
         cudaStreamSynchronize(b->stream);   // the frees complete before the stream goes
         cudaStreamDestroy(b->stream);

@@ -18,6 +18,7 @@
 
 #include "kernels.hpp"
 #include "ops.cuh"
+#include "prob_split.cuh"
 
 namespace hisv {
 
@@ -368,19 +369,40 @@ __device__ __forceinline__ void amp_parts(const float4 &v, double &re, double &i
     im = (double)v.z + (double)v.w;
 }
 
-template <typename E, typename Out>
-__global__ void __launch_bounds__(256) k_probs(const E *__restrict__ sv, uint64_t N,
-                                                Out *__restrict__ out, double *__restrict__ partials) {
-    __shared__ double red[8];
-    double acc = 0.0;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (uint64_t)gridDim.x * blockDim.x) {
-        const E v = __ldcs(sv + i);
-        double re, im;
-        amp_parts(v, re, im);
-        const double p = re * re + im * im;
-        if (out) out[i] = (Out)p;
-        acc += p;
+// The sum of a block's FP64 partials into partials[blockIdx.x]; the block that
+// ends last (ticket: blocks done, back at zero afterwards) also adds all
+// partials up, in the same order as k_sum, and writes the norm: one launch
+// less per measurement. ticket null: k_sum follows.
+__device__ __forceinline__ bool last_block(uint32_t *ticket, uint32_t &flag) {
+    if (threadIdx.x == 0) {
+        __threadfence();
+        const uint32_t t = atomicAdd(ticket, 1u);
+        flag = t + 1 == gridDim.x;
+        if (flag) {
+            *ticket = 0u;
+            __threadfence();
+        }
     }
+    __syncthreads();
+    return flag != 0;
+}
+
+// 256 threads: the sum of v[0..nb) in a fixed order, valid in thread 0.
+__device__ __forceinline__ double sum_partials(const double *v, int nb, double *red) {
+    double s = 0.0;
+    for (int i = threadIdx.x; i < nb; i += blockDim.x) s += __ldcg(v + i);
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
+        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+        __syncthreads();
+    }
+    return red[0];
+}
+
+__device__ __forceinline__ void finish_norm(double acc, double *partials, uint32_t *ticket, double *out) {
+    __shared__ double red[256];
+    __shared__ uint32_t flag;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
@@ -390,46 +412,136 @@ __global__ void __launch_bounds__(256) k_probs(const E *__restrict__ sv, uint64_
         for (int w = 0; w < (int)(blockDim.x >> 5); w++) s += red[w];
         partials[blockIdx.x] = s;
     }
+    if (!ticket || !last_block(ticket, flag)) return;
+    const double s = sum_partials(partials, gridDim.x, red);
+    if (threadIdx.x == 0) *out = s;
+}
+
+template <typename E, typename Out>
+__global__ void __launch_bounds__(256) k_probs(const E *__restrict__ sv, uint64_t N, Out *__restrict__ out,
+                                                double *__restrict__ partials, uint32_t *ticket, double *norm) {
+    double acc = 0.0;
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (uint64_t)gridDim.x * blockDim.x) {
+        const E v = __ldcs(sv + i);
+        double re, im;
+        amp_parts(v, re, im);
+        const double p = re * re + im * im;
+        if (out) out[i] = (Out)p;
+        acc += p;
+    }
+    finish_norm(acc, partials, ticket, norm);
 }
 
 __global__ void k_sum(const double *__restrict__ partials, int nb, double *__restrict__ out) {
     __shared__ double red[256];
-    double s = 0.0;
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) s += partials[i];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
+    const double s = sum_partials(partials, nb, red);
+    if (threadIdx.x == 0) *out = s;
+}
+
+// k_probs_fast: the same for float outputs of complex64 and double-float
+// states, on the FP32 pipes (split_prob, prob_split.cuh). In FP64 the two
+// conversions, the product, the multiply-add and the add of an amplitude
+// made the kernel FP64-bound on a GPU with ~2 FP64 lanes per SM (2^28
+// complex64 amplitudes: 3.05 ms against 0.47 ms of HBM time for the 3.2 GB;
+// 0.50 ms here, 0.94 of the measured copy rate).
+// Each thread takes 16 bytes at a time, PROB_U of them in flight, and sends
+// the FP64 pipe two conversions and two adds per PROB_U loads.
+constexpr int PROB_U = 4;
+constexpr int PROB_CHUNK = 256 * PROB_U;   // 16-byte loads per block and iteration
+
+template <bool DF>
+__global__ void __launch_bounds__(256, 4) k_probs_fast(const float4 *__restrict__ sv, uint64_t n_chunks,
+                                                        float *__restrict__ out, double *__restrict__ partials,
+                                                        uint32_t *ticket, double *norm) {
+    double acc = 0.0;
+    for (uint64_t c = blockIdx.x; c < n_chunks; c += gridDim.x) {
+        const uint64_t at = c * PROB_CHUNK + threadIdx.x;
+        float4 v[PROB_U];
+#pragma unroll
+        for (int u = 0; u < PROB_U; u++) v[u] = __ldcs(sv + at + 256 * u);
+        bool ok = true;
+#pragma unroll
+        for (int u = 0; u < PROB_U; u++) ok = ok && split_range<DF>(v[u]);
+        if (ok) {
+            float S = 0.0f, T = 0.0f;
+#pragma unroll
+            for (int u = 0; u < PROB_U; u++) {
+                if constexpr (DF) {
+                    const float2 p = split_prob_df(v[u]);
+                    split_add(S, T, p);
+                    if (out) out[at + 256 * u] = p.x + p.y;
+                } else {
+                    const float2 p = split_prob(v[u].x, v[u].y), q = split_prob(v[u].z, v[u].w);
+                    split_add(S, T, p);
+                    split_add(S, T, q);
+                    if (out) reinterpret_cast<float2 *>(out)[at + 256 * u] = make_float2(p.x + p.y, q.x + q.y);
+                }
+            }
+            acc += (double)S + (double)T;
+        } else {   // outside the split's range: FP64
+#pragma unroll
+            for (int u = 0; u < PROB_U; u++) {
+                if constexpr (DF) {
+                    double re, im;
+                    amp_parts(v[u], re, im);
+                    const double p = re * re + im * im;
+                    if (out) out[at + 256 * u] = (float)p;
+                    acc += p;
+                } else {
+                    const double p = (double)v[u].x * v[u].x + (double)v[u].y * v[u].y;
+                    const double q = (double)v[u].z * v[u].z + (double)v[u].w * v[u].w;
+                    if (out) reinterpret_cast<float2 *>(out)[at + 256 * u] = make_float2((float)p, (float)q);
+                    acc += p;
+                    acc += q;
+                }
+            }
+        }
     }
-    if (threadIdx.x == 0) *out = red[0];
+    finish_norm(acc, partials, ticket, norm);
+}
+
+// The FP32 kernels take whole chunks of 16-byte loads: at least one chunk,
+// and an output of pairs aligned to 8 bytes (one float per load otherwise).
+static bool fast_prob_ok(const void *sv, uint64_t N, bool fp64, bool df, int out_fp64, const void *out) {
+    const uint64_t loads = df ? N : N / 2;
+    return (!fp64 || df) && !(out && out_fp64) && loads >= (uint64_t)PROB_CHUNK &&
+           (reinterpret_cast<uintptr_t>(sv) & 15) == 0 && (df || (reinterpret_cast<uintptr_t>(out) & 7) == 0);
+}
+static int fast_grid(uint64_t n_chunks, int nblocks) {
+    const uint64_t cap = (uint64_t)(nblocks < 152 * 4 ? nblocks : 152 * 4);   // one wave of resident blocks
+    return (int)(n_chunks < cap ? n_chunks : cap);
 }
 
 cudaError_t launch_probs(bool fp64, const void *sv, int n, void *out, int out_fp64, double *partials,
-                         int nblocks, double *d_norm, cudaStream_t st, bool df) {
+                         int nblocks, double *d_norm, cudaStream_t st, bool df, uint32_t *ticket) {
     const uint64_t N = 1ull << n;
     uint64_t need = (N + 255) / 256;
     int nb = (int)(need < (uint64_t)nblocks ? need : (uint64_t)nblocks);
     if (nb < 1) nb = 1;
-    if (df) {
-        if (out_fp64) k_probs<float4, double><<<nb, 256, 0, st>>>((const float4 *)sv, N, (double *)out, partials);
-        else k_probs<float4, float><<<nb, 256, 0, st>>>((const float4 *)sv, N, (float *)out, partials);
+    if (fast_prob_ok(sv, N, fp64, df, out_fp64, out)) {
+        const uint64_t chunks = (df ? N : N / 2) / PROB_CHUNK;
+        nb = fast_grid(chunks, nblocks);
+        if (df) k_probs_fast<true><<<nb, 256, 0, st>>>((const float4 *)sv, chunks, (float *)out, partials, ticket, d_norm);
+        else k_probs_fast<false><<<nb, 256, 0, st>>>((const float4 *)sv, chunks, (float *)out, partials, ticket, d_norm);
+    } else if (df) {
+        if (out_fp64) k_probs<float4, double><<<nb, 256, 0, st>>>((const float4 *)sv, N, (double *)out, partials, ticket, d_norm);
+        else k_probs<float4, float><<<nb, 256, 0, st>>>((const float4 *)sv, N, (float *)out, partials, ticket, d_norm);
     } else if (!fp64) {
-        if (out_fp64) k_probs<float2, double><<<nb, 256, 0, st>>>((const float2 *)sv, N, (double *)out, partials);
-        else k_probs<float2, float><<<nb, 256, 0, st>>>((const float2 *)sv, N, (float *)out, partials);
+        if (out_fp64) k_probs<float2, double><<<nb, 256, 0, st>>>((const float2 *)sv, N, (double *)out, partials, ticket, d_norm);
+        else k_probs<float2, float><<<nb, 256, 0, st>>>((const float2 *)sv, N, (float *)out, partials, ticket, d_norm);
     } else {
-        if (out_fp64) k_probs<double2, double><<<nb, 256, 0, st>>>((const double2 *)sv, N, (double *)out, partials);
-        else k_probs<double2, float><<<nb, 256, 0, st>>>((const double2 *)sv, N, (float *)out, partials);
+        if (out_fp64) k_probs<double2, double><<<nb, 256, 0, st>>>((const double2 *)sv, N, (double *)out, partials, ticket, d_norm);
+        else k_probs<double2, float><<<nb, 256, 0, st>>>((const double2 *)sv, N, (float *)out, partials, ticket, d_norm);
     }
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || ticket) return e;
     k_sum<<<1, 256, 0, st>>>(partials, nb, d_norm);
     return cudaGetLastError();
 }
 
 // Summary of the probability distribution without writing it: per block the
 // FP64 sum of |a_x|^2 and the largest |a_x|^2 with its index (ties to the
-// smaller index), then one block combines them.
+// smaller index); the block that ends last combines them.
 __device__ __forceinline__ void better(double &p, uint64_t &i, double q, uint64_t j) {
     if (q > p || (q == p && j < i)) {
         p = q;
@@ -437,22 +549,13 @@ __device__ __forceinline__ void better(double &p, uint64_t &i, double q, uint64_
     }
 }
 
+// out[0] = sum |a|^2, out[1] = |a_0|^2, out[2] = max |a_x|^2, out[3] = its index (bits)
 template <typename E>
-__global__ void __launch_bounds__(256) k_summary(const E *__restrict__ sv, uint64_t N,
-                                                  double *__restrict__ sums, double *__restrict__ maxs,
-                                                  uint64_t *__restrict__ idxs) {
-    __shared__ double rs[8], rm[8];
-    __shared__ uint64_t ri[8];
-    double acc = 0.0, best = -1.0;
-    uint64_t bi = ~0ull;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (uint64_t)gridDim.x * blockDim.x) {
-        const E v = __ldcs(sv + i);
-        double re, im;
-        amp_parts(v, re, im);
-        const double p = re * re + im * im;
-        acc += p;
-        better(best, bi, p, i);
-    }
+__device__ __forceinline__ void finish_summary(const E *sv, double acc, double best, uint64_t bi, double *sums,
+                                               double *maxs, uint64_t *idxs, uint32_t *ticket, double *out) {
+    __shared__ double rs[256], rm[256];
+    __shared__ uint64_t ri[256];
+    __shared__ uint32_t flag;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -477,20 +580,12 @@ __global__ void __launch_bounds__(256) k_summary(const E *__restrict__ sv, uint6
         maxs[blockIdx.x] = m;
         idxs[blockIdx.x] = mi;
     }
-}
-
-// out[0] = sum |a|^2, out[1] = |a_0|^2, out[2] = max |a_x|^2, out[3] = its index (bits)
-template <typename E>
-__global__ void k_summary_final(const E *__restrict__ sv, const double *__restrict__ sums,
-                                const double *__restrict__ maxs, const uint64_t *__restrict__ idxs, int nb,
-                                double *__restrict__ out) {
-    __shared__ double rs[256], rm[256];
-    __shared__ uint64_t ri[256];
+    if (!last_block(ticket, flag)) return;
     double s = 0.0, m = -1.0;
     uint64_t mi = ~0ull;
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) {
-        s += sums[i];
-        better(m, mi, maxs[i], idxs[i]);
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
+        s += __ldcg(sums + i);
+        better(m, mi, __ldcg(maxs + i), __ldcg(reinterpret_cast<const unsigned long long *>(idxs) + i));
     }
     rs[threadIdx.x] = s;
     rm[threadIdx.x] = m;
@@ -513,23 +608,112 @@ __global__ void k_summary_final(const E *__restrict__ sv, const double *__restri
     }
 }
 
+template <typename E>
+__global__ void __launch_bounds__(256) k_summary(const E *__restrict__ sv, uint64_t N,
+                                                  double *__restrict__ sums, double *__restrict__ maxs,
+                                                  uint64_t *__restrict__ idxs, uint32_t *ticket, double *out) {
+    double acc = 0.0, best = -1.0;
+    uint64_t bi = ~0ull;
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (uint64_t)gridDim.x * blockDim.x) {
+        const E v = __ldcs(sv + i);
+        double re, im;
+        amp_parts(v, re, im);
+        const double p = re * re + im * im;
+        acc += p;
+        better(best, bi, p, i);
+    }
+    finish_summary(sv, acc, best, bi, sums, maxs, idxs, ticket, out);
+}
+
+// The norm on the FP32 pipes as in k_probs_fast. The maximum stays exact: a
+// group of loads goes through the FP64 comparison only if one of its FP32
+// probabilities (within 2^-23 of the true ones) comes within 2^-21 of the
+// warp's largest so far, so nothing that could win or tie is passed over.
+// For random states that is a few groups per warp (2^28 complex64
+// amplitudes: 3.57 ms with every amplitude in FP64, against 0.32 ms of HBM
+// time; 2^25: 0.48 ms, here 0.16 ms); for a state of equal probabilities it is every group, as before.
+template <bool DF>
+__global__ void __launch_bounds__(256, 4) k_summary_fast(const float4 *__restrict__ sv, uint64_t n_chunks,
+                                                          double *__restrict__ sums, double *__restrict__ maxs,
+                                                          uint64_t *__restrict__ idxs, uint32_t *ticket,
+                                                          double *out) {
+    double acc = 0.0, best = -1.0;
+    uint64_t bi = ~0ull;
+    float least = -1.0f;   // below this a probability cannot win (warp-wide)
+    for (uint64_t c = blockIdx.x; c < n_chunks; c += gridDim.x) {
+        const uint64_t at = c * PROB_CHUNK + threadIdx.x;
+        float4 v[PROB_U];
+#pragma unroll
+        for (int u = 0; u < PROB_U; u++) v[u] = __ldcs(sv + at + 256 * u);
+        bool ok = true;
+#pragma unroll
+        for (int u = 0; u < PROB_U; u++) ok = ok && split_range<DF>(v[u]);
+        float top = -1.0f;
+        if (ok) {
+            float S = 0.0f, T = 0.0f;
+#pragma unroll
+            for (int u = 0; u < PROB_U; u++) {
+                if constexpr (DF) {
+                    const float2 p = split_prob_df(v[u]);
+                    split_add(S, T, p);
+                    top = fmaxf(top, p.x + p.y);
+                } else {
+                    const float2 p = split_prob(v[u].x, v[u].y), q = split_prob(v[u].z, v[u].w);
+                    split_add(S, T, p);
+                    split_add(S, T, q);
+                    top = fmaxf(top, fmaxf(p.x, q.x));
+                }
+            }
+            acc += (double)S + (double)T;
+        }
+        if (__any_sync(0xffffffffu, !ok || top >= least)) {
+#pragma unroll
+            for (int u = 0; u < PROB_U; u++) {
+                if constexpr (DF) {
+                    double re, im;
+                    amp_parts(v[u], re, im);
+                    const double p = re * re + im * im;
+                    if (!ok) acc += p;
+                    better(best, bi, p, at + 256 * u);
+                } else {
+                    const double p = (double)v[u].x * v[u].x + (double)v[u].y * v[u].y;
+                    const double q = (double)v[u].z * v[u].z + (double)v[u].w * v[u].w;
+                    if (!ok) acc += p;
+                    if (!ok) acc += q;
+                    better(best, bi, p, 2 * (at + 256 * u));
+                    better(best, bi, q, 2 * (at + 256 * u) + 1);
+                }
+            }
+            float b = (float)best * (1.0f - 0x1p-21f);   // an infinite best stays infinite
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) b = fmaxf(b, __shfl_xor_sync(0xffffffffu, b, o));
+            least = b;
+        }
+    }
+    const typename std::conditional<DF, float4, float2>::type *amps =
+        reinterpret_cast<const typename std::conditional<DF, float4, float2>::type *>(sv);
+    finish_summary(amps, acc, best, bi, sums, maxs, idxs, ticket, out);
+}
+
 cudaError_t launch_summary(bool fp64, const void *sv, int n, double *scratch, int nblocks, double *out,
-                           cudaStream_t st, bool df) {
+                           cudaStream_t st, bool df, uint32_t *ticket) {
     const uint64_t N = 1ull << n;
     uint64_t need = (N + 255) / 256;
     int nb = (int)(need < (uint64_t)nblocks ? need : (uint64_t)nblocks);
     if (nb < 1) nb = 1;
     double *sums = scratch, *maxs = scratch + nblocks;
     uint64_t *idxs = reinterpret_cast<uint64_t *>(scratch + 2 * nblocks);
-    if (df) {
-        k_summary<float4><<<nb, 256, 0, st>>>((const float4 *)sv, N, sums, maxs, idxs);
-        k_summary_final<float4><<<1, 256, 0, st>>>((const float4 *)sv, sums, maxs, idxs, nb, out);
+    if (fast_prob_ok(sv, N, fp64, df, 0, nullptr)) {
+        const uint64_t chunks = (df ? N : N / 2) / PROB_CHUNK;
+        nb = fast_grid(chunks, nblocks);
+        if (df) k_summary_fast<true><<<nb, 256, 0, st>>>((const float4 *)sv, chunks, sums, maxs, idxs, ticket, out);
+        else k_summary_fast<false><<<nb, 256, 0, st>>>((const float4 *)sv, chunks, sums, maxs, idxs, ticket, out);
+    } else if (df) {
+        k_summary<float4><<<nb, 256, 0, st>>>((const float4 *)sv, N, sums, maxs, idxs, ticket, out);
     } else if (fp64) {
-        k_summary<double2><<<nb, 256, 0, st>>>((const double2 *)sv, N, sums, maxs, idxs);
-        k_summary_final<double2><<<1, 256, 0, st>>>((const double2 *)sv, sums, maxs, idxs, nb, out);
+        k_summary<double2><<<nb, 256, 0, st>>>((const double2 *)sv, N, sums, maxs, idxs, ticket, out);
     } else {
-        k_summary<float2><<<nb, 256, 0, st>>>((const float2 *)sv, N, sums, maxs, idxs);
-        k_summary_final<float2><<<1, 256, 0, st>>>((const float2 *)sv, sums, maxs, idxs, nb, out);
+        k_summary<float2><<<nb, 256, 0, st>>>((const float2 *)sv, N, sums, maxs, idxs, ticket, out);
     }
     return cudaGetLastError();
 }

@@ -22,15 +22,18 @@ cudaError_t launch_gate1(bool fp64, void *sv, int n, int q, const double *m, cud
 cudaError_t launch_gate2(bool fp64, void *sv, int n, int q0, int q1, const double *m, cudaStream_t st);
 
 // p[x] = |a_x|^2 (float or double out, may be null) and FP64 block partial sums
-// of the norm reduced into *d_norm. partials has nblocks doubles.
+// of the norm reduced into *d_norm. partials has nblocks doubles, of which at
+// most nblocks are used. ticket: a zeroed device word, left zero, that lets
+// the last block add the partials up; null takes a second launch for it
+// (callers whose scratch several calls may share).
 cudaError_t launch_probs(bool fp64, const void *sv, int n, void *out, int out_fp64, double *partials,
-                         int nblocks, double *d_norm, cudaStream_t st, bool df = false);
+                         int nblocks, double *d_norm, cudaStream_t st, bool df, uint32_t *ticket);
 
 // Norm, |a_0|^2 and the largest |a_x|^2 with its index (ties to the smaller
 // index), FP64, without a probability vector: scratch holds 3 * nblocks
-// doubles, out 4 (out[3] holds the index's bits).
+// doubles, out 4 (out[3] holds the index's bits); ticket as above, required.
 cudaError_t launch_summary(bool fp64, const void *sv, int n, double *scratch, int nblocks, double *out,
-                           cudaStream_t st, bool df = false);
+                           cudaStream_t st, bool df, uint32_t *ticket);
 // FMA throughput of the CUDA cores in FP64 (fp64) or FP32, in FLOP/s (best of
 // a few timed launches over every SM; synchronises the stream).
 cudaError_t alu_probe(bool fp64, double *flops_per_s, cudaStream_t st);

@@ -91,7 +91,7 @@ extern "C" sv_status sv_probs_noalloc(const void *dev_state, int n_qubits, sv_pr
     double *partials = static_cast<double *>(scratch);
     double *norm = dev_norm ? dev_norm : partials + SV_NOALLOC_MAX_BLOCKS;
     e = hisv::launch_probs(prec != SV_C64, dev_state, n_qubits, dev_probs, out_fp64, partials, n_blocks, norm,
-                           reinterpret_cast<cudaStream_t>(stream), prec == SV_C128DF);
+                           reinterpret_cast<cudaStream_t>(stream), prec == SV_C128DF, nullptr);
     if (e != cudaSuccess) {
         return noalloc_fail(SV_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
     }
