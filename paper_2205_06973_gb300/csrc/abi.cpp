@@ -17,6 +17,7 @@
 #include "kernels.hpp"
 #include "partition.hpp"
 #include "planner.hpp"
+#include "small.hpp"
 
 using namespace hisv;
 
@@ -78,6 +79,50 @@ const char *sv_last_error(void) { return g_err.c_str(); }
 const char *sv_version(void) { return "hisvsim-gb300 0.1 (sm_103a)"; }
 
 }  // extern "C"
+
+// The gate records of a small circuit in the kernel's precision.
+template <typename Real> static std::vector<SmallGate<Real>> small_gates(const sv_plan *p) {
+    std::vector<SmallGate<Real>> out(p->gates.size());
+    for (size_t i = 0; i < out.size(); i++) {
+        const GateRef &g = p->gates[i];
+        SmallGate<Real> &r = out[i];
+        std::memset(&r, 0, sizeof(r));
+        r.q0 = g.q[0];
+        r.q1 = g.q[1];
+        double m[8] = {0};
+        switch (g.kind) {
+        case SV_GATE_CX: r.kind = SMALL_CX; break;
+        case SV_GATE_SWAP: r.kind = SMALL_SWAP; break;
+        case SV_GATE_CZ: case SV_GATE_CP:
+            r.kind = SMALL_PHASE;
+            m[0] = g.kind == SV_GATE_CZ ? -1.0 : std::cos(g.theta);
+            m[1] = g.kind == SV_GATE_CZ ? 0.0 : std::sin(g.theta);
+            break;
+        default: {
+            double u[8];
+            gate_matrix_1q(g.kind, g.theta, u);
+            const bool diag = u[2] == 0 && u[3] == 0 && u[4] == 0 && u[5] == 0;
+            const bool real = u[1] == 0 && u[3] == 0 && u[5] == 0 && u[7] == 0;
+            if (g.kind == SV_GATE_RX) {
+                r.kind = SMALL_RX;
+                m[0] = u[0];
+                m[1] = -u[3];
+            } else if (real) {
+                r.kind = SMALL_REAL;
+                for (int j = 0; j < 4; j++) m[j] = u[2 * j];
+            } else if (diag) {
+                r.kind = SMALL_DIAG;
+                m[0] = u[0]; m[1] = u[1]; m[2] = u[6]; m[3] = u[7];
+            } else {
+                r.kind = SMALL_GENERAL;
+                std::memcpy(m, u, sizeof(m));
+            }
+        }
+        }
+        for (int j = 0; j < 8; j++) r.m[j] = (Real)m[j];
+    }
+    return out;
+}
 
 static sv_status create_state(int n, sv_precision prec, void *dev_buf, size_t dev_buf_bytes, void *stream, bool init,
                               sv_state **out) {
@@ -482,6 +527,7 @@ sv_status sv_plan_destroy(sv_plan *p) {
         dev_free(kv.second.d_coefs, 0);
         dev_free(kv.second.d_aimg, 0);
         dev_free(kv.second.d_pimg, 0);
+        dev_free(kv.second.d_small, 0);
     }
     cudaSetDevice(cur);
     delete p;
@@ -579,6 +625,55 @@ static sv_status apply_gatewise(sv_state *s, sv_plan *p) {
     return SV_OK;
 }
 
+// A circuit on fewer than 10 qubits in one launch; the gate records are
+// uploaded at the plan's first apply for the precision and device and kept in
+// the plan. Where that cannot be done now (no memory, or the stream is being
+// captured, which an upload with its wait would break) the circuit runs gate
+// by gate.
+static sv_status apply_small(sv_state *s, sv_plan *p) {
+    if (p->gates.empty()) return SV_OK;
+    const bool fp64 = is_fp64(s);
+    const void *prog = nullptr;
+    {
+        std::lock_guard<std::recursive_mutex> lk(p->mu);
+        auto key = std::make_tuple(s->dev, fp64, 0, 0);   // tile 0: no part program has it
+        auto it = p->dev_progs.find(key);
+        if (it == p->dev_progs.end()) {
+            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+            cudaError_t e = cudaStreamIsCapturing(s->stream, &cap);
+            if (e != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+                cudaGetLastError();
+                return apply_gatewise(s, p);
+            }
+            std::vector<SmallGate<float>> f;
+            std::vector<SmallGate<double>> d;
+            if (fp64) d = small_gates<double>(p);
+            else f = small_gates<float>(p);
+            const void *src = fp64 ? static_cast<const void *>(d.data()) : f.data();
+            const size_t bytes = p->gates.size() * (fp64 ? sizeof(SmallGate<double>) : sizeof(SmallGate<float>));
+            DevProgram dp;
+            dp.dev = s->dev;
+            e = dev_alloc(&dp.d_small, bytes, s->stream);
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                return apply_gatewise(s, p);
+            }
+            e = cudaMemcpyAsync(dp.d_small, src, bytes, cudaMemcpyHostToDevice, s->stream);
+            // shared by every state that applies the plan, on any stream:
+            // complete before it is published
+            if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+            if (e != cudaSuccess) {
+                dev_free(dp.d_small, s->stream);
+                return fail(SV_ERR_CUDA, std::string("program upload: ") + cudaGetErrorString(e));
+            }
+            it = p->dev_progs.emplace(key, dp).first;
+        }
+        prog = it->second.d_small;
+    }
+    CUDA_TRY(launch_small(fp64, s->buf, s->n, prog, (uint32_t)p->gates.size(), s->stream));
+    return SV_OK;
+}
+
 sv_status sv_apply_parts(sv_state *s, sv_plan *p, uint32_t flags) {
     if (!s || !p) return fail(SV_ERR_ARG, "NULL argument");
     if (p->n != s->n) return fail(SV_ERR_ARG, "plan and state qubit counts differ");
@@ -588,8 +683,10 @@ sv_status sv_apply_parts(sv_state *s, sv_plan *p, uint32_t flags) {
             return fail(SV_ERR_ARG, "a double-float state runs parts of a partitioned plan (n >= 10) only");
         flags = (flags | SV_FLAG_SPECIALISE) & ~SV_FLAG_TC_DENSE;
     }
-    if ((flags & SV_FLAG_GATEWISE) || p->method == SV_PART_NONE || s->n < part_tmin()) {
+    if ((flags & SV_FLAG_GATEWISE) || p->method == SV_PART_NONE) {
         st = apply_gatewise(s, p);
+    } else if (s->n < part_tmin()) {
+        st = apply_small(s, p);
     } else {
         const bool fp64 = is_fp64(s);
         const int t = s->tile ? s->tile : default_tile(fp64, p->max_part);

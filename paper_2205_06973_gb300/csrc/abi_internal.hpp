@@ -38,6 +38,7 @@ struct DevProgram {
     void *d_coefs = nullptr;
     uint8_t *d_aimg = nullptr;      // R images of the dense parts
     uint8_t *d_pimg = nullptr;      // R images of the dense pairs (two per pass)
+    void *d_small = nullptr;        // gate records of a circuit on fewer than 10 qubits
 };
 
 struct sv_state {
