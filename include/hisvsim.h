@@ -277,7 +277,9 @@ sv_status sv_measure_summary(sv_state *s, double *norm_out, double *p0_out, uint
  * CUDA graph captures once and replays (the batched workload: thousands of
  * uneven circuits of 10..30 qubits). States are complex64, contiguous in one
  * device buffer in circuit order (circuit i starts after the 2^n_j amplitudes
- * of every j < i). Each plan's parts run on 2^9-amplitude tiles, one warp
+ * of every j < i). A circuit of at most 12 qubits runs on one CTA, its state
+ * on chip from the first gate to the last. A larger one's parts run on
+ * 2^9-amplitude tiles, one warp
  * per tile; parts of one circuit run in order (a device work list in wave
  * order with per-circuit tile counters and bounded waits), parts of different
  * circuits overlap. Parts are limited to 9 qubits (plans with k <= 9).
@@ -288,7 +290,8 @@ sv_status sv_measure_summary(sv_state *s, double *norm_out, double *p0_out, uint
  * sv_batch_set_plan  plan for circuit i (qubit count must match); the plan
  *                  must stay alive until the next sv_batch_run has returned.
  * sv_batch_config  warps per CTA (1..8) and tiles per work item (1..4096);
- *                  0 keeps the default (8, 16). Changing plans or the
+ *                  0 keeps the default (8, and up to 16 by the batch's
+ *                  size). Changing plans or the
  *                  configuration rebuilds the work list and the graph.
  * sv_batch_run     apply every circuit once to its current state; the first
  *                  run builds the work list, uploads it and captures the

@@ -21,11 +21,11 @@ LIB = os.path.join(HERE, "libhisvsim.so")
 INCLUDE = os.path.join(ROOT, "include")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["kernels.cu", "dense.cu", "dense_pair.cu", "dense_batch.cu", "noalloc.cu", "small.cu", "batch.cu", "abi.cpp", "batch_abi.cpp",
-           "partition.cpp", "planner.cpp", "qasm.cpp", "jit.cpp"]
+SOURCES = ["kernels.cu", "part_f32.cu", "part_f64.cu", "dense.cu", "dense_pair.cu", "dense_batch.cu", "noalloc.cu", "small.cu", "batch.cu", "abi.cpp", "batch_abi.cpp",
+           "partition.cpp", "planner.cpp", "interp.cpp", "qasm.cpp", "jit.cpp"]
 # headers handed to the run-time compiler (NVRTC) by jit.cpp, embedded as
 # string literals: name in the generated include file -> source header
-JIT_HEADERS = (("kJitOpsCore", "ops_core.cuh"), ("kJitPrelude", "jit_prelude.cuh"))
+JIT_HEADERS = (("kJitOpsCore", "ops_core.cuh"), ("kJitPacked", "packed.cuh"), ("kJitPrelude", "jit_prelude.cuh"))
 JIT_INC = os.path.join(BUILD, "jit_sources.inc")
 
 
@@ -66,7 +66,7 @@ def _compile(src: str, verbose: bool) -> str:
 def _write_jit_sources():
     """The run-time compiler's headers as C++ raw string literals (rewritten
     only when their text changes, so the dependency check stays exact)."""
-    text = "// generated by build.py from csrc/ops_core.cuh and csrc/jit_prelude.cuh\n"
+    text = "// generated by build.py from csrc/ops_core.cuh, csrc/packed.cuh and csrc/jit_prelude.cuh\n"
     for name, hdr in JIT_HEADERS:
         with open(os.path.join(CSRC, hdr)) as f:
             body = f.read()

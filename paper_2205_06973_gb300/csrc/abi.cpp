@@ -80,6 +80,24 @@ const char *sv_version(void) { return "hisvsim-gb300 0.1 (sm_103a)"; }
 
 }  // extern "C"
 
+// Copy v to new device memory (stream-ordered).
+template <typename V> static cudaError_t upload_vec(void **d, const V &v, cudaStream_t st) {
+    if (v.empty()) return cudaSuccess;
+    const size_t bytes = v.size() * sizeof(v[0]);
+    cudaError_t e = dev_alloc(d, bytes, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(*d, v.data(), bytes, cudaMemcpyHostToDevice, st);
+    return e;
+}
+template <typename Real> static cudaError_t upload_lowered(const Program &prog, DevProgram &d, cudaStream_t st) {
+    Lowered<Real> lo;
+    lower_program<Real>(prog, lo);
+    cudaError_t e = upload_vec(reinterpret_cast<void **>(&d.d_phases), lo.phases, st);
+    if (e == cudaSuccess) e = upload_vec(&d.d_ops, lo.ops, st);
+    if (e == cudaSuccess) e = upload_vec(&d.d_table, lo.table, st);
+    cudaError_t se = cudaStreamSynchronize(st);   // lo goes out of scope
+    return e == cudaSuccess ? se : e;
+}
+
 // The gate records of a small circuit in the kernel's precision.
 template <typename Real> static std::vector<SmallGate<Real>> small_gates(const sv_plan *p) {
     std::vector<SmallGate<Real>> out(p->gates.size());
@@ -384,16 +402,24 @@ sv_status sv_plan_export(const sv_plan *p, uint32_t *pog, size_t n_gates, uint32
     return SV_OK;
 }
 
-static sv_status get_host_program(sv_plan *p, bool fp64, int t, int dense, const Program **out) {
+// Program variants of a plan (besides precision and tile): bit 0 = tensor-core
+// dense parts (complex64 only), bit 1 = two of them per pass where they fit
+// one tile, bits 4-7 = register bits per thread, and the bits below.
+constexpr int kModeWhole = 4;   // all gates as one part (the tile is the whole state)
+constexpr int kModeJit = 8;     // device program without the interpreter's op stream
+
+static sv_status get_host_program(sv_plan *p, bool fp64, int t, int mode, const Program **out) {
+    mode &= ~kModeJit;
     std::lock_guard<std::recursive_mutex> lk(p->mu);
-    auto key = std::make_tuple(fp64, t, dense);
+    auto key = std::make_tuple(fp64, t, mode);
     auto it = p->host_progs.find(key);
     if (it == p->host_progs.end()) {
         std::unique_ptr<Program> prog(new Program());
         std::string err;
-        const int R = (dense >> 4) ? (dense >> 4) : part_R(fp64);
-        if (!compile_program(p->gates, p->n, p->pog, p->n_parts, fp64, t, R, dense & 3, *prog, err,
-                             p->inner.empty() ? nullptr : &p->inner))
+        const bool whole = (mode & kModeWhole) != 0;
+        const std::vector<uint32_t> one(whole ? p->gates.size() : 0, 0u);
+        if (!compile_program(p->gates, p->n, whole ? one : p->pog, whole ? 1u : p->n_parts, fp64, t, mode >> 4,
+                             mode & 3, *prog, err, p->inner.empty() ? nullptr : &p->inner))
             return fail(SV_ERR_PARTITION, err);
         it = p->host_progs.emplace(key, std::move(prog)).first;
     }
@@ -401,12 +427,36 @@ static sv_status get_host_program(sv_plan *p, bool fp64, int t, int dense, const
     return SV_OK;
 }
 
-// Program variant of the flags: bit 0 = tensor-core dense parts (complex64
-// only), bit 1 = two of them per pass where they fit one tile, bits 4-7 =
-// register bits per thread when not the precision's default.
+// The variant of the flags on the kernels compiled for a plan (and in the
+// plan's statistics): the precision's default register bits unless given.
 static int dense_mode(uint32_t flags, bool fp64) {
     const bool tc = (flags & SV_FLAG_TC_DENSE) && !fp64;
-    return (tc ? 1 : 0) | ((tc && (flags & SV_FLAG_TC_PAIRS)) ? 2 : 0) | (int)(((flags >> 8) & 0xFu) << 4);
+    const int R = (int)((flags >> 8) & 0xFu);
+    return (tc ? 1 : 0) | ((tc && (flags & SV_FLAG_TC_PAIRS)) ? 2 : 0) | ((R ? R : part_R(fp64)) << 4);
+}
+
+// Tile and variant of an apply on the interpreter (no register bits given).
+//  * Multi-level plans keep the register bits their second level may use.
+//  * A complex64 state of at most 13 qubits on its default tile is one tile:
+//    all gates become one part, in their order, so the apply is one launch
+//    that keeps the state on chip from the first gate to the last.
+//  * A small complex128 state is cut into tiles down to 2^8 amplitudes until
+//    there are two per SM: an SM has about two FP64 lanes, so its tiles'
+//    arithmetic sets the time, and 14 qubits on 2^11 tiles keep 8 of 152 SMs
+//    busy (the 840-gate layered circuit: 1.11 ms; 2^8 tiles: see DESIGN).
+static int interp_mode(const sv_plan *p, bool fp64, uint32_t flags, int t_user, int &t) {
+    const int tc = dense_mode(flags, fp64) & 3;
+    const bool ml = !p->inner.empty();
+    const int R = ml ? part_R(fp64) : interp_R(fp64);
+    t = t_user ? t_user : default_tile(fp64, p->max_part);
+    if (t_user || ml) return tc | (R << 4);
+    if (!fp64 && p->n <= part_tmax(false) && !(tc && p->n >= DENSE_K + DENSE_COLS)) {
+        t = p->n;
+        return kModeWhole | (R << 4);
+    }
+    if (fp64)
+        while (t > 8 && t > p->max_part && (p->n <= t || (1ull << (p->n - t)) < 2 * 152)) t--;
+    return tc | (R << 4);
 }
 
 sv_status sv_plan_stats(sv_plan *p, sv_precision prec, int t, uint32_t flags, uint32_t *passes, uint32_t *phases,
@@ -434,10 +484,10 @@ sv_status sv_plan_stats(sv_plan *p, sv_precision prec, int t, uint32_t flags, ui
 
 // The plan's specialised part kernels for (precision, tile, dense mode),
 // compiled and loaded on first use.
-static sv_status get_jit_program(sv_plan *p, sv_precision prec, int t, int dense, const Program *hp,
+static sv_status get_jit_program(sv_plan *p, sv_precision prec, int t, int mode, const Program *hp,
                                  JitProgram **out) {
     std::lock_guard<std::recursive_mutex> lk(p->mu);
-    auto key = std::make_tuple((int)prec, t, dense);
+    auto key = std::make_tuple((int)prec, t, mode);
     auto it = p->jit_progs.find(key);
     if (it == p->jit_progs.end()) {
         std::unique_ptr<JitProgram> jp(new JitProgram());
@@ -524,7 +574,7 @@ sv_status sv_plan_destroy(sv_plan *p) {
         cudaSetDevice(kv.second.dev);
         dev_free(kv.second.d_phases, 0);
         dev_free(kv.second.d_ops, 0);
-        dev_free(kv.second.d_coefs, 0);
+        dev_free(kv.second.d_table, 0);
         dev_free(kv.second.d_aimg, 0);
         dev_free(kv.second.d_pimg, 0);
         dev_free(kv.second.d_small, 0);
@@ -537,60 +587,35 @@ sv_status sv_plan_destroy(sv_plan *p) {
 static void free_dev(DevProgram &d, cudaStream_t st) {
     dev_free(d.d_phases, st);
     dev_free(d.d_ops, st);
-    dev_free(d.d_coefs, st);
+    dev_free(d.d_table, st);
     dev_free(d.d_aimg, st);
     dev_free(d.d_pimg, st);
 }
 
-static sv_status get_dev_program(sv_state *s, sv_plan *p, int t, int dense, const Program **hp,
+static sv_status get_dev_program(sv_state *s, sv_plan *p, int t, int mode, const Program **hp,
                                  const DevProgram **dp) {
     std::lock_guard<std::recursive_mutex> lk(p->mu);
     const bool fp64 = is_fp64(s);
-    sv_status st = get_host_program(p, fp64, t, dense, hp);
+    sv_status st = get_host_program(p, fp64, t, mode, hp);
     if (st != SV_OK) return st;
-    auto key = std::make_tuple(s->dev, fp64, t, dense);
+    auto key = std::make_tuple(s->dev, fp64, t, mode);
     auto it = p->dev_progs.find(key);
     if (it == p->dev_progs.end()) {
         const Program &prog = **hp;
         DevProgram d;
         d.dev = s->dev;
-        const size_t nph = std::max<size_t>(1, prog.phases.size()), nop = std::max<size_t>(1, prog.ops.size());
-        const size_t ncf = std::max<size_t>(1, prog.coefs.size()), nim = std::max<size_t>(16, prog.a_img.size());
-        const size_t rsz = fp64 ? sizeof(double) : sizeof(float);
-        cudaStream_t st = s->stream;
-        cudaError_t e = dev_alloc(reinterpret_cast<void **>(&d.d_phases), sizeof(Phase) * nph, st);
-        if (e == cudaSuccess) e = dev_alloc(reinterpret_cast<void **>(&d.d_ops), sizeof(Op) * nop, st);
-        if (e == cudaSuccess) e = dev_alloc(&d.d_coefs, rsz * ncf, st);
-        if (e == cudaSuccess) e = dev_alloc(reinterpret_cast<void **>(&d.d_aimg), nim, st);
-        if (e == cudaSuccess && !prog.pair_img.empty())
-            e = dev_alloc(reinterpret_cast<void **>(&d.d_pimg), prog.pair_img.size(), st);
+        cudaError_t e = upload_vec(reinterpret_cast<void **>(&d.d_aimg), prog.a_img, s->stream);
+        if (e == cudaSuccess) e = upload_vec(reinterpret_cast<void **>(&d.d_pimg), prog.pair_img, s->stream);
+        if (e == cudaSuccess && !(mode & kModeJit))
+            e = fp64 ? upload_lowered<double>(prog, d, s->stream) : upload_lowered<float>(prog, d, s->stream);
+        // the program is shared by every state that applies the plan, on any
+        // stream: it is complete before it is published
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
         if (e != cudaSuccess) {
             cudaGetLastError();
-            free_dev(d, st);
-            return fail(SV_ERR_OOM, std::string("program upload: ") + cudaGetErrorString(e));
-        }
-        std::vector<float> cf32;
-        const void *cf = prog.coefs.data();
-        if (!fp64) {
-            cf32.assign(prog.coefs.begin(), prog.coefs.end());
-            cf = cf32.data();
-        }
-        if (!prog.phases.empty())
-            e = cudaMemcpyAsync(d.d_phases, prog.phases.data(), sizeof(Phase) * prog.phases.size(), cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess && !prog.ops.empty())
-            e = cudaMemcpyAsync(d.d_ops, prog.ops.data(), sizeof(Op) * prog.ops.size(), cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess && !prog.coefs.empty())
-            e = cudaMemcpyAsync(d.d_coefs, cf, rsz * prog.coefs.size(), cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess && !prog.a_img.empty())
-            e = cudaMemcpyAsync(d.d_aimg, prog.a_img.data(), prog.a_img.size(), cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess && !prog.pair_img.empty())
-            e = cudaMemcpyAsync(d.d_pimg, prog.pair_img.data(), prog.pair_img.size(), cudaMemcpyHostToDevice, st);
-        // the program is shared by every state that applies the plan, on any
-        // stream: it is complete before it is published (cf32 also dies here)
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) {
-            free_dev(d, st);
-            return fail(SV_ERR_CUDA, std::string("program upload: ") + cudaGetErrorString(e));
+            free_dev(d, s->stream);
+            return fail(e == cudaErrorMemoryAllocation ? SV_ERR_OOM : SV_ERR_CUDA,
+                        std::string("program upload: ") + cudaGetErrorString(e));
         }
         it = p->dev_progs.emplace(key, d).first;
     }
@@ -689,16 +714,18 @@ sv_status sv_apply_parts(sv_state *s, sv_plan *p, uint32_t flags) {
         st = apply_small(s, p);
     } else {
         const bool fp64 = is_fp64(s);
-        const int t = s->tile ? s->tile : default_tile(fp64, p->max_part);
+        const bool jit = (flags & SV_FLAG_SPECIALISE) != 0;
+        int t = s->tile ? s->tile : default_tile(fp64, p->max_part);
+        const int mode = jit ? dense_mode(flags, fp64) : interp_mode(p, fp64, flags, s->tile, t);
         const Program *hp = nullptr;
         const DevProgram *dp = nullptr;
-        st = get_dev_program(s, p, t, dense_mode(flags, fp64), &hp, &dp);
+        st = get_dev_program(s, p, t, mode | (jit ? kModeJit : 0), &hp, &dp);
         if (st != SV_OK) return st;
         JitProgram *jp = nullptr;
-        if (((flags >> 8) & 0xFu) && !(flags & SV_FLAG_SPECIALISE))
+        if (((flags >> 8) & 0xFu) && !jit)
             return fail(SV_ERR_ARG, "register bits other than the default need SV_FLAG_SPECIALISE");
-        if ((flags & SV_FLAG_SPECIALISE) && !hp->parts.empty()) {
-            st = get_jit_program(p, s->prec, t, dense_mode(flags, fp64), hp, &jp);
+        if (jit && !hp->parts.empty()) {
+            st = get_jit_program(p, s->prec, t, mode, hp, &jp);
             if (st != SV_OK) return st;
         }
         if (!hp->dense.empty() || !hp->pairs.empty()) {
@@ -723,8 +750,8 @@ sv_status sv_apply_parts(sv_state *s, sv_plan *p, uint32_t flags) {
             if (hp->kind[i] == 0 && jp)
                 e = jit_launch(*jp, j, s->buf, hp->n_tiles[j], s->stream);
             else if (hp->kind[i] == 0)
-                e = launch_part(fp64, hp->t, s->buf, hp->parts[j], dp->d_phases, dp->d_ops, dp->d_coefs,
-                                hp->n_tiles[j], s->stream);
+                e = (fp64 ? launch_part_f64 : launch_part_f32)(hp->t, hp->R, s->buf, hp->parts[j], dp->d_phases,
+                                                               dp->d_ops, dp->d_table, hp->n_tiles[j], s->stream);
             else if (hp->kind[i] == 1)
                 e = launch_dense6(s->buf, hp->dense[j], dp->d_aimg + (size_t)j * DENSE_A_BYTES, hp->dense_tiles[j],
                                   s->d_err, s->d_dnorm, didx++, s->stream);

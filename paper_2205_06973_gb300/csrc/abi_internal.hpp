@@ -10,13 +10,12 @@
 #include <vector>
 
 #include "../../include/hisvsim.h"
+#include "interp.hpp"
 #include "jit.hpp"
 #include "partition.hpp"
 #include "planner.hpp"
 
 using hisv::GateRef;
-using hisv::Op;
-using hisv::Phase;
 using hisv::Program;
 
 namespace hisv {
@@ -33,9 +32,9 @@ void set_last_error(const std::string &msg);
 
 struct DevProgram {
     int dev = -1;
-    Phase *d_phases = nullptr;
-    Op *d_ops = nullptr;
-    void *d_coefs = nullptr;
+    hisv::IPhase *d_phases = nullptr;   // the interpreter's program (interp.hpp)
+    void *d_ops = nullptr;
+    void *d_table = nullptr;
     uint8_t *d_aimg = nullptr;      // R images of the dense parts
     uint8_t *d_pimg = nullptr;      // R images of the dense pairs (two per pass)
     void *d_small = nullptr;        // gate records of a circuit on fewer than 10 qubits
@@ -70,10 +69,10 @@ struct sv_plan {
     std::vector<uint32_t> inner;        // second-level part of each gate (multi-level plans), else empty
     uint32_t n_inner = 0;
     int k2 = 0;
-    std::map<std::tuple<bool, int, int>, std::unique_ptr<Program>> host_progs;   // (fp64, t, dense)
-    std::map<std::tuple<int, bool, int, int>, DevProgram> dev_progs;             // (dev, fp64, t, dense)
+    std::map<std::tuple<bool, int, int>, std::unique_ptr<Program>> host_progs;   // (fp64, t, mode)
+    std::map<std::tuple<int, bool, int, int>, DevProgram> dev_progs;             // (dev, fp64, t, mode)
     std::vector<std::vector<double>> mats;                                 // gatewise matrices
-    std::map<std::tuple<int, int, int>, std::unique_ptr<hisv::JitProgram>> jit_progs;   // (precision, t, dense)
+    std::map<std::tuple<int, int, int>, std::unique_ptr<hisv::JitProgram>> jit_progs;   // (precision, t, mode)
     // the caches above are filled on first use; several host threads may
     // apply one plan (map nodes never move, so returned pointers stay valid)
     std::recursive_mutex mu;

@@ -51,10 +51,10 @@ __device__ __forceinline__ uint64_t deposit_b(uint64_t v, uint64_t mask) {
 
 __global__ void __launch_bounds__(256) k_batch(float2 *__restrict__ svbase, const BatchItem *__restrict__ items,
                                               uint32_t n_items, const uint64_t *__restrict__ circ_off,
-                                              const PartLaunch *__restrict__ parts, const Phase *__restrict__ phases,
-                                              const Op *__restrict__ ops, const float *__restrict__ coefs,
-                                              uint32_t *__restrict__ done, uint32_t *__restrict__ head,
-                                              int *__restrict__ err) {
+                                              const PartLaunch *__restrict__ parts,
+                                              const IPhase *__restrict__ phases, const IOp<float> *__restrict__ ops,
+                                              const float *__restrict__ table, uint32_t *__restrict__ done,
+                                              uint32_t *__restrict__ head, int *__restrict__ err) {
     extern __shared__ __align__(16) float2 bsm[];
     const int lane = threadIdx.x & 31;
     float2 *const wsm = bsm + (threadIdx.x >> 5) * (1 << BT);
@@ -110,36 +110,20 @@ __global__ void __launch_bounds__(256) k_batch(float2 *__restrict__ svbase, cons
             }
             __syncwarp();
             float tpr = 1.0f, tpi = 0.0f;
-            uint32_t s_thr = 0, s_reg[BR];
+            Slots<BR, BT - BR> S;
             for (uint32_t p = 0; p < P.n_phases; p++) {
-                const Phase ph = phases[P.phase_begin + p];
+                const IPhase *const ph = phases + P.phase_begin + p;
+                const uint2 span = __ldg(reinterpret_cast<const uint2 *>(&ph->op_begin));
                 if (p > 0) {   // transpose through the warp's shared tile
                     __syncwarp();
 #pragma unroll
-                    for (int i = 0; i < BNR; i++) {
-                        uint32_t o = s_thr;
-#pragma unroll
-                        for (int b = 0; b < BR; b++)
-                            if (i & (1 << b)) o ^= s_reg[b];
-                        wsm[o] = a[i];
-                    }
+                    for (int i = 0; i < BNR; i++) wsm[S.at(i)] = a[i];
                     __syncwarp();
                 }
-                s_thr = 0;
+                S.load(ph, lane);
 #pragma unroll
-                for (int j = 0; j < BT - BR; j++)
-                    if ((lane >> j) & 1) s_thr ^= swz<float>(ph.thr[j]);
-#pragma unroll
-                for (int b = 0; b < BR; b++) s_reg[b] = swz<float>(ph.reg[b]);
-#pragma unroll
-                for (int i = 0; i < BNR; i++) {
-                    uint32_t o = s_thr;
-#pragma unroll
-                    for (int b = 0; b < BR; b++)
-                        if (i & (1 << b)) o ^= s_reg[b];
-                    a[i] = wsm[o];
-                }
-                run_ops<float, BR>(a, ops + ph.op_begin, ph.op_count, coefs, lane, tpr, tpi, wsm, s_thr, s_reg);
+                for (int i = 0; i < BNR; i++) a[i] = wsm[S.at(i)];
+                run_ops<float, BR>(a, ops + span.x, span.y, table, lane, tpr, tpi);
             }
             if (P.flags & PL_STORE_FACTOR) {
                 const float gr = (float)P.gr, gi = (float)P.gi;
@@ -168,6 +152,73 @@ __global__ void __launch_bounds__(256) k_batch(float2 *__restrict__ svbase, cons
             red_release_add(done + I.circuit, I.tile_count);
         }
         __syncwarp();
+    }
+}
+
+// Whole circuits of T qubits, one CTA each: the state stays in shared memory
+// and registers from the first gate to the last (the planner's program of the
+// circuit as one part). On 2^9-amplitude tiles such a circuit is a chain of
+// parts of a few tiles each, every part a trip through L2 and the work queue
+// with little for the other warps to do: 45 parameterised circuits of 10 to
+// 12 qubits took 3.2 ms.
+template <int T>
+__global__ void __launch_bounds__(1 << (T - BR))
+k_batch_whole(float2 *__restrict__ svbase, const BatchWhole *__restrict__ circuits,
+              const PartLaunch *__restrict__ parts, const IPhase *__restrict__ phases,
+              const IOp<float> *__restrict__ ops, const float *__restrict__ table) {
+    constexpr int TB = T - BR;
+    extern __shared__ __align__(16) float2 bsm[];
+    const uint32_t tid = threadIdx.x;
+    const BatchWhole W = circuits[blockIdx.x];
+    const PartLaunch &P = parts[W.part];
+    float2 *const sv = svbase + W.sv_off;
+    uint32_t s_cthr = 0;
+#pragma unroll
+    for (int j = 0; j < TB; j++)
+        if ((tid >> j) & 1) s_cthr ^= swz<float>(j);
+#pragma unroll
+    for (int i = 0; i < BNR; i++) {
+        uint32_t so = s_cthr;
+#pragma unroll
+        for (int b = 0; b < BR; b++)
+            if (i & (1 << b)) so ^= swz<float>(TB + b);
+        bsm[so] = __ldcg(sv + (tid | ((uint32_t)i << TB)));
+    }
+    __syncthreads();
+    float2 a[BNR];
+    float tpr = 1.0f, tpi = 0.0f;
+    Slots<BR, TB> S;
+    for (uint32_t p = 0; p < P.n_phases; p++) {
+        const IPhase *const ph = phases + P.phase_begin + p;
+        const uint2 span = __ldg(reinterpret_cast<const uint2 *>(&ph->op_begin));
+        if (p > 0) {
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < BNR; i++) bsm[S.at(i)] = a[i];
+            __syncthreads();
+        }
+        S.load(ph, tid);
+#pragma unroll
+        for (int i = 0; i < BNR; i++) a[i] = bsm[S.at(i)];
+        run_ops<float, BR>(a, ops + span.x, span.y, table, tid, tpr, tpi);
+    }
+    if (P.flags & PL_STORE_FACTOR) {
+        const float gr = (float)P.gr, gi = (float)P.gi;
+        const float fr = gr * tpr - gi * tpi, fi = gr * tpi + gi * tpr;
+#pragma unroll
+        for (int i = 0; i < BNR; i++) cmul_in(a[i], fr, fi);
+    }
+    uint32_t toff = 0;
+#pragma unroll
+    for (int j = 0; j < TB; j++)
+        if ((tid >> j) & 1) toff |= 1u << P.store_thr_q[j];
+#pragma unroll
+    for (int i = 0; i < BNR; i++) {
+        uint32_t off = toff;
+#pragma unroll
+        for (int b = 0; b < BR; b++)
+            if (i & (1 << b)) off |= 1u << P.store_reg_q[b];
+        __stcg(sv + off, a[i]);
     }
 }
 
@@ -280,7 +331,19 @@ cudaError_t batch_prepare(int warps_per_cta, int *n_ctas) {
 cudaError_t launch_batch(const BatchLaunch &B, int warps_per_cta, int n_ctas, cudaStream_t st) {
     const size_t smem = (size_t)warps_per_cta * (1u << BT) * sizeof(float2);
     k_batch<<<n_ctas, warps_per_cta * 32, smem, st>>>(B.svbase, B.items, B.n_items, B.circ_off, B.parts, B.phases,
-                                                      B.ops, B.coefs, B.done, B.head, B.err);
+                                                      B.ops, B.table, B.done, B.head, B.err);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_batch_whole(int t, const BatchLaunch &B, const BatchWhole *circuits, uint32_t n, cudaStream_t st) {
+    const size_t smem = sizeof(float2) << t;
+    const unsigned threads = 1u << (t - BR);
+    switch (t) {
+    case 10: k_batch_whole<10><<<n, threads, smem, st>>>(B.svbase, circuits, B.parts, B.phases, B.ops, B.table); break;
+    case 11: k_batch_whole<11><<<n, threads, smem, st>>>(B.svbase, circuits, B.parts, B.phases, B.ops, B.table); break;
+    case 12: k_batch_whole<12><<<n, threads, smem, st>>>(B.svbase, circuits, B.parts, B.phases, B.ops, B.table); break;
+    default: return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
 }
 

@@ -4,6 +4,7 @@
 
 #include <cstdint>
 
+#include "interp.hpp"
 #include "program.hpp"
 
 namespace hisv {
@@ -19,15 +20,22 @@ struct BatchItem {
     uint32_t wait;
 };
 
+// A circuit that one CTA runs from start to end (its program is one part).
+struct BatchWhole {
+    uint64_t sv_off;             // first amplitude of its state
+    uint32_t part;
+    uint32_t pad;
+};
+
 struct BatchLaunch {
     float2 *svbase;              // concatenated complex64 states
     const BatchItem *items;
     uint32_t n_items;
     const uint64_t *circ_off;    // first amplitude of each circuit's state
     const PartLaunch *parts;     // all circuits' parts (tile of 2^9 amplitudes)
-    const Phase *phases;
-    const Op *ops;
-    const float *coefs;
+    const IPhase *phases;        // lowered programs (interp.hpp)
+    const IOp<float> *ops;
+    const float *table;
     uint32_t *done;              // per-circuit finished-tile counters (zeroed per run)
     uint32_t *head;              // queue ticket (zeroed per run)
     int *err;                    // bounded-wait failure flag
@@ -36,11 +44,16 @@ struct BatchLaunch {
 constexpr int BATCH_TILE_QUBITS = 9;   // one warp's tile: 32 lanes x 16 amplitudes
 constexpr int BATCH_REG_BITS = 4;      // tile qubits held in registers (16 amplitudes per lane)
 constexpr int BATCH_MIN_QUBITS = 10;
+// Circuits of at most this many qubits run on one CTA each: a 12-qubit state
+// is 32 KiB of shared memory for 256 threads, so several share an SM.
+constexpr int BATCH_WHOLE_QUBITS = 12;
 
 // Raise the shared-memory limit and return the persistent grid size (CTAs
 // resident on all SMs) for a CTA of warps_per_cta warps.
 cudaError_t batch_prepare(int warps_per_cta, int *n_ctas);
 cudaError_t launch_batch(const BatchLaunch &B, int warps_per_cta, int n_ctas, cudaStream_t st);
+// n circuits of t qubits (BATCH_MIN_QUBITS..BATCH_WHOLE_QUBITS), one CTA each.
+cudaError_t launch_batch_whole(int t, const BatchLaunch &B, const BatchWhole *circuits, uint32_t n, cudaStream_t st);
 // Probabilities of all states (out, may be null) and, with norms, each
 // circuit's norm: partials then holds total / 2^BATCH_MIN_QUBITS doubles.
 cudaError_t launch_batch_probs(float2 *svbase, uint64_t total, const uint64_t *circ_off, const uint32_t *circ_n,

@@ -39,8 +39,10 @@ struct sv_batch {
     cudaStream_t prep = nullptr;         // private: allocations, uploads and the graph capture, so that
                                          // building a batch never enqueues on (or captures) a stream that
                                          // another thread uses for earlier batches
+    cudaStream_t side = nullptr;         // second branch of the capture, with its fork and join
+    cudaEvent_t fork = nullptr, join = nullptr;
     int warps = 8;                       // warps per CTA
-    int chunk = 16;                      // tiles per queue item
+    int chunk = 0;                       // tiles per queue item (0 = by the batch's size)
     bool hold_last = false;              // testing: the last item waits for tiles that never complete
     int dense_min = 0;                   // circuits of >= this many qubits (and >= 13) with parts of <= 6
                                          // qubits run on the batched tensor-core kernel; 0 = off
@@ -80,6 +82,13 @@ static void drop_program(sv_batch *b) {
     b->built = false;
 }
 
+static void drop_streams(sv_batch *b) {
+    if (b->prep) cudaStreamDestroy(b->prep);
+    if (b->side) cudaStreamDestroy(b->side);
+    if (b->fork) cudaEventDestroy(b->fork);
+    if (b->join) cudaEventDestroy(b->join);
+}
+
 extern "C" {
 
 sv_status sv_batch_create(uint32_t n_circuits, const int *n_qubits, void *stream, sv_batch **out) {
@@ -105,7 +114,11 @@ sv_status sv_batch_create(uint32_t n_circuits, const int *n_qubits, void *stream
     }
     {
         cudaError_t pe = cudaStreamCreateWithFlags(&b->prep, cudaStreamNonBlocking);
+        if (pe == cudaSuccess) pe = cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking);
+        if (pe == cudaSuccess) pe = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
+        if (pe == cudaSuccess) pe = cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming);
         if (pe != cudaSuccess) {
+            drop_streams(b.get());
             if (b->own_stream) cudaStreamDestroy(b->stream);
             return bfail(SV_ERR_CUDA, std::string("batch stream: ") + cudaGetErrorString(pe));
         }
@@ -133,7 +146,7 @@ sv_status sv_batch_create(uint32_t n_circuits, const int *n_qubits, void *stream
         dev_free(b->sv, st); dev_free(b->d_off, st); dev_free(b->d_nq, st); dev_free(b->d_done, st);
         dev_free(b->d_err, st); dev_free(b->d_norms, st);
         cudaStreamSynchronize(st);
-        cudaStreamDestroy(b->prep);
+        drop_streams(b.get());
         if (b->own_stream) cudaStreamDestroy(b->stream);
         return bfail(e == cudaErrorMemoryAllocation ? SV_ERR_OOM : SV_ERR_CUDA,
                      std::string("batch allocation: ") + cudaGetErrorString(e));
@@ -158,7 +171,7 @@ sv_status sv_batch_config(sv_batch *b, int warps_per_cta, int tiles_per_item) {
     if (warps_per_cta < 0 || warps_per_cta > 8 || tiles_per_item < 0 || tiles_per_item > 4096)
         return bfail(SV_ERR_ARG, "warps_per_cta in [1, 8], tiles_per_item in [1, 4096] (0 = default)");
     b->warps = warps_per_cta ? warps_per_cta : 8;
-    b->chunk = tiles_per_item ? tiles_per_item : 16;
+    b->chunk = tiles_per_item;
     drop_program(b);
     return SV_OK;
 }
@@ -254,6 +267,9 @@ static sv_status build_program(sv_batch *b) {
     int dev = 0;
     BCUDA(cudaGetDevice(&dev));
     std::vector<Program> gl(b->n);                 // gate-list programs (circuits not on the dense kernel)
+    std::vector<Lowered<float>> lowered(b->n);
+    // the failure test holds back a work item, so it keeps the work queue
+    auto whole = [&](uint32_t c) { return !D.dense[c] && b->nq[c] <= BATCH_WHOLE_QUBITS && !b->hold_last; };
     std::vector<DenseBatchPart> dparts(D.n_parts);
     std::vector<std::string> errs(b->n);
     std::atomic<uint32_t> next(0);
@@ -262,9 +278,15 @@ static sv_status build_program(sv_batch *b) {
         for (uint32_t c = next++; c < b->n; c = next++) {
             sv_plan *p = b->plans[c];
             if (!D.dense[c]) {
-                if (!compile_program(p->gates, p->n, p->pog, p->n_parts, false, BATCH_TILE_QUBITS, BATCH_REG_BITS, 0,
-                                     gl[c], errs[c]) && errs[c].empty())
-                    errs[c] = "compile failed";
+                // a circuit that one CTA holds: all gates as one part
+                const bool w = whole(c);
+                const std::vector<uint32_t> one(w ? p->gates.size() : 0, 0u);
+                if (!compile_program(p->gates, p->n, w ? one : p->pog, w ? 1u : p->n_parts, false,
+                                     w ? p->n : BATCH_TILE_QUBITS, BATCH_REG_BITS, 0, gl[c], errs[c])) {
+                    if (errs[c].empty()) errs[c] = "compile failed";
+                } else {
+                    lower_program<float>(gl[c], lowered[c]);
+                }
                 continue;
             }
             Program pr;
@@ -320,50 +342,64 @@ static sv_status build_program(sv_batch *b) {
         b->n_dense_circ = D.n_circ;
     }
     std::vector<PartLaunch> parts;
-    std::vector<Phase> phases;
-    std::vector<Op> ops;
-    std::vector<float> coefs;
+    std::vector<IPhase> phases;
+    std::vector<IOp<float>> ops;
+    std::vector<float> table;
     std::vector<uint32_t> part_base(b->n), n_parts(b->n);
-    uint32_t maxP = 0;
+    std::vector<BatchWhole> wholes[BATCH_WHOLE_QUBITS + 1];   // by qubit count
+    uint32_t maxP = 0, n_whole = 0, whole_parts = 0;
+    uint64_t wave_tiles = 0;
     for (uint32_t c = 0; c < b->n; c++) {
         if (D.dense[c]) {
             n_parts[c] = 0;
             continue;
         }
         const Program &prog = gl[c];
-        const uint32_t ph0 = (uint32_t)phases.size(), op0 = (uint32_t)ops.size(), cf0 = (uint32_t)coefs.size();
+        const Lowered<float> &lo = lowered[c];
+        const uint32_t ph0 = (uint32_t)phases.size(), op0 = (uint32_t)ops.size(), tb0 = (uint32_t)table.size();
         part_base[c] = (uint32_t)parts.size();
-        n_parts[c] = (uint32_t)prog.parts.size();
+        if (whole(c)) {
+            n_parts[c] = 0;
+            if (!prog.parts.empty()) wholes[b->nq[c]].push_back({b->off[c], part_base[c], 0});
+            n_whole++;
+            whole_parts += b->plans[c]->n_parts;
+        } else {
+            n_parts[c] = (uint32_t)prog.parts.size();
+            wave_tiles += 1ull << (b->nq[c] - BATCH_TILE_QUBITS);
+        }
         maxP = std::max(maxP, n_parts[c]);
         for (PartLaunch L : prog.parts) {
             L.phase_begin += ph0;
-            L.op_begin += op0;
-            L.op_end += op0;
-            L.coef_begin += cf0;
-            L.coef_end += cf0;
             parts.push_back(L);
         }
-        for (Phase ph : prog.phases) {
+        for (IPhase ph : lo.phases) {
             ph.op_begin += op0;
             phases.push_back(ph);
         }
-        for (Op op : prog.ops) {
-            op.coef += cf0;
+        for (IOp<float> op : lo.ops) {
+            if (op.code == IM_DIAG || op.code / 8 == IK_U2) op.arg += tb0;
             ops.push_back(op);
         }
-        for (double v : prog.coefs) coefs.push_back((float)v);
+        table.insert(table.end(), lo.table.begin(), lo.table.end());
     }
+    int n_ctas = 0;
+    BCUDA(batch_prepare(b->warps, &n_ctas));
+    // tiles per item: the configured number, else as many as still leave the
+    // resident warps two items of a wave each (at most 16)
+    uint32_t chunk = (uint32_t)b->chunk;
+    if (!chunk)
+        chunk = (uint32_t)std::min<uint64_t>(16, std::max<uint64_t>(1, wave_tiles / (2ull * n_ctas * b->warps)));
     std::vector<BatchItem> items;
     for (uint32_t w = 0; w < maxP; w++)
         for (uint32_t c = 0; c < b->n; c++) {
             if (w >= n_parts[c]) continue;
             const uint32_t nt = 1u << (b->nq[c] - BATCH_TILE_QUBITS);
-            for (uint32_t t0 = 0; t0 < nt; t0 += (uint32_t)b->chunk) {
+            for (uint32_t t0 = 0; t0 < nt; t0 += chunk) {
                 BatchItem it;
                 it.circuit = c;
                 it.part = part_base[c] + w;
                 it.tile_begin = t0;
-                it.tile_count = std::min<uint32_t>((uint32_t)b->chunk, nt - t0);
+                it.tile_count = std::min<uint32_t>(chunk, nt - t0);
                 it.wait = w * nt;
                 items.push_back(it);
             }
@@ -371,25 +407,34 @@ static sv_status build_program(sv_batch *b) {
     if (b->hold_last && !items.empty()) items.back().wait = 0xFFFFFFFFu;
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t s_items = al(items.size() * sizeof(BatchItem)), s_parts = al(parts.size() * sizeof(PartLaunch));
-    const size_t s_ph = al(phases.size() * sizeof(Phase)), s_op = al(ops.size() * sizeof(Op));
-    const size_t s_cf = al(std::max<size_t>(1, coefs.size()) * sizeof(float));
+    const size_t s_ph = al(phases.size() * sizeof(IPhase)), s_op = al(ops.size() * sizeof(IOp<float>));
+    const size_t s_tb = al(table.size() * sizeof(float)), s_wh = al(n_whole * sizeof(BatchWhole));
+    const size_t s_all = std::max<size_t>(256, s_items + s_parts + s_ph + s_op + s_tb + s_wh);
     char *d = nullptr;
-    cudaError_t e = dev_alloc(reinterpret_cast<void **>(&d), s_items + s_parts + s_ph + s_op + s_cf, b->prep);
+    cudaError_t e = dev_alloc(reinterpret_cast<void **>(&d), s_all, b->prep);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return bfail(SV_ERR_OOM, std::string("batch program: ") + cudaGetErrorString(e));
     }
     b->d_prog = d;
-    std::vector<char> host(s_items + s_parts + s_ph + s_op + s_cf, 0);
+    std::vector<char> host(s_all, 0);
     // (an empty vector's data() may be null, which memcpy must not get)
     auto put = [&](size_t at, const void *src, size_t bytes) {
         if (bytes) std::memcpy(host.data() + at, src, bytes);
     };
-    put(0, items.data(), items.size() * sizeof(BatchItem));
-    put(s_items, parts.data(), parts.size() * sizeof(PartLaunch));
-    put(s_items + s_parts, phases.data(), phases.size() * sizeof(Phase));
-    put(s_items + s_parts + s_ph, ops.data(), ops.size() * sizeof(Op));
-    put(s_items + s_parts + s_ph + s_op, coefs.data(), coefs.size() * sizeof(float));
+    size_t at = 0;
+    put(at, items.data(), items.size() * sizeof(BatchItem));
+    put(at += s_items, parts.data(), parts.size() * sizeof(PartLaunch));
+    put(at += s_parts, phases.data(), phases.size() * sizeof(IPhase));
+    put(at += s_ph, ops.data(), ops.size() * sizeof(IOp<float>));
+    put(at += s_op, table.data(), table.size() * sizeof(float));
+    at += s_tb;
+    const BatchWhole *d_whole[BATCH_WHOLE_QUBITS + 1] = {};
+    for (int t = BATCH_MIN_QUBITS; t <= BATCH_WHOLE_QUBITS; t++) {
+        put(at, wholes[t].data(), wholes[t].size() * sizeof(BatchWhole));
+        d_whole[t] = reinterpret_cast<const BatchWhole *>(d + at);
+        at += wholes[t].size() * sizeof(BatchWhole);
+    }
     BCUDA(cudaMemcpyAsync(d, host.data(), host.size(), cudaMemcpyHostToDevice, b->prep));
     // every upload (gate lists, dense items, parts and R images) is complete
     // before the graph can be launched on any stream
@@ -400,23 +445,30 @@ static sv_status build_program(sv_batch *b) {
     B.n_items = (uint32_t)items.size();
     B.circ_off = b->d_off;
     B.parts = reinterpret_cast<const PartLaunch *>(d + s_items);
-    B.phases = reinterpret_cast<const Phase *>(d + s_items + s_parts);
-    B.ops = reinterpret_cast<const Op *>(d + s_items + s_parts + s_ph);
-    B.coefs = reinterpret_cast<const float *>(d + s_items + s_parts + s_ph + s_op);
+    B.phases = reinterpret_cast<const IPhase *>(d + s_items + s_parts);
+    B.ops = reinterpret_cast<const IOp<float> *>(d + s_items + s_parts + s_ph);
+    B.table = reinterpret_cast<const float *>(d + s_items + s_parts + s_ph + s_op);
     B.done = b->d_done;
     B.head = b->d_done + b->n;
     B.err = b->d_err;
-    b->n_items = B.n_items;
-    b->n_parts = (uint32_t)parts.size();
-    int n_ctas = 0;
-    BCUDA(batch_prepare(b->warps, &n_ctas));
+    b->n_items = B.n_items + n_whole;
+    b->n_parts = (uint32_t)parts.size() - n_whole + whole_parts;
     // one graph: zero the tile counters, the tickets and the dense passes'
     // norm slots, then the persistent launches (dense circuits, gate lists)
     const size_t ds_items = D.s_items, ds_parts = D.s_parts, ds_img = D.s_img;
     // captured on the private stream (nothing else is ever enqueued there),
     // launched on the caller's stream
     BCUDA(cudaStreamBeginCapture(b->prep, cudaStreamCaptureModeThreadLocal));
-    cudaError_t ce = cudaMemsetAsync(b->d_done, 0, sizeof(uint32_t) * (b->n + 2), b->prep);
+    // the whole circuits wait for nothing: they run beside the other kernels
+    // (a second branch of the graph), where these leave room on the SMs
+    cudaError_t ce = cudaSuccess;
+    if (n_whole) {
+        ce = cudaEventRecord(b->fork, b->prep);
+        if (ce == cudaSuccess) ce = cudaStreamWaitEvent(b->side, b->fork, 0);
+        for (int t = BATCH_WHOLE_QUBITS; ce == cudaSuccess && t >= BATCH_MIN_QUBITS; t--)
+            if (!wholes[t].empty()) ce = launch_batch_whole(t, B, d_whole[t], (uint32_t)wholes[t].size(), b->side);
+    }
+    if (ce == cudaSuccess) ce = cudaMemsetAsync(b->d_done, 0, sizeof(uint32_t) * (b->n + 2), b->prep);
     if (ce == cudaSuccess && b->n_dense_items) {
         double *dn = reinterpret_cast<double *>(dd + ds_items + ds_parts + ds_img);
         ce = cudaMemsetAsync(dn, 0, sizeof(double) * b->n_dense_parts, b->prep);
@@ -427,6 +479,10 @@ static sv_status build_program(sv_batch *b) {
                                      b->prep);
     }
     if (ce == cudaSuccess && B.n_items) ce = launch_batch(B, b->warps, n_ctas, b->prep);
+    if (ce == cudaSuccess && n_whole) {
+        ce = cudaEventRecord(b->join, b->side);
+        if (ce == cudaSuccess) ce = cudaStreamWaitEvent(b->prep, b->join, 0);
+    }
     cudaGraph_t g = nullptr;
     cudaError_t ee = cudaStreamEndCapture(b->prep, &g);
     if (ce != cudaSuccess || ee != cudaSuccess) {
@@ -582,7 +638,7 @@ sv_status sv_batch_destroy(sv_batch *b) {
         cudaStreamSynchronize(b->stream);   // the frees complete before the stream goes
         cudaStreamDestroy(b->stream);
     }
-    cudaStreamDestroy(b->prep);             // idle: drop_program synchronised it
+    drop_streams(b);                        // idle: drop_program synchronised prep
     delete b;
     if (e != cudaSuccess) return bfail(SV_ERR_CUDA, std::string("pending batch work failed: ") + cudaGetErrorString(e));
     return SV_OK;

@@ -20,7 +20,7 @@
 #include <sstream>
 #include <thread>
 
-#include "jit_sources.inc"   // kJitOpsCore, kJitPrelude (generated by build.py)
+#include "jit_sources.inc"   // kJitOpsCore, kJitPacked, kJitPrelude (generated by build.py)
 
 namespace hisv {
 namespace {
@@ -277,11 +277,6 @@ std::string jit_part_source(const Program &prog, size_t pi, bool df) {
                 if (mode == 0) o << "op_h2<" << A << ">(a);";   // packed f32x2
                 else o << "op_h<NR, " << A << ">(a);";
                 break;
-            case OP_U2:
-                o << "{ const Real m[8] = {";
-                for (int q = 0; q < 8; q++) o << (q ? ", " : "") << L_(c + q);
-                o << "}; op_u2<NR, " << A << ">(a, m); }";
-                break;
             case OP_RXS: o << "op_rxs<NR, " << A << ", " << B << ">(a, " << L_(c) << ");"; break;
             case OP_RYS:
                 if (mode == 0) o << "op_rys2<" << A << ", " << B << ">(a, " << L_(c) << ");";
@@ -292,13 +287,8 @@ std::string jit_part_source(const Program &prog, size_t pi, bool df) {
                 for (int q = 0; q < 6; q++) o << ", " << L_(c + q);
                 o << ");";
                 break;
-            case OP_RX: o << "op_rx<NR, " << A << ">(a, " << L_(c) << ", " << L_(c + 1) << ");"; break;
-            case OP_RY: o << "op_ry<NR, " << A << ">(a, " << L_(c) << ", " << L_(c + 1) << ");"; break;
             case OP_X: o << "op_x<" << A << ">(a);"; break;
             case OP_Y: o << "op_y<" << A << ">(a);"; break;
-            case OP_D:
-                o << "op_d<NR, " << A << ">(a, " << L_(c) << ", " << L_(c + 1) << ", " << L_(c + 2) << ", " << L_(c + 3) << ");";
-                break;
             case OP_P: o << "op_p<NR, " << A << ">(a, " << L_(c) << ", " << L_(c + 1) << ");"; break;
             case OP_Z: o << "op_z<NR, " << A << ">(a);"; break;
             case OP_CX: o << "op_cx<" << A << ", " << B << ">(a);"; break;
@@ -385,10 +375,10 @@ bool jit_compile(const Program &prog, JitProgram &out, std::string &err, bool lo
     auto work = [&](size_t ci) {
         std::string src = "#include \"jit_prelude.cuh\"\n";
         for (size_t i = ci; i < P; i += nchunks) src += jit_part_source(prog, i, df);
-        const char *hdrs[2] = {kJitOpsCore, kJitPrelude};
-        const char *hnames[2] = {"ops_core.cuh", "jit_prelude.cuh"};
+        const char *hdrs[3] = {kJitOpsCore, kJitPacked, kJitPrelude};
+        const char *hnames[3] = {"ops_core.cuh", "packed.cuh", "jit_prelude.cuh"};
         nvrtcProgram pr = nullptr;
-        nvrtcResult r = n.create(&pr, src.c_str(), "hisv_parts.cu", 2, hdrs, hnames);
+        nvrtcResult r = n.create(&pr, src.c_str(), "hisv_parts.cu", 3, hdrs, hnames);
         if (r != NVRTC_SUCCESS) {
             errs[ci] = std::string("nvrtcCreateProgram: ") + n.errstr(r);
             return;

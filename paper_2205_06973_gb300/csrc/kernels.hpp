@@ -3,18 +3,27 @@
 #include <cuda_runtime.h>
 #include <cstdint>
 
+#include "interp.hpp"
 #include "program.hpp"
 
 namespace hisv {
 
-// Register bits per thread of the part kernel: 5 for complex64, 4 for complex128.
+// Default register bits per thread (2^R amplitudes) of the kernels compiled
+// for a plan, and of the interpreter's on multi-level plans, whose
+// second-level parts may need that many register qubits.
 inline int part_R(bool fp64) { return fp64 ? 4 : 5; }
+// Register bits of the interpreter otherwise: its code must stay small.
+inline int interp_R(bool fp64) { return fp64 ? 3 : 4; }
 inline int part_tmin() { return 10; }
 inline int part_tmax(bool fp64) { return fp64 ? 12 : 13; }
 
-// One pass of a part over the whole state (Algorithm 1): n_tiles = 2^(n - t) CTAs.
-cudaError_t launch_part(bool fp64, int t, void *sv, const PartLaunch &L, const Phase *phases,
-                        const Op *ops, const void *coefs, uint64_t n_tiles, cudaStream_t st);
+// One pass of a part over the whole state (Algorithm 1) on the interpreter:
+// n_tiles = 2^(n - t) tiles, R register bits; phases, ops and table are the
+// lowered program (interp.hpp) in device memory.
+cudaError_t launch_part_f32(int t, int R, void *sv, const PartLaunch &L, const IPhase *phases, const void *ops,
+                            const void *table, uint64_t n_tiles, cudaStream_t st);
+cudaError_t launch_part_f64(int t, int R, void *sv, const PartLaunch &L, const IPhase *phases, const void *ops,
+                            const void *table, uint64_t n_tiles, cudaStream_t st);
 
 // Plain one-pass-per-gate kernels (Sec. III-A): m is the 2x2 (8 reals) or 4x4
 // (32 reals, local index l = b_q0 + 2 b_q1) complex matrix, row-major (re, im).

@@ -1,18 +1,27 @@
-// Register-level operations of the part interpreter (shared by the part
-// kernel and the batched warp-level kernel).
+// The gate-list interpreter's inner loop (shared by the part kernel and the
+// batched kernels): a phase's ops on a thread's 2^R amplitudes.
 //
-// A thread holds 2^R amplitudes a[0..2^R) of its tile; register bit b of the
-// index i is one tile slot (qubit). Every op acts on compile-time register
-// bits (with_bit turns a runtime bit into a template argument), so the
-// amplitudes stay in registers.
+// What bounds it is instruction supply. Every op has its own code per
+// register bit (the amplitudes stay in registers, so the bit must be a
+// compile-time index), and with 2^5 amplitudes per thread and two dispatch
+// levels that code was larger than the SM's instruction cache: on a 21-qubit
+// layered circuit (k = 10) 3.4 to 4.3 of 9 stall cycles per instruction were
+// "no instruction" and a pass took 36 us. So the code is kept small: 2^4
+// complex64 (2^3 complex128) amplitudes per thread, one packed instruction
+// for both halves of an amplitude where the arithmetic allows it, one form
+// per gate kind where the planner's can be reduced to another (interp.hpp),
+// permutations as selects (a permutation of registers, or through shared
+// memory, would cost more code or a round trip), one indirect branch per op.
+// The next op's record is fetched while an op runs.
 #pragma once
 #include <cuda_runtime.h>
 
 #include <cstdint>
 #include <type_traits>
 
+#include "interp.hpp"
 #include "ops_core.cuh"
-#include "program.hpp"
+#include "packed.cuh"
 
 namespace hisv {
 
@@ -20,174 +29,158 @@ template <typename Real> struct CT;
 template <> struct CT<float> { typedef float2 T; };
 template <> struct CT<double> { typedef double2 T; };
 
-// Call f(integral_constant<int, b>) for a runtime register bit b < R.
-template <int R, int B = 0, typename F>
-__device__ __forceinline__ void with_bit(int b, F &&f) {
-    if constexpr (B < R) {
-        if (b == B) f(std::integral_constant<int, B>());
-        else with_bit<R, B + 1>(b, static_cast<F &&>(f));
-    }
+__device__ __forceinline__ IOp<float> ld_op(const IOp<float> *p) {
+    const float4 v = __ldg(reinterpret_cast<const float4 *>(p));
+    IOp<float> o;
+    o.code = __float_as_uint(v.x);
+    o.arg = __float_as_uint(v.y);
+    o.c[0] = v.z;
+    o.c[1] = v.w;
+    return o;
+}
+__device__ __forceinline__ IOp<double> ld_op(const IOp<double> *p) {
+    const uint2 h = __ldg(reinterpret_cast<const uint2 *>(p));
+    const double *c = reinterpret_cast<const double *>(p) + 1;
+    IOp<double> o;
+    o.code = h.x;
+    o.arg = h.y;
+    o.c[0] = __ldg(c);
+    o.c[1] = __ldg(c + 1);
+    return o;
 }
 
-// Register permutations (X, Y, CX) go through shared memory: the thread
-// stores its amplitudes into its own slots of the tile buffer (slot of
-// register index i: s_thr ^ XOR of s_reg[b] over the bits b of i, the
-// layout the phase was loaded with) and loads them back permuted. No other
-// thread touches these slots, so no barrier is needed, and no register is
-// renamed inside the op switch: a permutation kept in registers renames them
-// differently on every path, and reconciling those renamings at the loop's
-// back edge costs every op of the interpreter (measured: about a third of
-// its instructions).
-// New a[i] = old a[i ^ (1 << t)] where the control holds (tctl, and bit cbit
-// of i when cbit >= 0), else a[i] stays; Y also multiplies by -i (bit t of i
-// clear) or +i (set).
-template <int NR, int R, typename C>
-__device__ __forceinline__ void perm_smem(C (&a)[NR], C *buf, uint32_t s_thr, const uint32_t (&s_reg)[R], int t,
-                                          int cbit, bool tctl, bool y) {
+// H, RY and RX of one register bit; float amplitudes packed where no
+// component changes place.
+template <int NR, int B> __device__ __forceinline__ void in_h(float2 (&a)[NR]) {
 #pragma unroll
     for (int i = 0; i < NR; i++) {
-        uint32_t o = s_thr;
-#pragma unroll
-        for (int b = 0; b < R; b++)
-            if (i & (1 << b)) o ^= s_reg[b];
-        buf[o] = a[i];
+        if (i & (1 << B)) continue;
+        const int j = i | (1 << B);
+        const float2 x = a[i], y = a[j];
+        a[i] = add2(x, y);
+        a[j] = sub2(x, y);
     }
-    uint32_t st = 0;   // s_reg[t] without a dynamic register index
-#pragma unroll
-    for (int b = 0; b < R; b++)
-        if (b == t) st = s_reg[b];
+}
+template <int NR, int B> __device__ __forceinline__ void in_h(double2 (&a)[NR]) { op_h<NR, B>(a); }
+
+template <int NR, int B, int F> __device__ __forceinline__ void in_ry(float2 (&a)[NR], float t) {
 #pragma unroll
     for (int i = 0; i < NR; i++) {
-        uint32_t o = s_thr;
-        asm volatile("" : "+r"(o));   // recompute the slots: keeping all of them live would spill
-#pragma unroll
-        for (int b = 0; b < R; b++)
-            if (i & (1 << b)) o ^= s_reg[b];
-        const bool ctl = tctl && (cbit < 0 || ((i >> cbit) & 1));
-        const C v = buf[ctl ? (o ^ st) : o];
-        if (y) {
-            if ((i >> t) & 1) { a[i].x = -v.y; a[i].y = v.x; }
-            else { a[i].x = v.y; a[i].y = -v.x; }
+        if (i & (1 << B)) continue;
+        const int j = i | (1 << B);
+        const float2 x = a[i], y = a[j];
+        if (F == 0) {
+            a[i] = fma2(-t, y, x);
+            a[j] = fma2(t, x, y);
         } else {
-            a[i] = v;
+            a[i] = fma2(t, x, make_float2(-y.x, -y.y));
+            a[j] = fma2(t, y, x);
         }
     }
 }
+template <int NR, int B, int F> __device__ __forceinline__ void in_ry(double2 (&a)[NR], double t) {
+    op_rys<NR, B, F>(a, t);
+}
 
-// Run a phase's ops on the thread's amplitudes. ops/coefs: the op records
-// and the coefficient array their coef indices refer to; (tpr, tpi): the
-// per-thread phase of diagonal gates on thread bits; buf, s_thr, s_reg: the
-// tile buffer and the thread's slot layout of this phase (permutations).
-template <typename Real, int R>
-__device__ __forceinline__ void run_ops(typename CT<Real>::T (&a)[1 << R], const Op *__restrict__ opsp, uint32_t count,
-                                        const Real *__restrict__ coefs, int tid, Real &tpr, Real &tpi,
-                                        typename CT<Real>::T *buf, uint32_t s_thr, const uint32_t (&s_reg)[R]) {
-    constexpr int NR = 1 << R;
-    for (uint32_t o = 0; o < count; o++) {
-        const Op op = opsp[o];
-        const Real *cf = coefs + op.coef;
-        switch (op.kind) {
-        case OP_X:
-            perm_smem<NR, R>(a, buf, s_thr, s_reg, op.a, -1, true, false);
-            break;
-        case OP_Y:
-            perm_smem<NR, R>(a, buf, s_thr, s_reg, op.a, -1, true, true);
-            break;
-        case OP_CX:
-            perm_smem<NR, R>(a, buf, s_thr, s_reg, op.b, op.a, true, false);
-            break;
-        case OP_CXT:
-            perm_smem<NR, R>(a, buf, s_thr, s_reg, op.b, -1, ((tid >> op.tb) & 1) != 0, false);
-            break;
-        case OP_H:
-            with_bit<R>(op.a, [&](auto bc) { op_h<NR, decltype(bc)::value>(a); });
-            break;
-        case OP_U2:
-            with_bit<R>(op.a, [&](auto bc) { op_u2<NR, decltype(bc)::value>(a, cf); });
-            break;
-        case OP_RX: {
-            const Real c = cf[0], s = cf[1];
-            with_bit<R>(op.a, [&](auto bc) { op_rx<NR, decltype(bc)::value>(a, c, s); });
-        } break;
-        case OP_RY: {
-            const Real c = cf[0], s = cf[1];
-            with_bit<R>(op.a, [&](auto bc) { op_ry<NR, decltype(bc)::value>(a, c, s); });
-        } break;
-        case OP_RXS: {
-            const Real t = cf[0];
-            if (op.b == 0) with_bit<R>(op.a, [&](auto bc) { op_rxs<NR, decltype(bc)::value, 0>(a, t); });
-            else with_bit<R>(op.a, [&](auto bc) { op_rxs<NR, decltype(bc)::value, 1>(a, t); });
-        } break;
-        case OP_RYS: {
-            const Real t = cf[0];
-            if (op.b == 0) with_bit<R>(op.a, [&](auto bc) { op_rys<NR, decltype(bc)::value, 0>(a, t); });
-            else with_bit<R>(op.a, [&](auto bc) { op_rys<NR, decltype(bc)::value, 1>(a, t); });
-        } break;
-        case OP_U2S: {
-            const Real ur = cf[0], ui = cf[1], vr = cf[2], vi = cf[3], wr = cf[4], wi = cf[5];
-            if (op.b == 0)
-                with_bit<R>(op.a, [&](auto bc) { op_u2s<NR, decltype(bc)::value, 0>(a, ur, ui, vr, vi, wr, wi); });
-            else
-                with_bit<R>(op.a, [&](auto bc) { op_u2s<NR, decltype(bc)::value, 1>(a, ur, ui, vr, vi, wr, wi); });
-        } break;
-        case OP_D: {
-            const Real d0r = cf[0], d0i = cf[1], d1r = cf[2], d1i = cf[3];
-            with_bit<R>(op.a, [&](auto bc) { op_d<NR, decltype(bc)::value>(a, d0r, d0i, d1r, d1i); });
-        } break;
-        case OP_P: {
-            const Real dr = cf[0], di = cf[1];
-            with_bit<R>(op.a, [&](auto bc) { op_p<NR, decltype(bc)::value>(a, dr, di); });
-        } break;
-        case OP_Z:
-            with_bit<R>(op.a, [&](auto bc) { op_z<NR, decltype(bc)::value>(a); });
-            break;
-        case OP_CP: {
-            const Real dr = cf[0], di = cf[1];
-            with_bit<R>(op.a, [&](auto ac) {
-                with_bit<R>(op.b, [&](auto bc) {
-                    constexpr int A = decltype(ac)::value, B = decltype(bc)::value;
-                    if constexpr (A != B) op_cp<NR, A, B>(a, dr, di);
-                });
-            });
-        } break;
-        case OP_CZ:
-            with_bit<R>(op.a, [&](auto ac) {
-                with_bit<R>(op.b, [&](auto bc) {
-                    constexpr int A = decltype(ac)::value, B = decltype(bc)::value;
-                    if constexpr (A != B) op_cz<NR, A, B>(a);
-                });
-            });
-            break;
-        case OP_CPT:
-            if ((tid >> op.tb) & 1) {
-                const Real dr = cf[0], di = cf[1];
-                with_bit<R>(op.a, [&](auto bc) { op_p<NR, decltype(bc)::value>(a, dr, di); });
-            }
-            break;
-        case OP_CZT:
-            if ((tid >> op.tb) & 1)
-                with_bit<R>(op.a, [&](auto bc) { op_z<NR, decltype(bc)::value>(a); });
-            break;
-        case OP_TD: {
-            const int bit = (tid >> op.tb) & 1;
-            const Real dr = bit ? cf[2] : cf[0], di = bit ? cf[3] : cf[1];
-            const Real x = tpr, y = tpi;
-            tpr = x * dr - y * di;
-            tpi = x * di + y * dr;
-        } break;
-        case OP_TP2:
-            if (((tid >> op.tb) & 1) && ((tid >> op.b) & 1)) {
-                const Real dr = cf[0], di = cf[1];
-                const Real x = tpr, y = tpi;
-                tpr = x * dr - y * di;
-                tpi = x * di + y * dr;
-            }
-            break;
-        case OP_DIAG:
+// Exchange a[i] and a[i | bit B] where the register index has all bits of
+// rm set and the thread condition holds: selects, so that no register is
+// renamed differently on the paths of the op switch.
+template <int NR, int B, typename C>
+__device__ __forceinline__ void in_swap(C (&a)[NR], uint32_t rm, bool tc) {
 #pragma unroll
-            for (int i = 0; i < NR; i++) cmul_in(a[i], cf[2 * i], cf[2 * i + 1]);
+    for (int i = 0; i < NR; i++) {
+        if (i & (1 << B)) continue;
+        const int j = i | (1 << B);
+        const bool p = tc && (i & rm) == rm;
+        const C x = a[i], y = a[j];
+        a[i].x = p ? y.x : x.x;
+        a[i].y = p ? y.y : x.y;
+        a[j].x = p ? x.x : y.x;
+        a[j].y = p ? x.y : y.y;
+    }
+}
+
+template <typename Real, int R>
+__device__ __forceinline__ void run_ops(typename CT<Real>::T (&a)[1 << R], const IOp<Real> *__restrict__ ops,
+                                        uint32_t count, const Real *__restrict__ table, uint32_t tid, Real &tpr,
+                                        Real &tpi) {
+    constexpr int NR = 1 << R;
+    if (count == 0) return;
+    IOp<Real> op = ld_op(ops);
+    for (uint32_t o = 1;; o++) {
+        const IOp<Real> cur = op;
+        if (o < count) op = ld_op(ops + o);
+        const uint32_t tm = cur.arg & 0xFFFFu;
+        const bool tc = (tid & tm) == tm;
+        switch (cur.code) {
+// one case per register bit below R
+#define HISV_BIT(K, B, BODY) \
+    case (K) * 8 + (B):      \
+        if constexpr ((B) < R) BODY; \
+        break;
+#define HISV_BITS(K, BODY0, BODY1, BODY2, BODY3, BODY4) \
+    HISV_BIT(K, 0, BODY0) HISV_BIT(K, 1, BODY1) HISV_BIT(K, 2, BODY2) HISV_BIT(K, 3, BODY3) HISV_BIT(K, 4, BODY4)
+#define HISV_EACH(K, CALL) HISV_BITS(K, CALL(0), CALL(1), CALL(2), CALL(3), CALL(4))
+#define HISV_H(B) (in_h<NR, B>(a))
+#define HISV_RX0(B) (op_rxs<NR, B, 0>(a, cur.c[0]))
+#define HISV_RX1(B) (op_rxs<NR, B, 1>(a, cur.c[0]))
+#define HISV_RY0(B) (in_ry<NR, B, 0>(a, cur.c[0]))
+#define HISV_RY1(B) (in_ry<NR, B, 1>(a, cur.c[0]))
+#define HISV_U2(B) \
+    (op_u2s<NR, B, 0>(a, __ldg(table + cur.arg), __ldg(table + cur.arg + 1), __ldg(table + cur.arg + 2), \
+                      __ldg(table + cur.arg + 3), __ldg(table + cur.arg + 4), __ldg(table + cur.arg + 5)))
+#define HISV_SWAP(B) (in_swap<NR, B>(a, cur.arg >> 16, tc))
+#define HISV_P(B) (op_p<NR, B>(a, tc ? cur.c[0] : Real(1), tc ? cur.c[1] : Real(0)))
+            HISV_EACH(IK_H, HISV_H)
+            HISV_EACH(IK_RX0, HISV_RX0)
+            HISV_EACH(IK_RX1, HISV_RX1)
+            HISV_EACH(IK_RY0, HISV_RY0)
+            HISV_EACH(IK_RY1, HISV_RY1)
+            HISV_EACH(IK_U2, HISV_U2)
+            HISV_EACH(IK_SWAP, HISV_SWAP)
+            HISV_EACH(IK_P, HISV_P)
+// one case per pair A < B of register bits below R
+#define HISV_CP(A, B)                             \
+    case IK_CP * 8 + (B) * ((B) - 1) / 2 + (A):   \
+        if constexpr ((B) < R) op_cp<NR, A, B>(a, cur.c[0], cur.c[1]); \
+        break;
+            HISV_CP(0, 1)
+            HISV_CP(0, 2) HISV_CP(1, 2)
+            HISV_CP(0, 3) HISV_CP(1, 3) HISV_CP(2, 3)
+            HISV_CP(0, 4) HISV_CP(1, 4) HISV_CP(2, 4) HISV_CP(3, 4)
+#undef HISV_BIT
+#undef HISV_BITS
+#undef HISV_EACH
+#undef HISV_H
+#undef HISV_RX0
+#undef HISV_RX1
+#undef HISV_RY0
+#undef HISV_RY1
+#undef HISV_U2
+#undef HISV_SWAP
+#undef HISV_P
+#undef HISV_CP
+        case IM_TPH:
+            if (tc) {
+                const Real x = tpr, y = tpi;
+                tpr = x * cur.c[0] - y * cur.c[1];
+                tpi = x * cur.c[1] + y * cur.c[0];
+            }
             break;
-        case OP_TAPPLY:
+        case IM_DIAG: {
+            const Real *const d = table + cur.arg;
+#pragma unroll
+            for (int i = 0; i < NR; i++) {
+                if constexpr (sizeof(Real) == 4) {
+                    const float2 v = __ldg(reinterpret_cast<const float2 *>(d) + i);
+                    cmul_in(a[i], v.x, v.y);
+                } else {
+                    const double2 v = __ldg(reinterpret_cast<const double2 *>(d) + i);
+                    cmul_in(a[i], v.x, v.y);
+                }
+            }
+        } break;
+        case IM_TAPPLY:
 #pragma unroll
             for (int i = 0; i < NR; i++) cmul_in(a[i], tpr, tpi);
             tpr = Real(1);
@@ -196,7 +189,38 @@ __device__ __forceinline__ void run_ops(typename CT<Real>::T (&a)[1 << R], const
         default:
             break;
         }
+        if (o >= count) break;
     }
 }
+
+// XOR of the offsets off[j] over the set bits j of v (TB bits).
+template <int TB>
+__device__ __forceinline__ uint32_t xor_bits(uint32_t v, const uint16_t *off) {
+    uint32_t s = 0;
+#pragma unroll
+    for (int j = 0; j < TB; j++) s ^= (v >> j) & 1 ? off[j] : 0u;
+    return s;
+}
+
+// A phase's layout for this thread: offset of its amplitude 0 and of each
+// register bit.
+template <int R, int TB> struct Slots {
+    uint32_t thr, reg[R];
+    __device__ __forceinline__ void load(const IPhase *__restrict__ ph, uint32_t tid) {
+        union { uint4 q[3]; uint16_t h[24]; } u;
+#pragma unroll
+        for (int i = 0; i < 3; i++) u.q[i] = __ldg(reinterpret_cast<const uint4 *>(ph) + i);
+#pragma unroll
+        for (int b = 0; b < R; b++) reg[b] = u.h[b];
+        thr = xor_bits<TB>(tid, u.h + 8);
+    }
+    __device__ __forceinline__ uint32_t at(int i) const {
+        uint32_t o = thr;
+#pragma unroll
+        for (int b = 0; b < R; b++)
+            if (i & (1 << b)) o ^= reg[b];
+        return o;
+    }
+};
 
 }  // namespace hisv

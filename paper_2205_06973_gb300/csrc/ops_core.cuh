@@ -26,46 +26,6 @@ __device__ __forceinline__ void op_h(C (&a)[NR]) {
     }
 }
 
-template <int NR, int B, typename C, typename Real>
-__device__ __forceinline__ void op_u2(C (&a)[NR], const Real *m) {
-    const Real m00r = m[0], m00i = m[1], m01r = m[2], m01i = m[3];
-    const Real m10r = m[4], m10i = m[5], m11r = m[6], m11i = m[7];
-#pragma unroll
-    for (int i = 0; i < NR; i++) {
-        if (i & (1 << B)) continue;
-        const int j = i | (1 << B);
-        const C x = a[i], y = a[j];
-        a[i].x = m00r * x.x - m00i * x.y + m01r * y.x - m01i * y.y;
-        a[i].y = m00r * x.y + m00i * x.x + m01r * y.y + m01i * y.x;
-        a[j].x = m10r * x.x - m10i * x.y + m11r * y.x - m11i * y.y;
-        a[j].y = m10r * x.y + m10i * x.x + m11r * y.y + m11i * y.x;
-    }
-}
-
-template <int NR, int B, typename C, typename Real>
-__device__ __forceinline__ void op_rx(C (&a)[NR], Real c, Real s) {
-#pragma unroll
-    for (int i = 0; i < NR; i++) {
-        if (i & (1 << B)) continue;
-        const int j = i | (1 << B);
-        const C x = a[i], y = a[j];
-        a[i].x = c * x.x + s * y.y; a[i].y = c * x.y - s * y.x;
-        a[j].x = s * x.y + c * y.x; a[j].y = c * y.y - s * x.x;
-    }
-}
-
-template <int NR, int B, typename C, typename Real>
-__device__ __forceinline__ void op_ry(C (&a)[NR], Real c, Real s) {
-#pragma unroll
-    for (int i = 0; i < NR; i++) {
-        if (i & (1 << B)) continue;
-        const int j = i | (1 << B);
-        const C x = a[i], y = a[j];
-        a[i].x = c * x.x - s * y.x; a[i].y = c * x.y - s * y.y;
-        a[j].x = s * x.x + c * y.x; a[j].y = s * x.y + c * y.y;
-    }
-}
-
 // Scaled rotations: the gate divided by its largest entry (the factor is
 // applied once, with the part's store factor), so every output component is
 // one multiply-add. F = form (see OP_RXS / OP_RYS / OP_U2S in program.hpp).
@@ -125,15 +85,6 @@ __device__ __forceinline__ void cmul_in(C &v, Real dr, Real di) {
     const Real x = v.x, y = v.y;
     v.x = x * dr - y * di;
     v.y = x * di + y * dr;
-}
-
-template <int NR, int B, typename C, typename Real>
-__device__ __forceinline__ void op_d(C (&a)[NR], Real d0r, Real d0i, Real d1r, Real d1i) {
-#pragma unroll
-    for (int i = 0; i < NR; i++) {
-        if (i & (1 << B)) cmul_in(a[i], d1r, d1i);
-        else cmul_in(a[i], d0r, d0i);
-    }
 }
 
 template <int NR, int B, typename C, typename Real>

@@ -1,0 +1,37 @@
+// Packed float arithmetic shared by the library's kernels and the part
+// kernels compiled at run time (no standard or CUDA headers).
+#pragma once
+
+namespace hisv {
+
+// Packed pairs of floats (sm_100+ f32x2 arithmetic): a complex64 amplitude is
+// one 64-bit register pair, so a complex sum or a real-scaled complex
+// multiply-add is one instruction.
+__device__ __forceinline__ unsigned long long pk(float2 v) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(v.x), "f"(v.y));
+    return r;
+}
+__device__ __forceinline__ float2 upk(unsigned long long r) {
+    float2 v;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(r));
+    return v;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pk(a)), "l"(pk(b)));
+    return upk(d);
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+    unsigned long long d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pk(a)), "l"(pk(b)));
+    return upk(d);
+}
+// t * b + c with the real t on both halves
+__device__ __forceinline__ float2 fma2(float t, float2 b, float2 c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(pk(make_float2(t, t))), "l"(pk(b)), "l"(pk(c)));
+    return upk(d);
+}
+
+}  // namespace hisv

@@ -385,6 +385,17 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
             fr = x * dr - y * di;
             fi = x * di + y * dr;
         };
+        // the part factor goes into a merged diagonal's coefficients
+        auto scale_diag = [&](const Op &op) {
+            double *c = prog.coefs.data() + op.coef;
+            for (int i = 0; i < (1 << R); i++) {
+                const double x = c[2 * i], y = c[2 * i + 1];
+                c[2 * i] = x * fr - y * fi;
+                c[2 * i + 1] = x * fi + y * fr;
+            }
+            fr = 1.0;
+            fi = 0.0;
+        };
         bool last_tphase = false;
         std::vector<int> remaining = gl;
         bool first = true;
@@ -680,9 +691,6 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
                     switch (op.kind) {
                     case OP_P: for (int i = 0; i < NR; i++) if ((i >> op.a) & 1) mulphase(i, c[0], c[1]); break;
                     case OP_Z: for (int i = 0; i < NR; i++) if ((i >> op.a) & 1) mulphase(i, -1.0, 0.0); break;
-                    case OP_D:
-                        for (int i = 0; i < NR; i++) mulphase(i, (i >> op.a) & 1 ? c[2] : c[0], (i >> op.a) & 1 ? c[3] : c[1]);
-                        break;
                     case OP_CZ:
                         for (int i = 0; i < NR; i++) if (((i >> op.a) & 1) && ((i >> op.b) & 1)) mulphase(i, -1.0, 0.0);
                         break;
@@ -701,8 +709,7 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
                     // register bits the op acts on non-diagonally
                     uint32_t touch = 0;
                     switch (op.kind) {
-                    case OP_H: case OP_U2: case OP_RX: case OP_RY: case OP_X: case OP_Y: case OP_RXS: case OP_RYS:
-                    case OP_U2S: touch = 1u << op.a; break;
+                    case OP_H: case OP_X: case OP_Y: case OP_RXS: case OP_RYS: case OP_U2S: touch = 1u << op.a; break;
                     case OP_CX: touch = (1u << op.a) | (1u << op.b); break;
                     case OP_CXT: touch = 1u << op.b; break;
                     default: touch = 0; break;   // thread-bit phases: diagonal, they commute
@@ -713,6 +720,19 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
                 flush();
             }
             if (tphase && !last) emit(OP_TAPPLY, 0, 0, 0, 0);
+            // a part of many phases (a whole circuit) applies the part factor
+            // before the unnormalised amplitudes grow out of range: into a
+            // merged diagonal of the phase, else as one of its own
+            if (!last && std::hypot(fr, fi) < 0x1p-24) {
+                uint32_t o = ph.op_begin;
+                while (o < (uint32_t)prog.ops.size() && prog.ops[o].kind != OP_DIAG) o++;
+                if (o == (uint32_t)prog.ops.size()) {
+                    const uint32_t at = (uint32_t)prog.coefs.size();
+                    for (int i = 0; i < (1 << R); i++) prog.coefs.insert(prog.coefs.end(), {1.0, 0.0});
+                    emit(OP_DIAG, 0, 0, 0, at);
+                }
+                scale_diag(prog.ops[o]);
+            }
             if (last) last_tphase = tphase;
             ph.op_count = (uint32_t)prog.ops.size() - ph.op_begin;
             prog.phases.push_back(ph);
@@ -733,14 +753,7 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
         if (!last_tphase && (fr != 1.0 || fi != 0.0)) {
             for (uint32_t o = L.op_begin; o < (uint32_t)prog.ops.size(); o++) {
                 if (prog.ops[o].kind != OP_DIAG) continue;
-                double *c = prog.coefs.data() + prog.ops[o].coef;
-                for (int i = 0; i < (1 << R); i++) {
-                    const double x = c[2 * i], y = c[2 * i + 1];
-                    c[2 * i] = x * fr - y * fi;
-                    c[2 * i + 1] = x * fi + y * fr;
-                }
-                fr = 1.0;
-                fi = 0.0;
+                scale_diag(prog.ops[o]);
                 break;
             }
         }
@@ -777,11 +790,9 @@ void program_flops(const Program &prog, double &alu_per_amp, double &tensor_per_
                 const Op &op = prog.ops[ph.op_begin + k];
                 switch (op.kind) {
                 case OP_H: alu_per_amp += 2.0; break;                 // a + b, a - b per component pair
-                case OP_RX: case OP_RY: alu_per_amp += 6.0; break;    // c x + s y per component
-                case OP_U2: alu_per_amp += 14.0; break;               // 2x2 complex matrix-vector
                 case OP_RXS: case OP_RYS: alu_per_amp += 4.0; break;  // one multiply-add per component
                 case OP_U2S: alu_per_amp += 11.0; break;              // x + u y (8), v x + w y (14) per pair
-                case OP_D: case OP_DIAG: case OP_TAPPLY: alu_per_amp += 6.0; break;   // complex product, all
+                case OP_DIAG: case OP_TAPPLY: alu_per_amp += 6.0; break;   // complex product, all
                 case OP_P: case OP_CPT: alu_per_amp += 3.0; break;    // complex product on half
                 case OP_CP: alu_per_amp += 1.5; break;                // complex product on a quarter
                 default: break;                                       // X, Y, Z, CX, CZ, SWAP, thread phases
