@@ -67,15 +67,17 @@ template <typename Real> void lower_program(const Program &prog, Lowered<Real> &
                 emit(IM_DIAG, table(d.data(), 2 * NR));
             } break;
             case OP_P: emit(kind(IK_P, op.a), 0, c[0], c[1]); break;
-            case OP_Z: emit(kind(IK_P, op.a), 0, -1.0, 0.0); break;
+            case OP_Z: emit(IM_SIGN, (1u << op.a) << 16); break;
             case OP_CPT: emit(kind(IK_P, op.a), tm, c[0], c[1]); break;
-            case OP_CZT: emit(kind(IK_P, op.a), tm, -1.0, 0.0); break;
+            case OP_CZT: emit(IM_SIGN, ((1u << op.a) << 16) | tm); break;
             case OP_CP: emit(pair(op.a, op.b), 0, c[0], c[1]); break;
-            case OP_CZ: emit(pair(op.a, op.b), 0, -1.0, 0.0); break;
+            case OP_CZ: emit(IM_SIGN, ((1u << op.a) | (1u << op.b)) << 16); break;
             case OP_TD: emit(IM_TPH, tm, c[2], c[3]); break;   // the planner's d0 is 1
             case OP_TP2: emit(IM_TPH, tm | (1u << op.b), c[0], c[1]); break;
             case OP_DIAG: emit(IM_DIAG, table(c, 2 * NR)); break;
             case OP_TAPPLY: emit(IM_TAPPLY, 0); break;
+            case OP_TSG: emit(IM_TSG, tm | (1u << op.b)); break;
+            case OP_TSAPPLY: emit(IM_TSAPPLY, 0); break;
             default: break;
             }
         }

@@ -29,10 +29,13 @@ enum InterpMisc : uint32_t {
     IM_TPH = IK_MISC * 8,   // per-thread phase *= c where the thread condition holds
     IM_DIAG,                // register amplitude i *= table[arg + 2 i] (re, im)
     IM_TAPPLY,              // multiply by the per-thread phase, reset it
+    IM_TSG,                 // per-thread sign flips where the thread condition holds
+    IM_TSAPPLY,             // negate where the per-thread sign is set, reset it
+    IM_SIGN,                // negate where the register mask and the thread condition hold: Z, CZ
 };
 
 // arg: low half = thread-bit mask (all set: the condition holds; 0 = always),
-// high half = register control mask of IK_SWAP; for IK_U2 and IM_DIAG the
+// high half = register mask of IK_SWAP and IM_SIGN; for IK_U2 and IM_DIAG the
 // table index (in reals).
 template <typename Real> struct alignas(16) IOp {
     uint32_t code;

@@ -192,7 +192,8 @@ std::string jit_part_source(const Program &prog, size_t pi, bool df) {
       << "        cp_wait1();\n"
       << "        __syncthreads();\n"
       << "        Real tpr = 1, tpi = 0;\n"
-      << "        (void)tpr; (void)tpi;\n";
+      << "        bool tsg = false;\n"
+      << "        (void)tpr; (void)tpi; (void)tsg;\n";
     const std::vector<double> &cf = prog.coefs;
     auto L_ = [&](uint32_t at) { return lit(cf[at], mode); };
     auto L_lit = [&](double v) { return lit(v, mode); };
@@ -314,6 +315,12 @@ std::string jit_part_source(const Program &prog, size_t pi, bool df) {
             case OP_TP2:
                 o << "{ const bool c_ = " << tb << " && ((tid >> " << B << ") & 1); tmul(tpr, tpi, c_ ? " << L_(c)
                   << " : (Real)1, c_ ? " << L_(c + 1) << " : (Real)0); }";
+                break;
+            case OP_TSG:
+                o << "tsg ^= " << tb << " && ((tid >> " << B << ") & 1);";
+                break;
+            case OP_TSAPPLY:
+                o << "op_flip<NR>(a, tsg); tsg = false;";
                 break;
             case OP_DIAG:
                 // entries of exactly 1, -1, i or -i are a copy, negation or

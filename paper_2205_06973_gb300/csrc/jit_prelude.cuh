@@ -179,7 +179,8 @@ __device__ __forceinline__ void op_cxt(C (&a)[NR], bool ctl) {
 }
 // The amplitudes with register bit B set are negated where neg holds (a
 // controlled Z whose control is a thread bit): one packed multiply by (s, s)
-// per amplitude for complex64, a multiply of each part otherwise.
+// per amplitude for complex64, sign-bit flips for complex128, a multiply of
+// each part for double-float.
 template <int B>
 __device__ __forceinline__ void op_sgn(C (&a)[NR], bool neg) {
 #if HISV_DF
@@ -191,10 +192,14 @@ __device__ __forceinline__ void op_sgn(C (&a)[NR], bool neg) {
             a[i].y.hi *= s; a[i].y.lo *= s;
         }
 #elif HISV_FP64
-    const double s = neg ? -1.0 : 1.0;
+    // a sign-bit flip: a product would be FP64 work
+    const int m = neg ? (int)0x80000000 : 0;
 #pragma unroll
     for (int i = 0; i < NR; i++)
-        if (i & (1 << B)) { a[i].x *= s; a[i].y *= s; }
+        if (i & (1 << B)) {
+            a[i].x = __hiloint2double(__double2hiint(a[i].x) ^ m, __double2loint(a[i].x));
+            a[i].y = __hiloint2double(__double2hiint(a[i].y) ^ m, __double2loint(a[i].y));
+        }
 #else
     const float s = neg ? -1.f : 1.f;
     unsigned long long ss;

@@ -100,12 +100,19 @@ __device__ __forceinline__ void in_swap(C (&a)[NR], uint32_t rm, bool tc) {
     }
 }
 
+// v negated where p holds: a sign-bit flip (not FP64 work for doubles).
+__device__ __forceinline__ float flip(float v, uint32_t m) { return __uint_as_float(__float_as_uint(v) ^ m); }
+__device__ __forceinline__ double flip(double v, uint32_t m) {
+    return __hiloint2double(__double2hiint(v) ^ (int)m, __double2loint(v));
+}
+
 template <typename Real, int R>
 __device__ __forceinline__ void run_ops(typename CT<Real>::T (&a)[1 << R], const IOp<Real> *__restrict__ ops,
                                         uint32_t count, const Real *__restrict__ table, uint32_t tid, Real &tpr,
                                         Real &tpi) {
     constexpr int NR = 1 << R;
     if (count == 0) return;
+    uint32_t tsg = 0u;   // the per-thread sign, applied within the phase
     IOp<Real> op = ld_op(ops);
     for (uint32_t o = 1;; o++) {
         const IOp<Real> cur = op;
@@ -186,6 +193,26 @@ __device__ __forceinline__ void run_ops(typename CT<Real>::T (&a)[1 << R], const
             tpr = Real(1);
             tpi = Real(0);
             break;
+        case IM_TSG:
+            tsg ^= tc ? 0x80000000u : 0u;
+            break;
+        case IM_TSAPPLY:
+#pragma unroll
+            for (int i = 0; i < NR; i++) {
+                a[i].x = flip(a[i].x, tsg);
+                a[i].y = flip(a[i].y, tsg);
+            }
+            tsg = 0u;
+            break;
+        case IM_SIGN: {
+            const uint32_t rm = cur.arg >> 16;
+#pragma unroll
+            for (int i = 0; i < NR; i++) {
+                const uint32_t m = tc && (i & rm) == rm ? 0x80000000u : 0u;
+                a[i].x = flip(a[i].x, m);
+                a[i].y = flip(a[i].y, m);
+            }
+        } break;
         default:
             break;
         }

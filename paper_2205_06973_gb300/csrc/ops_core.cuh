@@ -115,6 +115,23 @@ __device__ __forceinline__ void op_cz(C (&a)[NR]) {
         if ((i & (1 << A)) && (i & (1 << B))) { a[i].x = -a[i].x; a[i].y = -a[i].y; }
 }
 
+// Every amplitude negated where neg holds (a controlled Z of two thread bits):
+// a product for single floats, selects (no FP64 work) for the wider forms.
+template <int NR, typename C>
+__device__ __forceinline__ void op_flip(C (&a)[NR], bool neg) {
+#pragma unroll
+    for (int i = 0; i < NR; i++) {
+        if constexpr (sizeof(C) == 8) {
+            const auto s = neg ? -1.0f : 1.0f;
+            a[i].x = a[i].x * s;
+            a[i].y = a[i].y * s;
+        } else {
+            a[i].x = neg ? -a[i].x : a[i].x;
+            a[i].y = neg ? -a[i].y : a[i].y;
+        }
+    }
+}
+
 // Swizzled shared-memory index contribution of tile slot p. The swizzle XORs
 // the slot bits above the bank group into the low bits (linear over GF(2)),
 // so a warp whose lane bits sit on slots of distinct residues touches

@@ -18,6 +18,7 @@
 #include "planner.hpp"
 
 #include <algorithm>
+#include <array>
 #include <cstdint>
 #include <cmath>
 #include <cstring>
@@ -76,6 +77,22 @@ static uint32_t needed_slots(const GateRef &g, const int *slot_of) {
     default:
         return 0u;
     }
+}
+
+static bool is_diagonal(int kind) {
+    switch (kind) {
+    case SV_GATE_Z: case SV_GATE_S: case SV_GATE_T: case SV_GATE_RZ: case SV_GATE_P: case SV_GATE_CZ: case SV_GATE_CP:
+        return true;
+    default:
+        return false;
+    }
+}
+
+// qubits that the gate acts on non-diagonally (not as a phase or a control)
+static uint64_t acts_nondiag(const GateRef &g) {
+    if (is_diagonal(g.kind)) return 0;
+    if (g.kind == SV_GATE_SWAP) return (1ull << g.q[0]) | (1ull << g.q[1]);
+    return 1ull << (g.kind == SV_GATE_CX ? g.q[1] : g.q[0]);
 }
 
 // Thread-bit order of a phase: lane bits first. The first lanes cover
@@ -404,8 +421,9 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
             int sim_slot[64];
             std::memcpy(sim_slot, slot_of, sizeof(slot_of));
             uint32_t Rset = 0;
-            uint64_t blocked = 0;
+            uint64_t blocked = 0, blocked_nd = 0;   // for every gate; for gates non-diagonal on the qubit
             std::vector<int> sched, rest;
+            std::vector<std::array<int, 2>> slot_before;   // tile slots of a scheduled gate's qubits
             if (inner && !inner->empty()) {
                 // multi-level partitioning: the phase is the next second-level
                 // part (the smallest inner id left; its gates in order)
@@ -428,21 +446,62 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
                 }
             } else
             for (int g : remaining) {
+                // gates that are diagonal on every qubit they share (phases,
+                // controls) commute: a gate that stays behind blocks its
+                // non-diagonal qubits for all others, its diagonal ones only
+                // for gates that are not diagonal there
                 const GateRef &gr = gates[g];
-                if (gmask[g] & blocked) {
-                    blocked |= gmask[g];
-                    rest.push_back(g);
-                    continue;
-                }
-                uint32_t need = needed_slots(gr, sim_slot);
-                if ((need & ~Rset) && popc(Rset | need) > R) {
-                    blocked |= gmask[g];
+                const uint64_t nd = acts_nondiag(gr), dg = gmask[g] & ~nd;
+                const uint32_t need = needed_slots(gr, sim_slot);
+                if ((nd & (blocked | blocked_nd)) || (dg & blocked) ||
+                    ((need & ~Rset) && popc(Rset | need) > R)) {
+                    blocked |= nd;
+                    blocked_nd |= dg;
                     rest.push_back(g);
                     continue;
                 }
                 Rset |= need;
                 sched.push_back(g);
+                slot_before.push_back({sim_slot[gr.q[0]], sim_slot[gr.q[1]]});
                 if (gr.kind == SV_GATE_SWAP) std::swap(sim_slot[gr.q[0]], sim_slot[gr.q[1]]);
+            }
+            if (!(inner && !inner->empty())) {
+                // A diagonal gate on thread bits alone costs a complex product
+                // of every amplitude at the phase's end, while on a register
+                // bit it joins the phase's merged diagonal. So it is left to a
+                // later phase if one of its qubits must be resident in one
+                // anyway and the gates of this phase that follow it on its
+                // qubits are diagonal there too.
+                uint64_t later = 0, need = 0;   // qubits that must be resident after this phase
+                for (int g : rest)
+                    if (gates[g].kind != SV_GATE_SWAP) need |= acts_nondiag(gates[g]);
+                std::vector<int> keep;
+                bool moved = false;
+                for (size_t i = sched.size(); i-- > 0;) {
+                    const int g = sched[i];
+                    bool thread = Rset != 0 && is_diagonal(gates[g].kind) && (gmask[g] & need) && !(gmask[g] & later);
+                    for (int j = 0; thread && j < gates[g].arity; j++) thread = !((Rset >> slot_before[i][j]) & 1);
+                    if (thread) {
+                        rest.push_back(g);
+                        moved = true;
+                        continue;
+                    }
+                    later |= acts_nondiag(gates[g]);
+                    keep.push_back(g);
+                }
+                if (moved) {
+                    std::sort(rest.begin(), rest.end());
+                    std::reverse(keep.begin(), keep.end());
+                    sched.swap(keep);
+                }
+                // spare register bits go to the thread bits of diagonal gates
+                std::memcpy(sim_slot, slot_of, sizeof(slot_of));
+                for (int g : sched) {
+                    if (is_diagonal(gates[g].kind))
+                        for (int j = 0; j < gates[g].arity; j++)
+                            if (popc(Rset) < R) Rset |= 1u << sim_slot[gates[g].q[j]];
+                    if (gates[g].kind == SV_GATE_SWAP) std::swap(sim_slot[gates[g].q[0]], sim_slot[gates[g].q[1]]);
+                }
             }
             for (int p = t - 1; p >= 0 && popc(Rset) < R; p--) Rset |= 1u << p;
             const bool last = rest.empty();
@@ -471,7 +530,7 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
             }
             // pass 2: emit ops
             ph.op_begin = (uint32_t)prog.ops.size();
-            bool tphase = false;
+            bool tphase = false, tsign = false;
             auto coef = [&](std::initializer_list<double> v) {
                 uint32_t at = (uint32_t)prog.coefs.size();
                 prog.coefs.insert(prog.coefs.end(), v.begin(), v.end());
@@ -521,6 +580,9 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
                     if (r0) {
                         if (gr.kind == SV_GATE_Z) emit(OP_Z, rb[s0], 0, 0, 0);
                         else emit(OP_P, rb[s0], 0, 0, coef({dr, di}));
+                    } else if (gr.kind == SV_GATE_Z) {
+                        emit(OP_TSG, 0, tbit[s0], tbit[s0], 0);
+                        tsign = true;
                     } else {
                         emit(OP_TD, 0, 0, tbit[s0], coef({1.0, 0.0, dr, di}));
                         tphase = true;
@@ -552,6 +614,9 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
                         const int rs = r0 ? s0 : s1, ts = r0 ? s1 : s0;
                         if (cz) emit(OP_CZT, rb[rs], 0, tbit[ts], 0);
                         else emit(OP_CPT, rb[rs], 0, tbit[ts], coef({dr, di}));
+                    } else if (cz) {
+                        emit(OP_TSG, 0, tbit[s1], tbit[s0], 0);
+                        tsign = true;
                     } else {
                         emit(OP_TP2, 0, tbit[s1], tbit[s0], coef({dr, di}));
                         tphase = true;
@@ -566,11 +631,8 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
                 }
                 return true;
             };
-            // Runs of one-qubit gates on one qubit with no multi-qubit gate on it
-            // in between (gates on other qubits commute with them) become one
-            // op: their product, as a phase (diagonal; the entry of |0> joins
-            // the part factor) or a general 2x2 matrix.
-            auto emit_fused = [&](int q, const std::vector<int> &run) -> bool {
+            // the product of a run of one-qubit gates on qubit q as one op
+            auto emit_product = [&](int q, const std::vector<int> &run) -> bool {
                 if (run.size() == 1) return emit_one(run[0]);
                 double M[8] = {1, 0, 0, 0, 0, 0, 1, 0};
                 for (int g : run) {
@@ -627,6 +689,29 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
                     emit(OP_U2S, rb[sq], f1 ? 1 : 0, 0, coef({ur, ui, vr, vi, wr, wi}));
                 }
                 return true;
+            };
+            // Runs of one-qubit gates on one qubit with no multi-qubit gate on it
+            // in between (gates on other qubits commute with them) become one
+            // op: their product, as a phase (diagonal; the entry of |0> joins
+            // the part factor) or a general 2x2 matrix. With fewer than three
+            // non-diagonal gates the run stays those gates and one phase
+            // between them: 2 or 4 flops per amplitude and gate, and the
+            // phases mostly join a merged diagonal, against 11 for the matrix.
+            auto emit_fused = [&](int q, const std::vector<int> &whole) -> bool {
+                int nondiag = 0;
+                for (int g : whole) nondiag += !is_diagonal(gates[g].kind);
+                if (nondiag == 0 || nondiag > 2) return emit_product(q, whole);
+                std::vector<int> diag;
+                for (int g : whole) {
+                    if (is_diagonal(gates[g].kind)) {
+                        diag.push_back(g);
+                        continue;
+                    }
+                    if (!diag.empty() && !emit_product(q, diag)) return false;
+                    diag.clear();
+                    if (!emit_one(g)) return false;
+                }
+                return diag.empty() || emit_product(q, diag);
             };
             std::vector<std::vector<int>> pend(n);
             std::vector<int> pend_order;
@@ -720,6 +805,7 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
                 flush();
             }
             if (tphase && !last) emit(OP_TAPPLY, 0, 0, 0, 0);
+            if (tsign) emit(OP_TSAPPLY, 0, 0, 0, 0);
             // a part of many phases (a whole circuit) applies the part factor
             // before the unnormalised amplitudes grow out of range: into a
             // merged diagonal of the phase, else as one of its own

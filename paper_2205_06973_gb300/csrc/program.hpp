@@ -33,6 +33,8 @@ enum OpKind : uint8_t {
     OP_TD,       // tb; coef: d0, d1: per-thread phase *= (bit ? d1 : d0)
     OP_TP2,      // tb, b = second thread bit; coef: d: per-thread phase *= d if both set
     OP_TAPPLY,   // multiply the thread's amplitudes by its phase, reset the phase to 1
+    OP_TSG,      // tb, b: per-thread sign flips if both thread bits are set (Z, CZ on thread bits)
+    OP_TSAPPLY,  // negate the thread's amplitudes where its sign is set, reset the sign
     OP_DIAG,     // coef: 2^R phases (re, im): register amplitude i *= phase i (merged diagonal gates)
     // Rotations with their largest entry factored out into the part factor
     // (one multiply-add per output component instead of two); b = form:
