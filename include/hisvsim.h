@@ -105,8 +105,10 @@ typedef struct sv_plan sv_plan;
 /* Register bits per thread of the gate-list part kernels (amplitudes per
  * thread = 2^r, the register level of the tile): r in [3, 6] with
  * SV_FLAG_SPECIALISE (the tile must keep at least 2^5 threads, t - r >= 5);
- * 0 = the default (5 for complex64, 4 for complex128). The interpreter runs
- * the default only (SV_ERR_ARG otherwise). */
+ * 0 = 5 for complex64 and 4 for the complex128 forms; but where the tile is
+ * left to the library too, sv_apply_parts and sv_plan_specialise choose both
+ * by the state's size. The interpreter runs the library's choice only
+ * (SV_ERR_ARG otherwise). */
 #define SV_FLAG_REGBITS(r) (((uint32_t)(r) & 0xFu) << 8)
 #define SV_FLAG_SPECIALISE 0x8u /* gate-list parts run as kernels generated for this plan, with
                                    the tile layout, register phases and every gate (with its
@@ -161,7 +163,8 @@ sv_status sv_sync(sv_state *s);
 /* CTA tile size used by the part kernels for this state: tile_qubits t in
  * [10, 13] for SV_C64 and [10, 12] for SV_C128 and SV_C128DF (2^t
  * amplitudes per CTA); 0 restores the default: 12 (complex64) / 11 (the
- * complex128 forms), grown to the plan's largest part plus the lowest free
+ * complex128 forms; an apply takes less for states of few tiles and 12 for
+ * large double-float states), grown to the plan's largest part plus the lowest free
  * qubits that make each contiguous run of the tile fill a 32-byte sector
  * (two for complex64, one for the complex128 forms), within the limits
  * above. The tile always contains the part's qubits and is padded with the
@@ -192,7 +195,8 @@ sv_status sv_plan_build(const sv_gate *gates, size_t n_gates, int n_qubits, sv_m
 sv_status sv_plan_export(const sv_plan *p, uint32_t *part_of_gate, size_t n_gates, uint32_t *n_parts);
 /* Statistics of the compiled device program for a precision, tile and apply
  * flags (SV_FLAG_TC_DENSE changes the program): passes = parts run on the
- * GPU, phases = register phases of the gate-list parts, ops = their kernel
+ * GPU (without SV_FLAG_SPECIALISE a complex64 state of at most 13 qubits on
+ * the default tile runs them in one launch), phases = register phases of the gate-list parts, ops = their kernel
  * ops, dense = parts run as fused unitaries on the tensor cores (any output
  * pointer may be NULL). Compiles on the host if needed; no device work. */
 sv_status sv_plan_stats(sv_plan *p, sv_precision prec, int tile_qubits, uint32_t flags, uint32_t *passes,

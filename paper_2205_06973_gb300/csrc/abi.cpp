@@ -88,12 +88,12 @@ template <typename V> static cudaError_t upload_vec(void **d, const V &v, cudaSt
     if (e == cudaSuccess) e = cudaMemcpyAsync(*d, v.data(), bytes, cudaMemcpyHostToDevice, st);
     return e;
 }
-template <typename Real> static cudaError_t upload_lowered(const Program &prog, DevProgram &d, cudaStream_t st) {
-    Lowered<Real> lo;
-    lower_program<Real>(prog, lo);
-    cudaError_t e = upload_vec(reinterpret_cast<void **>(&d.d_phases), lo.phases, st);
-    if (e == cudaSuccess) e = upload_vec(&d.d_ops, lo.ops, st);
-    if (e == cudaSuccess) e = upload_vec(&d.d_table, lo.table, st);
+static cudaError_t upload_lowered(const Program &prog, DevProgram &d, cudaStream_t st) {
+    Lowered lo;
+    lower_program(prog, lo);
+    d.parts = lo.parts;
+    cudaError_t e = upload_vec(&d.d_stream, lo.stream, st);
+    if (e == cudaSuccess) e = upload_vec(reinterpret_cast<void **>(&d.d_windows), lo.windows, st);
     cudaError_t se = cudaStreamSynchronize(st);   // lo goes out of scope
     return e == cudaSuccess ? se : e;
 }
@@ -427,12 +427,54 @@ static sv_status get_host_program(sv_plan *p, bool fp64, int t, int mode, const 
     return SV_OK;
 }
 
-// The variant of the flags on the kernels compiled for a plan (and in the
-// plan's statistics): the precision's default register bits unless given.
+// A smaller tile for a state that gives fewer than two tiles per SM, down to
+// 2^8 amplitudes and the plan's largest part.
+static int small_tiles(const sv_plan *p, int t) {
+    while (t > 8 && t > p->max_part && (p->n <= t || (1ull << (p->n - t)) < 2 * 152)) t--;
+    return t;
+}
+
+// The variant of the flags with the precision's default register bits unless
+// given (statistics, sources, flop counts).
 static int dense_mode(uint32_t flags, bool fp64) {
     const bool tc = (flags & SV_FLAG_TC_DENSE) && !fp64;
     const int R = (int)((flags >> 8) & 0xFu);
     return (tc ? 1 : 0) | ((tc && (flags & SV_FLAG_TC_PAIRS)) ? 2 : 0) | ((R ? R : part_R(fp64)) << 4);
+}
+
+// Tile (t_user, 0 = the default) and variant of the kernels that an apply (or
+// sv_plan_specialise) compiles for a plan. With tile and register bits left to the library they go by the
+// state's size (measured on layered and parameterised circuits, 20 layers):
+//  * complex64 up to 19 qubits: 2^4 amplitudes per thread instead of 2^5 give
+//    the SMs twice the warps where a pass is a tile or less per SM (14 to 19
+//    qubits: 8 to 17 % shorter applies; even at 20 and 21, 5 to 13 % longer
+//    above), and up to 17 qubits half the tile (15 to 30 % shorter at 12 to
+//    16 qubits; even at 18);
+//  * double-float: 2^3 amplitudes per thread; with 2^4 the straight-line code
+//    (about 40 instructions per amplitude and gate) outran the instruction
+//    cache (4.6 of 7 stall cycles; 25 qubits: 12.6 against 8.3 ms, on 2^12
+//    tiles, which above 21 qubits are 8 to 14 % faster than 2^11);
+//  * complex128: small states in tiles down to 2^8 amplitudes until there
+//    are two per SM (14 qubits, 20 layers: 385 -> 173 us), since an SM has
+//    about two FP64 lanes and its tiles' arithmetic sets the time.
+// Multi-level plans keep the register bits their second level may use.
+static int spec_mode(const sv_plan *p, sv_precision prec, uint32_t flags, int t_user, int &t) {
+    const bool fp64 = prec != SV_C64;
+    t = t_user ? t_user : default_tile(fp64, p->max_part);
+    int mode = dense_mode(flags, fp64);
+    if (t_user || ((flags >> 8) & 0xFu) || !p->inner.empty()) return mode;
+    int R = part_R(fp64);
+    if (!fp64) {
+        if (p->n <= 19) R = 4;
+        if (p->n <= 17 && t == 12) t = 11;
+    } else if (prec == SV_C128DF) {
+        R = 3;
+        if (p->n >= 22) t = part_tmax(true);
+    } else if (small_tiles(p, t) < t) {
+        t = small_tiles(p, t);
+        R = 3;
+    }
+    return (mode & 15) | (R << 4);
 }
 
 // Tile and variant of an apply on the interpreter (no register bits given).
@@ -443,7 +485,7 @@ static int dense_mode(uint32_t flags, bool fp64) {
 //  * A small complex128 state is cut into tiles down to 2^8 amplitudes until
 //    there are two per SM: an SM has about two FP64 lanes, so its tiles'
 //    arithmetic sets the time, and 14 qubits on 2^11 tiles keep 8 of 152 SMs
-//    busy (the 840-gate layered circuit: 1.11 ms; 2^8 tiles: see DESIGN).
+//    busy (the 840-gate layered circuit: 1.11 ms; on 2^8 tiles 0.49 ms).
 static int interp_mode(const sv_plan *p, bool fp64, uint32_t flags, int t_user, int &t) {
     const int tc = dense_mode(flags, fp64) & 3;
     const bool ml = !p->inner.empty();
@@ -455,7 +497,7 @@ static int interp_mode(const sv_plan *p, bool fp64, uint32_t flags, int t_user, 
         return kModeWhole | (R << 4);
     }
     if (fp64) {
-        while (t > 8 && t > p->max_part && (p->n <= t || (1ull << (p->n - t)) < 2 * 152)) t--;
+        t = small_tiles(p, t);
     } else if (t == 12 && p->max_part < 12 && p->n < t + 6) {
         t = 11;   // fewer than 64 tiles: halves (16 qubits, 15 layers, k = 10: 110 -> 94 us)
     }
@@ -468,6 +510,7 @@ sv_status sv_plan_stats(sv_plan *p, sv_precision prec, int t, uint32_t flags, ui
     const bool fp64 = prec != SV_C64;
     if (t == 0) t = default_tile(fp64, p->max_part);
     if (t < part_tmin() || t > part_tmax(fp64)) return fail(SV_ERR_ARG, "tile_qubits out of range");
+    const int mode = dense_mode(flags, fp64);
     if (p->method == SV_PART_NONE || p->n < part_tmin() || (flags & SV_FLAG_GATEWISE)) {
         if (passes) *passes = (uint32_t)p->gates.size();
         if (phases) *phases = 0;
@@ -476,7 +519,7 @@ sv_status sv_plan_stats(sv_plan *p, sv_precision prec, int t, uint32_t flags, ui
         return SV_OK;
     }
     const Program *prog = nullptr;
-    sv_status st = get_host_program(p, fp64, t, dense_mode(flags, fp64), &prog);
+    sv_status st = get_host_program(p, fp64, t, mode, &prog);
     if (st != SV_OK) return st;
     if (passes) *passes = (uint32_t)prog->kind.size();
     if (phases) *phases = (uint32_t)prog->phases.size();
@@ -506,14 +549,14 @@ static sv_status get_jit_program(sv_plan *p, sv_precision prec, int t, int mode,
 sv_status sv_plan_specialise(sv_plan *p, sv_precision prec, int t, uint32_t flags, int load, double *compile_s) {
     if (!p) return fail(SV_ERR_ARG, "plan is NULL");
     const bool fp64 = prec != SV_C64;
-    if (t == 0) t = default_tile(fp64, p->max_part);
-    if (t < part_tmin() || t > part_tmax(fp64)) return fail(SV_ERR_ARG, "tile_qubits out of range");
+    if (t != 0 && (t < part_tmin() || t > part_tmax(fp64))) return fail(SV_ERR_ARG, "tile_qubits out of range");
+    const int mode = spec_mode(p, prec, flags, t, t);
     const Program *hp = nullptr;
-    sv_status st = get_host_program(p, fp64, t, dense_mode(flags, fp64), &hp);
+    sv_status st = get_host_program(p, fp64, t, mode, &hp);
     if (st != SV_OK) return st;
     if (load) {
         JitProgram *jp = nullptr;
-        st = get_jit_program(p, prec, t, dense_mode(flags, fp64), hp, &jp);
+        st = get_jit_program(p, prec, t, mode, hp, &jp);
         if (st != SV_OK) return st;
         if (compile_s) *compile_s = jp->compile_s;
         return SV_OK;
@@ -532,8 +575,9 @@ sv_status sv_plan_source(sv_plan *p, sv_precision prec, int t, uint32_t flags, u
     const bool fp64 = prec != SV_C64;
     if (t == 0) t = default_tile(fp64, p->max_part);
     if (t < part_tmin() || t > part_tmax(fp64)) return fail(SV_ERR_ARG, "tile_qubits out of range");
+    const int mode = dense_mode(flags, fp64);
     const Program *hp = nullptr;
-    sv_status st = get_host_program(p, fp64, t, dense_mode(flags, fp64), &hp);
+    sv_status st = get_host_program(p, fp64, t, mode, &hp);
     if (st != SV_OK) return st;
     if (part >= hp->parts.size()) return fail(SV_ERR_ARG, "part index out of range");
     const std::string src = jit_part_source(*hp, part, prec == SV_C128DF);
@@ -552,13 +596,14 @@ sv_status sv_plan_flops(sv_plan *p, sv_precision prec, int t, uint32_t flags, do
     const bool fp64 = prec != SV_C64;
     if (t == 0) t = default_tile(fp64, p->max_part);
     if (t < part_tmin() || t > part_tmax(fp64)) return fail(SV_ERR_ARG, "tile_qubits out of range");
+    const int mode = dense_mode(flags, fp64);
     double a = 0.0, b = 0.0;
     if (p->method == SV_PART_NONE || p->n < part_tmin() || (flags & SV_FLAG_GATEWISE)) {
         // one general matrix per gate: 14 flops per amplitude for a 2x2, 30 for a 4x4
         for (const GateRef &g : p->gates) a += g.arity == 1 ? 14.0 : 30.0;
     } else {
         const Program *hp = nullptr;
-        sv_status st = get_host_program(p, fp64, t, dense_mode(flags, fp64), &hp);
+        sv_status st = get_host_program(p, fp64, t, mode, &hp);
         if (st != SV_OK) return st;
         program_flops(*hp, a, b);
     }
@@ -575,9 +620,8 @@ sv_status sv_plan_destroy(sv_plan *p) {
     cudaGetDevice(&cur);
     for (auto &kv : p->dev_progs) {   // no apply of the plan may be in flight
         cudaSetDevice(kv.second.dev);
-        dev_free(kv.second.d_phases, 0);
-        dev_free(kv.second.d_ops, 0);
-        dev_free(kv.second.d_table, 0);
+        dev_free(kv.second.d_stream, 0);
+        dev_free(kv.second.d_windows, 0);
         dev_free(kv.second.d_aimg, 0);
         dev_free(kv.second.d_pimg, 0);
         dev_free(kv.second.d_small, 0);
@@ -588,9 +632,8 @@ sv_status sv_plan_destroy(sv_plan *p) {
 }
 
 static void free_dev(DevProgram &d, cudaStream_t st) {
-    dev_free(d.d_phases, st);
-    dev_free(d.d_ops, st);
-    dev_free(d.d_table, st);
+    dev_free(d.d_stream, st);
+    dev_free(d.d_windows, st);
     dev_free(d.d_aimg, st);
     dev_free(d.d_pimg, st);
 }
@@ -610,7 +653,7 @@ static sv_status get_dev_program(sv_state *s, sv_plan *p, int t, int mode, const
         cudaError_t e = upload_vec(reinterpret_cast<void **>(&d.d_aimg), prog.a_img, s->stream);
         if (e == cudaSuccess) e = upload_vec(reinterpret_cast<void **>(&d.d_pimg), prog.pair_img, s->stream);
         if (e == cudaSuccess && !(mode & kModeJit))
-            e = fp64 ? upload_lowered<double>(prog, d, s->stream) : upload_lowered<float>(prog, d, s->stream);
+            e = upload_lowered(prog, d, s->stream);
         // the program is shared by every state that applies the plan, on any
         // stream: it is complete before it is published
         if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
@@ -718,8 +761,8 @@ sv_status sv_apply_parts(sv_state *s, sv_plan *p, uint32_t flags) {
     } else {
         const bool fp64 = is_fp64(s);
         const bool jit = (flags & SV_FLAG_SPECIALISE) != 0;
-        int t = s->tile ? s->tile : default_tile(fp64, p->max_part);
-        const int mode = jit ? dense_mode(flags, fp64) : interp_mode(p, fp64, flags, s->tile, t);
+        int t = 0;
+        const int mode = jit ? spec_mode(p, s->prec, flags, s->tile, t) : interp_mode(p, fp64, flags, s->tile, t);
         const Program *hp = nullptr;
         const DevProgram *dp = nullptr;
         st = get_dev_program(s, p, t, mode | (jit ? kModeJit : 0), &hp, &dp);
@@ -753,8 +796,8 @@ sv_status sv_apply_parts(sv_state *s, sv_plan *p, uint32_t flags) {
             if (hp->kind[i] == 0 && jp)
                 e = jit_launch(*jp, j, s->buf, hp->n_tiles[j], s->stream);
             else if (hp->kind[i] == 0)
-                e = (fp64 ? launch_part_f64 : launch_part_f32)(hp->t, hp->R, s->buf, hp->parts[j], dp->d_phases,
-                                                               dp->d_ops, dp->d_table, hp->n_tiles[j], s->stream);
+                e = (fp64 ? launch_part_f64 : launch_part_f32)(hp->t, hp->R, s->buf, dp->parts[j], dp->d_stream,
+                                                               dp->d_windows, hp->n_tiles[j], s->stream);
             else if (hp->kind[i] == 1)
                 e = launch_dense6(s->buf, hp->dense[j], dp->d_aimg + (size_t)j * DENSE_A_BYTES, hp->dense_tiles[j],
                                   s->d_err, s->d_dnorm, didx++, s->stream);

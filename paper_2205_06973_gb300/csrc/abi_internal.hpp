@@ -32,9 +32,9 @@ void set_last_error(const std::string &msg);
 
 struct DevProgram {
     int dev = -1;
-    hisv::IPhase *d_phases = nullptr;   // the interpreter's program (interp.hpp)
-    void *d_ops = nullptr;
-    void *d_table = nullptr;
+    void *d_stream = nullptr;       // the interpreter's program (interp.hpp), its windows
+    hisv::IWindow *d_windows = nullptr;
+    std::vector<hisv::PartLaunch> parts;   // and its parts (launch arguments)
     uint8_t *d_aimg = nullptr;      // R images of the dense parts
     uint8_t *d_pimg = nullptr;      // R images of the dense pairs (two per pass)
     void *d_small = nullptr;        // gate records of a circuit on fewer than 10 qubits

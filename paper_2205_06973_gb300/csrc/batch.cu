@@ -52,9 +52,9 @@ __device__ __forceinline__ uint64_t deposit_b(uint64_t v, uint64_t mask) {
 __global__ void __launch_bounds__(256) k_batch(float2 *__restrict__ svbase, const BatchItem *__restrict__ items,
                                               uint32_t n_items, const uint64_t *__restrict__ circ_off,
                                               const PartLaunch *__restrict__ parts,
-                                              const IPhase *__restrict__ phases, const IOp<float> *__restrict__ ops,
-                                              const float *__restrict__ table, uint32_t *__restrict__ done,
-                                              uint32_t *__restrict__ head, int *__restrict__ err) {
+                                              const uint4 *__restrict__ stream, const IWindow *__restrict__ windows,
+                                              uint32_t *__restrict__ done, uint32_t *__restrict__ head,
+                                              int *__restrict__ err) {
     extern __shared__ __align__(16) float2 bsm[];
     const int lane = threadIdx.x & 31;
     float2 *const wsm = bsm + (threadIdx.x >> 5) * (1 << BT);
@@ -110,20 +110,12 @@ __global__ void __launch_bounds__(256) k_batch(float2 *__restrict__ svbase, cons
             }
             __syncwarp();
             float tpr = 1.0f, tpi = 0.0f;
+            uint32_t tsg = 0u;
             Slots<BR, BT - BR> S;
-            for (uint32_t p = 0; p < P.n_phases; p++) {
-                const IPhase *const ph = phases + P.phase_begin + p;
-                const uint2 span = __ldg(reinterpret_cast<const uint2 *>(&ph->op_begin));
-                if (p > 0) {   // transpose through the warp's shared tile
-                    __syncwarp();
-#pragma unroll
-                    for (int i = 0; i < BNR; i++) wsm[S.at(i)] = a[i];
-                    __syncwarp();
-                }
-                S.load(ph, lane);
-#pragma unroll
-                for (int i = 0; i < BNR; i++) a[i] = wsm[S.at(i)];
-                run_ops<float, BR>(a, ops + span.x, span.y, table, lane, tpr, tpi);
+            for (uint32_t w = 0; w < P.n_phases; w++) {   // read in place: a warp's items share few programs
+                const IWindow W = windows[P.phase_begin + w];
+                run_window<float, BR, BT - BR>(a, wsm, S, reinterpret_cast<const char *>(stream + W.at), W.phases, w == 0,
+                                               lane, tpr, tpi, tsg, [] { __syncwarp(); });
             }
             if (P.flags & PL_STORE_FACTOR) {
                 const float gr = (float)P.gr, gi = (float)P.gi;
@@ -161,62 +153,56 @@ __global__ void __launch_bounds__(256) k_batch(float2 *__restrict__ svbase, cons
 // parts of a few tiles each, every part a trip through L2 and the work queue
 // with little for the other warps to do: 45 parameterised circuits of 10 to
 // 12 qubits took 3.2 ms.
-template <int T>
-__global__ void __launch_bounds__(1 << (T - BR))
+template <int T, int R>
+__global__ void __launch_bounds__(1 << (T - R))
 k_batch_whole(float2 *__restrict__ svbase, const BatchWhole *__restrict__ circuits,
-              const PartLaunch *__restrict__ parts, const IPhase *__restrict__ phases,
-              const IOp<float> *__restrict__ ops, const float *__restrict__ table) {
-    constexpr int TB = T - BR;
+              const PartLaunch *__restrict__ parts, const uint4 *__restrict__ stream,
+              const IWindow *__restrict__ windows) {
+    constexpr int TB = T - R, NR = 1 << R;
     extern __shared__ __align__(16) float2 bsm[];
+    char *const prog = reinterpret_cast<char *>(bsm + (1 << T));   // INTERP_WINDOW bytes
     const uint32_t tid = threadIdx.x;
-    const BatchWhole W = circuits[blockIdx.x];
-    const PartLaunch &P = parts[W.part];
-    float2 *const sv = svbase + W.sv_off;
+    const BatchWhole C = circuits[blockIdx.x];
+    const PartLaunch &P = parts[C.part];
+    float2 *const sv = svbase + C.sv_off;
     uint32_t s_cthr = 0;
 #pragma unroll
     for (int j = 0; j < TB; j++)
         if ((tid >> j) & 1) s_cthr ^= swz<float>(j);
 #pragma unroll
-    for (int i = 0; i < BNR; i++) {
+    for (int i = 0; i < NR; i++) {
         uint32_t so = s_cthr;
 #pragma unroll
-        for (int b = 0; b < BR; b++)
+        for (int b = 0; b < R; b++)
             if (i & (1 << b)) so ^= swz<float>(TB + b);
         bsm[so] = __ldcg(sv + (tid | ((uint32_t)i << TB)));
     }
-    __syncthreads();
-    float2 a[BNR];
+    float2 a[NR];
     float tpr = 1.0f, tpi = 0.0f;
-    Slots<BR, TB> S;
-    for (uint32_t p = 0; p < P.n_phases; p++) {
-        const IPhase *const ph = phases + P.phase_begin + p;
-        const uint2 span = __ldg(reinterpret_cast<const uint2 *>(&ph->op_begin));
-        if (p > 0) {
-            __syncthreads();
-#pragma unroll
-            for (int i = 0; i < BNR; i++) bsm[S.at(i)] = a[i];
-            __syncthreads();
-        }
-        S.load(ph, tid);
-#pragma unroll
-        for (int i = 0; i < BNR; i++) a[i] = bsm[S.at(i)];
-        run_ops<float, BR>(a, ops + span.x, span.y, table, tid, tpr, tpi);
+    uint32_t tsg = 0u;
+    Slots<R, TB> S;
+    for (uint32_t w = 0; w < P.n_phases; w++) {
+        const IWindow W = windows[P.phase_begin + w];
+        if (w > 0) __syncthreads();   // every thread is done with the previous window
+        copy_window(prog, stream, W, tid, 1u << TB);
+        __syncthreads();
+        run_window<float, R, TB>(a, bsm, S, prog, W.phases, w == 0, tid, tpr, tpi, tsg, [] { __syncthreads(); });
     }
     if (P.flags & PL_STORE_FACTOR) {
         const float gr = (float)P.gr, gi = (float)P.gi;
         const float fr = gr * tpr - gi * tpi, fi = gr * tpi + gi * tpr;
 #pragma unroll
-        for (int i = 0; i < BNR; i++) cmul_in(a[i], fr, fi);
+        for (int i = 0; i < NR; i++) cmul_in(a[i], fr, fi);
     }
     uint32_t toff = 0;
 #pragma unroll
     for (int j = 0; j < TB; j++)
         if ((tid >> j) & 1) toff |= 1u << P.store_thr_q[j];
 #pragma unroll
-    for (int i = 0; i < BNR; i++) {
+    for (int i = 0; i < NR; i++) {
         uint32_t off = toff;
 #pragma unroll
-        for (int b = 0; b < BR; b++)
+        for (int b = 0; b < R; b++)
             if (i & (1 << b)) off |= 1u << P.store_reg_q[b];
         __stcg(sv + off, a[i]);
     }
@@ -330,18 +316,23 @@ cudaError_t batch_prepare(int warps_per_cta, int *n_ctas) {
 
 cudaError_t launch_batch(const BatchLaunch &B, int warps_per_cta, int n_ctas, cudaStream_t st) {
     const size_t smem = (size_t)warps_per_cta * (1u << BT) * sizeof(float2);
-    k_batch<<<n_ctas, warps_per_cta * 32, smem, st>>>(B.svbase, B.items, B.n_items, B.circ_off, B.parts, B.phases,
-                                                      B.ops, B.table, B.done, B.head, B.err);
+    k_batch<<<n_ctas, warps_per_cta * 32, smem, st>>>(B.svbase, B.items, B.n_items, B.circ_off, B.parts, B.stream,
+                                                      B.windows, B.done, B.head, B.err);
     return cudaGetLastError();
 }
 
+template <int T>
+static void whole_t(const BatchLaunch &B, const BatchWhole *circuits, uint32_t n, cudaStream_t st) {
+    constexpr int R = batch_whole_R(T);
+    const size_t smem = (sizeof(float2) << T) + INTERP_WINDOW;
+    k_batch_whole<T, R><<<n, 1u << (T - R), smem, st>>>(B.svbase, circuits, B.parts, B.stream, B.windows);
+}
+
 cudaError_t launch_batch_whole(int t, const BatchLaunch &B, const BatchWhole *circuits, uint32_t n, cudaStream_t st) {
-    const size_t smem = sizeof(float2) << t;
-    const unsigned threads = 1u << (t - BR);
     switch (t) {
-    case 10: k_batch_whole<10><<<n, threads, smem, st>>>(B.svbase, circuits, B.parts, B.phases, B.ops, B.table); break;
-    case 11: k_batch_whole<11><<<n, threads, smem, st>>>(B.svbase, circuits, B.parts, B.phases, B.ops, B.table); break;
-    case 12: k_batch_whole<12><<<n, threads, smem, st>>>(B.svbase, circuits, B.parts, B.phases, B.ops, B.table); break;
+    case 10: whole_t<10>(B, circuits, n, st); break;
+    case 11: whole_t<11>(B, circuits, n, st); break;
+    case 12: whole_t<12>(B, circuits, n, st); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

@@ -33,9 +33,8 @@ struct BatchLaunch {
     uint32_t n_items;
     const uint64_t *circ_off;    // first amplitude of each circuit's state
     const PartLaunch *parts;     // all circuits' parts (tile of 2^9 amplitudes)
-    const IPhase *phases;        // lowered programs (interp.hpp)
-    const IOp<float> *ops;
-    const float *table;
+    const uint4 *stream;         // lowered programs (interp.hpp)
+    const IWindow *windows;
     uint32_t *done;              // per-circuit finished-tile counters (zeroed per run)
     uint32_t *head;              // queue ticket (zeroed per run)
     int *err;                    // bounded-wait failure flag
@@ -47,6 +46,9 @@ constexpr int BATCH_MIN_QUBITS = 10;
 // Circuits of at most this many qubits run on one CTA each: a 12-qubit state
 // is 32 KiB of shared memory for 256 threads, so several share an SM.
 constexpr int BATCH_WHOLE_QUBITS = 12;
+// Their register bits: a 10-qubit state on 2^4 amplitudes per thread would
+// leave two of the SM's four schedulers without a warp.
+constexpr int batch_whole_R(int n) { return n < 12 ? 3 : BATCH_REG_BITS; }
 
 // Raise the shared-memory limit and return the persistent grid size (CTAs
 // resident on all SMs) for a CTA of warps_per_cta warps.

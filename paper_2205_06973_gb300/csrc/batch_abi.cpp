@@ -39,8 +39,11 @@ struct sv_batch {
     cudaStream_t prep = nullptr;         // private: allocations, uploads and the graph capture, so that
                                          // building a batch never enqueues on (or captures) a stream that
                                          // another thread uses for earlier batches
-    cudaStream_t side = nullptr;         // second branch of the capture, with its fork and join
-    cudaEvent_t fork = nullptr, join = nullptr;
+    // further branches of the capture (one per size of the whole circuits)
+    // with their fork and joins
+    static constexpr int SIDES = BATCH_WHOLE_QUBITS - BATCH_MIN_QUBITS + 1;
+    cudaStream_t side[SIDES] = {};
+    cudaEvent_t fork = nullptr, join[SIDES] = {};
     int warps = 8;                       // warps per CTA
     int chunk = 0;                       // tiles per queue item (0 = by the batch's size)
     bool hold_last = false;              // testing: the last item waits for tiles that never complete
@@ -84,9 +87,11 @@ static void drop_program(sv_batch *b) {
 
 static void drop_streams(sv_batch *b) {
     if (b->prep) cudaStreamDestroy(b->prep);
-    if (b->side) cudaStreamDestroy(b->side);
     if (b->fork) cudaEventDestroy(b->fork);
-    if (b->join) cudaEventDestroy(b->join);
+    for (int i = 0; i < sv_batch::SIDES; i++) {
+        if (b->side[i]) cudaStreamDestroy(b->side[i]);
+        if (b->join[i]) cudaEventDestroy(b->join[i]);
+    }
 }
 
 extern "C" {
@@ -114,9 +119,11 @@ sv_status sv_batch_create(uint32_t n_circuits, const int *n_qubits, void *stream
     }
     {
         cudaError_t pe = cudaStreamCreateWithFlags(&b->prep, cudaStreamNonBlocking);
-        if (pe == cudaSuccess) pe = cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking);
         if (pe == cudaSuccess) pe = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
-        if (pe == cudaSuccess) pe = cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming);
+        for (int i = 0; pe == cudaSuccess && i < sv_batch::SIDES; i++) {
+            pe = cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking);
+            if (pe == cudaSuccess) pe = cudaEventCreateWithFlags(&b->join[i], cudaEventDisableTiming);
+        }
         if (pe != cudaSuccess) {
             drop_streams(b.get());
             if (b->own_stream) cudaStreamDestroy(b->stream);
@@ -266,8 +273,7 @@ static sv_status build_program(sv_batch *b) {
     }
     int dev = 0;
     BCUDA(cudaGetDevice(&dev));
-    std::vector<Program> gl(b->n);                 // gate-list programs (circuits not on the dense kernel)
-    std::vector<Lowered<float>> lowered(b->n);
+    std::vector<Lowered> lowered(b->n);            // gate-list programs (circuits not on the dense kernel)
     // the failure test holds back a work item, so it keeps the work queue
     auto whole = [&](uint32_t c) { return !D.dense[c] && b->nq[c] <= BATCH_WHOLE_QUBITS && !b->hold_last; };
     std::vector<DenseBatchPart> dparts(D.n_parts);
@@ -281,11 +287,13 @@ static sv_status build_program(sv_batch *b) {
                 // a circuit that one CTA holds: all gates as one part
                 const bool w = whole(c);
                 const std::vector<uint32_t> one(w ? p->gates.size() : 0, 0u);
+                Program pr;
                 if (!compile_program(p->gates, p->n, w ? one : p->pog, w ? 1u : p->n_parts, false,
-                                     w ? p->n : BATCH_TILE_QUBITS, BATCH_REG_BITS, 0, gl[c], errs[c])) {
+                                     w ? p->n : BATCH_TILE_QUBITS, w ? batch_whole_R(p->n) : BATCH_REG_BITS, 0, pr,
+                                     errs[c])) {
                     if (errs[c].empty()) errs[c] = "compile failed";
                 } else {
-                    lower_program<float>(gl[c], lowered[c]);
+                    lower_program(pr, lowered[c]);
                 }
                 continue;
             }
@@ -342,9 +350,8 @@ static sv_status build_program(sv_batch *b) {
         b->n_dense_circ = D.n_circ;
     }
     std::vector<PartLaunch> parts;
-    std::vector<IPhase> phases;
-    std::vector<IOp<float>> ops;
-    std::vector<float> table;
+    std::vector<uint32_t> stream;
+    std::vector<IWindow> windows;
     std::vector<uint32_t> part_base(b->n), n_parts(b->n);
     std::vector<BatchWhole> wholes[BATCH_WHOLE_QUBITS + 1];   // by qubit count
     uint32_t maxP = 0, n_whole = 0, whole_parts = 0;
@@ -354,33 +361,28 @@ static sv_status build_program(sv_batch *b) {
             n_parts[c] = 0;
             continue;
         }
-        const Program &prog = gl[c];
-        const Lowered<float> &lo = lowered[c];
-        const uint32_t ph0 = (uint32_t)phases.size(), op0 = (uint32_t)ops.size(), tb0 = (uint32_t)table.size();
+        const Lowered &lo = lowered[c];
+        const uint32_t w0 = (uint32_t)windows.size(), at0 = (uint32_t)(stream.size() / 4);
         part_base[c] = (uint32_t)parts.size();
         if (whole(c)) {
             n_parts[c] = 0;
-            if (!prog.parts.empty()) wholes[b->nq[c]].push_back({b->off[c], part_base[c], 0});
+            if (!lo.parts.empty()) wholes[b->nq[c]].push_back({b->off[c], part_base[c], 0});
             n_whole++;
             whole_parts += b->plans[c]->n_parts;
         } else {
-            n_parts[c] = (uint32_t)prog.parts.size();
+            n_parts[c] = (uint32_t)lo.parts.size();
             wave_tiles += 1ull << (b->nq[c] - BATCH_TILE_QUBITS);
         }
         maxP = std::max(maxP, n_parts[c]);
-        for (PartLaunch L : prog.parts) {
-            L.phase_begin += ph0;
+        for (PartLaunch L : lo.parts) {
+            L.phase_begin += w0;
             parts.push_back(L);
         }
-        for (IPhase ph : lo.phases) {
-            ph.op_begin += op0;
-            phases.push_back(ph);
+        for (IWindow w : lo.windows) {
+            w.at += at0;
+            windows.push_back(w);
         }
-        for (IOp<float> op : lo.ops) {
-            if (op.code == IM_DIAG || op.code / 8 == IK_U2) op.arg += tb0;
-            ops.push_back(op);
-        }
-        table.insert(table.end(), lo.table.begin(), lo.table.end());
+        stream.insert(stream.end(), lo.stream.begin(), lo.stream.end());
     }
     int n_ctas = 0;
     BCUDA(batch_prepare(b->warps, &n_ctas));
@@ -407,9 +409,9 @@ static sv_status build_program(sv_batch *b) {
     if (b->hold_last && !items.empty()) items.back().wait = 0xFFFFFFFFu;
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t s_items = al(items.size() * sizeof(BatchItem)), s_parts = al(parts.size() * sizeof(PartLaunch));
-    const size_t s_ph = al(phases.size() * sizeof(IPhase)), s_op = al(ops.size() * sizeof(IOp<float>));
-    const size_t s_tb = al(table.size() * sizeof(float)), s_wh = al(n_whole * sizeof(BatchWhole));
-    const size_t s_all = std::max<size_t>(256, s_items + s_parts + s_ph + s_op + s_tb + s_wh);
+    const size_t s_st = al(stream.size() * sizeof(uint32_t)), s_wi = al(windows.size() * sizeof(IWindow));
+    const size_t s_wh = al(n_whole * sizeof(BatchWhole));
+    const size_t s_all = std::max<size_t>(256, s_items + s_parts + s_st + s_wi + s_wh);
     char *d = nullptr;
     cudaError_t e = dev_alloc(reinterpret_cast<void **>(&d), s_all, b->prep);
     if (e != cudaSuccess) {
@@ -425,10 +427,9 @@ static sv_status build_program(sv_batch *b) {
     size_t at = 0;
     put(at, items.data(), items.size() * sizeof(BatchItem));
     put(at += s_items, parts.data(), parts.size() * sizeof(PartLaunch));
-    put(at += s_parts, phases.data(), phases.size() * sizeof(IPhase));
-    put(at += s_ph, ops.data(), ops.size() * sizeof(IOp<float>));
-    put(at += s_op, table.data(), table.size() * sizeof(float));
-    at += s_tb;
+    put(at += s_parts, stream.data(), stream.size() * sizeof(uint32_t));
+    put(at += s_st, windows.data(), windows.size() * sizeof(IWindow));
+    at += s_wi;
     const BatchWhole *d_whole[BATCH_WHOLE_QUBITS + 1] = {};
     for (int t = BATCH_MIN_QUBITS; t <= BATCH_WHOLE_QUBITS; t++) {
         put(at, wholes[t].data(), wholes[t].size() * sizeof(BatchWhole));
@@ -445,9 +446,8 @@ static sv_status build_program(sv_batch *b) {
     B.n_items = (uint32_t)items.size();
     B.circ_off = b->d_off;
     B.parts = reinterpret_cast<const PartLaunch *>(d + s_items);
-    B.phases = reinterpret_cast<const IPhase *>(d + s_items + s_parts);
-    B.ops = reinterpret_cast<const IOp<float> *>(d + s_items + s_parts + s_ph);
-    B.table = reinterpret_cast<const float *>(d + s_items + s_parts + s_ph + s_op);
+    B.stream = reinterpret_cast<const uint4 *>(d + s_items + s_parts);
+    B.windows = reinterpret_cast<const IWindow *>(d + s_items + s_parts + s_st);
     B.done = b->d_done;
     B.head = b->d_done + b->n;
     B.err = b->d_err;
@@ -460,13 +460,17 @@ static sv_status build_program(sv_batch *b) {
     // launched on the caller's stream
     BCUDA(cudaStreamBeginCapture(b->prep, cudaStreamCaptureModeThreadLocal));
     // the whole circuits wait for nothing: they run beside the other kernels
-    // (a second branch of the graph), where these leave room on the SMs
+    // and each other (branches of the graph), where these leave room on the
+    // SMs; they come first, the largest before the others, as their time is
+    // the latency of a circuit's gates
     cudaError_t ce = cudaSuccess;
-    if (n_whole) {
-        ce = cudaEventRecord(b->fork, b->prep);
-        if (ce == cudaSuccess) ce = cudaStreamWaitEvent(b->side, b->fork, 0);
-        for (int t = BATCH_WHOLE_QUBITS; ce == cudaSuccess && t >= BATCH_MIN_QUBITS; t--)
-            if (!wholes[t].empty()) ce = launch_batch_whole(t, B, d_whole[t], (uint32_t)wholes[t].size(), b->side);
+    if (n_whole) ce = cudaEventRecord(b->fork, b->prep);
+    for (int t = BATCH_WHOLE_QUBITS; t >= BATCH_MIN_QUBITS; t--) {
+        const int i = t - BATCH_MIN_QUBITS;
+        if (wholes[t].empty()) continue;
+        if (ce == cudaSuccess) ce = cudaStreamWaitEvent(b->side[i], b->fork, 0);
+        if (ce == cudaSuccess) ce = launch_batch_whole(t, B, d_whole[t], (uint32_t)wholes[t].size(), b->side[i]);
+        if (ce == cudaSuccess) ce = cudaEventRecord(b->join[i], b->side[i]);
     }
     if (ce == cudaSuccess) ce = cudaMemsetAsync(b->d_done, 0, sizeof(uint32_t) * (b->n + 2), b->prep);
     if (ce == cudaSuccess && b->n_dense_items) {
@@ -479,10 +483,9 @@ static sv_status build_program(sv_batch *b) {
                                      b->prep);
     }
     if (ce == cudaSuccess && B.n_items) ce = launch_batch(B, b->warps, n_ctas, b->prep);
-    if (ce == cudaSuccess && n_whole) {
-        ce = cudaEventRecord(b->join, b->side);
-        if (ce == cudaSuccess) ce = cudaStreamWaitEvent(b->prep, b->join, 0);
-    }
+    for (int i = 0; i < sv_batch::SIDES; i++)
+        if (ce == cudaSuccess && !wholes[i + BATCH_MIN_QUBITS].empty())
+            ce = cudaStreamWaitEvent(b->prep, b->join[i], 0);
     cudaGraph_t g = nullptr;
     cudaError_t ee = cudaStreamEndCapture(b->prep, &g);
     if (ce != cudaSuccess || ee != cudaSuccess) {

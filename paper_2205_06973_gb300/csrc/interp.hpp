@@ -1,10 +1,15 @@
-// The op stream that the gate-list interpreter runs: the planner's program
-// (program.hpp) lowered for a number format and register-bit count.
+// The instruction stream that the gate-list interpreter runs: the planner's
+// program (program.hpp) lowered for a number format and register-bit count.
 //
-// An op is one record (16 bytes for float) with its opcode, thread condition
-// and coefficients together, so that a warp fetches an op with one load; the
+// A part's phases follow one another in the stream, each as a header with its
+// shared-memory layout, its op records and the tables these refer to. An op
+// is one record (16 bytes for float) with its opcode, thread condition and
+// coefficients together, so that a warp fetches an op with one load; the
 // opcode holds the register bit, so that the kernel reaches the op's code
-// with one indirect branch.
+// with one indirect branch. The stream is cut into windows that a CTA copies
+// into shared memory as a whole: read from global memory op by op, a circuit
+// that is run once waits for L2 at every eighth op and at every table (16
+// parameterised 10-qubit circuits of up to 50 layers, a CTA each: 0.38 ms).
 #pragma once
 #include <cstdint>
 #include <vector>
@@ -14,12 +19,12 @@
 namespace hisv {
 
 // Opcode = kind * 8 + register bit; IK_CP = kind * 8 + index of the register
-// bit pair (a < b): b (b - 1) / 2 + a (up to 15 pairs, two opcode rows).
+// bit pair (a < b): b (b - 1) / 2 + a (up to 10 pairs, two opcode rows).
 enum InterpKind : uint32_t {
     IK_H = 0,
     IK_RX0, IK_RX1,   // OP_RXS forms; c[0] = t
     IK_RY0, IK_RY1,   // OP_RYS forms; c[0] = t
-    IK_U2,            // [[1, u], [v, w]]; table[arg..]: u, v, w (re, im)
+    IK_U2,            // [[1, u], [v, w]]; table: u, v, w (re, im)
     IK_SWAP,          // exchange the halves where the conditions hold: X, CX, CXT
     IK_P,             // phase c on the set half where the thread condition holds
     IK_CP, IK_CP2,    // phase c where both register bits are set
@@ -27,7 +32,7 @@ enum InterpKind : uint32_t {
 };
 enum InterpMisc : uint32_t {
     IM_TPH = IK_MISC * 8,   // per-thread phase *= c where the thread condition holds
-    IM_DIAG,                // register amplitude i *= table[arg + 2 i] (re, im)
+    IM_DIAG,                // register amplitude i *= table[2 i], table[2 i + 1] (re, im)
     IM_TAPPLY,              // multiply by the per-thread phase, reset it
     IM_TSG,                 // per-thread sign flips where the thread condition holds
     IM_TSAPPLY,             // negate where the per-thread sign is set, reset it
@@ -35,33 +40,45 @@ enum InterpMisc : uint32_t {
 };
 
 // arg: low half = thread-bit mask (all set: the condition holds; 0 = always),
-// high half = register mask of IK_SWAP and IM_SIGN; for IK_U2 and IM_DIAG the
-// table index (in reals).
+// high half = register mask of IK_SWAP and IM_SIGN; for IK_U2 and IM_DIAG
+// the table's distance in bytes from the phase's header.
 template <typename Real> struct alignas(16) IOp {
     uint32_t code;
     uint32_t arg;
-    Real c[2];
+    alignas(2 * sizeof(Real) < 16 ? 8 : 16) Real c[2];
 };
 static_assert(sizeof(IOp<float>) == 16 && sizeof(IOp<double>) == 32, "IOp layout");
 
-// A register phase with its shared-memory layout: swizzled offsets of the
-// register and thread bits.
+// Header of a register phase: swizzled offsets of the register and thread
+// bits in the tile's buffer, then n_ops op records and the tables. A phase
+// whose ops do not fit a window is continued (IPH_CONT) under a second
+// header with the same layout and no transpose in between.
 struct alignas(16) IPhase {
     uint16_t sreg[8];
     uint16_t sthr[MAX_TB];
-    uint32_t op_begin;
-    uint32_t op_count;
-    uint32_t pad[2];
+    uint32_t n_ops;
+    uint32_t bytes;      // header, ops and tables: the next header follows
+    uint32_t flags;
+    uint32_t pad;
 };
 static_assert(sizeof(IPhase) == 64, "IPhase layout");
+constexpr uint32_t IPH_CONT = 1u;
+
+struct IWindow {
+    uint32_t at;         // in 16-byte units from the stream's start
+    uint32_t bytes;      // at most INTERP_WINDOW, a multiple of 16
+    uint32_t phases;     // headers
+    uint32_t pad;
+};
+constexpr uint32_t INTERP_WINDOW = 8192;
 
 struct Program;
-template <typename Real> struct Lowered {
-    std::vector<IPhase> phases;
-    std::vector<IOp<Real>> ops;
-    std::vector<Real> table;   // 16-byte aligned entries (IM_DIAG, IK_U2)
+struct Lowered {
+    std::vector<uint32_t> stream;
+    std::vector<IWindow> windows;
+    // the program's parts with phase_begin / n_phases = first window / windows
+    std::vector<PartLaunch> parts;
 };
-// Lower every phase of the program (its parts keep their phase indices).
-template <typename Real> void lower_program(const Program &prog, Lowered<Real> &out);
+void lower_program(const Program &prog, Lowered &out);
 
 }  // namespace hisv

@@ -171,6 +171,8 @@ std::string jit_part_source(const Program &prog, size_t pi, bool df) {
     o << "    C a[NR];\n"
       << "    u64 tile = blockIdx.x;\n"
       << "    u64 base = tile < n_tiles ? deposit64(tile, OUTER) : 0ull;\n"
+      << "    const u64 DGRID = deposit64(gridDim.x, OUTER);\n"
+      << "    pdl_wait();\n"
       << "    if (tile < n_tiles) {\n"
       << "        const C *src = sv + (base | c_thr);\n"
       << "#pragma unroll\n"
@@ -182,12 +184,12 @@ std::string jit_part_source(const Program &prog, size_t pi, bool df) {
       << "        C *const nxt = (it & 1) ? buf0 : buf1;\n"
       << "        __syncthreads();\n"
       << "        const u64 ntile = tile + gridDim.x;\n"
-      << "        const u64 nbase = ntile < n_tiles ? deposit64(ntile, OUTER) : 0ull;\n"
+      << "        const u64 nbase = ((base | ~OUTER) + DGRID) & OUTER;\n"   // carries run over the tile's qubits
       << "        if (ntile < n_tiles) {\n"
       << "            const C *src = sv + (nbase | c_thr);\n"
       << "#pragma unroll\n"
       << "            for (int i = 0; i < NR; i++) cp_async(nxt + (s_cthr ^ SO[i]), src + GO[i]);\n"
-      << "        }\n"
+      << "        } else pdl_launch();\n"
       << "        cp_commit();\n"
       << "        cp_wait1();\n"
       << "        __syncthreads();\n"
@@ -473,8 +475,19 @@ cudaError_t jit_launch(JitProgram &jp, size_t i, void *sv, uint64_t n_tiles, cud
     if (grid < 1) grid = 1;
     unsigned long long nt = n_tiles;
     void *args[2] = {&sv, &nt};
-    e = cudaLaunchKernel(reinterpret_cast<const void *>(jp.kern[i]), dim3((unsigned)grid), dim3(jp.threads), args,
-                         jp.smem, st);
+    // programmatic dependent launch: the next pass launches and runs its
+    // prologue while this one's last tiles are computed (see k_part)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(jp.threads);
+    cfg.dynamicSmemBytes = jp.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(jp.kern[i]), args);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }

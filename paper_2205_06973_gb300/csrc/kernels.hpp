@@ -18,12 +18,12 @@ inline int part_tmin() { return 10; }
 inline int part_tmax(bool fp64) { return fp64 ? 12 : 13; }
 
 // One pass of a part over the whole state (Algorithm 1) on the interpreter:
-// n_tiles = 2^(n - t) tiles, R register bits; phases, ops and table are the
-// lowered program (interp.hpp) in device memory.
-cudaError_t launch_part_f32(int t, int R, void *sv, const PartLaunch &L, const IPhase *phases, const void *ops,
-                            const void *table, uint64_t n_tiles, cudaStream_t st);
-cudaError_t launch_part_f64(int t, int R, void *sv, const PartLaunch &L, const IPhase *phases, const void *ops,
-                            const void *table, uint64_t n_tiles, cudaStream_t st);
+// n_tiles = 2^(n - t) tiles, R register bits; L is a lowered part, stream and
+// windows the lowered program (interp.hpp) in device memory.
+cudaError_t launch_part_f32(int t, int R, void *sv, const PartLaunch &L, const void *stream, const IWindow *windows,
+                            uint64_t n_tiles, cudaStream_t st);
+cudaError_t launch_part_f64(int t, int R, void *sv, const PartLaunch &L, const void *stream, const IWindow *windows,
+                            uint64_t n_tiles, cudaStream_t st);
 
 // Plain one-pass-per-gate kernels (Sec. III-A): m is the 2x2 (8 reals) or 4x4
 // (32 reals, local index l = b_q0 + 2 b_q1) complex matrix, row-major (re, im).

@@ -29,8 +29,9 @@ template <typename Real> struct CT;
 template <> struct CT<float> { typedef float2 T; };
 template <> struct CT<double> { typedef double2 T; };
 
+// One op record; p may point to shared or global memory.
 __device__ __forceinline__ IOp<float> ld_op(const IOp<float> *p) {
-    const float4 v = __ldg(reinterpret_cast<const float4 *>(p));
+    const float4 v = *reinterpret_cast<const float4 *>(p);
     IOp<float> o;
     o.code = __float_as_uint(v.x);
     o.arg = __float_as_uint(v.y);
@@ -39,13 +40,13 @@ __device__ __forceinline__ IOp<float> ld_op(const IOp<float> *p) {
     return o;
 }
 __device__ __forceinline__ IOp<double> ld_op(const IOp<double> *p) {
-    const uint2 h = __ldg(reinterpret_cast<const uint2 *>(p));
-    const double *c = reinterpret_cast<const double *>(p) + 1;
+    const uint2 h = *reinterpret_cast<const uint2 *>(p);
+    const double2 c = *reinterpret_cast<const double2 *>(&p->c[0]);
     IOp<double> o;
     o.code = h.x;
     o.arg = h.y;
-    o.c[0] = __ldg(c);
-    o.c[1] = __ldg(c + 1);
+    o.c[0] = c.x;
+    o.c[1] = c.y;
     return o;
 }
 
@@ -106,17 +107,18 @@ __device__ __forceinline__ double flip(double v, uint32_t m) {
     return __hiloint2double(__double2hiint(v) ^ (int)m, __double2loint(v));
 }
 
+// The ops of one phase header (hdr: in shared or global memory).
 template <typename Real, int R>
-__device__ __forceinline__ void run_ops(typename CT<Real>::T (&a)[1 << R], const IOp<Real> *__restrict__ ops,
-                                        uint32_t count, const Real *__restrict__ table, uint32_t tid, Real &tpr,
-                                        Real &tpi) {
+__device__ __forceinline__ void run_ops(typename CT<Real>::T (&a)[1 << R], const char *hdr, uint32_t count,
+                                        uint32_t tid, Real &tpr, Real &tpi, uint32_t &tsg) {
     constexpr int NR = 1 << R;
     if (count == 0) return;
-    uint32_t tsg = 0u;   // the per-thread sign, applied within the phase
+    const IOp<Real> *const ops = reinterpret_cast<const IOp<Real> *>(hdr + sizeof(IPhase));
     IOp<Real> op = ld_op(ops);
     for (uint32_t o = 1;; o++) {
         const IOp<Real> cur = op;
         if (o < count) op = ld_op(ops + o);
+        const Real *const table = reinterpret_cast<const Real *>(hdr + cur.arg);   // IK_U2, IM_DIAG
         const uint32_t tm = cur.arg & 0xFFFFu;
         const bool tc = (tid & tm) == tm;
         switch (cur.code) {
@@ -134,8 +136,7 @@ __device__ __forceinline__ void run_ops(typename CT<Real>::T (&a)[1 << R], const
 #define HISV_RY0(B) (in_ry<NR, B, 0>(a, cur.c[0]))
 #define HISV_RY1(B) (in_ry<NR, B, 1>(a, cur.c[0]))
 #define HISV_U2(B) \
-    (op_u2s<NR, B, 0>(a, __ldg(table + cur.arg), __ldg(table + cur.arg + 1), __ldg(table + cur.arg + 2), \
-                      __ldg(table + cur.arg + 3), __ldg(table + cur.arg + 4), __ldg(table + cur.arg + 5)))
+    (op_u2s<NR, B, 0>(a, table[0], table[1], table[2], table[3], table[4], table[5]))
 #define HISV_SWAP(B) (in_swap<NR, B>(a, cur.arg >> 16, tc))
 #define HISV_P(B) (op_p<NR, B>(a, tc ? cur.c[0] : Real(1), tc ? cur.c[1] : Real(0)))
             HISV_EACH(IK_H, HISV_H)
@@ -174,19 +175,20 @@ __device__ __forceinline__ void run_ops(typename CT<Real>::T (&a)[1 << R], const
                 tpi = x * cur.c[1] + y * cur.c[0];
             }
             break;
-        case IM_DIAG: {
-            const Real *const d = table + cur.arg;
+        case IM_DIAG:
 #pragma unroll
             for (int i = 0; i < NR; i++) {
                 if constexpr (sizeof(Real) == 4) {
-                    const float2 v = __ldg(reinterpret_cast<const float2 *>(d) + i);
+                    if (i & 1) continue;
+                    const float4 v = reinterpret_cast<const float4 *>(table)[i / 2];
                     cmul_in(a[i], v.x, v.y);
+                    cmul_in(a[i + 1], v.z, v.w);
                 } else {
-                    const double2 v = __ldg(reinterpret_cast<const double2 *>(d) + i);
+                    const double2 v = reinterpret_cast<const double2 *>(table)[i];
                     cmul_in(a[i], v.x, v.y);
                 }
             }
-        } break;
+            break;
         case IM_TAPPLY:
 #pragma unroll
             for (int i = 0; i < NR; i++) cmul_in(a[i], tpr, tpi);
@@ -233,10 +235,10 @@ __device__ __forceinline__ uint32_t xor_bits(uint32_t v, const uint16_t *off) {
 // register bit.
 template <int R, int TB> struct Slots {
     uint32_t thr, reg[R];
-    __device__ __forceinline__ void load(const IPhase *__restrict__ ph, uint32_t tid) {
+    __device__ __forceinline__ void load(const char *hdr, uint32_t tid) {
         union { uint4 q[3]; uint16_t h[24]; } u;
 #pragma unroll
-        for (int i = 0; i < 3; i++) u.q[i] = __ldg(reinterpret_cast<const uint4 *>(ph) + i);
+        for (int i = 0; i < 3; i++) u.q[i] = reinterpret_cast<const uint4 *>(hdr)[i];
 #pragma unroll
         for (int b = 0; b < R; b++) reg[b] = u.h[b];
         thr = xor_bits<TB>(tid, u.h + 8);
@@ -249,5 +251,39 @@ template <int R, int TB> struct Slots {
         return o;
     }
 };
+
+// The phases of one window (w: in shared or global memory) on the tile in
+// buf. first: the tile's first phase, which loads without a transpose. sync()
+// orders the tile's threads.
+template <typename Real, int R, int TB, typename Sync>
+__device__ __forceinline__ void run_window(typename CT<Real>::T (&a)[1 << R], typename CT<Real>::T *buf,
+                                           Slots<R, TB> &S, const char *w, uint32_t n_phases, bool first,
+                                           uint32_t tid, Real &tpr, Real &tpi, uint32_t &tsg, Sync &&sync) {
+    constexpr int NR = 1 << R;
+    for (uint32_t p = 0; p < n_phases; p++) {
+        const uint4 h = *reinterpret_cast<const uint4 *>(w + 48);   // n_ops, bytes, flags
+        if (!(h.z & IPH_CONT)) {
+            if (!first) {   // transpose through shared memory: write with the previous layout
+                sync();
+#pragma unroll
+                for (int i = 0; i < NR; i++) buf[S.at(i)] = a[i];
+                sync();
+            }
+            first = false;
+            S.load(w, tid);
+#pragma unroll
+            for (int i = 0; i < NR; i++) a[i] = buf[S.at(i)];
+        }
+        run_ops<Real, R>(a, w, h.x, tid, tpr, tpi, tsg);
+        w += h.y;
+    }
+}
+
+// Copy a window into shared memory (all threads of the CTA; the caller
+// synchronises).
+__device__ __forceinline__ void copy_window(char *dst, const uint4 *__restrict__ stream, const IWindow &W, uint32_t tid,
+                                            uint32_t nt) {
+    for (uint32_t i = tid; i < W.bytes / 16; i += nt) reinterpret_cast<uint4 *>(dst)[i] = __ldg(stream + W.at + i);
+}
 
 }  // namespace hisv

@@ -115,6 +115,19 @@ __device__ __forceinline__ void op_cz(C (&a)[NR]) {
         if ((i & (1 << A)) && (i & (1 << B))) { a[i].x = -a[i].x; a[i].y = -a[i].y; }
 }
 
+// Programmatic dependent launch: wait until the previous kernel on the stream
+// has completed and its writes are visible; let the next one launch.
+__device__ __forceinline__ void pdl_wait() {
+#if defined(__CUDA_ARCH__)
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+#endif
+}
+__device__ __forceinline__ void pdl_launch() {
+#if defined(__CUDA_ARCH__)
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+#endif
+}
+
 // Every amplitude negated where neg holds (a controlled Z of two thread bits):
 // a product for single floats, selects (no FP64 work) for the wider forms.
 template <int NR, typename C>

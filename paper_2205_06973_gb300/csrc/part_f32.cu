@@ -3,21 +3,21 @@
 
 namespace hisv {
 
-cudaError_t launch_part_f32(int t, int R, void *sv, const PartLaunch &L, const IPhase *phases, const void *ops,
-                            const void *table, uint64_t n_tiles, cudaStream_t st) {
+cudaError_t launch_part_f32(int t, int R, void *sv, const PartLaunch &L, const void *stream,
+                            const IWindow *windows, uint64_t n_tiles, cudaStream_t st) {
     if (R == 4) {
         switch (t) {
-        case 10: return launch_part_t<float, 10, 4>(sv, L, phases, ops, table, n_tiles, st);
-        case 11: return launch_part_t<float, 11, 4>(sv, L, phases, ops, table, n_tiles, st);
-        case 12: return launch_part_t<float, 12, 4>(sv, L, phases, ops, table, n_tiles, st);
-        case 13: return launch_part_t<float, 13, 4>(sv, L, phases, ops, table, n_tiles, st);
+        case 10: return launch_part_t<float, 10, 4>(sv, L, stream, windows, n_tiles, st);
+        case 11: return launch_part_t<float, 11, 4>(sv, L, stream, windows, n_tiles, st);
+        case 12: return launch_part_t<float, 12, 4>(sv, L, stream, windows, n_tiles, st);
+        case 13: return launch_part_t<float, 13, 4>(sv, L, stream, windows, n_tiles, st);
         }
     } else if (R == 5) {   // multi-level plans: a second-level part may need five register qubits
         switch (t) {
-        case 10: return launch_part_t<float, 10, 5>(sv, L, phases, ops, table, n_tiles, st);
-        case 11: return launch_part_t<float, 11, 5>(sv, L, phases, ops, table, n_tiles, st);
-        case 12: return launch_part_t<float, 12, 5>(sv, L, phases, ops, table, n_tiles, st);
-        case 13: return launch_part_t<float, 13, 5>(sv, L, phases, ops, table, n_tiles, st);
+        case 10: return launch_part_t<float, 10, 5>(sv, L, stream, windows, n_tiles, st);
+        case 11: return launch_part_t<float, 11, 5>(sv, L, stream, windows, n_tiles, st);
+        case 12: return launch_part_t<float, 12, 5>(sv, L, stream, windows, n_tiles, st);
+        case 13: return launch_part_t<float, 13, 5>(sv, L, stream, windows, n_tiles, st);
         }
     }
     return cudaErrorInvalidValue;

@@ -1,5 +1,6 @@
 // k_part: one HBM pass of one part (Algorithm 1, Gather-Execute-Scatter), with
-// the part's gates interpreted from an op stream. Persistent CTAs walk the
+// the part's gates interpreted from a stream (interp.hpp) whose window the
+// CTA copies into shared memory before the first tile. Persistent CTAs walk the
 // tiles (outer assignments) with a two-stage pipeline: while tile i is
 // computed from registers, the cp.async copy of tile i + 1 streams into the
 // other shared buffer. The tile's register phases (2^R amplitudes per thread)
@@ -51,7 +52,7 @@ __device__ __forceinline__ uint64_t deposit64(uint64_t v, uint64_t mask) {
 template <typename Real, int T, int R>
 struct PartCfg {
     static constexpr int NT = 1 << (T - R);
-    static constexpr int SMEM = 2 * (1 << T) * 2 * (int)sizeof(Real);
+    static constexpr int SMEM = 2 * (1 << T) * 2 * (int)sizeof(Real) + (int)INTERP_WINDOW;
     static constexpr int REGS = sizeof(Real) == 8 ? (R == 4 ? 168 : 120) : (R == 5 ? 168 : 104);
     static constexpr int BY_REG = 65536 / (REGS * NT);
     static constexpr int BY_SMEM = (227 * 1024) / (SMEM + 1024);
@@ -62,8 +63,7 @@ struct PartCfg {
 template <typename Real, int T, int R>
 __global__ void __launch_bounds__(PartCfg<Real, T, R>::NT, PartCfg<Real, T, R>::MINB)
 k_part(typename CT<Real>::T *__restrict__ sv, const __grid_constant__ PartLaunch L,
-       const IPhase *__restrict__ phases, const IOp<Real> *__restrict__ ops, const Real *__restrict__ table,
-       uint64_t n_tiles) {
+       const uint4 *__restrict__ stream, const IWindow *__restrict__ windows, uint64_t n_tiles) {
     typedef typename CT<Real>::T C;
     constexpr int NR = 1 << R;
     constexpr int TB = T - R;
@@ -71,7 +71,10 @@ k_part(typename CT<Real>::T *__restrict__ sv, const __grid_constant__ PartLaunch
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *const buf0 = reinterpret_cast<C *>(smem_raw);
     C *const buf1 = buf0 + TILE;
+    char *const prog = reinterpret_cast<char *>(buf1 + TILE);   // INTERP_WINDOW bytes
     const uint32_t tid = threadIdx.x;
+    IWindow W = windows[L.phase_begin];
+    copy_window(prog, stream, W, tid, 1u << TB);   // ordered by the first tile's barriers
 
     // copy layout: tile index = tid | (c << TB); thread bits on the lowest slots
     uint64_t c_thr = 0, s_thr = 0;
@@ -103,7 +106,7 @@ k_part(typename CT<Real>::T *__restrict__ sv, const __grid_constant__ PartLaunch
     uint64_t tile = blockIdx.x;
     const uint64_t dgrid = deposit64(gridDim.x, L.outer_mask);
     uint64_t base = deposit64(tile, L.outer_mask);
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");   // the previous pass has written the state
+    pdl_wait();   // the previous pass has written the state
     if (tile < n_tiles) issue(base, buf0);
     cp_async_commit();
     for (uint32_t it = 0; tile < n_tiles; tile += gridDim.x, it++) {
@@ -113,28 +116,22 @@ k_part(typename CT<Real>::T *__restrict__ sv, const __grid_constant__ PartLaunch
         // the next tile's outer bits: an add whose carries run over the tile's qubits
         const uint64_t nbase = ((base | ~L.outer_mask) + dgrid) & L.outer_mask;
         if (tile + gridDim.x < n_tiles) issue(nbase, nxt);
-        else asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+        else pdl_launch();
         cp_async_commit();
         cp_async_wait<1>();  // this tile's copies have landed
         __syncthreads();
 
         Real tpr = Real(1), tpi = Real(0);   // per-thread phase of diagonal gates on thread bits
+        uint32_t tsg = 0u;                   // and its sign
         Slots<R, TB> S;
-        for (uint32_t p = 0; p < L.n_phases; p++) {
-            const IPhase *const ph = phases + L.phase_begin + p;
-            const uint2 span = __ldg(reinterpret_cast<const uint2 *>(&ph->op_begin));
-            if (p > 0) {
-                // transpose through shared memory: write with the previous layout
+        for (uint32_t w = 0; w < L.n_phases; w++) {
+            if (L.n_phases > 1 && (w > 0 || it > 0)) {   // a program of several windows
                 __syncthreads();
-#pragma unroll
-                for (int i = 0; i < NR; i++) cur[S.at(i)] = a[i];
+                W = windows[L.phase_begin + w];
+                copy_window(prog, stream, W, tid, 1u << TB);
                 __syncthreads();
             }
-            S.load(ph, tid);
-#pragma unroll
-            for (int i = 0; i < NR; i++) a[i] = cur[S.at(i)];
-            // Execute: the phase's gates
-            run_ops<Real, R>(a, ops + span.x, span.y, table, tid, tpr, tpi);
+            run_window<Real, R, TB>(a, cur, S, prog, W.phases, w == 0, tid, tpr, tpi, tsg, [] { __syncthreads(); });
         }
         // Scatter: the last phase's layout, with SWAP relabels applied; the
         // part factor and the last phase's per-thread phase are applied here
@@ -159,12 +156,12 @@ k_part(typename CT<Real>::T *__restrict__ sv, const __grid_constant__ PartLaunch
 }
 
 template <typename Real, int T, int R>
-static cudaError_t launch_part_t(void *sv, const PartLaunch &L, const IPhase *phases, const void *ops,
-                                 const void *table, uint64_t n_tiles, cudaStream_t st) {
+static cudaError_t launch_part_t(void *sv, const PartLaunch &L, const void *stream, const IWindow *windows,
+                                 uint64_t n_tiles, cudaStream_t st) {
     typedef typename CT<Real>::T C;
     typedef PartCfg<Real, T, R> Cfg;
     auto kern = k_part<Real, T, R>;
-    const size_t smem = 2 * (sizeof(C) << T);
+    const size_t smem = Cfg::SMEM;
     // per instantiation: devices on which the shared-memory limit was raised,
     // and the resident CTAs per SM found there
     // (set once under a lock; a thread that sees the device's bit sees its counts)
@@ -203,8 +200,8 @@ static cudaError_t launch_part_t(void *sv, const PartLaunch &L, const IPhase *ph
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, kern, reinterpret_cast<C *>(sv), L, phases,
-                           reinterpret_cast<const IOp<Real> *>(ops), reinterpret_cast<const Real *>(table), n_tiles);
+    e = cudaLaunchKernelEx(&cfg, kern, reinterpret_cast<C *>(sv), L, reinterpret_cast<const uint4 *>(stream), windows,
+                           n_tiles);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
