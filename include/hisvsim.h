@@ -167,8 +167,9 @@ sv_status sv_sync(sv_state *s);
  * large double-float states), grown to the plan's largest part plus the lowest free
  * qubits that make each contiguous run of the tile fill a 32-byte sector
  * (two for complex64, one for the complex128 forms), within the limits
- * above. The tile always contains the part's qubits and is padded with the
- * lowest remaining qubits (Sec. IV-B, multi-level: parts smaller than the
+ * above. The tile always contains the part's qubits (on the specialised
+ * kernels those that its gates act on other than as phases and controls) and
+ * is padded with the lowest remaining qubits (Sec. IV-B, multi-level: parts smaller than the
  * limit take extra qubits for spatial locality). */
 sv_status sv_set_tile(sv_state *s, int tile_qubits);
 

@@ -348,9 +348,13 @@ sv_status sv_plan_build(const sv_gate *gates, size_t n_gates, int n, sv_method m
         else if (m == SV_PART_BEAM) p->pog = part_beam(dag, k, dfs_trials);
         else if (!part_exact(dag, k, p->pog, err)) return fail(SV_ERR_ARG, err);
         for (uint32_t x : p->pog) p->n_parts = std::max(p->n_parts, x + 1);
-        std::vector<uint64_t> pm(p->n_parts, 0);
-        for (size_t i = 0; i < n_gates; i++) pm[p->pog[i]] |= dag.qmask[i];
+        std::vector<uint64_t> pm(p->n_parts, 0), nd(p->n_parts, 0);
+        for (size_t i = 0; i < n_gates; i++) {
+            pm[p->pog[i]] |= dag.qmask[i];
+            nd[p->pog[i]] |= tile_need(p->gates[i]);
+        }
         for (uint64_t m : pm) p->max_part = std::max(p->max_part, __builtin_popcountll(m));
+        for (uint64_t m : nd) p->max_tile = std::max(p->max_tile, __builtin_popcountll(m));
     } else {
         p->pog.resize(n_gates);
         for (size_t i = 0; i < n_gates; i++) p->pog[i] = (uint32_t)i;
@@ -406,10 +410,9 @@ sv_status sv_plan_export(const sv_plan *p, uint32_t *pog, size_t n_gates, uint32
 // dense parts (complex64 only), bit 1 = two of them per pass where they fit
 // one tile, bits 4-7 = register bits per thread, and the bits below.
 constexpr int kModeWhole = 4;   // all gates as one part (the tile is the whole state)
-constexpr int kModeJit = 8;     // device program without the interpreter's op stream
+constexpr int kModeJit = 8;     // for the specialised kernels (outer_diag), no interpreter stream
 
 static sv_status get_host_program(sv_plan *p, bool fp64, int t, int mode, const Program **out) {
-    mode &= ~kModeJit;
     std::lock_guard<std::recursive_mutex> lk(p->mu);
     auto key = std::make_tuple(fp64, t, mode);
     auto it = p->host_progs.find(key);
@@ -419,7 +422,7 @@ static sv_status get_host_program(sv_plan *p, bool fp64, int t, int mode, const 
         const bool whole = (mode & kModeWhole) != 0;
         const std::vector<uint32_t> one(whole ? p->gates.size() : 0, 0u);
         if (!compile_program(p->gates, p->n, whole ? one : p->pog, whole ? 1u : p->n_parts, fp64, t, mode >> 4,
-                             mode & 3, *prog, err, p->inner.empty() ? nullptr : &p->inner))
+                             mode & 3, *prog, err, p->inner.empty() ? nullptr : &p->inner, (mode & kModeJit) != 0))
             return fail(SV_ERR_PARTITION, err);
         it = p->host_progs.emplace(key, std::move(prog)).first;
     }
@@ -435,11 +438,11 @@ static int small_tiles(const sv_plan *p, int t) {
 }
 
 // The variant of the flags with the precision's default register bits unless
-// given (statistics, sources, flop counts).
+// given (sources; without kModeJit, statistics and flop counts).
 static int dense_mode(uint32_t flags, bool fp64) {
     const bool tc = (flags & SV_FLAG_TC_DENSE) && !fp64;
     const int R = (int)((flags >> 8) & 0xFu);
-    return (tc ? 1 : 0) | ((tc && (flags & SV_FLAG_TC_PAIRS)) ? 2 : 0) | ((R ? R : part_R(fp64)) << 4);
+    return (tc ? 1 : 0) | ((tc && (flags & SV_FLAG_TC_PAIRS)) ? 2 : 0) | kModeJit | ((R ? R : part_R(fp64)) << 4);
 }
 
 // Tile (t_user, 0 = the default) and variant of the kernels that an apply (or
@@ -462,6 +465,9 @@ static int spec_mode(const sv_plan *p, sv_precision prec, uint32_t flags, int t_
     const bool fp64 = prec != SV_C64;
     t = t_user ? t_user : default_tile(fp64, p->max_part);
     int mode = dense_mode(flags, fp64);
+    // a part's controls and two-qubit phases need not be in its tile
+    if (!t_user && p->inner.empty()) t = std::max(default_tile(fp64, p->max_tile), p->max_part);
+    if (t > part_tmax(fp64)) t = part_tmax(fp64);
     if (t_user || ((flags >> 8) & 0xFu) || !p->inner.empty()) return mode;
     int R = part_R(fp64);
     if (!fp64) {
@@ -510,7 +516,7 @@ sv_status sv_plan_stats(sv_plan *p, sv_precision prec, int t, uint32_t flags, ui
     const bool fp64 = prec != SV_C64;
     if (t == 0) t = default_tile(fp64, p->max_part);
     if (t < part_tmin() || t > part_tmax(fp64)) return fail(SV_ERR_ARG, "tile_qubits out of range");
-    const int mode = dense_mode(flags, fp64);
+    const int mode = dense_mode(flags, fp64) & ~kModeJit;
     if (p->method == SV_PART_NONE || p->n < part_tmin() || (flags & SV_FLAG_GATEWISE)) {
         if (passes) *passes = (uint32_t)p->gates.size();
         if (phases) *phases = 0;
@@ -596,7 +602,7 @@ sv_status sv_plan_flops(sv_plan *p, sv_precision prec, int t, uint32_t flags, do
     const bool fp64 = prec != SV_C64;
     if (t == 0) t = default_tile(fp64, p->max_part);
     if (t < part_tmin() || t > part_tmax(fp64)) return fail(SV_ERR_ARG, "tile_qubits out of range");
-    const int mode = dense_mode(flags, fp64);
+    const int mode = dense_mode(flags, fp64) & ~kModeJit;
     double a = 0.0, b = 0.0;
     if (p->method == SV_PART_NONE || p->n < part_tmin() || (flags & SV_FLAG_GATEWISE)) {
         // one general matrix per gate: 14 flops per amplitude for a 2x2, 30 for a 4x4
@@ -765,7 +771,7 @@ sv_status sv_apply_parts(sv_state *s, sv_plan *p, uint32_t flags) {
         const int mode = jit ? spec_mode(p, s->prec, flags, s->tile, t) : interp_mode(p, fp64, flags, s->tile, t);
         const Program *hp = nullptr;
         const DevProgram *dp = nullptr;
-        st = get_dev_program(s, p, t, mode | (jit ? kModeJit : 0), &hp, &dp);
+        st = get_dev_program(s, p, t, mode, &hp, &dp);
         if (st != SV_OK) return st;
         JitProgram *jp = nullptr;
         if (((flags >> 8) & 0xFu) && !jit)

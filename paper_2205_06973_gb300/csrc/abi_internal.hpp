@@ -66,6 +66,7 @@ struct sv_plan {
     std::vector<uint32_t> pog;
     uint32_t n_parts = 0;
     int max_part = 0;                                                      // qubits of the largest part
+    int max_tile = 0;                   // most qubits a part needs in its tile (tile_need)
     std::vector<uint32_t> inner;        // second-level part of each gate (multi-level plans), else empty
     uint32_t n_inner = 0;
     int k2 = 0;

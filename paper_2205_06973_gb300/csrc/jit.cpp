@@ -197,6 +197,11 @@ std::string jit_part_source(const Program &prog, size_t pi, bool df) {
       << "        bool tsg = false;\n"
       << "        (void)tpr; (void)tpi; (void)tsg;\n";
     const std::vector<double> &cf = prog.coefs;
+    // a thread bit, or the bit of a qubit outside the tile
+    auto cond = [](int b) {
+        return b < OP_OUTER ? "((tid >> " + std::to_string(b) + ") & 1)"
+                            : "((int)(base >> " + std::to_string(b - OP_OUTER) + ") & 1)";
+    };
     auto L_ = [&](uint32_t at) { return lit(cf[at], mode); };
     auto L_lit = [&](double v) { return lit(v, mode); };
     // Per-thread phases (OP_TD / OP_TP2) multiply every amplitude a thread
@@ -235,11 +240,28 @@ std::string jit_part_source(const Program &prog, size_t pi, bool df) {
             if (fold && (kd == OP_TD || kd == OP_TP2 || kd == OP_TAPPLY)) continue;
             order.push_back(k);
         }
+        // Phases on a register bit under a thread or outer bit (OP_CPT) gather
+        // in one factor per register bit until an op acts non-diagonally on
+        // it: a QFT part applies one product per target qubit instead of one
+        // for each of its controls outside the registers.
+        uint32_t gathered = 0;
+        auto apply_gathered = [&](uint32_t bits) {
+            for (int b = 0; b < R; b++)
+                if ((gathered & bits) >> b & 1)
+                    o << "        op_p<NR, " << b << ">(a, w" << p << "_" << b << "r, w" << p << "_" << b << "i);\n";
+            gathered &= ~bits;
+        };
+        uint32_t declared = 0;
         for (uint32_t k : order) {
             const Op &op = prog.ops[ph.op_begin + k];
             const uint32_t c = op.coef;
-            const std::string tb = "((tid >> " + std::to_string(op.tb) + ") & 1)";
+            const std::string tb = cond(op.tb);
             const int A = op.a, B = op.b;
+            switch (op.kind) {
+            case OP_H: case OP_RXS: case OP_RYS: case OP_U2S: case OP_X: case OP_Y: apply_gathered(1u << A); break;
+            case OP_CX: case OP_CXT: apply_gathered(1u << B); break;
+            default: break;
+            }
             o << "        ";
             if (fold && (int)k == first_diag) {
                 // coefficient q = d_q x g x (per-thread phase), g the part
@@ -302,10 +324,15 @@ std::string jit_part_source(const Program &prog, size_t pi, bool df) {
                 if (A != B) o << "op_cz<NR, " << A << ", " << B << ">(a);";
                 break;
             case OP_CXT: o << "op_cxt<" << B << ">(a, " << tb << " != 0);"; break;
-            case OP_CPT:
-                o << "{ const bool c_ = " << tb << " != 0; op_p<NR, " << A << ">(a, c_ ? " << L_(c) << " : (Real)1, c_ ? "
-                  << L_(c + 1) << " : (Real)0); }";
-                break;
+            case OP_CPT: {
+                const std::string w = "w" + std::to_string(p) + "_" + std::to_string(A);
+                if (!((declared >> A) & 1)) o << "Real " << w << "r = 1, " << w << "i = 0; ";
+                else if (!((gathered >> A) & 1)) o << w << "r = 1; " << w << "i = 0; ";
+                o << "{ const bool c_ = " << tb << " != 0; tmul(" << w << "r, " << w << "i, c_ ? " << L_(c)
+                  << " : (Real)1, c_ ? " << L_(c + 1) << " : (Real)0); }";
+                declared |= 1u << A;
+                gathered |= 1u << A;
+            } break;
             case OP_CZT:
                 // a sign, not a complex product
                 o << "op_sgn<" << A << ">(a, " << tb << " != 0);";
@@ -315,11 +342,11 @@ std::string jit_part_source(const Program &prog, size_t pi, bool df) {
                   << L_(c + 3) << " : " << L_(c + 1) << "); }";
                 break;
             case OP_TP2:
-                o << "{ const bool c_ = " << tb << " && ((tid >> " << B << ") & 1); tmul(tpr, tpi, c_ ? " << L_(c)
+                o << "{ const bool c_ = " << tb << " && " << cond(B) << "; tmul(tpr, tpi, c_ ? " << L_(c)
                   << " : (Real)1, c_ ? " << L_(c + 1) << " : (Real)0); }";
                 break;
             case OP_TSG:
-                o << "tsg ^= " << tb << " && ((tid >> " << B << ") & 1);";
+                o << "tsg ^= " << tb << " && " << cond(B) << ";";
                 break;
             case OP_TSAPPLY:
                 o << "op_flip<NR>(a, tsg); tsg = false;";
@@ -344,6 +371,7 @@ std::string jit_part_source(const Program &prog, size_t pi, bool df) {
             }
             o << "\n";
         }
+        apply_gathered(~0u);
     }
     if ((L.flags & PL_STORE_FACTOR) && !store_folded) {
         o << "        { const Real gr = " << lit(L.gr, mode) << ", gi = " << lit(L.gi, mode) << ";\n"

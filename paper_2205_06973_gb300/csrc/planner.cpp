@@ -12,7 +12,9 @@
 //    that does not fit blocks its qubits for the rest of the phase, so every
 //    qubit keeps its gate order (the schedule rule of Sec. IV-A).
 //    Diagonal gates and CX controls need no residency: on a thread bit they
-//    become per-thread conditions or a per-thread phase.
+//    become per-thread conditions or a per-thread phase (and in programs for
+//    the specialised kernels the same on a qubit outside the tile, whose bit
+//    is the tile index's: outer_diag).
 //  * SWAP gates cost nothing: they exchange the slots of their two qubits
 //    for the rest of the part, and the store uses the final slot map.
 #include "planner.hpp"
@@ -93,6 +95,12 @@ static uint64_t acts_nondiag(const GateRef &g) {
     if (is_diagonal(g.kind)) return 0;
     if (g.kind == SV_GATE_SWAP) return (1ull << g.q[0]) | (1ull << g.q[1]);
     return 1ull << (g.kind == SV_GATE_CX ? g.q[1] : g.q[0]);
+}
+
+// A one-qubit phase on a qubit outside the tile would multiply every
+// amplitude; inside, it joins a merged diagonal.
+uint64_t tile_need(const GateRef &g) {
+    return is_diagonal(g.kind) && g.arity == 1 ? 1ull << g.q[0] : acts_nondiag(g);
 }
 
 // Thread-bit order of a phase: lane bits first. The first lanes cover
@@ -252,7 +260,7 @@ static void pair_swizzle(DensePairLaunch &D) {
 
 bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector<uint32_t> &pog,
                      uint32_t n_parts, bool fp64, int t_cfg, int R, int dense_mode, Program &prog,
-                     std::string &err, const std::vector<uint32_t> *inner) {
+                     std::string &err, const std::vector<uint32_t> *inner, bool outer_diag) {
     prog = Program();
     prog.fp64 = fp64;
     prog.R = R;
@@ -377,15 +385,27 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
             err = "part " + std::to_string(pi) + " has " + std::to_string(popc(S)) + " qubits > tile " + std::to_string(t);
             return false;
         }
+        // the tile: with outer_diag only the qubits of tile_need must be in it,
+        // and more low qubits (longer contiguous runs) take the places of the
+        // others
         uint64_t Tm = S;
+        if (outer_diag) {
+            Tm = 0;
+            for (int g : gl) Tm |= tile_need(gates[g]);
+        }
         for (int q = 0; q < n && popc(Tm) < t; q++) Tm |= 1ull << q;
         int slot_of[64], q_at[64];
-        for (int q = 0, p = 0; q < n; q++)
+        for (int q = 0, p = 0, o = t; q < n; q++) {
             if ((Tm >> q) & 1) {
                 slot_of[q] = p;
                 q_at[p] = q;
                 p++;
+            } else if ((S >> q) & 1) {
+                slot_of[q] = o++;   // a part qubit outside the tile: a slot past its slots
             }
+        }
+        int rank[64];   // place of a tile qubit among the tile's qubits
+        std::memcpy(rank, slot_of, sizeof(rank));
         PartLaunch L;
         std::memset(&L, 0, sizeof(L));
         L.outer_mask = all & ~Tm;
@@ -494,26 +514,37 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
                     std::reverse(keep.begin(), keep.end());
                     sched.swap(keep);
                 }
-                // spare register bits go to the thread bits of diagonal gates
-                // (the last phase keeps its lowest slots for the lanes of the
-                // store: 28-qubit passes lost 1 to 3 % otherwise)
-                const int lowest = rest.empty() ? 5 : 0;
                 std::memcpy(sim_slot, slot_of, sizeof(slot_of));
-                for (int g : sched) {
-                    if (is_diagonal(gates[g].kind))
-                        for (int j = 0; j < gates[g].arity; j++) {
-                            const int sl = sim_slot[gates[g].q[j]];
-                            if (popc(Rset) < R && sl >= lowest) Rset |= 1u << sl;
-                        }
+                for (int g : sched)
                     if (gates[g].kind == SV_GATE_SWAP) std::swap(sim_slot[gates[g].q[0]], sim_slot[gates[g].q[1]]);
-                }
             }
-            for (int p = t - 1; p >= 0 && popc(Rset) < R; p--) Rset |= 1u << p;
             const bool last = rest.empty();
-            // slot -> qubit at the start and at the end of this phase
+            // slot -> qubit at the end of this phase
             int q_end[64];
             for (int q = 0; q < n; q++)
                 if ((Tm >> q) & 1) q_end[sim_slot[q]] = q;
+            // Spare register bits go to the thread bits of diagonal gates, then
+            // to the highest slots; in the last phase, which stores the tile,
+            // to the slots that end on the highest qubits, since the lowest
+            // five are the lanes of the store (with a register bit on one of
+            // them 28-qubit passes lost 1 to 3 %; the QFT's swap passes, whose
+            // high slots end on low qubits, ran at 0.34 to 0.46 of HBM).
+            auto key_of = [&](int p) { return last ? rank[q_end[p]] : p; };
+            if (!(inner && !inner->empty())) {
+                int at[64];
+                std::memcpy(at, slot_of, sizeof(slot_of));
+                for (int g : sched) {
+                    if (is_diagonal(gates[g].kind))
+                        for (int j = 0; j < gates[g].arity; j++) {
+                            const int sl = at[gates[g].q[j]];
+                            if (popc(Rset) < R && sl < t && (!last || key_of(sl) >= 5)) Rset |= 1u << sl;
+                        }
+                    if (gates[g].kind == SV_GATE_SWAP) std::swap(at[gates[g].q[0]], at[gates[g].q[1]]);
+                }
+            }
+            for (int v = t - 1; v >= 0 && popc(Rset) < R; v--)
+                for (int p = 0; p < t; p++)
+                    if (key_of(p) == v) Rset |= 1u << p;
             Phase ph;
             std::memset(&ph, 0, sizeof(ph));
             int rb[64], tbit[64];
@@ -526,13 +557,15 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
             std::vector<int> key(t, 0);
             for (int p = 0; p < t; p++) {
                 if (!((Rset >> p) & 1)) cand.push_back(p);
-                key[p] = last ? q_end[p] : p;   // the last phase stores: lanes on the lowest qubits
+                key[p] = key_of(p);   // the last phase stores: lanes on the lowest qubits
             }
             std::vector<int> thr = order_thread_slots(cand, key, fp64);
             for (size_t j = 0; j < thr.size(); j++) {
                 ph.thr[j] = (uint8_t)thr[j];
                 tbit[thr[j]] = (int)j;
             }
+            for (int q = 0; q < n; q++)
+                if (((S & ~Tm) >> q) & 1) tbit[slot_of[q]] = OP_OUTER + q;
             // pass 2: emit ops
             ph.op_begin = (uint32_t)prog.ops.size();
             bool tphase = false, tsign = false;

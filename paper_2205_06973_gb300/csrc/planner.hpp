@@ -37,6 +37,9 @@ struct Program {
 void gate_matrix_1q(int kind, double theta, double m[8]);
 void gate_matrix_2q(int kind, double theta, double m[32]);
 bool gate_is_two_qubit(int kind);
+// Qubits of the gate that belong in its part's tile: those it acts on other
+// than as a two-qubit phase or a control.
+uint64_t tile_need(const GateRef &g);
 
 // Compile the parts (part_of_gate numbered in execution order) for a tile of
 // t_cfg qubits (t = min(n, t_cfg)) and R register bits.
@@ -47,9 +50,13 @@ bool gate_is_two_qubit(int kind);
 // partitioning, Sec. IV-B); each becomes one register phase of its
 // first-level part instead of the greedy phase split (error if one needs
 // more than R register qubits).
+// outer_diag: qubits that the part's gates act on only as two-qubit phases or
+// controls may lie outside its tile; conditions on them are thread-bit
+// numbers from OP_OUTER (not for the interpreter, whose conditions are thread
+// masks).
 bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector<uint32_t> &pog,
                      uint32_t n_parts, bool fp64, int t_cfg, int R, int dense_mode, Program &prog,
-                     std::string &err, const std::vector<uint32_t> *inner = nullptr);
+                     std::string &err, const std::vector<uint32_t> *inner = nullptr, bool outer_diag = false);
 
 // Floating-point operations per state amplitude that the program's kernels
 // execute: CUDA-core arithmetic (alu) and tensor-core products (tensor).

@@ -52,6 +52,9 @@ struct Op {
     uint32_t coef;   // index of the first coefficient (in reals)
 };
 
+// A thread-bit number of OP_OUTER + q stands for qubit q outside the tile.
+constexpr int OP_OUTER = 32;
+
 constexpr int MAX_R = 6;
 constexpr int MAX_TB = 16;
 
