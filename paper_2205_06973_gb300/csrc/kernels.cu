@@ -205,7 +205,7 @@ __global__ void k_sum(const double *__restrict__ partials, int nb, double *__res
 // complex64 amplitudes: 3.05 ms against 0.47 ms of HBM time for the 3.2 GB;
 // 0.50 ms here, 0.94 of the measured copy rate).
 // Each thread takes 16 bytes at a time, PROB_U of them in flight, and sends
-// the FP64 pipe two conversions and two adds per PROB_U loads.
+// the FP64 pipe two conversions and two adds per four chunks.
 constexpr int PROB_U = 4;
 constexpr int PROB_CHUNK = 256 * PROB_U;   // 16-byte loads per block and iteration
 
@@ -214,7 +214,9 @@ __global__ void __launch_bounds__(256, 4) k_probs_fast(const float4 *__restrict_
                                                         float *__restrict__ out, double *__restrict__ partials,
                                                         uint32_t *ticket, double *norm) {
     double acc = 0.0;
-    for (uint64_t c = blockIdx.x; c < n_chunks; c += gridDim.x) {
+    float S = 0.0f, T = 0.0f;
+    uint32_t it = 0;
+    for (uint64_t c = blockIdx.x; c < n_chunks; c += gridDim.x, it++) {
         const uint64_t at = c * PROB_CHUNK + threadIdx.x;
         float4 v[PROB_U];
 #pragma unroll
@@ -223,7 +225,6 @@ __global__ void __launch_bounds__(256, 4) k_probs_fast(const float4 *__restrict_
 #pragma unroll
         for (int u = 0; u < PROB_U; u++) ok = ok && split_range<DF>(v[u]);
         if (ok) {
-            float S = 0.0f, T = 0.0f;
 #pragma unroll
             for (int u = 0; u < PROB_U; u++) {
                 if constexpr (DF) {
@@ -237,7 +238,6 @@ __global__ void __launch_bounds__(256, 4) k_probs_fast(const float4 *__restrict_
                     if (out) reinterpret_cast<float2 *>(out)[at + 256 * u] = make_float2(p.x + p.y, q.x + q.y);
                 }
             }
-            acc += (double)S + (double)T;
         } else {   // outside the split's range: FP64
 #pragma unroll
             for (int u = 0; u < PROB_U; u++) {
@@ -256,8 +256,12 @@ __global__ void __launch_bounds__(256, 4) k_probs_fast(const float4 *__restrict_
                 }
             }
         }
+        if ((it & 3) == 3) {
+            acc += (double)S + (double)T;
+            S = T = 0.0f;
+        }
     }
-    finish_norm(acc, partials, ticket, norm);
+    finish_norm(acc + ((double)S + (double)T), partials, ticket, norm);
 }
 
 // The FP32 kernels take whole chunks of 16-byte loads: at least one chunk,
@@ -385,22 +389,26 @@ __global__ void __launch_bounds__(256) k_summary(const E *__restrict__ sv, uint6
     finish_summary(sv, acc, best, bi, sums, maxs, idxs, ticket, out);
 }
 
-// The norm on the FP32 pipes as in k_probs_fast. The maximum stays exact: a
-// group of loads goes through the FP64 comparison only if one of its FP32
-// probabilities (within 2^-23 of the true ones) comes within 2^-21 of the
-// warp's largest so far, so nothing that could win or tie is passed over.
-// For random states that is a few groups per warp (2^28 complex64
-// amplitudes: 3.57 ms with every amplitude in FP64, against 0.32 ms of HBM
-// time; 2^25: 0.48 ms, here 0.16 ms); for a state of equal probabilities it is every group, as before.
+// The norm on the FP32 pipes as in k_probs_fast. The maximum stays exact: an
+// amplitude goes through the FP64 comparison only if its FP32 probability
+// (within 2^-22 of the true one) comes within 2^-21 of the warp's largest so
+// far, so nothing that could win or tie is passed over. For random states
+// that is a few amplitudes per warp (2^28 complex64 amplitudes: 3.57 ms with
+// every amplitude in FP64, against 0.32 ms of HBM time; 2^25: 0.48 ms, 0.16 ms
+// with whole groups of loads in FP64, 0.08 ms here); for a state of equal
+// probabilities it is every amplitude, as before.
 template <bool DF>
 __global__ void __launch_bounds__(256, 4) k_summary_fast(const float4 *__restrict__ sv, uint64_t n_chunks,
                                                           double *__restrict__ sums, double *__restrict__ maxs,
                                                           uint64_t *__restrict__ idxs, uint32_t *ticket,
                                                           double *out) {
+    constexpr int PER = DF ? 1 : 2;   // amplitudes per load
     double acc = 0.0, best = -1.0;
     uint64_t bi = ~0ull;
     float least = -1.0f;   // below this a probability cannot win (warp-wide)
-    for (uint64_t c = blockIdx.x; c < n_chunks; c += gridDim.x) {
+    float S = 0.0f, T = 0.0f;
+    uint32_t it = 0;
+    for (uint64_t c = blockIdx.x; c < n_chunks; c += gridDim.x, it++) {
         const uint64_t at = c * PROB_CHUNK + threadIdx.x;
         float4 v[PROB_U];
 #pragma unroll
@@ -408,48 +416,48 @@ __global__ void __launch_bounds__(256, 4) k_summary_fast(const float4 *__restric
         bool ok = true;
 #pragma unroll
         for (int u = 0; u < PROB_U; u++) ok = ok && split_range<DF>(v[u]);
-        float top = -1.0f;
+        float p[PROB_U * PER], top = -1.0f;
         if (ok) {
-            float S = 0.0f, T = 0.0f;
 #pragma unroll
             for (int u = 0; u < PROB_U; u++) {
                 if constexpr (DF) {
-                    const float2 p = split_prob_df(v[u]);
-                    split_add(S, T, p);
-                    top = fmaxf(top, p.x + p.y);
+                    const float2 a = split_prob_df(v[u]);
+                    split_add(S, T, a);
+                    p[u] = a.x + a.y;
                 } else {
-                    const float2 p = split_prob(v[u].x, v[u].y), q = split_prob(v[u].z, v[u].w);
-                    split_add(S, T, p);
-                    split_add(S, T, q);
-                    top = fmaxf(top, fmaxf(p.x, q.x));
+                    const float2 a = split_prob(v[u].x, v[u].y), b = split_prob(v[u].z, v[u].w);
+                    split_add(S, T, a);
+                    split_add(S, T, b);
+                    p[2 * u] = a.x;
+                    p[2 * u + 1] = b.x;
                 }
             }
-            acc += (double)S + (double)T;
+#pragma unroll
+            for (int j = 0; j < PROB_U * PER; j++) top = fmaxf(top, p[j]);
         }
         if (__any_sync(0xffffffffu, !ok || top >= least)) {
+            float w = top;
 #pragma unroll
-            for (int u = 0; u < PROB_U; u++) {
-                if constexpr (DF) {
-                    double re, im;
-                    amp_parts(v[u], re, im);
-                    const double p = re * re + im * im;
-                    if (!ok) acc += p;
-                    better(best, bi, p, at + 256 * u);
-                } else {
-                    const double p = (double)v[u].x * v[u].x + (double)v[u].y * v[u].y;
-                    const double q = (double)v[u].z * v[u].z + (double)v[u].w * v[u].w;
-                    if (!ok) acc += p;
-                    if (!ok) acc += q;
-                    better(best, bi, p, 2 * (at + 256 * u));
-                    better(best, bi, q, 2 * (at + 256 * u) + 1);
-                }
+            for (int o = 16; o > 0; o >>= 1) w = fmaxf(w, __shfl_xor_sync(0xffffffffu, w, o));
+            least = fmaxf(least, w * (1.0f - 0x1p-21f));
+#pragma unroll
+            for (int j = 0; j < PROB_U * PER; j++) {
+                if (ok && p[j] < least) continue;
+                const float4 x = v[j / PER];
+                double re, im;
+                if constexpr (DF) amp_parts(x, re, im);
+                else amp_parts(j % 2 ? make_float2(x.z, x.w) : make_float2(x.x, x.y), re, im);
+                const double q = re * re + im * im;
+                if (!ok) acc += q;
+                better(best, bi, q, PER * (at + 256 * (j / PER)) + j % PER);
             }
-            float b = (float)best * (1.0f - 0x1p-21f);   // an infinite best stays infinite
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) b = fmaxf(b, __shfl_xor_sync(0xffffffffu, b, o));
-            least = b;
+        }
+        if ((it & 3) == 3) {   // the FP64 pipe gets two conversions and adds per four chunks
+            acc += (double)S + (double)T;
+            S = T = 0.0f;
         }
     }
+    acc += (double)S + (double)T;
     const typename std::conditional<DF, float4, float2>::type *amps =
         reinterpret_cast<const typename std::conditional<DF, float4, float2>::type *>(sv);
     finish_summary(amps, acc, best, bi, sums, maxs, idxs, ticket, out);
