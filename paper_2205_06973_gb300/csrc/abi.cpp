@@ -2,6 +2,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -98,47 +99,101 @@ static cudaError_t upload_lowered(const Program &prog, DevProgram &d, cudaStream
     return e == cudaSuccess ? se : e;
 }
 
-// The gate records of a small circuit in the kernel's precision.
-template <typename Real> static std::vector<SmallGate<Real>> small_gates(const sv_plan *p) {
-    std::vector<SmallGate<Real>> out(p->gates.size());
-    for (size_t i = 0; i < out.size(); i++) {
-        const GateRef &g = p->gates[i];
-        SmallGate<Real> &r = out[i];
+// The ops of a small circuit in the kernel's precision: runs of one-qubit
+// gates on a qubit as one matrix (any gate on other qubits between them
+// commutes with them), runs of CX and SWAP gates as one permutation.
+template <typename Real> static std::vector<SmallOp<Real>> small_ops(const sv_plan *p) {
+    std::vector<SmallOp<Real>> out;
+    const int n = p->n;
+    std::vector<std::array<double, 8>> pend(n);   // product of the qubit's pending gates
+    std::vector<char> has(n, 0);
+    auto flush = [&](int q) {
+        if (!has[q]) return;
+        has[q] = 0;
+        const double *u = pend[q].data();
+        SmallOp<Real> r;
         std::memset(&r, 0, sizeof(r));
-        r.q0 = g.q[0];
-        r.q1 = g.q[1];
+        r.q0 = q;
         double m[8] = {0};
-        switch (g.kind) {
-        case SV_GATE_CX: r.kind = SMALL_CX; break;
-        case SV_GATE_SWAP: r.kind = SMALL_SWAP; break;
-        case SV_GATE_CZ: case SV_GATE_CP:
-            r.kind = SMALL_PHASE;
-            m[0] = g.kind == SV_GATE_CZ ? -1.0 : std::cos(g.theta);
-            m[1] = g.kind == SV_GATE_CZ ? 0.0 : std::sin(g.theta);
-            break;
-        default: {
-            double u[8];
-            gate_matrix_1q(g.kind, g.theta, u);
-            const bool diag = u[2] == 0 && u[3] == 0 && u[4] == 0 && u[5] == 0;
-            const bool real = u[1] == 0 && u[3] == 0 && u[5] == 0 && u[7] == 0;
-            if (g.kind == SV_GATE_RX) {
-                r.kind = SMALL_RX;
-                m[0] = u[0];
-                m[1] = -u[3];
-            } else if (real) {
-                r.kind = SMALL_REAL;
-                for (int j = 0; j < 4; j++) m[j] = u[2 * j];
-            } else if (diag) {
-                r.kind = SMALL_DIAG;
-                m[0] = u[0]; m[1] = u[1]; m[2] = u[6]; m[3] = u[7];
-            } else {
-                r.kind = SMALL_GENERAL;
-                std::memcpy(m, u, sizeof(m));
-            }
-        }
+        if (u[2] == 0 && u[3] == 0 && u[4] == 0 && u[5] == 0) {
+            r.kind = SMALL_DIAG;
+            m[0] = u[0]; m[1] = u[1]; m[2] = u[6]; m[3] = u[7];
+        } else if (u[1] == 0 && u[3] == 0 && u[5] == 0 && u[7] == 0) {
+            r.kind = SMALL_REAL;
+            for (int j = 0; j < 4; j++) m[j] = u[2 * j];
+        } else if (u[1] == 0 && u[2] == 0 && u[4] == 0 && u[7] == 0) {
+            r.kind = SMALL_CROSS;
+            m[0] = u[0]; m[1] = u[3]; m[2] = u[5]; m[3] = u[6];
+        } else {
+            r.kind = SMALL_GENERAL;
+            std::memcpy(m, u, sizeof(m));
         }
         for (int j = 0; j < 8; j++) r.m[j] = (Real)m[j];
+        out.push_back(r);
+    };
+    // the pending permutation new[x] = old[L x]: columns of L
+    std::vector<uint16_t> cols(n);
+    bool perm = false;
+    auto flush_perm = [&]() {
+        if (!perm) return;
+        perm = false;
+        SmallOp<Real> r;
+        std::memset(&r, 0, sizeof(r));
+        r.kind = SMALL_PERM;
+        for (int b = 0; b < n; b++) r.perm[b] = cols[b];
+        out.push_back(r);
+    };
+    for (const GateRef &g : p->gates) {
+        if (g.arity == 1) {
+            // gates on qubits that the permutation moves come after it
+            const int q = g.q[0];
+            if (perm) flush_perm();
+            double u[8];
+            gate_matrix_1q(g.kind, g.theta, u);
+            if (!has[q]) {
+                std::copy(u, u + 8, pend[q].begin());
+                has[q] = 1;
+                continue;
+            }
+            std::array<double, 8> t;
+            for (int r = 0; r < 2; r++)
+                for (int c = 0; c < 2; c++) {
+                    double re = 0, im = 0;
+                    for (int k = 0; k < 2; k++) {
+                        const double ar = u[2 * (2 * r + k)], ai = u[2 * (2 * r + k) + 1];
+                        const double br = pend[q][2 * (2 * k + c)], bi = pend[q][2 * (2 * k + c) + 1];
+                        re += ar * br - ai * bi;
+                        im += ar * bi + ai * br;
+                    }
+                    t[2 * (2 * r + c)] = re;
+                    t[2 * (2 * r + c) + 1] = im;
+                }
+            pend[q] = t;
+            continue;
+        }
+        flush(g.q[0]);
+        flush(g.q[1]);
+        if (g.kind == SV_GATE_CX || g.kind == SV_GATE_SWAP) {
+            if (!perm)
+                for (int b = 0; b < n; b++) cols[b] = (uint16_t)(1u << b);
+            perm = true;
+            // new state y[x] = old[L x]; the gate then maps z[x] = y[G x], so L <- L G
+            if (g.kind == SV_GATE_CX) cols[g.q[0]] ^= cols[g.q[1]];   // G e_c = e_c + e_t
+            else std::swap(cols[g.q[0]], cols[g.q[1]]);
+            continue;
+        }
+        flush_perm();
+        SmallOp<Real> r;
+        std::memset(&r, 0, sizeof(r));
+        r.kind = SMALL_PHASE;
+        r.q0 = g.q[0];
+        r.q1 = g.q[1];
+        r.m[0] = (Real)(g.kind == SV_GATE_CZ ? -1.0 : std::cos(g.theta));
+        r.m[1] = (Real)(g.kind == SV_GATE_CZ ? 0.0 : std::sin(g.theta));
+        out.push_back(r);
     }
+    flush_perm();
+    for (int q = 0; q < n; q++) flush(q);
     return out;
 }
 
@@ -702,7 +757,7 @@ static sv_status apply_gatewise(sv_state *s, sv_plan *p) {
     return SV_OK;
 }
 
-// A circuit on fewer than 10 qubits in one launch; the gate records are
+// A circuit on fewer than 10 qubits in one launch; the op records are
 // uploaded at the plan's first apply for the precision and device and kept in
 // the plan. Where that cannot be done now (no memory, or the stream is being
 // captured, which an upload with its wait would break) the circuit runs gate
@@ -710,7 +765,7 @@ static sv_status apply_gatewise(sv_state *s, sv_plan *p) {
 static sv_status apply_small(sv_state *s, sv_plan *p) {
     if (p->gates.empty()) return SV_OK;
     const bool fp64 = is_fp64(s);
-    const void *prog = nullptr;
+    const DevProgram *prog = nullptr;
     {
         std::lock_guard<std::recursive_mutex> lk(p->mu);
         auto key = std::make_tuple(s->dev, fp64, 0, 0);   // tile 0: no part program has it
@@ -722,14 +777,15 @@ static sv_status apply_small(sv_state *s, sv_plan *p) {
                 cudaGetLastError();
                 return apply_gatewise(s, p);
             }
-            std::vector<SmallGate<float>> f;
-            std::vector<SmallGate<double>> d;
-            if (fp64) d = small_gates<double>(p);
-            else f = small_gates<float>(p);
+            std::vector<SmallOp<float>> f;
+            std::vector<SmallOp<double>> d;
+            if (fp64) d = small_ops<double>(p);
+            else f = small_ops<float>(p);
             const void *src = fp64 ? static_cast<const void *>(d.data()) : f.data();
-            const size_t bytes = p->gates.size() * (fp64 ? sizeof(SmallGate<double>) : sizeof(SmallGate<float>));
+            const size_t bytes = fp64 ? d.size() * sizeof(d[0]) : f.size() * sizeof(f[0]);
             DevProgram dp;
             dp.dev = s->dev;
+            dp.n_small = (uint32_t)(fp64 ? d.size() : f.size());
             e = dev_alloc(&dp.d_small, bytes, s->stream);
             if (e != cudaSuccess) {
                 cudaGetLastError();
@@ -745,9 +801,9 @@ static sv_status apply_small(sv_state *s, sv_plan *p) {
             }
             it = p->dev_progs.emplace(key, dp).first;
         }
-        prog = it->second.d_small;
+        prog = &it->second;   // map nodes do not move
     }
-    CUDA_TRY(launch_small(fp64, s->buf, s->n, prog, (uint32_t)p->gates.size(), s->stream));
+    CUDA_TRY(launch_small(fp64, s->buf, s->n, prog->d_small, prog->n_small, s->stream));
     return SV_OK;
 }
 

@@ -37,7 +37,8 @@ struct DevProgram {
     std::vector<hisv::PartLaunch> parts;   // and its parts (launch arguments)
     uint8_t *d_aimg = nullptr;      // R images of the dense parts
     uint8_t *d_pimg = nullptr;      // R images of the dense pairs (two per pass)
-    void *d_small = nullptr;        // gate records of a circuit on fewer than 10 qubits
+    void *d_small = nullptr;        // op records of a circuit on fewer than 10 qubits
+    uint32_t n_small = 0;
 };
 
 struct sv_state {

@@ -4,10 +4,13 @@
 //
 // Gate by gate, such a circuit is one launch of a few hundred threads per
 // gate, bound by the launches: 2.5 us each, 347 us for the 138 gates of a
-// 8-qubit parameterised circuit (complex64), 22.5 us here. A gate costs a shared-memory
-// round trip of its pairs and a barrier. One thread per pair (2^(n-1) threads,
-// at least a warp); the gate records are staged in shared memory a block at a
-// time, so that a gate's coefficients are broadcast reads. Gates do only the
+// 8-qubit parameterised circuit (complex64). Here an op costs a shared-memory
+// round trip of its pairs and a barrier, about 0.12 us of latency, so the host
+// makes fewer ops of the gates: the product of a run of one-qubit gates on a
+// qubit, and one permutation of a run of CX and SWAP gates (GF(2)-linear in
+// the index): 12.3 us, 22.5 us with one op per gate. One thread per pair (2^(n-1) threads,
+// at least a warp); the op records are staged in shared memory a block at a
+// time, so that an op's coefficients are broadcast reads. Ops do only the
 // arithmetic their form needs (a real matrix, a diagonal, a permutation): in
 // complex128 the SM's two FP64 lanes would otherwise set the time.
 #include "small.hpp"
@@ -17,27 +20,28 @@
 namespace hisv {
 namespace {
 
-constexpr int STAGE = 64;   // gate records staged per block of the list
+constexpr int STAGE = 64;   // op records staged per block of the list
 
 template <typename Real>
 __global__ void __launch_bounds__(256) k_small(typename CT<Real>::T *__restrict__ sv, int n,
-                                                const SmallGate<Real> *__restrict__ gates, uint32_t n_gates) {
+                                                const SmallOp<Real> *__restrict__ ops, uint32_t n_ops) {
     typedef typename CT<Real>::T C;
     __shared__ C a[1 << SMALL_MAX_QUBITS];
-    __shared__ __align__(16) SmallGate<Real> stage[STAGE];
+    __shared__ __align__(16) unsigned char stage_raw[STAGE * sizeof(SmallOp<Real>)];
+    const SmallOp<Real> *const stage = reinterpret_cast<const SmallOp<Real> *>(stage_raw);
     const uint32_t tid = threadIdx.x, N = 1u << n;
     for (uint32_t x = tid; x < N; x += blockDim.x) a[x] = sv[x];
-    for (uint32_t g0 = 0; g0 < n_gates; g0 += STAGE) {
-        const uint32_t m = min((uint32_t)STAGE, n_gates - g0);
+    for (uint32_t g0 = 0; g0 < n_ops; g0 += STAGE) {
+        const uint32_t m = min((uint32_t)STAGE, n_ops - g0);
         __syncthreads();
-        const uint4 *src = reinterpret_cast<const uint4 *>(gates + g0);
-        for (uint32_t i = tid; i < m * (uint32_t)(sizeof(SmallGate<Real>) / 16); i += blockDim.x)
-            reinterpret_cast<uint4 *>(stage)[i] = src[i];
+        const uint4 *src = reinterpret_cast<const uint4 *>(ops + g0);
+        for (uint32_t i = tid; i < m * (uint32_t)(sizeof(SmallOp<Real>) / 16); i += blockDim.x)
+            reinterpret_cast<uint4 *>(stage_raw)[i] = src[i];
         __syncthreads();
         for (uint32_t g = 0; g < m; g++) {
-            const SmallGate<Real> &G = stage[g];
+            const SmallOp<Real> &G = stage[g];
             const int kind = G.kind;
-            if (kind < SMALL_CX) {
+            if (kind < SMALL_PHASE) {
                 const uint32_t lo = (1u << G.q0) - 1, x0 = ((tid & ~lo) << 1) | (tid & lo), x1 = x0 | (1u << G.q0);
                 if (tid < N / 2) {
                     const C x = a[x0], y = a[x1];
@@ -52,11 +56,11 @@ __global__ void __launch_bounds__(256) k_small(typename CT<Real>::T *__restrict_
                         u.y = G.m[0] * x.y + G.m[1] * x.x;
                         v.x = G.m[2] * y.x - G.m[3] * y.y;
                         v.y = G.m[2] * y.y + G.m[3] * y.x;
-                    } else if (kind == SMALL_RX) {
-                        u.x = G.m[0] * x.x + G.m[1] * y.y;
-                        u.y = G.m[0] * x.y - G.m[1] * y.x;
-                        v.x = G.m[1] * x.y + G.m[0] * y.x;
-                        v.y = G.m[0] * y.y - G.m[1] * x.x;
+                    } else if (kind == SMALL_CROSS) {
+                        u.x = G.m[0] * x.x - G.m[1] * y.y;
+                        u.y = G.m[0] * x.y + G.m[1] * y.x;
+                        v.x = G.m[3] * y.x - G.m[2] * x.y;
+                        v.y = G.m[3] * y.y + G.m[2] * x.x;
                     } else {
                         u.x = G.m[0] * x.x - G.m[1] * x.y + G.m[2] * y.x - G.m[3] * y.y;
                         u.y = G.m[0] * x.y + G.m[1] * x.x + G.m[2] * y.y + G.m[3] * y.x;
@@ -66,21 +70,29 @@ __global__ void __launch_bounds__(256) k_small(typename CT<Real>::T *__restrict_
                     a[x0] = u;
                     a[x1] = v;
                 }
-            } else if (tid < N / 4) {
+            } else if (kind == SMALL_PHASE) {
                 const int ql = min(G.q0, G.q1), qh = max(G.q0, G.q1);
                 const uint32_t ml = (1u << ql) - 1, mh = (1u << qh) - 1;
-                uint32_t x = ((tid & ~ml) << 1) | (tid & ml);   // zero bits inserted at ql, then qh
-                x = ((x & ~mh) << 1) | (x & mh);
-                const uint32_t x01 = x | (1u << G.q0), x10 = x | (1u << G.q1), x11 = x01 | x10;
-                if (kind == SMALL_PHASE) {
-                    C v = a[x11];
+                if (tid < N / 4) {
+                    uint32_t x = ((tid & ~ml) << 1) | (tid & ml);   // zero bits inserted at ql, then qh
+                    x = ((x & ~mh) << 1) | (x & mh) | (1u << ql) | (1u << qh);
+                    C v = a[x];
                     cmul_in(v, G.m[0], G.m[1]);
-                    a[x11] = v;
-                } else {   // CX: the control's two amplitudes change places; SWAP: the unequal bits'
-                    const uint32_t y = kind == SMALL_CX ? x11 : x10;
-                    const C u = a[x01], v = a[y];
-                    a[x01] = v;
-                    a[y] = u;
+                    a[x] = v;
+                }
+            } else {   // every amplitude is read before any is written
+                const uint32_t x = 2 * tid;
+                uint32_t y = G.perm[n];
+                for (int b = 1; b < n; b++) y ^= (x >> b) & 1 ? G.perm[b] : 0u;
+                C u{}, v{};
+                if (x < N) {
+                    u = a[y];
+                    v = a[y ^ G.perm[0]];
+                }
+                __syncthreads();
+                if (x < N) {
+                    a[x] = u;
+                    a[x + 1] = v;
                 }
             }
             __syncthreads();
@@ -91,13 +103,13 @@ __global__ void __launch_bounds__(256) k_small(typename CT<Real>::T *__restrict_
 
 }  // namespace
 
-cudaError_t launch_small(bool fp64, void *sv, int n, const void *gates, uint32_t n_gates, cudaStream_t st) {
+cudaError_t launch_small(bool fp64, void *sv, int n, const void *ops, uint32_t n_ops, cudaStream_t st) {
     if (n < 1 || n > SMALL_MAX_QUBITS) return cudaErrorInvalidValue;
     const unsigned threads = n > 6 ? 1u << (n - 1) : 32u;
     if (fp64)
-        k_small<double><<<1, threads, 0, st>>>((double2 *)sv, n, (const SmallGate<double> *)gates, n_gates);
+        k_small<double><<<1, threads, 0, st>>>((double2 *)sv, n, (const SmallOp<double> *)ops, n_ops);
     else
-        k_small<float><<<1, threads, 0, st>>>((float2 *)sv, n, (const SmallGate<float> *)gates, n_gates);
+        k_small<float><<<1, threads, 0, st>>>((float2 *)sv, n, (const SmallOp<float> *)ops, n_ops);
     return cudaGetLastError();
 }
 
