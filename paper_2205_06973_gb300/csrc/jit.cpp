@@ -15,6 +15,7 @@
 
 #include <algorithm>
 #include <chrono>
+#include <cmath>
 #include <cstdio>
 #include <mutex>
 #include <sstream>
@@ -80,6 +81,20 @@ std::string lit(double v, int mode) {
         std::snprintf(b, sizeof(b), "(df(%af, %af))", (double)hi, (double)lo);
     } else std::snprintf(b, sizeof(b), "(%af)", (double)(float)v);
     return b;
+}
+
+// d = i^quad e^{i phi} with |phi| <= pi / 4, as the shears of rot_in; false if
+// d is not a phase (a merged diagonal may hold the part factor).
+bool shears(double dr, double di, int &quad, double &t, double &s) {
+    const double r = std::hypot(dr, di);   // a product of phases: 1 up to its rounding
+    if (std::fabs(r - 1.0) > 1e-13) return false;
+    dr /= r;
+    di /= r;
+    quad = std::fabs(dr) >= std::fabs(di) ? (dr > 0 ? 0 : 2) : (di > 0 ? 1 : 3);
+    const double c = quad == 0 ? dr : quad == 1 ? di : quad == 2 ? -dr : -di;
+    s = quad == 0 ? di : quad == 1 ? -dr : quad == 2 ? -di : dr;   // d i^-quad = c + i s
+    t = s / (1.0 + c);
+    return true;
 }
 
 unsigned swz_host(int p, bool fp64) {
@@ -314,7 +329,14 @@ std::string jit_part_source(const Program &prog, size_t pi, bool df) {
                 break;
             case OP_X: o << "op_x<" << A << ">(a);"; break;
             case OP_Y: o << "op_y<" << A << ">(a);"; break;
-            case OP_P: o << "op_p<NR, " << A << ">(a, " << L_(c) << ", " << L_(c + 1) << ");"; break;
+            case OP_P: {
+                int quad;
+                double rt, rs;
+                if (mode == 1 && shears(cf[c], cf[c + 1], quad, rt, rs))
+                    o << "op_prot<NR, " << A << ", " << quad << ">(a, " << L_lit(rt) << ", " << L_lit(rs) << ");";
+                else
+                    o << "op_p<NR, " << A << ">(a, " << L_(c) << ", " << L_(c + 1) << ");";
+            } break;
             case OP_Z: o << "op_z<NR, " << A << ">(a);"; break;
             case OP_CX: o << "op_cx<" << A << ", " << B << ">(a);"; break;
             case OP_CP:
@@ -358,9 +380,13 @@ std::string jit_part_source(const Program &prog, size_t pi, bool df) {
                     const double dr = cf[c + 2 * q], di = cf[c + 2 * q + 1];
                     const std::string aq = "a[" + std::to_string(q) + "]";
                     if (dr == 1.0 && di == 0.0) continue;
-                    if (dr == -1.0 && di == 0.0) o << aq << ".x = -" << aq << ".x; " << aq << ".y = -" << aq << ".y; ";
-                    else if (dr == 0.0 && di == 1.0) o << "{ const Real x_ = " << aq << ".x; " << aq << ".x = -" << aq << ".y; " << aq << ".y = x_; } ";
-                    else if (dr == 0.0 && di == -1.0) o << "{ const Real x_ = " << aq << ".x; " << aq << ".x = " << aq << ".y; " << aq << ".y = -x_; } ";
+                    int quad;
+                    double rt, rs;
+                    if (dr == -1.0 && di == 0.0) o << aq << ".x = neg_of(" << aq << ".x); " << aq << ".y = neg_of(" << aq << ".y); ";
+                    else if (dr == 0.0 && di == 1.0) o << "{ const Real x_ = " << aq << ".x; " << aq << ".x = neg_of(" << aq << ".y); " << aq << ".y = x_; } ";
+                    else if (dr == 0.0 && di == -1.0) o << "{ const Real x_ = " << aq << ".x; " << aq << ".x = " << aq << ".y; " << aq << ".y = neg_of(x_); } ";
+                    else if (mode == 1 && shears(dr, di, quad, rt, rs))
+                        o << "rotq_in<" << quad << ">(" << aq << ", " << L_lit(rt) << ", " << L_lit(rs) << "); ";
                     else o << "cmul_in(" << aq << ", " << L_(c + 2 * q) << ", " << L_(c + 2 * q + 1) << "); ";
                 }
                 break;
