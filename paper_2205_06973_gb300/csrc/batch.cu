@@ -127,13 +127,13 @@ __global__ void __launch_bounds__(256) k_batch(float2 *__restrict__ svbase, cons
                 uint64_t toff = deposit_b(tile, P.outer_mask);
 #pragma unroll
                 for (int j = 0; j < BT - BR; j++)
-                    if ((lane >> j) & 1) toff |= 1ull << P.store_thr_q[j];
+                    if ((lane >> j) & 1) toff ^= P.store_thr[j];
 #pragma unroll
                 for (int i = 0; i < BNR; i++) {
                     uint64_t off = toff;
 #pragma unroll
                     for (int b = 0; b < BR; b++)
-                        if (i & (1 << b)) off |= 1ull << P.store_reg_q[b];
+                        if (i & (1 << b)) off ^= P.store_reg[b];
                     __stcg(sv + off, a[i]);
                 }
             }
@@ -197,13 +197,13 @@ k_batch_whole(float2 *__restrict__ svbase, const BatchWhole *__restrict__ circui
     uint32_t toff = 0;
 #pragma unroll
     for (int j = 0; j < TB; j++)
-        if ((tid >> j) & 1) toff |= 1u << P.store_thr_q[j];
+        if ((tid >> j) & 1) toff ^= (uint32_t)P.store_thr[j];
 #pragma unroll
     for (int i = 0; i < NR; i++) {
         uint32_t off = toff;
 #pragma unroll
         for (int b = 0; b < R; b++)
-            if (i & (1 << b)) off |= 1u << P.store_reg_q[b];
+            if (i & (1 << b)) off ^= (uint32_t)P.store_reg[b];
         __stcg(sv + off, a[i]);
     }
 }

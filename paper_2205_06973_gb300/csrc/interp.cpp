@@ -15,6 +15,13 @@ uint16_t swz_of(int p, bool wide) {
     return (uint16_t)(p < 3 ? (1u << p) : ((1u << p) | (1u << (p % 3))));
 }
 
+uint16_t swz_mask(uint16_t v, bool wide) {
+    uint16_t o = 0;
+    for (int p = 0; p < 16; p++)
+        if ((v >> p) & 1) o = (uint16_t)(o ^ swz_of(p, wide));
+    return o;
+}
+
 // A phase under construction: its op records and the tables (their place in
 // the stream is known once the op count is).
 template <typename Real> struct PhaseOut {
@@ -22,7 +29,8 @@ template <typename Real> struct PhaseOut {
     std::vector<uint32_t> table_at;   // per op: index into table + 1, or 0
     std::vector<Real> table;
 
-    size_t bytes() const { return sizeof(IPhase) + ops.size() * sizeof(IOp<Real>) + table.size() * sizeof(Real); }
+    // two headers: a phase may have a write layout
+    size_t bytes() const { return 2 * sizeof(IPhase) + ops.size() * sizeof(IOp<Real>) + table.size() * sizeof(Real); }
     void emit(uint32_t code, uint32_t arg, double c0 = 0.0, double c1 = 0.0) {
         IOp<Real> o{};
         o.code = code;
@@ -54,12 +62,18 @@ template <typename Real> void lower(const Program &prog, Lowered &out) {
             bool cont = false;
             auto close = [&]() {   // append q to the stream
                 IPhase h{};
-                for (int b = 0; b < R; b++) h.sreg[b] = swz_of(ph.reg[b], wide);
-                for (int j = 0; j < TB; j++) h.sthr[j] = swz_of(ph.thr[j], wide);
+                auto layout = [&](const Layout &l, IPhase &d) {
+                    for (int b = 0; b < R; b++) d.sreg[b] = swz_mask(l.reg[b], wide);
+                    for (int j = 0; j < TB; j++) d.sthr[j] = swz_mask(l.thr[j], wide);
+                };
+                layout(ph.rd, h);
+                // the last phase's write layout is the part's store layout
+                const bool write = !cont && p + 1 < L.n_phases && std::memcmp(&ph.rd, &ph.wr, sizeof(Layout)) != 0;
                 h.n_ops = (uint32_t)q.ops.size();
-                h.bytes = (uint32_t)q.bytes();
-                h.flags = cont ? IPH_CONT : 0u;
-                const uint32_t t0 = (uint32_t)(sizeof(IPhase) + q.ops.size() * sizeof(IOp<Real>));
+                h.ops_at = (uint32_t)(write ? 2 * sizeof(IPhase) : sizeof(IPhase));
+                const uint32_t t0 = h.ops_at + (uint32_t)(q.ops.size() * sizeof(IOp<Real>));
+                h.bytes = t0 + (uint32_t)(q.table.size() * sizeof(Real));
+                h.flags = (cont ? IPH_CONT : 0u) | (write ? IPH_WRITE : 0u);
                 for (size_t i = 0; i < q.ops.size(); i++)
                     if (q.table_at[i]) q.ops[i].arg = t0 + (q.table_at[i] - 1) * (uint32_t)sizeof(Real);
                 if (out.windows.size() == w0 || out.windows.back().bytes + h.bytes > INTERP_WINDOW)
@@ -70,7 +84,12 @@ template <typename Real> void lower(const Program &prog, Lowered &out) {
                 out.stream.resize(at + h.bytes / 4);
                 char *d = reinterpret_cast<char *>(out.stream.data() + at);
                 std::memcpy(d, &h, sizeof(h));
-                if (!q.ops.empty()) std::memcpy(d + sizeof(h), q.ops.data(), q.ops.size() * sizeof(IOp<Real>));
+                if (write) {
+                    IPhase wr{};
+                    layout(ph.wr, wr);
+                    std::memcpy(d + sizeof(h), &wr, sizeof(wr));
+                }
+                if (!q.ops.empty()) std::memcpy(d + h.ops_at, q.ops.data(), q.ops.size() * sizeof(IOp<Real>));
                 if (!q.table.empty()) std::memcpy(d + t0, q.table.data(), q.table.size() * sizeof(Real));
                 q = PhaseOut<Real>();
                 cont = true;

@@ -51,18 +51,20 @@ static_assert(sizeof(IOp<float>) == 16 && sizeof(IOp<double>) == 32, "IOp layout
 
 // Header of a register phase: swizzled offsets of the register and thread
 // bits in the tile's buffer, then n_ops op records and the tables. A phase
-// whose ops do not fit a window is continued (IPH_CONT) under a second
-// header with the same layout and no transpose in between.
+// that is written with another layout than it is read (IPH_WRITE) has that
+// one, in the form of the first 64 bytes, before its ops. A phase whose ops
+// do not fit a window is continued (IPH_CONT) under a second header with the
+// same layout and no transpose in between.
 struct alignas(16) IPhase {
     uint16_t sreg[8];
     uint16_t sthr[MAX_TB];
     uint32_t n_ops;
-    uint32_t bytes;      // header, ops and tables: the next header follows
+    uint32_t bytes;      // all of it: the next header follows
     uint32_t flags;
-    uint32_t pad;
+    uint32_t ops_at;     // bytes from the header to the op records
 };
 static_assert(sizeof(IPhase) == 64, "IPhase layout");
-constexpr uint32_t IPH_CONT = 1u;
+constexpr uint32_t IPH_CONT = 1u, IPH_WRITE = 2u;
 
 struct IWindow {
     uint32_t at;         // in 16-byte units from the stream's start

@@ -102,6 +102,16 @@ unsigned swz_host(int p, bool fp64) {
     return p < 3 ? (1u << p) : ((1u << p) | (1u << (p % 3)));
 }
 
+// Shared-memory offset of a set of tile slots (the swizzle is linear). The
+// programs of these kernels have no CX folded into their layouts: each phase
+// is written as it is read.
+unsigned swz_mask(unsigned v, bool fp64) {
+    unsigned o = 0;
+    for (int p = 0; p < 16; p++)
+        if ((v >> p) & 1) o ^= swz_host(p, fp64);
+    return o;
+}
+
 template <typename T>
 std::string table(const char *type, const char *name, const std::vector<T> &v) {
     std::ostringstream o;
@@ -151,9 +161,9 @@ std::string jit_part_source(const Program &prog, size_t pi, bool df) {
     o << ";\n";
     for (int j = 0; j < TB; j++) {
         o << "    if ((tid >> " << j << ") & 1) { c_thr |= 0x" << std::hex << (1ull << L.tile_q[j]) << "ull; st_thr |= 0x"
-          << (1ull << L.store_thr_q[j]) << "ull; s_cthr ^= 0x" << swz_host(j, fp64) << "u;";
+          << L.store_thr[j] << "ull; s_cthr ^= 0x" << swz_host(j, fp64) << "u;";
         for (uint32_t p = 0; p < nph; p++)
-            o << " sp" << std::dec << p << " ^= 0x" << std::hex << swz_host(prog.phases[L.phase_begin + p].thr[j], fp64) << "u;";
+            o << " sp" << std::dec << p << " ^= 0x" << std::hex << swz_mask(prog.phases[L.phase_begin + p].rd.thr[j], fp64) << "u;";
         o << std::dec << " }\n";
     }
     std::vector<uint64_t> GO(NRr), SG(NRr);
@@ -165,7 +175,7 @@ std::string jit_part_source(const Program &prog, size_t pi, bool df) {
             if ((i >> b) & 1) {
                 g |= 1ull << L.tile_q[TB + b];
                 so ^= swz_host(TB + b, fp64);
-                s |= 1ull << L.store_reg_q[b];
+                s |= L.store_reg[b];
             }
         GO[i] = g;
         SO[i] = so;
@@ -178,7 +188,7 @@ std::string jit_part_source(const Program &prog, size_t pi, bool df) {
         for (int i = 0; i < NRr; i++) {
             uint32_t v = 0;
             for (int b = 0; b < R; b++)
-                if ((i >> b) & 1) v ^= swz_host(ph.reg[b], fp64);
+                if ((i >> b) & 1) v ^= swz_mask(ph.rd.reg[b], fp64);
             SR[i] = v;
         }
         o << table("u32", ("SR" + std::to_string(p)).c_str(), SR);

@@ -107,13 +107,14 @@ __device__ __forceinline__ double flip(double v, uint32_t m) {
     return __hiloint2double(__double2hiint(v) ^ (int)m, __double2loint(v));
 }
 
-// The ops of one phase header (hdr: in shared or global memory).
+// The ops of one phase header (hdr: in shared or global memory), at ops_at.
 template <typename Real, int R>
-__device__ __forceinline__ void run_ops(typename CT<Real>::T (&a)[1 << R], const char *hdr, uint32_t count,
+__device__ __forceinline__ void run_ops(typename CT<Real>::T (&a)[1 << R], const char *hdr, uint32_t ops_at,
+                                        uint32_t count,
                                         uint32_t tid, Real &tpr, Real &tpi, uint32_t &tsg) {
     constexpr int NR = 1 << R;
     if (count == 0) return;
-    const IOp<Real> *const ops = reinterpret_cast<const IOp<Real> *>(hdr + sizeof(IPhase));
+    const IOp<Real> *const ops = reinterpret_cast<const IOp<Real> *>(hdr + ops_at);
     IOp<Real> op = ld_op(ops);
     for (uint32_t o = 1;; o++) {
         const IOp<Real> cur = op;
@@ -261,7 +262,7 @@ __device__ __forceinline__ void run_window(typename CT<Real>::T (&a)[1 << R], ty
                                            uint32_t tid, Real &tpr, Real &tpi, uint32_t &tsg, Sync &&sync) {
     constexpr int NR = 1 << R;
     for (uint32_t p = 0; p < n_phases; p++) {
-        const uint4 h = *reinterpret_cast<const uint4 *>(w + 48);   // n_ops, bytes, flags
+        const uint4 h = *reinterpret_cast<const uint4 *>(w + 48);   // n_ops, bytes, flags, ops_at
         if (!(h.z & IPH_CONT)) {
             if (!first) {   // transpose through shared memory: write with the previous layout
                 sync();
@@ -273,8 +274,9 @@ __device__ __forceinline__ void run_window(typename CT<Real>::T (&a)[1 << R], ty
             S.load(w, tid);
 #pragma unroll
             for (int i = 0; i < NR; i++) a[i] = buf[S.at(i)];
+            if (h.z & IPH_WRITE) S.load(w + sizeof(IPhase), tid);
         }
-        run_ops<Real, R>(a, w, h.x, tid, tpr, tpi, tsg);
+        run_ops<Real, R>(a, w, h.w, h.x, tid, tpr, tpi, tsg);
         w += h.y;
     }
 }

@@ -84,7 +84,7 @@ k_part(typename CT<Real>::T *__restrict__ sv, const __grid_constant__ PartLaunch
         if ((tid >> j) & 1) {
             c_thr |= 1ull << L.tile_q[j];
             s_cthr ^= swz<Real>(j);
-            s_thr |= 1ull << L.store_thr_q[j];
+            s_thr ^= L.store_thr[j];
         }
     auto issue = [&](uint64_t base, C *dst) {
         const C *src = sv + (base | c_thr);
@@ -141,14 +141,14 @@ k_part(typename CT<Real>::T *__restrict__ sv, const __grid_constant__ PartLaunch
 #pragma unroll
             for (int i = 0; i < NR; i++) cmul_in(a[i], fr, fi);
         }
-        C *const dst = sv + (base | s_thr);
+        const uint64_t dst = base | s_thr;
 #pragma unroll
         for (int i = 0; i < NR; i++) {
-            uint64_t off = 0;
+            uint64_t off = dst;
 #pragma unroll
             for (int b = 0; b < R; b++)
-                if (i & (1 << b)) off |= 1ull << L.store_reg_q[b];
-            __stcs(dst + off, a[i]);
+                if (i & (1 << b)) off ^= L.store_reg[b];
+            __stcs(sv + off, a[i]);
         }
         base = nbase;
     }

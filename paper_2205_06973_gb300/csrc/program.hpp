@@ -58,13 +58,21 @@ constexpr int OP_OUTER = 32;
 constexpr int MAX_R = 6;
 constexpr int MAX_TB = 16;
 
+// A phase's layouts in the tile's buffer. The bits of a tile index are the
+// tile's slots; a layout gives each register and thread bit the set of slots
+// it flips (a bit mask). The phase reads with rd, and the transpose after it
+// writes with wr. Both are the plain slots of the bits, except that CX gates
+// before all or after all of the phase's other gates on their qubits are
+// folded into them: linear maps of the index, which cost nothing there.
+struct Layout {
+    uint16_t reg[8];         // register bit b (b < R)
+    uint16_t thr[MAX_TB];    // thread bit j (j < t - R)
+};
 struct Phase {
-    uint8_t reg[8];          // tile slot of register bit b (b < R)
-    uint8_t thr[MAX_TB];     // tile slot of thread bit j (j < t - R)
+    Layout rd, wr;
     uint32_t op_begin;
     uint32_t op_count;
 };
-static_assert(sizeof(Phase) == 32, "Phase layout");
 
 // Launch record of one part (passed by value to the kernel).
 struct PartLaunch {
@@ -79,8 +87,9 @@ struct PartLaunch {
     uint32_t coef_begin, coef_end;
     double gr, gi;           // part factor: 2^{-h/2} for h unnormalised H gates times RZ global phases
     uint8_t tile_q[32];      // global qubit of tile slot p (p < t); the gather/copy layout
-    uint8_t store_reg_q[8];  // global qubit of register bit b in the last phase (after SWAP relabels)
-    uint8_t store_thr_q[MAX_TB];
+    // the last phase's write layout in the state (after SWAP relabels): the
+    // qubits that a register or thread bit flips
+    uint64_t store_reg[8], store_thr[MAX_TB];
 };
 
 constexpr uint32_t PL_STORE_FACTOR = 1u;

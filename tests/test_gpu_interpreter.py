@@ -78,3 +78,38 @@ def test_batch_of_small_and_large(dense):
     assert info["items"] > 0 and info["parts"] >= len(circs) - info["dense_circuits"] - 1
     b.close()
     torch.cuda.synchronize()
+
+
+def _cx_net(n, depth, seed):
+    """Runs of CX (chains both ways, fans, random pairs, onto and off the
+    lowest five qubits), SWAPs among them, separated by gates that do and do
+    not commute with a CX on either qubit."""
+    rng = np.random.default_rng(seed)
+    g = [("H", (q,), 0.0) for q in range(n)]
+    for _ in range(depth):
+        kind = int(rng.integers(4))
+        if kind == 0:
+            g += [("CX", (q, q + 1), 0.0) for q in range(n - 1)]
+        elif kind == 1:
+            g += [("CX", (q + 1, q), 0.0) for q in reversed(range(n - 1))]
+        elif kind == 2:
+            c = int(rng.integers(n))
+            g += [("CX", (c, q), 0.0) for q in range(n) if q != c]
+        for _ in range(n):
+            a, b = (int(x) for x in rng.choice(n, 2, replace=False))
+            g.append(("SWAP" if rng.random() < 0.1 else "CX", (a, b), 0.0))
+        for q in rng.choice(n, n // 3, replace=False):
+            name = ("RZ", "RX", "T", "X", "H", "RY")[int(rng.integers(6))]
+            g.append((name, (int(q),), float(rng.uniform(0, 6))))
+    return g
+
+
+@pytest.mark.parametrize("precision", ["c64", "c128", "c128df"])
+@pytest.mark.parametrize("n", [10, 13, 16])
+def test_cx_at_the_ends_of_phases(n, precision):
+    g = _cx_net(n, 8, n)
+    psi = random_state(n, 3 * n)
+    ref = sim.run(n, g, psi)
+    for method, k, tile in (("nat", 8, 10), ("dagp", 7, 0), ("beam", 9, 0), ("dfs", 6, 11)):
+        out = run_gpu(n, g, method=method, k=k, precision=precision, psi=psi, tile=min(tile, n))
+        assert max_abs(out, ref) <= TOL[precision], (method, k, tile)
