@@ -52,6 +52,7 @@ struct sv_state {
     int dev = 0;
     double *d_partials = nullptr;   // kProbBlocks + 1 doubles; the last holds the norm
     double h_norm = 0.0;            // norm read back from the device
+    double *h_slot = nullptr;       // pinned result slot (taken at the first measurement)
     int *d_err = nullptr;           // device error word of bounded waits (0 = none), then the
                                     // block tickets of the measurements
     double *d_dnorm = nullptr;      // norm accumulators of one apply's dense passes

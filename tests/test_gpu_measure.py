@@ -102,3 +102,22 @@ def test_batch_probs_alignment_and_norms():
     b.sync()
     assert only[1] is None
     b.close()
+
+
+def test_more_states_than_result_slots():
+    """The 65th live state that measures copies its results."""
+    _, api = native()
+    n = 6
+    states = []
+    for i in range(66):
+        st = api.State(n)
+        st.set_basis(i % 64)
+        states.append(st)
+    for i, st in enumerate(states):
+        assert st.summary() == (1.0, float(i % 64 == 0), i % 64, 1.0)
+        p = torch.empty(1 << n, device="cuda")
+        assert st.probs(p) == 1.0 and int(p.argmax()) == i % 64
+    states[3].close()
+    assert states[65].summary() == (1.0, 0.0, 1, 1.0)
+    for st in states:
+        st.close()
