@@ -549,7 +549,9 @@ static int dense_mode(uint32_t flags, bool fp64) {
 //    the SMs twice the warps where a pass is a tile or less per SM (14 to 19
 //    qubits: 8 to 17 % shorter applies; even at 20 and 21, 5 to 13 % longer
 //    above), and up to 17 qubits half the tile (15 to 30 % shorter at 12 to
-//    16 qubits; even at 18);
+//    16 qubits; even at 18); at 20 qubits twice the tile, 128 tiles of 152
+//    SMs in one wave (k = 10: 130 -> 90 us layered, 155 -> 133 parameterised;
+//    at 19 and 21 even to 60 % longer);
 //  * double-float: 2^3 amplitudes per thread; with 2^4 the straight-line code
 //    (about 40 instructions per amplitude and gate) outran the instruction
 //    cache (4.6 of 7 stall cycles; 25 qubits: 12.6 against 8.3 ms, on 2^12
@@ -568,8 +570,9 @@ static int spec_mode(const sv_plan *p, sv_precision prec, uint32_t flags, int t_
     if (t_user || ((flags >> 8) & 0xFu) || !p->inner.empty()) return mode;
     int R = part_R(fp64);
     if (!fp64) {
-        if (p->n <= 19) R = 4;
+        if (p->n <= 20) R = 4;
         if (p->n <= 17 && t == 12) t = 11;
+        if (p->n == 20) t = 13;
     } else if (prec == SV_C128DF) {
         R = 3;
         if (p->n >= 22) t = part_tmax(true);
@@ -584,25 +587,37 @@ static int spec_mode(const sv_plan *p, sv_precision prec, uint32_t flags, int t_
 //  * Multi-level plans keep the register bits their second level may use.
 //  * A complex64 state of at most 13 qubits on its default tile is one tile:
 //    all gates become one part, in their order, so the apply is one launch
-//    that keeps the state on chip from the first gate to the last.
+//    that keeps the state on chip from the first gate to the last. At 10
+//    qubits 2^3 amplitudes per thread (15 layers: 34 -> 31 us, parameterised
+//    52 -> 49; at 11 and 12 qubits 38 -> 38, 82 -> 92).
 //  * A small complex128 state is cut into tiles down to 2^8 amplitudes until
 //    there are two per SM: an SM has about two FP64 lanes, so its tiles'
 //    arithmetic sets the time, and 14 qubits on 2^11 tiles keep 8 of 152 SMs
 //    busy (the 840-gate layered circuit: 1.11 ms; on 2^8 tiles 0.49 ms).
+//  * A complex64 state of 14 to 18 qubits is cut into smaller tiles while
+//    there is no more than one per SM, of 2^3 amplitudes per thread up to 17
+//    qubits: 15 layers, k = 10, in us on 2^12 / 2^11 / 2^10 tiles with 2^4 and
+//    on 2^10 with 2^3 amplitudes: 14 qubits 79 / 65 / 66 / 56, 17 qubits 102 /
+//    83 / 91 / 80 (parameterised 153 / 122 / 124 / 114); 18 qubits 111 / 93 /
+//    138 / 129, 19 qubits 117 / 149 / 170 / 168.
 static int interp_mode(const sv_plan *p, bool fp64, uint32_t flags, int t_user, int &t) {
     const int tc = dense_mode(flags, fp64) & 3;
     const bool ml = !p->inner.empty();
-    const int R = ml ? part_R(fp64) : interp_R(fp64);
+    int R = ml ? part_R(fp64) : interp_R(fp64);
     t = t_user ? t_user : default_tile(fp64, p->max_part);
     if (t_user || ml) return tc | (R << 4);
     if (!fp64 && p->n <= part_tmax(false) && !(tc && p->n >= DENSE_K + DENSE_COLS)) {
         t = p->n;
+        if (t == 10) R = 3;
         return kModeWhole | (R << 4);
     }
     if (fp64) {
         t = small_tiles(p, t);
-    } else if (t == 12 && p->max_part < 12 && p->n < t + 6) {
-        t = 11;   // fewer than 64 tiles: halves (16 qubits, 15 layers, k = 10: 110 -> 94 us)
+    } else if (p->n <= 17 && p->max_part <= 10) {
+        t = 10;
+        R = 3;
+    } else if (t == 12 && p->max_part < 12 && p->n <= 18) {
+        t = 11;
     }
     return tc | (R << 4);
 }

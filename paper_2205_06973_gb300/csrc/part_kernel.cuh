@@ -53,7 +53,7 @@ template <typename Real, int T, int R>
 struct PartCfg {
     static constexpr int NT = 1 << (T - R);
     static constexpr int SMEM = 2 * (1 << T) * 2 * (int)sizeof(Real) + (int)INTERP_WINDOW;
-    static constexpr int REGS = sizeof(Real) == 8 ? (R == 4 ? 168 : 120) : (R == 5 ? 168 : 104);
+    static constexpr int REGS = sizeof(Real) == 8 ? (R == 4 ? 168 : 120) : (R == 5 ? 168 : R == 4 ? 104 : 64);
     static constexpr int BY_REG = 65536 / (REGS * NT);
     static constexpr int BY_SMEM = (227 * 1024) / (SMEM + 1024);
     static constexpr int MINB0 = BY_REG < BY_SMEM ? BY_REG : BY_SMEM;
