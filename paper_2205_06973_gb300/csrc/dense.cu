@@ -74,25 +74,27 @@ k_dense6(float2 *__restrict__ sv, const __grid_constant__ DenseLaunch L, const u
     uint8_t *const base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t *const sR = base;                                               // R image (B operand)
     uint64_t *const bars = reinterpret_cast<uint64_t *>(base + DENSE_A_BYTES);
-    uint64_t *const afull = bars, *const dfull = bars + 2, *const dempty = bars + 4;
+    uint64_t *const afull = bars, *const dfull = bars + 2, *const dempty = bars + 4, *const rfull = bars + 6;
     uint32_t *const tslot = reinterpret_cast<uint32_t *>(base + DENSE_A_BYTES + 128);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-    for (int i = tid; i < DENSE_A_BYTES / 16; i += DENSE_THREADS)
-        reinterpret_cast<uint4 *>(sR)[i] = reinterpret_cast<const uint4 *>(a_img)[i];
     if (tid == 0) {
         for (int b = 0; b < 2; b++) {
             mbar_init(&afull[b], CONV_THREADS);
             mbar_init(&dfull[b], 1);
             mbar_init(&dempty[b], EPI_THREADS);
         }
+        mbar_init(rfull, 1);
         mbar_init_fence();
+        // R in one bulk copy that only the MMA thread waits for (loads and
+        // shared-memory stores of all threads before the first barrier: 8.2
+        // instead of 7.1 us a pass of 20 qubits)
+        bulk_copy(sR, a_img, DENSE_A_BYTES, rfull);
     }
     if (warp == MMA_WARP) {
         tmem_alloc(tslot, TMEM_COLS);
         tmem_relinquish();
     }
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // R image visible to the MMAs
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -190,7 +192,12 @@ k_dense6(float2 *__restrict__ sv, const __grid_constant__ DenseLaunch L, const u
             const uint32_t idesc = idesc_bf16_f32(128, 128);
             const uint32_t sb = smem_u32(sR);
             uint32_t i = 0;
-            for (uint64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, i++) {
+            const bool image = mbar_wait(rfull, 0, WAIT_LIMIT);
+            if (!image) {
+                atomicExch(err, 1);
+                mbar_wait(rfull, 0, WAIT_LIMIT);   // its own copy in flight
+            }
+            for (uint64_t tile = blockIdx.x; image && tile < n_tiles; tile += gridDim.x, i++) {
                 const uint32_t b = i & 1, u = i >> 1;
                 if (!mbar_wait(&afull[b], u & 1, WAIT_LIMIT) ||
                     (i >= 2 && !mbar_wait(&dempty[b], (u - 1) & 1, WAIT_LIMIT))) {
