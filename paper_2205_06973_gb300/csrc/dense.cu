@@ -116,6 +116,7 @@ k_dense6(float2 *__restrict__ sv, const __grid_constant__ DenseLaunch L, const u
     for (int b = 0; b < DENSE_K; b++) pbit[b] = 1ull << L.part_q[b];
     const uint64_t hoff = h ? pbit[DENSE_K - 1] : 0ull;  // amplitude bit 5 = the half
     const uint64_t dgrid = deposit_bits(gridDim.x, L.outer_mask);
+    const uint64_t flip = L.reverse ? L.outer_mask : 0ull;   // the tiles backwards
 
     if (warp >= EPI_WARPS && warp < MMA_WARP) {
         // ------------------------------------------------------ converters
@@ -143,9 +144,9 @@ k_dense6(float2 *__restrict__ sv, const __grid_constant__ DenseLaunch L, const u
             tc_fence_after();
             if (tile + gridDim.x < n_tiles) {
 #pragma unroll
-                for (int u = 0; u < 2; u++) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(sv + (tpf | lineoff[u])));
+                for (int u = 0; u < 2; u++) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(sv + ((tpf ^ flip) | lineoff[u])));
             }
-            const float2 *const src = sv + (tb | coff | hoff);
+            const float2 *const src = sv + ((tb ^ flip) | coff | hoff);
             const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + 256 + 128 * b + 32 * h;
             float tile_in = 0.0f;   // FP32 partial of this tile, folded into the FP64 sum
 #pragma unroll
@@ -243,7 +244,7 @@ k_dense6(float2 *__restrict__ sv, const __grid_constant__ DenseLaunch L, const u
             }
             tc_fence_after();
             const uint32_t td = tmem + ((uint32_t)(32 * q) << 16) + 128 * b;
-            float2 *const dst = sv + (tb | coff);
+            float2 *const dst = sv + ((tb ^ flip) | coff);
             float tile_out = 0.0f;
 #pragma unroll
             for (int g = 0; g < 4; g++) {   // 16 amplitudes (32 columns) at a time

@@ -22,7 +22,7 @@ struct DenseLaunch {
     uint8_t col_q[DENSE_COLS]; // qubit of column bit j (ascending)
     uint8_t slot_q[16];        // the 13 tile qubits in ascending order (gather layout)
     uint16_t slot_part;        // bit s set: slot s is a part qubit
-    uint16_t pad;
+    uint16_t reverse;          // 1: the tiles from the last to the first
 };
 
 // Launch record of a pass that applies two dense parts (by value): the tile

@@ -193,9 +193,10 @@ std::string jit_part_source(const Program &prog, size_t pi, bool df) {
         }
         o << table("u32", ("SR" + std::to_string(p)).c_str(), SR);
     }
+    const bool reverse = L.flags & PL_REVERSE;
     o << "    C a[NR];\n"
       << "    u64 tile = blockIdx.x;\n"
-      << "    u64 base = tile < n_tiles ? deposit64(tile, OUTER) : 0ull;\n"
+      << "    u64 base = tile < n_tiles ? deposit64(tile, OUTER)" << (reverse ? " ^ OUTER" : "") << " : 0ull;\n"
       << "    const u64 DGRID = deposit64(gridDim.x, OUTER);\n"
       << "    pdl_wait();\n"
       << "    if (tile < n_tiles) {\n"
@@ -209,7 +210,8 @@ std::string jit_part_source(const Program &prog, size_t pi, bool df) {
       << "        C *const nxt = (it & 1) ? buf0 : buf1;\n"
       << "        __syncthreads();\n"
       << "        const u64 ntile = tile + gridDim.x;\n"
-      << "        const u64 nbase = ((base | ~OUTER) + DGRID) & OUTER;\n"   // carries run over the tile's qubits
+      << (reverse ? "        const u64 nbase = (base - DGRID) & OUTER;\n"   // carries and borrows run over the tile's qubits
+                  : "        const u64 nbase = ((base | ~OUTER) + DGRID) & OUTER;\n")
       << "        if (ntile < n_tiles) {\n"
       << "            const C *src = sv + (nbase | c_thr);\n"
       << "#pragma unroll\n"

@@ -105,9 +105,10 @@ k_part(typename CT<Real>::T *__restrict__ sv, const __grid_constant__ PartLaunch
     C a[NR];
     uint64_t tile = blockIdx.x;
     const uint64_t dgrid = deposit64(gridDim.x, L.outer_mask);
+    const uint64_t flip = L.flags & PL_REVERSE ? L.outer_mask : 0ull;
     uint64_t base = deposit64(tile, L.outer_mask);
     pdl_wait();   // the previous pass has written the state
-    if (tile < n_tiles) issue(base, buf0);
+    if (tile < n_tiles) issue(base ^ flip, buf0);
     cp_async_commit();
     for (uint32_t it = 0; tile < n_tiles; tile += gridDim.x, it++) {
         C *const cur = (it & 1) ? buf1 : buf0;
@@ -115,7 +116,7 @@ k_part(typename CT<Real>::T *__restrict__ sv, const __grid_constant__ PartLaunch
         __syncthreads();   // every thread is done with nxt (it was cur two stages ago)
         // the next tile's outer bits: an add whose carries run over the tile's qubits
         const uint64_t nbase = ((base | ~L.outer_mask) + dgrid) & L.outer_mask;
-        if (tile + gridDim.x < n_tiles) issue(nbase, nxt);
+        if (tile + gridDim.x < n_tiles) issue(nbase ^ flip, nxt);
         else pdl_launch();
         cp_async_commit();
         cp_async_wait<1>();  // this tile's copies have landed
@@ -141,7 +142,7 @@ k_part(typename CT<Real>::T *__restrict__ sv, const __grid_constant__ PartLaunch
 #pragma unroll
             for (int i = 0; i < NR; i++) cmul_in(a[i], fr, fi);
         }
-        const uint64_t dst = base | s_thr;
+        const uint64_t dst = (base ^ flip) | s_thr;
 #pragma unroll
         for (int i = 0; i < NR; i++) {
             uint64_t off = dst;

@@ -399,6 +399,7 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
             fused_unitary(gates, gl, qs, DENSE_K, U);
             std::vector<uint8_t> img;
             dense_a_image(U.data(), img);
+            D.reverse = prog.kind.size() & 1;
             prog.kind.push_back(1);
             prog.index.push_back((uint32_t)prog.dense.size());
             prog.dense.push_back(D);
@@ -994,6 +995,12 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
         L.gr = fr;
         L.gi = fi;
         L.flags = (last_tphase || fr != 1.0 || fi != 0.0) ? PL_STORE_FACTOR : 0u;
+        // every other pass takes the tiles backwards: it begins with what the
+        // pass before wrote last, which L2 still holds (layered circuits, k =
+        // 7 to 9 specialised: 24 qubits 699 -> 610 and 1156 -> 1072 us, 26 qubits
+        // 4.60 -> 4.51 ms, 28 qubits 21.29 -> 21.24; tensor-core passes at 24
+        // qubits 1.64 -> 1.52 ms; up to 23 qubits the state stays in L2 anyway)
+        if (prog.kind.size() & 1) L.flags |= PL_REVERSE;
         prog.kind.push_back(0);
         prog.index.push_back((uint32_t)prog.parts.size());
         prog.parts.push_back(L);

@@ -93,5 +93,6 @@ struct PartLaunch {
 };
 
 constexpr uint32_t PL_STORE_FACTOR = 1u;
+constexpr uint32_t PL_REVERSE = 2u;   // the tiles from the last to the first
 
 }  // namespace hisv
