@@ -66,7 +66,62 @@ constexpr uint32_t DENSE_SMEM = 120 * 1024;
 constexpr uint32_t WAIT_LIMIT = 1u << 24;            // bounded mbarrier polls
 static_assert(DENSE_A_BYTES + 1024 + 16 * CONV_THREADS + 1024 <= (int)DENSE_SMEM, "shared memory layout");
 
+__device__ __forceinline__ void pass_dependency() {
+    // the previous kernel on the stream (another pass) has completed and its
+    // writes (state, norm accumulators) are visible from here on
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+// Amplitude m's bits on the part's qubits (m's low log2(W) bits are 0: W
+// consecutive amplitudes).
+template <int B>
+__device__ __forceinline__ uint64_t part_offset(int m, const uint64_t (&pbit)[DENSE_K]) {
+    uint64_t o = 0;
+#pragma unroll
+    for (int b = 0; b < B; b++)
+        if ((m >> b) & 1) o |= pbit[b];
+    return o;
+}
+// 16 amplitudes of this lane's column, as BF16 hi at ta and lo at ta + 64;
+// their |a|^2 added to norm.
+__device__ __forceinline__ void split_to_tmem(const float2 *x, uint32_t ta, float &norm) {
+    uint32_t hi[16], lo[16];
+#pragma unroll
+    for (int j = 0; j < 16; j++) {
+        const float2 v = x[j];
+        norm = fmaf(v.x, v.x, fmaf(v.y, v.y, norm));
+        const __nv_bfloat162 bh = __floats2bfloat162_rn(v.x, v.y);
+        const float2 hf = __bfloat1622float2(bh);
+        const __nv_bfloat162 bl = __floats2bfloat162_rn(v.x - hf.x, v.y - hf.y);
+        hi[j] = *reinterpret_cast<const uint32_t *>(&bh);
+        lo[j] = *reinterpret_cast<const uint32_t *>(&bl);
+    }
+    tmem_st16(ta, hi);
+    tmem_st16(ta + 64, lo);
+}
+// 16 accumulated amplitudes, scaled, to amplitudes m0.. of the column dst.
 template <int W>
+__device__ __forceinline__ void store_amps(float2 *dst, int m0, const uint64_t (&pbit)[DENSE_K],
+                                           const uint32_t (&r)[32], float scale, float &norm) {
+#pragma unroll
+    for (int j = 0; j < 16; j += W) {
+        float2 y[W];
+#pragma unroll
+        for (int w = 0; w < W; w++) {
+            y[w] = make_float2(__uint_as_float(r[2 * (j + w)]) * scale, __uint_as_float(r[2 * (j + w) + 1]) * scale);
+            norm = fmaf(y[w].x, y[w].x, fmaf(y[w].y, y[w].y, norm));
+        }
+        st_amps<W>(dst + part_offset<6>(m0 + j, pbit), y);
+    }
+}
+
+// ONE: no more tiles than SMs, so each CTA has a single tile and a pass is
+// the latency of its chain. The geometry is then computed before the wait
+// for the previous pass, all loads are in flight at once, and the converter
+// warps run the epilogue (15 parameterised layers, us against the loop over
+// tiles: 13 qubits 111 -> 106, 16 qubits 148 -> 131, 18 qubits 177 -> 150, 20
+// qubits 207 -> 180). More tiles need the loop, whose four epilogue warps
+// store one tile while the next is loaded.
+template <int W, bool ONE>
 __global__ void __launch_bounds__(DENSE_THREADS, 1)
 k_dense6(float2 *__restrict__ sv, const __grid_constant__ DenseLaunch L, const uint8_t *__restrict__ a_img,
          uint64_t n_tiles, int *__restrict__ err, double *__restrict__ dn, uint32_t dense_idx) {
@@ -99,10 +154,6 @@ k_dense6(float2 *__restrict__ sv, const __grid_constant__ DenseLaunch L, const u
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
-    // the previous kernel on the stream (another pass) has completed and its
-    // writes (state, norm accumulators) are visible from here on
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
-
     // per-thread geometry shared by converters and epilogue: TMEM lane
     // quarter q and amplitude half h of the warp; column n = 32 q + lane
     const int q = warp & 3, h = warp >= EPI_WARPS ? ((warp - EPI_WARPS) >> 2) & 1 : 0;
@@ -118,7 +169,59 @@ k_dense6(float2 *__restrict__ sv, const __grid_constant__ DenseLaunch L, const u
     const uint64_t dgrid = deposit_bits(gridDim.x, L.outer_mask);
     const uint64_t flip = L.reverse ? L.outer_mask : 0ull;   // the tiles backwards
 
-    if (warp >= EPI_WARPS && warp < MMA_WARP) {
+    if constexpr (ONE) {
+        // a single tile: the 8 converter warps also run the epilogue, each
+        // for its own half of the amplitudes
+        const uint64_t tb = deposit_bits(blockIdx.x, L.outer_mask) ^ flip;
+        float2 *const col = sv + (tb | coff | hoff);
+        pass_dependency();
+        if (warp >= EPI_WARPS && warp < MMA_WARP) {
+            const uint32_t tq = tmem + ((uint32_t)(32 * q) << 16);
+            float2 x[32];
+#pragma unroll
+            for (int m = 0; m < 32; m += W) ld_amps<W>(col + part_offset<5>(m, pbit), x + m);
+            double n0 = 0.0, prev = 0.0;
+            if (dense_idx > 0) {
+                n0 = dn[0];
+                prev = dn[dense_idx];
+            }
+            float in = 0.0f;
+#pragma unroll
+            for (int g = 0; g < 2; g++) split_to_tmem(x + 16 * g, tq + 256 + 32 * h + 16 * g, in);
+            tmem_st_wait();
+            tc_fence_before();
+            mbar_arrive(&afull[0]);
+            const float scale = n0 > 0.0 && prev > 0.0 ? (float)sqrt(n0 / prev) : 1.0f;
+            if (__all_sync(0xffffffffu, mbar_wait(&dfull[0], 0, WAIT_LIMIT))) {   // warp-uniform (tcgen05.ld)
+                tc_fence_after();
+                float out = 0.0f;
+#pragma unroll
+                for (int g = 0; g < 2; g++) {
+                    uint32_t r[32];
+                    tmem_ld32(tq + 64 * h + 32 * g, r);
+                    tmem_ld_wait();
+                    store_amps<W>(col, 16 * g, pbit, r, scale, out);
+                }
+                tc_fence_before();
+                double sum = (double)out;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                if (lane == 0) atomicAdd(dn + 1 + dense_idx, sum);
+            } else {
+                atomicExch(err, 1);
+            }
+            if (dense_idx == 0) {
+                double sum = (double)in;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                if (lane == 0) atomicAdd(dn, sum);
+            }
+        }
+    } else {
+        pass_dependency();
+    }
+
+    if (!ONE && warp >= EPI_WARPS && warp < MMA_WARP) {
         // ------------------------------------------------------ converters
         // L2 warm-up lines of a tile: qubits 0..3 are tile qubits, so a tile
         // is 512 lines of 128 bytes, line lam at the deposit of lam into the
@@ -153,27 +256,8 @@ k_dense6(float2 *__restrict__ sv, const __grid_constant__ DenseLaunch L, const u
             for (int g = 0; g < 2; g++) {   // two rounds of 16 loads (the lines are in L2 by now)
                 float2 x[16];
 #pragma unroll
-                for (int j = 0; j < 16; j += W) {
-                    const int m = 16 * g + j;   // its low log2(W) bits are 0: W consecutive amplitudes
-                    uint64_t o = 0;
-#pragma unroll
-                    for (int bb = 0; bb < 5; bb++)
-                        if ((m >> bb) & 1) o |= pbit[bb];
-                    ld_amps<W>(src + o, x + j);
-                }
-                uint32_t hi[16], lo[16];
-#pragma unroll
-                for (int j = 0; j < 16; j++) {
-                    const float2 v = x[j];
-                    tile_in = fmaf(v.x, v.x, fmaf(v.y, v.y, tile_in));
-                    const __nv_bfloat162 bh = __floats2bfloat162_rn(v.x, v.y);
-                    const float2 hf = __bfloat1622float2(bh);
-                    const __nv_bfloat162 bl = __floats2bfloat162_rn(v.x - hf.x, v.y - hf.y);
-                    hi[j] = *reinterpret_cast<const uint32_t *>(&bh);
-                    lo[j] = *reinterpret_cast<const uint32_t *>(&bl);
-                }
-                tmem_st16(ta + 16 * g, hi);
-                tmem_st16(ta + 64 + 16 * g, lo);
+                for (int j = 0; j < 16; j += W) ld_amps<W>(src + part_offset<5>(16 * g + j, pbit), x + j);
+                split_to_tmem(x, ta + 16 * g, tile_in);
             }
             tmem_st_wait();
             tc_fence_before();
@@ -224,7 +308,7 @@ k_dense6(float2 *__restrict__ sv, const __grid_constant__ DenseLaunch L, const u
             // the MMAs of the last tile complete before the TMEM is freed
             if (i > 0 && !mbar_wait(&dfull[(i - 1) & 1], ((i - 1) >> 1) & 1, WAIT_LIMIT)) atomicExch(err, 1);
         }
-    } else {
+    } else if (!ONE) {
         // ------------------------------------------------------ epilogue
         // unitarity: rescale to the input norm N0 measured by the first dense
         // pass, correcting the drift measured on the previous dense pass
@@ -255,22 +339,7 @@ k_dense6(float2 *__restrict__ sv, const __grid_constant__ DenseLaunch L, const u
                     tc_fence_before();
                     mbar_arrive(&dempty[b]);
                 }
-#pragma unroll
-                for (int j = 0; j < 16; j += W) {
-                    const int m = 16 * g + j;
-                    uint64_t o = 0;
-#pragma unroll
-                    for (int bb = 0; bb < 6; bb++)
-                        if ((m >> bb) & 1) o |= pbit[bb];
-                    float2 y[W];
-#pragma unroll
-                    for (int w = 0; w < W; w++) {
-                        y[w] = make_float2(__uint_as_float(r[2 * (j + w)]) * scale,
-                                           __uint_as_float(r[2 * (j + w) + 1]) * scale);
-                        tile_out = fmaf(y[w].x, y[w].x, fmaf(y[w].y, y[w].y, tile_out));
-                    }
-                    st_amps<W>(dst + o, y);
-                }
+                store_amps<W>(dst, 16 * g, pbit, r, scale, tile_out);
             }
             out_norm += (double)tile_out;
             tb = masked_add(tb, dgrid, L.outer_mask);
@@ -325,6 +394,10 @@ void dense_a_image(const double *U, std::vector<uint8_t> &img) {
         }
 }
 
+template <int W, bool ONE> static cudaError_t dense_attr() {
+    return cudaFuncSetAttribute(k_dense6<W, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DENSE_SMEM);
+}
+
 cudaError_t launch_dense6(void *sv, const DenseLaunch &L, const void *a_img, uint64_t n_tiles, int *d_err,
                           double *d_norms, uint32_t dense_idx, cudaStream_t st) {
     // per device: shared-memory limit raised and SM count cached, once
@@ -339,12 +412,10 @@ cudaError_t launch_dense6(void *sv, const DenseLaunch &L, const void *a_img, uin
     if (!((attr_set.load(std::memory_order_acquire) >> dev) & 1)) {
         std::lock_guard<std::mutex> lk(mu);
         if (!((attr_set.load(std::memory_order_relaxed) >> dev) & 1)) {
-            e = cudaFuncSetAttribute(k_dense6<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DENSE_SMEM);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_dense6<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DENSE_SMEM);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_dense6<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DENSE_SMEM);
-            if (e != cudaSuccess) return e;
+            const cudaError_t es[6] = {dense_attr<1, false>(), dense_attr<2, false>(), dense_attr<4, false>(),
+                                       dense_attr<1, true>(), dense_attr<2, true>(), dense_attr<4, true>()};
+            for (cudaError_t x : es)
+                if (x != cudaSuccess) return x;
             e = cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev);
             if (e != cudaSuccess) return e;
             attr_set.fetch_or(1ull << dev, std::memory_order_release);
@@ -371,12 +442,13 @@ cudaError_t launch_dense6(void *sv, const DenseLaunch &L, const void *a_img, uin
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (z >= 2 && a32)
-        e = cudaLaunchKernelEx(&cfg, k_dense6<4>, p, L, a, n_tiles, d_err, d_norms, dense_idx);
-    else if (z >= 1)
-        e = cudaLaunchKernelEx(&cfg, k_dense6<2>, p, L, a, n_tiles, d_err, d_norms, dense_idx);
+    const bool one = n_tiles <= (uint64_t)sms[dev];
+    const int w = z >= 2 && a32 ? 4 : z >= 1 ? 2 : 1;
+    auto go = [&](auto kern) { return cudaLaunchKernelEx(&cfg, kern, p, L, a, n_tiles, d_err, d_norms, dense_idx); };
+    if (one)
+        e = w == 4 ? go(k_dense6<4, true>) : w == 2 ? go(k_dense6<2, true>) : go(k_dense6<1, true>);
     else
-        e = cudaLaunchKernelEx(&cfg, k_dense6<1>, p, L, a, n_tiles, d_err, d_norms, dense_idx);
+        e = w == 4 ? go(k_dense6<4, false>) : w == 2 ? go(k_dense6<2, false>) : go(k_dense6<1, false>);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
