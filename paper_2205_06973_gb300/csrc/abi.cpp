@@ -589,7 +589,12 @@ static int spec_mode(const sv_plan *p, sv_precision prec, uint32_t flags, int t_
 //    all gates become one part, in their order, so the apply is one launch
 //    that keeps the state on chip from the first gate to the last. At 10
 //    qubits 2^3 amplitudes per thread (15 layers: 34 -> 31 us, parameterised
-//    52 -> 49; at 11 and 12 qubits 38 -> 38, 82 -> 92).
+//    52 -> 49; at 11 and 12 qubits 38 -> 38, 82 -> 92). At 12 and 13 qubits
+//    one SM's issue (about 0.17 and 0.25 us a gate) takes longer than the
+//    passes of a plan with enough gates to a part (about 2 us a pass and 0.13
+//    us a gate on 2^10 tiles): k = 10, 12 qubits 54 -> 47 us, parameterised
+//    82 -> 70, but with k = 6 and 33 gates to a part 82 -> 92; 13 qubits 78 ->
+//    50 and 134 -> 78, with k = 6 and 31 gates to a part 134 -> 104.
 //  * A small complex128 state is cut into tiles down to 2^8 amplitudes until
 //    there are two per SM: an SM has about two FP64 lanes, so its tiles'
 //    arithmetic sets the time, and 14 qubits on 2^11 tiles keep 8 of 152 SMs
@@ -606,7 +611,8 @@ static int interp_mode(const sv_plan *p, bool fp64, uint32_t flags, int t_user, 
     int R = ml ? part_R(fp64) : interp_R(fp64);
     t = t_user ? t_user : default_tile(fp64, p->max_part);
     if (t_user || ml) return tc | (R << 4);
-    if (!fp64 && p->n <= part_tmax(false) && !(tc && p->n >= DENSE_K + DENSE_COLS)) {
+    const bool cut = p->n >= 12 && p->max_part <= 10 && p->gates.size() >= (p->n == 12 ? 40 : 20) * (size_t)p->n_parts;
+    if (!fp64 && p->n <= part_tmax(false) && !cut && !(tc && p->n >= DENSE_K + DENSE_COLS)) {
         t = p->n;
         if (t == 10) R = 3;
         return kModeWhole | (R << 4);
