@@ -449,7 +449,7 @@ def run_e2e_only(a):
     tc, jit = int(a.tc), bool(a.jit)
     if jit:
         plan.specialise("c64", a.tile, tc=tc, regbits=a.regbits)
-    passes = plan.stats("c64", a.tile, tc=tc, regbits=a.regbits)["passes"]
+    passes = plan.stats("c64", a.tile, tc=tc, regbits=a.regbits, jit=jit)["passes"]
     e2e = e2e_loop(n, plan, tc, jit, a.regbits, a.tile, S, host_in, host_out, 1, torch.device("cuda", 0),
                    passes * 2 * (8 << n))
     e2e["host_buffers"] = "pinned, allocated at process start"
@@ -555,7 +555,7 @@ def grid_section(n, gates, st, peak, fp32_peak=None):
                 if jit:
                     row["compile_s"] = round(plan.specialise("c64"), 2)
                 ms = _timed(st, plan, jit=jit)
-                gbs = passes * 2 * st.nbytes / (ms / 1e3) / 1e9
+                gbs = plan.stats("c64", jit=jit)["passes"] * 2 * st.nbytes / (ms / 1e3) / 1e9
                 row[name] = {"ms": round(ms, 2), "GBs": round(gbs, 1), "frac": round(gbs / peak, 4)}
                 if fp32_peak:
                     fl = flops / (ms / 1e3)
@@ -570,7 +570,7 @@ def grid_section(n, gates, st, peak, fp32_peak=None):
                 plan.specialise("c64", 12)
                 ms = _timed(st, plan, jit=True)
                 st.set_tile(0)
-                gbs = passes * 2 * st.nbytes / (ms / 1e3) / 1e9
+                gbs = plan.stats("c64", 12, jit=True)["passes"] * 2 * st.nbytes / (ms / 1e3) / 1e9
                 row["specialised_tile12"] = {"ms": round(ms, 2), "GBs": round(gbs, 1), "frac": round(gbs / peak, 4)}
             plan.close()
             rows.append(row)
@@ -597,7 +597,7 @@ def c128_section(n, gates, peak, fp64_peak):
                                  ("beam", 10, True, "c128df"), ("beam", 8, True, "c128df"),
                                  ("dagp", 10, True, "c128df")):
         plan = api.Plan(gates, n, method, k, dfs_trials=16)
-        passes = plan.stats("c128")["passes"]
+        passes = plan.stats("c128", jit=jit)["passes"]
         flops = plan.flops("c128")[0]
         cs = plan.specialise(prec) if jit else 0.0
         ms = _timed(st if prec == "c128" else sdf, plan, jit=jit, reps=1)
@@ -634,7 +634,7 @@ def multilevel_section(peak):
         for m, k in (("dagp", 10), ("beam", 10), ("beam", 12)):
             for inner in (None, ("dagp", 5), ("beam", 5)):
                 plan = api.Plan(g, n, m, k, inner=inner)
-                stt = plan.stats("c64")
+                stt = plan.stats("c64", jit=True)
                 cs = plan.specialise("c64")
                 ms = _timed(st, plan, jit=True, reps=2 if n < 30 else 1)
                 gbs = stt["passes"] * 2 * st.nbytes / (ms / 1e3) / 1e9
@@ -660,7 +660,7 @@ def qft33_section(peak):
     for m, k, tc, jit in (("beam", 6, True, False), ("beam", 6, 2, False), ("beam", 10, False, True),
                           ("beam", 12, False, True)):
         plan = api.Plan(g, n, m, k, dfs_trials=64 if k <= 6 else 16)
-        stt = plan.stats("c64", tc=tc)
+        stt = plan.stats("c64", tc=tc, jit=jit)
         cs = plan.specialise("c64", tc=tc) if jit else 0.0
         st.set_basis(x)
         ms = _timed(st, plan, tc=tc, jit=jit, reps=1)
@@ -707,7 +707,7 @@ def run_ours(a):
         st = api.State(n, "c64", tile=choice["tile"])
     from paper_2205_06973_gb300.autotune import BEAM_WIDTH
     plan = api.Plan(gates, n, method, k, dfs_trials=BEAM_WIDTH if method == "beam" else 16)
-    stats = plan.stats("c64", choice.get("tile", 0), tc=tc, regbits=regbits)
+    stats = plan.stats("c64", choice.get("tile", 0), tc=tc, regbits=regbits, jit=jit)
     if jit:
         plan.specialise("c64", choice.get("tile", 0), tc=tc, regbits=regbits)
     passes = stats["passes"]

@@ -197,7 +197,9 @@ sv_status sv_plan_export(const sv_plan *p, uint32_t *part_of_gate, size_t n_gate
 /* Statistics of the compiled device program for a precision, tile and apply
  * flags (SV_FLAG_TC_DENSE changes the program): passes = parts run on the
  * GPU (without SV_FLAG_SPECIALISE a complex64 state of at most 13 qubits on
- * the default tile runs them in one launch), phases = register phases of the gate-list parts, ops = their kernel
+ * the default tile may run them in one launch; with it, the passes of the
+ * specialised kernels, which cut parts whose tiles would have short runs and
+ * join parts of two-qubit phases to others), phases = register phases of the gate-list parts, ops = their kernel
  * ops, dense = parts run as fused unitaries on the tensor cores (any output
  * pointer may be NULL). Compiles on the host if needed; no device work. */
 sv_status sv_plan_stats(sv_plan *p, sv_precision prec, int tile_qubits, uint32_t flags, uint32_t *passes,

@@ -48,10 +48,10 @@ class Plan:
         N.check(N.lib.sv_plan_export(self.h, pog.ctypes.data, self.G, ctypes.byref(P)))
         return pog[: self.G], P.value
 
-    def stats(self, precision="c64", tile=0, tc=False, regbits=0):
+    def stats(self, precision="c64", tile=0, tc=False, regbits=0, jit=False):
         a, b, c, d = ctypes.c_uint32(), ctypes.c_uint32(), ctypes.c_uint32(), ctypes.c_uint32()
         N.check(N.lib.sv_plan_stats(self.h, N.PRECISIONS[precision], tile,
-                                    N.tc_flags(tc) | N.SV_FLAG_REGBITS(regbits),
+                                    N.tc_flags(tc) | N.SV_FLAG_REGBITS(regbits) | (N.SV_FLAG_SPECIALISE if jit else 0),
                                     ctypes.byref(a), ctypes.byref(b), ctypes.byref(c), ctypes.byref(d)))
         return {"passes": a.value, "phases": b.value, "ops": c.value, "dense": d.value}
 

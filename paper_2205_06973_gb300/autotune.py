@@ -114,7 +114,7 @@ def tune_state(workload, n, gates, precision="c64", candidates=STATE_CANDIDATES,
             if jit:
                 compile_s = plan.specialise(precision, tile, tc=tc, regbits=regbits)
             ms = _time_apply(st, plan, tc, reps, jit=jit, regbits=regbits)
-            stats = plan.stats(precision, tile, tc=tc, regbits=regbits)
+            stats = plan.stats(precision, tile, tc=tc, regbits=regbits, jit=jit)
         except Exception as e:   # a configuration the library rejects (tile too small, no NVRTC)
             if log:
                 log(f"tune: skip {method} k={k} tc={tc} tile={tile} jit={jit}: {e}")

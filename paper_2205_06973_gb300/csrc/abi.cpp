@@ -508,6 +508,7 @@ sv_status sv_plan_export(const sv_plan *p, uint32_t *pog, size_t n_gates, uint32
 // one tile, bits 4-7 = register bits per thread, and the bits below.
 constexpr int kModeWhole = 4;   // all gates as one part (the tile is the whole state)
 constexpr int kModeJit = 8;     // for the specialised kernels (outer_diag), no interpreter stream
+constexpr int kModeRefine = 128;   // the plan's parts cut and joined (refine_parts)
 
 static sv_status get_host_program(sv_plan *p, bool fp64, int t, int mode, const Program **out) {
     std::lock_guard<std::recursive_mutex> lk(p->mu);
@@ -516,10 +517,19 @@ static sv_status get_host_program(sv_plan *p, bool fp64, int t, int mode, const 
     if (it == p->host_progs.end()) {
         std::unique_ptr<Program> prog(new Program());
         std::string err;
-        const bool whole = (mode & kModeWhole) != 0;
-        const std::vector<uint32_t> one(whole ? p->gates.size() : 0, 0u);
-        if (!compile_program(p->gates, p->n, whole ? one : p->pog, whole ? 1u : p->n_parts, fp64, t, mode >> 4,
-                             mode & 3, *prog, err, p->inner.empty() ? nullptr : &p->inner, (mode & kModeJit) != 0))
+        const bool refined = (mode & kModeRefine) && p->max_part <= t;   // else refused below
+        const bool own = (mode & kModeWhole) || refined;
+        std::vector<uint32_t> pog;
+        uint32_t n_parts = p->n_parts;
+        if (mode & kModeWhole) {
+            pog.assign(p->gates.size(), 0u);
+            n_parts = 1;
+        } else if (refined) {
+            n_parts = refine_parts(p->gates, p->n, p->pog, p->n_parts, fp64, t, pog);
+        }
+        if (!compile_program(p->gates, p->n, own ? pog : p->pog, n_parts, fp64, t, (mode >> 4) & 7,
+                             mode & 3, *prog, err, p->inner.empty() ? nullptr : &p->inner, (mode & kModeJit) != 0,
+                             refined))
             return fail(SV_ERR_PARTITION, err);
         it = p->host_progs.emplace(key, std::move(prog)).first;
     }
@@ -567,6 +577,9 @@ static int spec_mode(const sv_plan *p, sv_precision prec, uint32_t flags, int t_
     // a part's controls and two-qubit phases need not be in its tile
     if (!t_user && p->inner.empty()) t = std::max(default_tile(fp64, p->max_tile), p->max_part);
     if (t > part_tmax(fp64)) t = part_tmax(fp64);
+    // (a complex128 state in L2 is bound by FP64 work alone: a 20-qubit QFT
+    // takes 455 us on joined parts, 445 on its own)
+    if (p->inner.empty() && !(mode & 3) && !(prec == SV_C128 && p->n <= 21)) mode |= kModeRefine;
     if (t_user || ((flags >> 8) & 0xFu) || !p->inner.empty()) return mode;
     int R = part_R(fp64);
     if (!fp64) {
@@ -580,7 +593,7 @@ static int spec_mode(const sv_plan *p, sv_precision prec, uint32_t flags, int t_
         t = small_tiles(p, t);
         R = 3;
     }
-    return (mode & 15) | (R << 4);
+    return (mode & ~(7 << 4)) | (R << 4);
 }
 
 // Tile and variant of an apply on the interpreter (no register bits given).
@@ -632,6 +645,7 @@ sv_status sv_plan_stats(sv_plan *p, sv_precision prec, int t, uint32_t flags, ui
                         uint32_t *ops, uint32_t *dense) {
     if (!p) return fail(SV_ERR_ARG, "plan is NULL");
     const bool fp64 = prec != SV_C64;
+    const int t_user = t;
     if (t == 0) t = default_tile(fp64, p->max_part);
     if (t < part_tmin() || t > part_tmax(fp64)) return fail(SV_ERR_ARG, "tile_qubits out of range");
     const int mode = dense_mode(flags, fp64) & ~kModeJit;
@@ -646,6 +660,13 @@ sv_status sv_plan_stats(sv_plan *p, sv_precision prec, int t, uint32_t flags, ui
     sv_status st = get_host_program(p, fp64, t, mode, &prog);
     if (st != SV_OK) return st;
     if (passes) *passes = (uint32_t)prog->kind.size();
+    if (passes && (flags & SV_FLAG_SPECIALISE)) {   // the specialised kernels' passes
+        int ts = 0;
+        if ((spec_mode(p, prec, flags, t_user, ts) & kModeRefine) && p->max_part <= ts) {
+            std::vector<uint32_t> pog;
+            *passes = refine_parts(p->gates, p->n, p->pog, p->n_parts, fp64, ts, pog);
+        }
+    }
     if (phases) *phases = (uint32_t)prog->phases.size();
     if (ops) *ops = (uint32_t)prog->ops.size();
     if (dense) *dense = (uint32_t)(prog->dense.size() + prog->pairs.size());

@@ -103,6 +103,94 @@ uint64_t tile_need(const GateRef &g) {
     return is_diagonal(g.kind) && g.arity == 1 ? 1ull << g.q[0] : acts_nondiag(g);
 }
 
+// QFT, beam k = 12: the part with the 12 highest targets read and wrote runs
+// of 16 bytes (30 qubits: 27 of the circuit's 55.5 ms), its halves read whole
+// lines; the parts of phases alone cost a pass each. us with the plan's
+// parts / with these: 20 qubits 26 / 20, 24 qubits 435 / 298, 26 qubits 1910
+// / 1251, 28 qubits 11268 / 7026, 30 qubits 55532 / 25782; k = 9 at 28 qubits
+// 14271 / 7511. Layered circuits, k = 12 at 28 qubits 17659 / 17333.
+uint32_t refine_parts(const std::vector<GateRef> &gates, int n, const std::vector<uint32_t> &pog, uint32_t n_parts,
+                      bool fp64, int t, std::vector<uint32_t> &out) {
+    struct Group {
+        std::vector<int> gates;
+        uint64_t need = 0, all = 0;   // qubits of the tile, qubits
+    };
+    auto add = [&](Group &g, int i) {
+        g.gates.push_back(i);
+        g.need |= tile_need(gates[i]);
+        for (int j = 0; j < gates[i].arity; j++) g.all |= 1ull << gates[i].q[j];
+    };
+    // time of a pass, in passes at full rate, by the bytes of its tile's runs
+    // (the lowest qubits in the tile): 8 and 16 (3.3 against 0.64 ms at 28
+    // qubits), 32 (0.54 of HBM), 64 (0.91), 128 and more
+    auto cost = [&](uint64_t need) {
+        int spare = std::min(n, t) - popc(need), run = fp64 ? 1 : 0;
+        for (int q = 0; q < n && (((need >> q) & 1) || spare-- > 0); q++) run++;
+        return run >= 4 ? 1.0 : run == 3 ? 1.1 : run == 2 ? 1.8 : 5.0;
+    };
+    std::vector<Group> parts(n_parts), cut;
+    for (size_t i = 0; i < gates.size(); i++) add(parts[pog[i]], (int)i);
+    for (Group &p : parts) {
+        if (p.gates.empty()) continue;
+        double best = cost(p.need);
+        size_t at = 0;
+        std::vector<uint64_t> tail(p.gates.size() + 1, 0);
+        for (size_t i = p.gates.size(); i-- > 0;) tail[i] = tail[i + 1] | tile_need(gates[p.gates[i]]);
+        uint64_t head = 0;
+        for (size_t i = 1; best > 2.0 && i < p.gates.size(); i++) {
+            head |= tile_need(gates[p.gates[i - 1]]);
+            const double c = cost(head) + cost(tail[i]);
+            const size_t half = p.gates.size() / 2;
+            auto far = [&](size_t x) { return x > half ? x - half : half - x; };
+            if (c < best || (at && c == best && far(i) < far(at))) {
+                best = c;
+                at = i;
+            }
+        }
+        if (at == 0) {
+            cut.push_back(std::move(p));
+            continue;
+        }
+        Group a, b;
+        for (size_t i = 0; i < p.gates.size(); i++) add(i < at ? a : b, p.gates[i]);
+        cut.push_back(std::move(a));
+        cut.push_back(std::move(b));
+    }
+    // joined parts stay within 192 gates (30-qubit QFT: 9 passes, 25.8 ms;
+    // with 128 gates 11 passes, 29.9; with 320 still 9), for the size of their
+    // code, and within 32 slots
+    std::vector<Group> done;
+    auto fits = [&](const Group &a, const Group &b) {
+        return a.gates.size() + b.gates.size() <= 192 && popc(a.need | b.need) <= t &&
+               (n <= 32 || t + popc(a.all | b.all) <= 32) &&
+               cost(a.need | b.need) <= std::max(cost(a.need), cost(b.need));
+    };
+    auto phases_only = [&](const Group &g) {
+        for (int i : g.gates)
+            if (!is_diagonal(gates[i].kind) || gates[i].arity == 1) return false;
+        return true;
+    };
+    auto join = [&](Group &a, const Group &b) {
+        for (int i : b.gates) add(a, i);
+    };
+    for (size_t i = 0; i < cut.size(); i++) {
+        Group &g = cut[i];
+        const bool prev = !done.empty() && fits(done.back(), g), next = i + 1 < cut.size() && fits(g, cut[i + 1]);
+        if (phases_only(g) && prev && (!next || done.back().gates.size() <= cut[i + 1].gates.size()))
+            join(done.back(), g);
+        else if (phases_only(g) && next) {
+            join(g, cut[i + 1]);
+            cut[i + 1] = std::move(g);
+        } else {
+            done.push_back(std::move(g));
+        }
+    }
+    out.assign(gates.size(), 0);
+    for (size_t p = 0; p < done.size(); p++)
+        for (int i : done[p].gates) out[i] = (uint32_t)p;
+    return (uint32_t)done.size();
+}
+
 // Thread-bit order of a phase: lane bits first. The first lanes cover
 // distinct slot residues (mod 4 for 8-byte, mod 3 for 16-byte amplitudes) so
 // the swizzled shared-memory accesses are conflict free; otherwise slots
@@ -285,7 +373,7 @@ static int bank_rank(const Layout &l, bool wide) {
 
 bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector<uint32_t> &pog,
                      uint32_t n_parts, bool fp64, int t_cfg, int R, int dense_mode, Program &prog,
-                     std::string &err, const std::vector<uint32_t> *inner, bool outer_diag) {
+                     std::string &err, const std::vector<uint32_t> *inner, bool outer_diag, bool refined) {
     prog = Program();
     prog.fp64 = fp64;
     prog.R = R;
@@ -407,7 +495,7 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
             prog.a_img.insert(prog.a_img.end(), img.begin(), img.end());
             continue;
         }
-        if (popc(S) > t) {
+        if (popc(S) > t && !refined) {
             err = "part " + std::to_string(pi) + " has " + std::to_string(popc(S)) + " qubits > tile " + std::to_string(t);
             return false;
         }

@@ -41,6 +41,14 @@ bool gate_is_two_qubit(int kind);
 // than as a two-qubit phase or a control.
 uint64_t tile_need(const GateRef &g);
 
+// The parts of a plan as the specialised kernels pass over the state: a part
+// whose tile of t qubits would have short contiguous runs is cut in two where
+// both halves have longer ones, and a part of two-qubit phases alone, which
+// needs no tile of its own, joins a neighbour. Writes the new part of every
+// gate and returns their number.
+uint32_t refine_parts(const std::vector<GateRef> &gates, int n, const std::vector<uint32_t> &pog, uint32_t n_parts,
+                      bool fp64, int t, std::vector<uint32_t> &out);
+
 // Compile the parts (part_of_gate numbered in execution order) for a tile of
 // t_cfg qubits (t = min(n, t_cfg)) and R register bits.
 // dense_mode: bit 0 = every part of at most 6 qubits runs as a dense
@@ -53,10 +61,12 @@ uint64_t tile_need(const GateRef &g);
 // outer_diag: qubits that the part's gates act on only as two-qubit phases or
 // controls may lie outside its tile; conditions on them are thread-bit
 // numbers from OP_OUTER (not for the interpreter, whose conditions are thread
-// masks).
+// masks). refined (with outer_diag): the parts are refine_parts', whose tiles
+// fit although all their qubits may not.
 bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector<uint32_t> &pog,
                      uint32_t n_parts, bool fp64, int t_cfg, int R, int dense_mode, Program &prog,
-                     std::string &err, const std::vector<uint32_t> *inner = nullptr, bool outer_diag = false);
+                     std::string &err, const std::vector<uint32_t> *inner = nullptr, bool outer_diag = false,
+                     bool refined = false);
 
 // Floating-point operations per state amplitude that the program's kernels
 // execute: CUDA-core arithmetic (alu) and tensor-core products (tensor).

@@ -169,3 +169,29 @@ def test_register_bits(precision, regbits, tile):
         st.close()
         plan.close()
         assert max_abs(out, ref) <= TOL[precision], (method, k)
+
+
+def _phase_ladders(n, seed):
+    """Runs of two-qubit phases (parts that need no tile), H and SWAP on the
+    highest qubits (parts whose tiles have short runs), mixed gates between."""
+    rng = np.random.default_rng(seed)
+    g = synth.qft(n)
+    for _ in range(3):
+        g += [("CP", tuple(int(x) for x in rng.choice(n, 2, replace=False)), float(rng.uniform(0, 6)))
+              for _ in range(40)]
+        g += [("CZ", (q, (q + n // 2) % n), 0.0) for q in range(n // 2)]
+        g += [("H", (q,), 0.0) for q in range(n - 8, n)]
+        g += [("SWAP", (q, q - 4), 0.0) for q in range(n - 4, n)]
+        g += [("RZ", (int(rng.integers(n)),), float(rng.uniform(0, 6))) for _ in range(4)]
+    return g
+
+
+@pytest.mark.parametrize("precision", ["c64", "c128", "c128df"])
+@pytest.mark.parametrize("n", [13, 16, 18])
+def test_parts_cut_and_joined(n, precision):
+    g = _phase_ladders(n, n)
+    psi = random_state(n, 5 * n)
+    ref = sim.run(n, g, psi)
+    for method, k, tile in (("beam", 11, 0), ("nat", 10, 12), ("dagp", 6, 10), ("dfs", 4, 0)):
+        out = run_gpu(n, g, method=method, k=k, precision=precision, psi=psi, jit=True, tile=tile)
+        assert max_abs(out, ref) <= TOL[precision], (method, k, tile)
