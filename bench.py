@@ -100,7 +100,8 @@ def peaks():
 KERNEL_SOURCES = {
     "k_dense6": ("dense.cu", "dense.hpp", "dense_common.cuh", "planner.cpp"),
     "k_dense6_pair": ("dense_pair.cu", "dense.hpp", "dense_common.cuh", "planner.cpp"),
-    "k_part": ("kernels.cu", "ops.cuh", "ops_core.cuh", "program.hpp", "planner.cpp"),
+    "k_part": ("part_kernel.cuh", "part_f32.cu", "part_f64.cu", "interp.cpp", "interp.hpp", "ops.cuh", "packed.cuh",
+               "ops_core.cuh", "program.hpp", "planner.cpp"),
     "hisv_part": ("jit.cpp", "jit_prelude.cuh", "ops_core.cuh", "program.hpp", "planner.cpp"),
 }
 

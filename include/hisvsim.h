@@ -199,8 +199,8 @@ sv_status sv_plan_export(const sv_plan *p, uint32_t *part_of_gate, size_t n_gate
  * GPU (without SV_FLAG_SPECIALISE a complex64 state of at most 13 qubits on
  * the default tile may run them in one launch; with it, the passes of the
  * specialised kernels, which cut parts whose tiles would have short runs and
- * join parts of two-qubit phases to others), phases = register phases of the gate-list parts, ops = their kernel
- * ops, dense = parts run as fused unitaries on the tensor cores (any output
+ * join parts of two-qubit phases to others), phases = register phases of the
+ * plan's gate-list parts, ops = their kernel ops, dense = parts run as fused unitaries on the tensor cores (any output
  * pointer may be NULL). Compiles on the host if needed; no device work. */
 sv_status sv_plan_stats(sv_plan *p, sv_precision prec, int tile_qubits, uint32_t flags, uint32_t *passes,
                         uint32_t *phases, uint32_t *ops, uint32_t *dense);
@@ -237,7 +237,8 @@ sv_status sv_plan_specialise(sv_plan *p, sv_precision prec, int tile_qubits, uin
 /* sv_plan_source: the generated CUDA source of gate-list part i (execution
  * order among the gate-list parts) of the plan's program for prec, tile and
  * flags, copied NUL-terminated into buf (cap bytes); *len receives the
- * source length. Host only. */
+ * source length. Host only. It is the plan's own part in the default shape; an
+ * apply may cut and join parts (sv_plan_stats) and choose another tile. */
 sv_status sv_plan_source(sv_plan *p, sv_precision prec, int tile_qubits, uint32_t flags, uint32_t part, char *buf,
                          size_t cap, size_t *len);
 /* sv_plan_flops: the floating-point operations one apply of the plan
