@@ -106,9 +106,9 @@ uint64_t tile_need(const GateRef &g) {
 // QFT, beam k = 12: the part with the 12 highest targets read and wrote runs
 // of 16 bytes (30 qubits: 27 of the circuit's 55.5 ms), its halves read whole
 // lines; the parts of phases alone cost a pass each. us with the plan's
-// parts / with these: 20 qubits 26 / 20, 24 qubits 435 / 298, 26 qubits 1910
-// / 1251, 28 qubits 11268 / 7026, 30 qubits 55532 / 25782; k = 9 at 28 qubits
-// 14271 / 7511. Layered circuits, k = 12 at 28 qubits 17659 / 17333.
+// parts / with these: 20 qubits 26 / 19, 24 qubits 435 / 288, 26 qubits 1910
+// / 1208, 28 qubits 11268 / 6870, 30 qubits 55532 / 25103; k = 9 at 28 qubits
+// 14271 / 7571. Layered circuits, k = 12 at 28 qubits 17659 / 17333.
 uint32_t refine_parts(const std::vector<GateRef> &gates, int n, const std::vector<uint32_t> &pog, uint32_t n_parts,
                       bool fp64, int t, std::vector<uint32_t> &out) {
     struct Group {
@@ -132,12 +132,13 @@ uint32_t refine_parts(const std::vector<GateRef> &gates, int n, const std::vecto
     for (size_t i = 0; i < gates.size(); i++) add(parts[pog[i]], (int)i);
     for (Group &p : parts) {
         if (p.gates.empty()) continue;
-        double best = cost(p.need);
+        const double whole = cost(p.need);
+        double best = whole;
         size_t at = 0;
         std::vector<uint64_t> tail(p.gates.size() + 1, 0);
         for (size_t i = p.gates.size(); i-- > 0;) tail[i] = tail[i + 1] | tile_need(gates[p.gates[i]]);
         uint64_t head = 0;
-        for (size_t i = 1; best > 2.0 && i < p.gates.size(); i++) {
+        for (size_t i = 1; whole > 2.0 && i < p.gates.size(); i++) {   // of equal cuts the most even
             head |= tile_need(gates[p.gates[i - 1]]);
             const double c = cost(head) + cost(tail[i]);
             const size_t half = p.gates.size() / 2;
@@ -156,8 +157,8 @@ uint32_t refine_parts(const std::vector<GateRef> &gates, int n, const std::vecto
         cut.push_back(std::move(a));
         cut.push_back(std::move(b));
     }
-    // joined parts stay within 192 gates (30-qubit QFT: 9 passes, 25.8 ms;
-    // with 128 gates 11 passes, 29.9; with 320 still 9), for the size of their
+    // joined parts stay within 192 gates (30-qubit QFT: 9 passes, 25.1 ms;
+    // with 128 gates 11 passes, 4 ms more; with 320 still 9), for the size of their
     // code, and within 32 slots
     std::vector<Group> done;
     auto fits = [&](const Group &a, const Group &b) {
