@@ -349,6 +349,19 @@ static void pair_swizzle(DensePairLaunch &D) {
     for (int p = 0; p < NS; p++) D.xsw[p] = (uint16_t)(p < 4 ? (1u << p) : ((1u << p) | v[p]));
 }
 
+// Modulus of the factor that the planner gathered for an op (the op alone
+// grows a state by up to its inverse): the first row of a scaled matrix has
+// the norm of 1 and its smaller entry.
+static double factor_of(const Op &op, const std::vector<double> &coefs) {
+    const double *c = coefs.data() + op.coef;
+    switch (op.kind) {
+    case OP_H: return std::sqrt(0.5);
+    case OP_RXS: case OP_RYS: return 1.0 / std::hypot(1.0, c[0]);
+    case OP_U2S: return 1.0 / std::sqrt(1.0 + c[0] * c[0] + c[1] * c[1]);
+    default: return 1.0;
+    }
+}
+
 // Rank of a warp's 32 lanes in the shared-memory banks (bank groups of one
 // amplitude: 4 index bits for 8-byte amplitudes, 3 for 16-byte ones).
 static int bank_rank(const Layout &l, bool wide) {
@@ -539,16 +552,24 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
             fr = x * dr - y * di;
             fi = x * di + y * dr;
         };
-        // the part factor goes into a merged diagonal's coefficients
-        auto scale_diag = [&](const Op &op) {
+        // a factor goes into a merged diagonal's coefficients
+        auto scale_by = [&](const Op &op, double dr, double di) {
             double *c = prog.coefs.data() + op.coef;
             for (int i = 0; i < (1 << R); i++) {
                 const double x = c[2 * i], y = c[2 * i + 1];
-                c[2 * i] = x * fr - y * fi;
-                c[2 * i + 1] = x * fi + y * fr;
+                c[2 * i] = x * dr - y * di;
+                c[2 * i + 1] = x * di + y * dr;
             }
+        };
+        auto scale_diag = [&](const Op &op) {   // the part factor
+            scale_by(op, fr, fi);
             fr = 1.0;
             fi = 0.0;
+        };
+        auto unit_diag = [&]() {   // coefficients of a diagonal of ones
+            const uint32_t at = (uint32_t)prog.coefs.size();
+            for (int i = 0; i < (1 << R); i++) prog.coefs.insert(prog.coefs.end(), {1.0, 0.0});
+            return at;
         };
         bool last_tphase = false;
         std::vector<int> remaining = gl;
@@ -685,6 +706,7 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
                 if (((S & ~Tm) >> q) & 1) tbit[slot_of[q]] = OP_OUTER + q;
             // pass 2: emit ops
             ph.op_begin = (uint32_t)prog.ops.size();
+            const double grown_before = std::hypot(fr, fi);   // not yet applied, of earlier phases
             bool tphase = false, tsign = false;
             auto coef = [&](std::initializer_list<double> v) {
                 uint32_t at = (uint32_t)prog.coefs.size();
@@ -959,6 +981,26 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
                 }
                 flush();
             }
+            // A phase may hold any number of gates on its register bits, each
+            // growing the unnormalised amplitudes by up to sqrt2: where their
+            // factors reach 2^-40 the modulus gathered so far is applied in
+            // the middle of the phase, long before a float's range ends (the
+            // part factor below may join the same diagonal: 2^-80).
+            {
+                const std::vector<Op> in(prog.ops.begin() + ph.op_begin, prog.ops.end());
+                prog.ops.resize(ph.op_begin);
+                double grown = grown_before;
+                for (const Op &op : in) {
+                    prog.ops.push_back(op);
+                    grown *= factor_of(op, prog.coefs);
+                    if (grown >= 0x1p-40) continue;
+                    emit(OP_DIAG, 0, 0, 0, unit_diag());
+                    scale_by(prog.ops.back(), grown, 0.0);
+                    fr /= grown;
+                    fi /= grown;
+                    grown = 1.0;
+                }
+            }
             if (tphase && !last) emit(OP_TAPPLY, 0, 0, 0, 0);
             if (tsign) emit(OP_TSAPPLY, 0, 0, 0, 0);
             // a part of many phases (a whole circuit) applies the part factor
@@ -967,11 +1009,7 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
             if (!last && std::hypot(fr, fi) < 0x1p-24) {
                 uint32_t o = ph.op_begin;
                 while (o < (uint32_t)prog.ops.size() && prog.ops[o].kind != OP_DIAG) o++;
-                if (o == (uint32_t)prog.ops.size()) {
-                    const uint32_t at = (uint32_t)prog.coefs.size();
-                    for (int i = 0; i < (1 << R); i++) prog.coefs.insert(prog.coefs.end(), {1.0, 0.0});
-                    emit(OP_DIAG, 0, 0, 0, at);
-                }
+                if (o == (uint32_t)prog.ops.size()) emit(OP_DIAG, 0, 0, 0, unit_diag());
                 scale_diag(prog.ops[o]);
             }
             if (last) last_tphase = tphase;
