@@ -584,7 +584,7 @@ static int spec_mode(const sv_plan *p, sv_precision prec, uint32_t flags, int t_
     int R = part_R(fp64);
     if (!fp64) {
         if (p->n <= 20) R = 4;
-        if (p->n <= 17 && t == 12) t = 11;
+        if (p->n <= 17 && t == 12 && p->max_part < 12) t = 11;
         if (p->n == 20) t = 13;
     } else if (prec == SV_C128DF) {
         R = 3;
