@@ -505,10 +505,12 @@ sv_status sv_plan_export(const sv_plan *p, uint32_t *pog, size_t n_gates, uint32
 
 // Program variants of a plan (besides precision and tile): bit 0 = tensor-core
 // dense parts (complex64 only), bit 1 = two of them per pass where they fit
-// one tile, bits 4-7 = register bits per thread, and the bits below.
+// one tile, bits 4-7 = register bits per thread (the flags' whole field: what
+// compile_program has no program for it refuses), and the bits below.
 constexpr int kModeWhole = 4;   // all gates as one part (the tile is the whole state)
 constexpr int kModeJit = 8;     // for the specialised kernels (outer_diag), no interpreter stream
-constexpr int kModeRefine = 128;   // the plan's parts cut and joined (refine_parts)
+constexpr int kModeRefine = 256;   // the plan's parts cut and joined (refine_parts)
+static int mode_R(int mode) { return (mode >> 4) & 15; }
 
 static sv_status get_host_program(sv_plan *p, bool fp64, int t, int mode, const Program **out) {
     std::lock_guard<std::recursive_mutex> lk(p->mu);
@@ -527,7 +529,7 @@ static sv_status get_host_program(sv_plan *p, bool fp64, int t, int mode, const 
         } else if (refined) {
             n_parts = refine_parts(p->gates, p->n, p->pog, p->n_parts, fp64, t, pog);
         }
-        if (!compile_program(p->gates, p->n, own ? pog : p->pog, n_parts, fp64, t, (mode >> 4) & 7,
+        if (!compile_program(p->gates, p->n, own ? pog : p->pog, n_parts, fp64, t, mode_R(mode),
                              mode & 3, *prog, err, p->inner.empty() ? nullptr : &p->inner, (mode & kModeJit) != 0,
                              refined))
             return fail(SV_ERR_PARTITION, err);
@@ -593,7 +595,7 @@ static int spec_mode(const sv_plan *p, sv_precision prec, uint32_t flags, int t_
         t = small_tiles(p, t);
         R = 3;
     }
-    return (mode & ~(7 << 4)) | (R << 4);
+    return (mode & ~(15 << 4)) | (R << 4);
 }
 
 // Tile and variant of an apply on the interpreter (no register bits given).

@@ -395,7 +395,7 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
     prog.R = R;
     const int t = std::min(n, t_cfg);
     prog.t = t;
-    if (t - R > MAX_TB || R > MAX_R || t < R + 5) {
+    if (t - R > MAX_TB || R < 1 || R > MAX_R || t < R + 5) {
         err = "tile configuration out of range";
         return false;
     }
@@ -657,6 +657,10 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
                     if (gates[g].kind == SV_GATE_SWAP) std::swap(sim_slot[gates[g].q[0]], sim_slot[gates[g].q[1]]);
             }
             const bool last = rest.empty();
+            if (sched.empty()) {
+                err = "no gate of part " + std::to_string(pi) + " fits the register bits";
+                return false;
+            }
             // slot -> qubit at the end of this phase
             int q_end[64];
             for (int q = 0; q < n; q++)
