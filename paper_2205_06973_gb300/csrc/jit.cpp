@@ -83,8 +83,9 @@ std::string lit(double v, int mode) {
     return b;
 }
 
-// d = i^quad e^{i phi} with |phi| <= pi / 4, as the shears of rot_in; false if
-// d is not a phase (a merged diagonal may hold the part factor).
+// The phase d = i^quad e^{i phi} with |phi| <= pi / 4, as the shears of rot_in;
+// false if d is none by far. A modulus near 1 is lost: not for diagonals that
+// hold one (a part factor of small rotations is within 1e-13 of 1).
 bool shears(double dr, double di, int &quad, double &t, double &s) {
     const double r = std::hypot(dr, di);   // a product of phases: 1 up to its rounding
     if (std::fabs(r - 1.0) > 1e-13) return false;
@@ -397,7 +398,7 @@ std::string jit_part_source(const Program &prog, size_t pi, bool df) {
                     if (dr == -1.0 && di == 0.0) o << aq << ".x = neg_of(" << aq << ".x); " << aq << ".y = neg_of(" << aq << ".y); ";
                     else if (dr == 0.0 && di == 1.0) o << "{ const Real x_ = " << aq << ".x; " << aq << ".x = neg_of(" << aq << ".y); " << aq << ".y = x_; } ";
                     else if (dr == 0.0 && di == -1.0) o << "{ const Real x_ = " << aq << ".x; " << aq << ".x = " << aq << ".y; " << aq << ".y = neg_of(x_); } ";
-                    else if (mode == 1 && shears(dr, di, quad, rt, rs))
+                    else if (mode == 1 && A == 0 && shears(dr, di, quad, rt, rs))
                         o << "rotq_in<" << quad << ">(" << aq << ", " << L_lit(rt) << ", " << L_lit(rs) << "); ";
                     else o << "cmul_in(" << aq << ", " << L_(c + 2 * q) << ", " << L_(c + 2 * q + 1) << "); ";
                 }

@@ -18,10 +18,11 @@ __device__ __forceinline__ double neg_of(double v) {
 }
 #endif
 
-// (x + i y) times e^{i phi} by three shears, t = tan(phi / 2), s = sin(phi):
-// three multiply-adds instead of two products and two multiply-adds. Used for
-// complex128, whose kernels are bound by FP64 work (24 qubits, 20 layers,
-// k = 10: 29.9 -> 28.6 ms, the error against exact arithmetic unchanged).
+// (x + i y) times e^{i phi} by three shears (Paeth, Graphics Interface 1986),
+// t = tan(phi / 2), s = sin(phi): three multiply-adds instead of two products
+// and two multiply-adds. Used for complex128, whose kernels are bound by FP64
+// work (24 qubits, 20 layers, k = 10: 29.9 -> 28.6 ms; largest error against
+// exact arithmetic 1.87e-15 with products, 1.90e-15 with shears).
 template <typename C, typename Real>
 __device__ __forceinline__ void rot_in(C &v, Real t, Real s) {
     v.x = v.x - t * v.y;

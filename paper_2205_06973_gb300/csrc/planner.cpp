@@ -547,6 +547,7 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
         for (int p = 0; p < t; p++) L.tile_q[p] = (uint8_t)q_at[p];
         // part factor: 1/sqrt2 per (unnormalised) H and e^{-i theta/2} per RZ
         double fr = 1.0, fi = 0.0;
+        bool modulus = false;   // it holds more than phases
         auto fmul = [&](double dr, double di) {
             const double x = fr, y = fi;
             fr = x * dr - y * di;
@@ -561,10 +562,12 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
                 c[2 * i + 1] = x * di + y * dr;
             }
         };
-        auto scale_diag = [&](const Op &op) {   // the part factor
+        auto scale_diag = [&](Op &op) {   // the part factor
             scale_by(op, fr, fi);
+            if (modulus) op.a = 1;
             fr = 1.0;
             fi = 0.0;
+            modulus = false;
         };
         auto unit_diag = [&]() {   // coefficients of a diagonal of ones
             const uint32_t at = (uint32_t)prog.coefs.size();
@@ -736,6 +739,7 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
                 case SV_GATE_H:
                     emit(OP_H, rb[s0], 0, 0, 0);
                     fmul(std::sqrt(0.5), 0.0);
+                    modulus = true;
                     break;
                 case SV_GATE_X: emit(OP_X, rb[s0], 0, 0, 0); break;
                 case SV_GATE_Y: emit(OP_Y, rb[s0], 0, 0, 0); break;
@@ -745,6 +749,7 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
                     // or s [[t, -1], [1, t]], whichever keeps |t| <= 1
                     const double c = std::cos(th / 2), sn = std::sin(th / 2);
                     const bool rx = gr.kind == SV_GATE_RX;
+                    modulus = true;
                     if (std::fabs(c) >= std::fabs(sn)) {
                         fmul(c, 0.0);
                         emit(rx ? OP_RXS : OP_RYS, rb[s0], 0, 0, coef({sn / c}));
@@ -867,6 +872,7 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
                     div(M[4], M[5], vr, vi);
                     div(M[6], M[7], wr, wi);
                     fmul(pr, pi);
+                    modulus = true;
                     emit(OP_U2S, rb[sq], f1 ? 1 : 0, 0, coef({ur, ui, vr, vi, wr, wi}));
                 }
                 return true;
@@ -998,7 +1004,7 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
                     prog.ops.push_back(op);
                     grown *= factor_of(op, prog.coefs);
                     if (grown >= 0x1p-40) continue;
-                    emit(OP_DIAG, 0, 0, 0, unit_diag());
+                    emit(OP_DIAG, 1, 0, 0, unit_diag());
                     scale_by(prog.ops.back(), grown, 0.0);
                     fr /= grown;
                     fi /= grown;

@@ -36,6 +36,7 @@ enum OpKind : uint8_t {
     OP_TSG,      // tb, b: per-thread sign flips if both thread bits are set (Z, CZ on thread bits)
     OP_TSAPPLY,  // negate the thread's amplitudes where its sign is set, reset the sign
     OP_DIAG,     // coef: 2^R phases (re, im): register amplitude i *= phase i (merged diagonal gates)
+                     // a = 1: they hold the modulus of a part factor
     // Rotations with their largest entry factored out into the part factor
     // (one multiply-add per output component instead of two); b = form:
     OP_RXS,      // a; coef t. b = 0: RX = c [[1, -it], [-it, 1]], t = s/c; b = 1: RX = -is [[it, 1], [1, it]], t = c/s
