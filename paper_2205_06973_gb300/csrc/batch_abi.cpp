@@ -366,9 +366,11 @@ static sv_status build_program(sv_batch *b) {
         part_base[c] = (uint32_t)parts.size();
         if (whole(c)) {
             n_parts[c] = 0;
-            if (!lo.parts.empty()) wholes[b->nq[c]].push_back({b->off[c], part_base[c], 0});
-            n_whole++;
-            whole_parts += b->plans[c]->n_parts;
+            if (!lo.parts.empty()) {   // a circuit without gates has none
+                wholes[b->nq[c]].push_back({b->off[c], part_base[c], 0});
+                n_whole++;
+                whole_parts += b->plans[c]->n_parts;
+            }
         } else {
             n_parts[c] = (uint32_t)lo.parts.size();
             wave_tiles += 1ull << (b->nq[c] - BATCH_TILE_QUBITS);
