@@ -547,7 +547,7 @@ static int small_tiles(const sv_plan *p, int t) {
 }
 
 // The variant of the flags with the precision's default register bits unless
-// given (sources; without kModeJit, statistics and flop counts).
+// given (sources; without kModeJit, what stats_mode says).
 static int dense_mode(uint32_t flags, bool fp64) {
     const bool tc = (flags & SV_FLAG_TC_DENSE) && !fp64;
     const int R = (int)((flags >> 8) & 0xFu);
@@ -620,14 +620,15 @@ static int spec_mode(const sv_plan *p, sv_precision prec, uint32_t flags, int t_
 //    on 2^10 with 2^3 amplitudes: 14 qubits 79 / 65 / 66 / 56, 17 qubits 102 /
 //    83 / 91 / 80 (parameterised 153 / 122 / 124 / 114); 18 qubits 111 / 93 /
 //    138 / 129, 19 qubits 117 / 149 / 170 / 168.
-static int interp_mode(const sv_plan *p, bool fp64, uint32_t flags, int t_user, int &t) {
+// whole: false for the plan's own parts where they would become one.
+static int interp_mode(const sv_plan *p, bool fp64, uint32_t flags, int t_user, int &t, bool whole = true) {
     const int tc = dense_mode(flags, fp64) & 3;
     const bool ml = !p->inner.empty();
     int R = ml ? part_R(fp64) : interp_R(fp64);
     t = t_user ? t_user : default_tile(fp64, p->max_part);
     if (t_user || ml) return tc | (R << 4);
     const bool cut = p->n >= 12 && p->max_part <= 10 && p->gates.size() >= (p->n == 12 ? 40 : 20) * (size_t)p->n_parts;
-    if (!fp64 && p->n <= part_tmax(false) && !cut && !(tc && p->n >= DENSE_K + DENSE_COLS)) {
+    if (whole && !fp64 && p->n <= part_tmax(false) && !cut && !(tc && p->n >= DENSE_K + DENSE_COLS)) {
         t = p->n;
         if (t == 10) R = 3;
         return kModeWhole | (R << 4);
@@ -643,14 +644,26 @@ static int interp_mode(const sv_plan *p, bool fp64, uint32_t flags, int t_user, 
     return tc | (R << 4);
 }
 
+// Tile and variant of the program that sv_plan_stats and sv_plan_flops
+// describe: the one that an apply with these flags runs, so that a caller who
+// asks for the statistics first (on a thread that plans) has compiled it for
+// the apply; but the plan's own parts where the apply makes them one, and the
+// default shape for register bits that the interpreter does not take and for
+// double-float states.
+static int stats_mode(const sv_plan *p, sv_precision prec, uint32_t flags, int t_user, int &t) {
+    const bool fp64 = prec != SV_C64;
+    if (!((flags >> 8) & 0xFu) && prec != SV_C128DF) return interp_mode(p, fp64, flags, t_user, t, false);
+    t = t_user ? t_user : default_tile(fp64, p->max_part);
+    return dense_mode(flags, fp64) & ~kModeJit;
+}
+
 sv_status sv_plan_stats(sv_plan *p, sv_precision prec, int t, uint32_t flags, uint32_t *passes, uint32_t *phases,
                         uint32_t *ops, uint32_t *dense) {
     if (!p) return fail(SV_ERR_ARG, "plan is NULL");
     const bool fp64 = prec != SV_C64;
     const int t_user = t;
-    if (t == 0) t = default_tile(fp64, p->max_part);
-    if (t < part_tmin() || t > part_tmax(fp64)) return fail(SV_ERR_ARG, "tile_qubits out of range");
-    const int mode = dense_mode(flags, fp64) & ~kModeJit;
+    if (t != 0 && (t < part_tmin() || t > part_tmax(fp64))) return fail(SV_ERR_ARG, "tile_qubits out of range");
+    const int mode = stats_mode(p, prec, flags, t_user, t);
     if (p->method == SV_PART_NONE || p->n < part_tmin() || (flags & SV_FLAG_GATEWISE)) {
         if (passes) *passes = (uint32_t)p->gates.size();
         if (phases) *phases = 0;
@@ -741,9 +754,8 @@ sv_status sv_plan_flops(sv_plan *p, sv_precision prec, int t, uint32_t flags, do
                         double *tensor_flops) {
     if (!p) return fail(SV_ERR_ARG, "plan is NULL");
     const bool fp64 = prec != SV_C64;
-    if (t == 0) t = default_tile(fp64, p->max_part);
-    if (t < part_tmin() || t > part_tmax(fp64)) return fail(SV_ERR_ARG, "tile_qubits out of range");
-    const int mode = dense_mode(flags, fp64) & ~kModeJit;
+    if (t != 0 && (t < part_tmin() || t > part_tmax(fp64))) return fail(SV_ERR_ARG, "tile_qubits out of range");
+    const int mode = stats_mode(p, prec, flags, t, t);
     double a = 0.0, b = 0.0;
     if (p->method == SV_PART_NONE || p->n < part_tmin() || (flags & SV_FLAG_GATEWISE)) {
         // one general matrix per gate: 14 flops per amplitude for a 2x2, 30 for a 4x4
@@ -799,7 +811,7 @@ static sv_status get_dev_program(sv_state *s, sv_plan *p, int t, int mode, const
         d.dev = s->dev;
         cudaError_t e = upload_vec(reinterpret_cast<void **>(&d.d_aimg), prog.a_img, s->stream);
         if (e == cudaSuccess) e = upload_vec(reinterpret_cast<void **>(&d.d_pimg), prog.pair_img, s->stream);
-        if (e == cudaSuccess && !(mode & kModeJit))
+        if (e == cudaSuccess && !(mode & kModeJit) && !prog.parts.empty())
             e = upload_lowered(prog, d, s->stream);
         // the program is shared by every state that applies the plan, on any
         // stream: it is complete before it is published
