@@ -268,14 +268,17 @@ sv_status sv_apply_parts(sv_state *s, sv_plan *p, uint32_t flags);
 /* -------------------------------------------------------------- measure ---
  * Probabilities p[x] = |a_x|^2 (Sec. II-A) into dev_out (device memory of
  * 2^n floats, or doubles when out_fp64 != 0; may be NULL to get the norm only)
- * and the norm sum_x |a_x|^2 accumulated in FP64 into *norm_out (host, may be
- * NULL). Synchronises the stream when norm_out is not NULL. */
+ * and the norm sum_x |a_x|^2 into *norm_out (host, may be NULL), to no less
+ * than the accuracy of FP64 arithmetic: for complex64 and double-float states
+ * (without doubles as output) from exact squares summed in three floats per
+ * thread, then in FP64; otherwise in FP64 throughout. Synchronises the stream
+ * when norm_out is not NULL. */
 sv_status sv_measure_probs(sv_state *s, void *dev_out, int out_fp64, double *norm_out);
 /* Summary of the same distribution without writing it (no device memory
  * beyond the state's own scratch): *norm_out = sum_x |a_x|^2, *p0_out =
  * |a_0|^2, *pmax_out = max_x |a_x|^2 and *argmax_out = the smallest x that
- * reaches it, all computed in FP64 from the stored amplitudes (Sec. II-A:
- * measuring gives x with probability |a_x|^2). Any output may be NULL.
+ * reaches it, from the stored amplitudes, the norm as above and the rest in
+ * FP64 (Sec. II-A: measuring gives x with probability |a_x|^2). Any output may be NULL.
  * Synchronises the stream. */
 sv_status sv_measure_summary(sv_state *s, double *norm_out, double *p0_out, uint64_t *argmax_out,
                              double *pmax_out);
@@ -309,7 +312,7 @@ sv_status sv_measure_summary(sv_state *s, double *norm_out, double *p0_out, uint
  * sv_batch_reset   every state back to |0...0> (stream-ordered).
  * sv_batch_probs   p[x] = |a_x|^2 of all states into dev_out (floats,
  *                  concatenated like the states; may be NULL) and each
- *                  state's norm (FP64 accumulation) into norms_host[n] (may
+ *                  state's norm (as sv_measure_probs) into norms_host[n] (may
  *                  be NULL; synchronises when not NULL).
  * sv_batch_state   device address and byte size of circuit i's state.
  * sv_batch_copy_state  copy circuit i's state (bytes = its size) to host
@@ -362,7 +365,7 @@ sv_status sv_batch_hold_last_item(sv_batch *b, int on);
 sv_status sv_batch_destroy(sv_batch *b);
 
 /* ------------------------------------------------- allocation-free probs ---
- * sv_probs_noalloc: the same probabilities and FP64-accumulated norm as
+ * sv_probs_noalloc: the same probabilities and norm as
  * sv_measure_probs, for callers that must not allocate device memory: a host
  * framework that owns all device memory through its own pool under a fixed
  * budget, or a latency-critical loop where a device allocation could stall

@@ -4,6 +4,7 @@
 //  k_probs / k_sum   : |a_x|^2 and the norm with FP64 accumulation.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 
@@ -199,48 +200,48 @@ __global__ void k_sum(const double *__restrict__ partials, int nb, double *__res
 }
 
 // k_probs_fast: the same for float outputs of complex64 and double-float
-// states, on the FP32 pipes (split_prob, prob_split.cuh). In FP64 the two
-// conversions, the product, the multiply-add and the add of an amplitude
-// made the kernel FP64-bound on a GPU with ~2 FP64 lanes per SM (2^28
-// complex64 amplitudes: 3.05 ms against 0.47 ms of HBM time for the 3.2 GB;
-// 0.50 ms here, 0.94 of the measured copy rate).
-// Each thread takes 16 bytes at a time, PROB_U of them in flight, and sends
-// the FP64 pipe two conversions and two adds per four chunks.
-constexpr int PROB_U = 4;
-constexpr int PROB_CHUNK = 256 * PROB_U;   // 16-byte loads per block and iteration
+// states, on the FP32 pipes (prob_split.cuh). In FP64 the two conversions,
+// the product, the multiply-add and the add of an amplitude made the kernel
+// FP64-bound on a GPU with ~2 FP64 lanes per SM (2^28 complex64 amplitudes:
+// 3.05 ms against 0.47 ms of HBM time for the 3.2 GB; 0.49 ms here).
+// Each thread takes 16 bytes at a time, U of them in flight, and sends the
+// FP64 pipe three conversions and three adds per PROB_SUM amplitudes at most.
+// Probabilities leave with streaming stores. Two loads and six blocks per SM:
+// 469 us of kernel; two loads and plain stores 494, four loads and four blocks
+// 492, eight and two 478. Four loads and four blocks up to 2^25 amplitudes
+// (63 us of kernel there against 68; 2^20: 19.7 us a call against 22.5) and
+// for double-floats (2^27: 450 us a call against 466).
+constexpr int SUMMARY_U = 4;   // loads in flight per thread of k_summary_fast
 
-template <bool DF>
-__global__ void __launch_bounds__(256, 4) k_probs_fast(const float4 *__restrict__ sv, uint64_t n_chunks,
-                                                        float *__restrict__ out, double *__restrict__ partials,
-                                                        uint32_t *ticket, double *norm) {
+template <bool DF, int U, int BLOCKS>
+__global__ void __launch_bounds__(256, BLOCKS)
+k_probs_fast(const float4 *__restrict__ sv, uint64_t n_chunks, float *__restrict__ out, double *__restrict__ partials,
+             uint32_t *ticket, double *norm) {
     double acc = 0.0;
-    float S = 0.0f, T = 0.0f;
+    NormSum sum;
     uint32_t it = 0;
-    for (uint64_t c = blockIdx.x; c < n_chunks; c += gridDim.x, it++) {
-        const uint64_t at = c * PROB_CHUNK + threadIdx.x;
-        float4 v[PROB_U];
+    for (uint64_t c = blockIdx.x; c < n_chunks; c += gridDim.x) {
+        const uint64_t at = c * (256 * U) + threadIdx.x;
+        float4 v[U];
 #pragma unroll
-        for (int u = 0; u < PROB_U; u++) v[u] = __ldcs(sv + at + 256 * u);
-        bool ok = true;
+        for (int u = 0; u < U; u++) v[u] = __ldcs(sv + at + 256 * u);
+        if (sum.fits<DF>(v, acc)) {
 #pragma unroll
-        for (int u = 0; u < PROB_U; u++) ok = ok && split_range<DF>(v[u]);
-        if (ok) {
-#pragma unroll
-            for (int u = 0; u < PROB_U; u++) {
+            for (int u = 0; u < U; u++) {
                 if constexpr (DF) {
-                    const float2 p = split_prob_df(v[u]);
-                    split_add(S, T, p);
-                    if (out) out[at + 256 * u] = p.x + p.y;
+                    const SquaresDf q(v[u]);
+                    sum.add(q);
+                    if (out) __stcs(out + at + 256 * u, q.prob());
                 } else {
-                    const float2 p = split_prob(v[u].x, v[u].y), q = split_prob(v[u].z, v[u].w);
-                    split_add(S, T, p);
-                    split_add(S, T, q);
-                    if (out) reinterpret_cast<float2 *>(out)[at + 256 * u] = make_float2(p.x + p.y, q.x + q.y);
+                    const Squares q(make_float2(v[u].x, v[u].y)), r(make_float2(v[u].z, v[u].w));
+                    sum.add(q);
+                    sum.add(r);
+                    if (out) __stcs(reinterpret_cast<float2 *>(out) + at + 256 * u, make_float2(q.prob(), r.prob()));
                 }
             }
         } else {   // outside the split's range: FP64
 #pragma unroll
-            for (int u = 0; u < PROB_U; u++) {
+            for (int u = 0; u < U; u++) {
                 if constexpr (DF) {
                     double re, im;
                     amp_parts(v[u], re, im);
@@ -256,26 +257,26 @@ __global__ void __launch_bounds__(256, 4) k_probs_fast(const float4 *__restrict_
                 }
             }
         }
-        if ((it & 3) == 3) {
-            acc += (double)S + (double)T;
-            S = T = 0.0f;
-        }
+        if (++it % (PROB_SUM / ((DF ? 1 : 2) * U)) == 0) acc += sum.take();
     }
-    finish_norm(acc + ((double)S + (double)T), partials, ticket, norm);
+    finish_norm(acc + sum.take(), partials, ticket, norm);
 }
 
-// The FP32 kernels take whole chunks of 16-byte loads: at least one chunk,
-// and an output of pairs aligned to 8 bytes (one float per load otherwise).
+template <bool DF, int U, int BLOCKS>
+static int probs_fast(const void *sv, uint64_t loads, void *out, double *partials, int nblocks, uint32_t *ticket,
+                      double *d_norm, cudaStream_t st) {
+    const uint64_t chunks = loads / (256 * U), wave = std::min<uint64_t>(nblocks, 152 * BLOCKS);
+    const int nb = (int)std::min(chunks, wave);
+    k_probs_fast<DF, U, BLOCKS><<<nb, 256, 0, st>>>((const float4 *)sv, chunks, (float *)out, partials, ticket, d_norm);
+    return nb;
+}
+
+// The FP32 kernels take whole chunks of at most 1024 16-byte loads, and an output of pairs aligned to 8 bytes (one float per load otherwise).
 static bool fast_prob_ok(const void *sv, uint64_t N, bool fp64, bool df, int out_fp64, const void *out) {
     const uint64_t loads = df ? N : N / 2;
-    return (!fp64 || df) && !(out && out_fp64) && loads >= (uint64_t)PROB_CHUNK &&
+    return (!fp64 || df) && !(out && out_fp64) && loads >= 1024 &&
            (reinterpret_cast<uintptr_t>(sv) & 15) == 0 && (df || (reinterpret_cast<uintptr_t>(out) & 7) == 0);
 }
-static int fast_grid(uint64_t n_chunks, int nblocks) {
-    const uint64_t cap = (uint64_t)(nblocks < 152 * 4 ? nblocks : 152 * 4);   // one wave of resident blocks
-    return (int)(n_chunks < cap ? n_chunks : cap);
-}
-
 cudaError_t launch_probs(bool fp64, const void *sv, int n, void *out, int out_fp64, double *partials,
                          int nblocks, double *d_norm, cudaStream_t st, bool df, uint32_t *ticket) {
     const uint64_t N = 1ull << n;
@@ -283,10 +284,10 @@ cudaError_t launch_probs(bool fp64, const void *sv, int n, void *out, int out_fp
     int nb = (int)(need < (uint64_t)nblocks ? need : (uint64_t)nblocks);
     if (nb < 1) nb = 1;
     if (fast_prob_ok(sv, N, fp64, df, out_fp64, out)) {
-        const uint64_t chunks = (df ? N : N / 2) / PROB_CHUNK;
-        nb = fast_grid(chunks, nblocks);
-        if (df) k_probs_fast<true><<<nb, 256, 0, st>>>((const float4 *)sv, chunks, (float *)out, partials, ticket, d_norm);
-        else k_probs_fast<false><<<nb, 256, 0, st>>>((const float4 *)sv, chunks, (float *)out, partials, ticket, d_norm);
+        const uint64_t loads = df ? N : N / 2;
+        nb = df ? probs_fast<true, 4, 4>(sv, loads, out, partials, nblocks, ticket, d_norm, st)
+             : loads <= 1ull << 24 ? probs_fast<false, 4, 4>(sv, loads, out, partials, nblocks, ticket, d_norm, st)
+                                             : probs_fast<false, 2, 6>(sv, loads, out, partials, nblocks, ticket, d_norm, st);
     } else if (df) {
         if (out_fp64) k_probs<float4, double><<<nb, 256, 0, st>>>((const float4 *)sv, N, (double *)out, partials, ticket, d_norm);
         else k_probs<float4, float><<<nb, 256, 0, st>>>((const float4 *)sv, N, (float *)out, partials, ticket, d_norm);
@@ -395,45 +396,46 @@ __global__ void __launch_bounds__(256) k_summary(const E *__restrict__ sv, uint6
 // far, so nothing that could win or tie is passed over. For random states
 // that is a few amplitudes per warp (2^28 complex64 amplitudes: 3.57 ms with
 // every amplitude in FP64, against 0.32 ms of HBM time; 2^25: 0.48 ms, 0.16 ms
-// with whole groups of loads in FP64, 0.08 ms here); for a state of equal
-// probabilities it is every amplitude, as before.
+// with whole groups of loads in FP64, 0.074 ms here); for a state of equal
+// probabilities it is every amplitude, as before. At most 48 registers for
+// complex64: a block then fits on an SM beside a block of a tensor-core pass
+// (53,248 of 65,536 registers), so that the summary of one state need not wait
+// for the end of another's long pass.
+constexpr int summary_blocks(bool df) { return df ? 4 : 5; }   // per SM
 template <bool DF>
-__global__ void __launch_bounds__(256, 4) k_summary_fast(const float4 *__restrict__ sv, uint64_t n_chunks,
-                                                          double *__restrict__ sums, double *__restrict__ maxs,
-                                                          uint64_t *__restrict__ idxs, uint32_t *ticket,
-                                                          double *out) {
+__global__ void __launch_bounds__(256, summary_blocks(DF))
+k_summary_fast(const float4 *__restrict__ sv, uint64_t n_chunks, double *__restrict__ sums, double *__restrict__ maxs,
+               uint64_t *__restrict__ idxs, uint32_t *ticket, double *out) {
     constexpr int PER = DF ? 1 : 2;   // amplitudes per load
     double acc = 0.0, best = -1.0;
     uint64_t bi = ~0ull;
     float least = -1.0f;   // below this a probability cannot win (warp-wide)
-    float S = 0.0f, T = 0.0f;
+    NormSum sum;
     uint32_t it = 0;
-    for (uint64_t c = blockIdx.x; c < n_chunks; c += gridDim.x, it++) {
-        const uint64_t at = c * PROB_CHUNK + threadIdx.x;
-        float4 v[PROB_U];
+    for (uint64_t c = blockIdx.x; c < n_chunks; c += gridDim.x) {
+        const uint64_t at = c * (256 * SUMMARY_U) + threadIdx.x;
+        float4 v[SUMMARY_U];
 #pragma unroll
-        for (int u = 0; u < PROB_U; u++) v[u] = __ldcs(sv + at + 256 * u);
-        bool ok = true;
-#pragma unroll
-        for (int u = 0; u < PROB_U; u++) ok = ok && split_range<DF>(v[u]);
-        float p[PROB_U * PER], top = -1.0f;
+        for (int u = 0; u < SUMMARY_U; u++) v[u] = __ldcs(sv + at + 256 * u);
+        const bool ok = sum.fits<DF>(v, acc);
+        float p[SUMMARY_U * PER], top = -1.0f;
         if (ok) {
 #pragma unroll
-            for (int u = 0; u < PROB_U; u++) {
+            for (int u = 0; u < SUMMARY_U; u++) {
                 if constexpr (DF) {
-                    const float2 a = split_prob_df(v[u]);
-                    split_add(S, T, a);
-                    p[u] = a.x + a.y;
+                    const SquaresDf q(v[u]);
+                    sum.add(q);
+                    p[u] = q.rough();
                 } else {
-                    const float2 a = split_prob(v[u].x, v[u].y), b = split_prob(v[u].z, v[u].w);
-                    split_add(S, T, a);
-                    split_add(S, T, b);
-                    p[2 * u] = a.x;
-                    p[2 * u + 1] = b.x;
+                    const Squares q(make_float2(v[u].x, v[u].y)), r(make_float2(v[u].z, v[u].w));
+                    sum.add(q);
+                    sum.add(r);
+                    p[2 * u] = q.rough();
+                    p[2 * u + 1] = r.rough();
                 }
             }
 #pragma unroll
-            for (int j = 0; j < PROB_U * PER; j++) top = fmaxf(top, p[j]);
+            for (int j = 0; j < SUMMARY_U * PER; j++) top = fmaxf(top, p[j]);
         }
         if (__any_sync(0xffffffffu, !ok || top >= least)) {
             float w = top;
@@ -441,7 +443,7 @@ __global__ void __launch_bounds__(256, 4) k_summary_fast(const float4 *__restric
             for (int o = 16; o > 0; o >>= 1) w = fmaxf(w, __shfl_xor_sync(0xffffffffu, w, o));
             least = fmaxf(least, w * (1.0f - 0x1p-21f));
 #pragma unroll
-            for (int j = 0; j < PROB_U * PER; j++) {
+            for (int j = 0; j < SUMMARY_U * PER; j++) {
                 if (ok && p[j] < least) continue;
                 const float4 x = v[j / PER];
                 double re, im;
@@ -452,12 +454,9 @@ __global__ void __launch_bounds__(256, 4) k_summary_fast(const float4 *__restric
                 better(best, bi, q, PER * (at + 256 * (j / PER)) + j % PER);
             }
         }
-        if ((it & 3) == 3) {   // the FP64 pipe gets two conversions and adds per four chunks
-            acc += (double)S + (double)T;
-            S = T = 0.0f;
-        }
+        if (++it % (PROB_SUM / (PER * SUMMARY_U)) == 0) acc += sum.take();
     }
-    acc += (double)S + (double)T;
+    acc += sum.take();
     const typename std::conditional<DF, float4, float2>::type *amps =
         reinterpret_cast<const typename std::conditional<DF, float4, float2>::type *>(sv);
     finish_summary(amps, acc, best, bi, sums, maxs, idxs, ticket, out);
@@ -472,8 +471,8 @@ cudaError_t launch_summary(bool fp64, const void *sv, int n, double *scratch, in
     double *sums = scratch, *maxs = scratch + nblocks;
     uint64_t *idxs = reinterpret_cast<uint64_t *>(scratch + 2 * nblocks);
     if (fast_prob_ok(sv, N, fp64, df, 0, nullptr)) {
-        const uint64_t chunks = (df ? N : N / 2) / PROB_CHUNK;
-        nb = fast_grid(chunks, nblocks);
+        const uint64_t chunks = (df ? N : N / 2) / (256 * SUMMARY_U);
+        nb = (int)std::min<uint64_t>(chunks, std::min(nblocks, 152 * summary_blocks(df)));
         if (df) k_summary_fast<true><<<nb, 256, 0, st>>>((const float4 *)sv, chunks, sums, maxs, idxs, ticket, out);
         else k_summary_fast<false><<<nb, 256, 0, st>>>((const float4 *)sv, chunks, sums, maxs, idxs, ticket, out);
     } else if (df) {
