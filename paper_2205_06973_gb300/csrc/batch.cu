@@ -145,6 +145,7 @@ __global__ void __launch_bounds__(256) k_batch(float2 *__restrict__ svbase, cons
         }
         __syncwarp();
     }
+    pdl_wait();   // done when the kernel before is (BatchLaunch::beside)
 }
 
 // Whole circuits of T qubits, one CTA each: the state stays in shared memory
@@ -153,6 +154,10 @@ __global__ void __launch_bounds__(256) k_batch(float2 *__restrict__ svbase, cons
 // parts of a few tiles each, every part a trip through L2 and the work queue
 // with little for the other warps to do: 45 parameterised circuits of 10 to
 // 12 qubits took 3.2 ms.
+// The kernels of a batch's sizes and the one after them share nothing: each
+// lets the next launch as soon as its own CTAs have started, and ends when the
+// one before has ended, so that they run beside each other and still form a
+// chain (BatchLaunch::beside).
 template <int T, int R>
 __global__ void __launch_bounds__(1 << (T - R))
 k_batch_whole(float2 *__restrict__ svbase, const BatchWhole *__restrict__ circuits,
@@ -164,6 +169,7 @@ k_batch_whole(float2 *__restrict__ svbase, const BatchWhole *__restrict__ circui
     const uint32_t tid = threadIdx.x;
     const BatchWhole C = circuits[blockIdx.x];
     const PartLaunch &P = parts[C.part];
+    pdl_launch();   // the next kernel of the graph shares nothing with this one
     float2 *const sv = svbase + C.sv_off;
     uint32_t s_cthr = 0;
 #pragma unroll
@@ -206,6 +212,7 @@ k_batch_whole(float2 *__restrict__ svbase, const BatchWhole *__restrict__ circui
             if (i & (1 << b)) off ^= (uint32_t)P.store_reg[b];
         __stcg(sv + off, a[i]);
     }
+    pdl_wait();   // done when the kernel before is
 }
 
 // p[i] = |a_i|^2 over the concatenated states, 2^10 amplitudes per warp and
@@ -315,27 +322,27 @@ cudaError_t batch_prepare(int warps_per_cta, int *n_ctas) {
 }
 
 cudaError_t launch_batch(const BatchLaunch &B, int warps_per_cta, int n_ctas, cudaStream_t st) {
-    const size_t smem = (size_t)warps_per_cta * (1u << BT) * sizeof(float2);
-    k_batch<<<n_ctas, warps_per_cta * 32, smem, st>>>(B.svbase, B.items, B.n_items, B.circ_off, B.parts, B.stream,
-                                                      B.windows, B.done, B.head, B.err);
-    return cudaGetLastError();
+    BatchConfig c(n_ctas, warps_per_cta * 32, (size_t)warps_per_cta * (1u << BT) * sizeof(float2), st, B.beside);
+    cudaError_t e = cudaLaunchKernelEx(&c.cfg, k_batch, B.svbase, B.items, B.n_items, B.circ_off, B.parts, B.stream,
+                                       B.windows, B.done, B.head, B.err);
+    return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 template <int T>
-static void whole_t(const BatchLaunch &B, const BatchWhole *circuits, uint32_t n, cudaStream_t st) {
+static cudaError_t whole_t(const BatchLaunch &B, const BatchWhole *circuits, uint32_t n, cudaStream_t st) {
     constexpr int R = batch_whole_R(T);
-    const size_t smem = (sizeof(float2) << T) + INTERP_WINDOW;
-    k_batch_whole<T, R><<<n, 1u << (T - R), smem, st>>>(B.svbase, circuits, B.parts, B.stream, B.windows);
+    BatchConfig c(n, 1u << (T - R), (sizeof(float2) << T) + INTERP_WINDOW, st, B.beside);
+    cudaError_t e = cudaLaunchKernelEx(&c.cfg, k_batch_whole<T, R>, B.svbase, circuits, B.parts, B.stream, B.windows);
+    return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 cudaError_t launch_batch_whole(int t, const BatchLaunch &B, const BatchWhole *circuits, uint32_t n, cudaStream_t st) {
     switch (t) {
-    case 10: whole_t<10>(B, circuits, n, st); break;
-    case 11: whole_t<11>(B, circuits, n, st); break;
-    case 12: whole_t<12>(B, circuits, n, st); break;
-    default: return cudaErrorInvalidValue;
+    case 10: return whole_t<10>(B, circuits, n, st);
+    case 11: return whole_t<11>(B, circuits, n, st);
+    case 12: return whole_t<12>(B, circuits, n, st);
     }
-    return cudaGetLastError();
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_batch_probs(float2 *svbase, uint64_t total, const uint64_t *circ_off, const uint32_t *circ_n,

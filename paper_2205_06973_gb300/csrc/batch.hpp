@@ -38,6 +38,26 @@ struct BatchLaunch {
     uint32_t *done;              // per-circuit finished-tile counters (zeroed per run)
     uint32_t *head;              // queue ticket (zeroed per run)
     int *err;                    // bounded-wait failure flag
+    bool beside;                 // the kernel before on the stream is one of the whole circuits: launched
+                                 // without waiting for it, ends after it
+};
+
+// Launch configuration of a batch's kernel; beside: as a dependent that may run
+// with the kernel before (griddepcontrol.wait at its end).
+struct BatchConfig {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    BatchConfig(unsigned grid, unsigned threads, size_t smem, cudaStream_t st, bool beside) {
+        cfg.gridDim = dim3(grid);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = beside ? 1 : 0;
+    }
+    BatchConfig(const BatchConfig &) = delete;   // cfg points into it
 };
 
 constexpr int BATCH_TILE_QUBITS = 9;   // one warp's tile: 32 lanes x 16 amplitudes

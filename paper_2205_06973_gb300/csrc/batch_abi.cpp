@@ -39,11 +39,6 @@ struct sv_batch {
     cudaStream_t prep = nullptr;         // private: allocations, uploads and the graph capture, so that
                                          // building a batch never enqueues on (or captures) a stream that
                                          // another thread uses for earlier batches
-    // further branches of the capture (one per size of the whole circuits)
-    // with their fork and joins
-    static constexpr int SIDES = BATCH_WHOLE_QUBITS - BATCH_MIN_QUBITS + 1;
-    cudaStream_t side[SIDES] = {};
-    cudaEvent_t fork = nullptr, join[SIDES] = {};
     int warps = 8;                       // warps per CTA
     int chunk = 0;                       // tiles per queue item (0 = by the batch's size)
     bool hold_last = false;              // testing: the last item waits for tiles that never complete
@@ -85,15 +80,6 @@ static void drop_program(sv_batch *b) {
     b->built = false;
 }
 
-static void drop_streams(sv_batch *b) {
-    if (b->prep) cudaStreamDestroy(b->prep);
-    if (b->fork) cudaEventDestroy(b->fork);
-    for (int i = 0; i < sv_batch::SIDES; i++) {
-        if (b->side[i]) cudaStreamDestroy(b->side[i]);
-        if (b->join[i]) cudaEventDestroy(b->join[i]);
-    }
-}
-
 extern "C" {
 
 sv_status sv_batch_create(uint32_t n_circuits, const int *n_qubits, void *stream, sv_batch **out) {
@@ -119,13 +105,7 @@ sv_status sv_batch_create(uint32_t n_circuits, const int *n_qubits, void *stream
     }
     {
         cudaError_t pe = cudaStreamCreateWithFlags(&b->prep, cudaStreamNonBlocking);
-        if (pe == cudaSuccess) pe = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
-        for (int i = 0; pe == cudaSuccess && i < sv_batch::SIDES; i++) {
-            pe = cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking);
-            if (pe == cudaSuccess) pe = cudaEventCreateWithFlags(&b->join[i], cudaEventDisableTiming);
-        }
         if (pe != cudaSuccess) {
-            drop_streams(b.get());
             if (b->own_stream) cudaStreamDestroy(b->stream);
             return bfail(SV_ERR_CUDA, std::string("batch stream: ") + cudaGetErrorString(pe));
         }
@@ -153,7 +133,7 @@ sv_status sv_batch_create(uint32_t n_circuits, const int *n_qubits, void *stream
         dev_free(b->sv, st); dev_free(b->d_off, st); dev_free(b->d_nq, st); dev_free(b->d_done, st);
         dev_free(b->d_err, st); dev_free(b->d_norms, st);
         cudaStreamSynchronize(st);
-        drop_streams(b.get());
+        cudaStreamDestroy(b->prep);
         if (b->own_stream) cudaStreamDestroy(b->stream);
         return bfail(e == cudaErrorMemoryAllocation ? SV_ERR_OOM : SV_ERR_CUDA,
                      std::string("batch allocation: ") + cudaGetErrorString(e));
@@ -461,33 +441,32 @@ static sv_status build_program(sv_batch *b) {
     // captured on the private stream (nothing else is ever enqueued there),
     // launched on the caller's stream
     BCUDA(cudaStreamBeginCapture(b->prep, cudaStreamCaptureModeThreadLocal));
-    // the whole circuits wait for nothing: they run beside the other kernels
-    // and each other (branches of the graph), where these leave room on the
-    // SMs; they come first, the largest before the others, as their time is
-    // the latency of a circuit's gates
-    cudaError_t ce = cudaSuccess;
-    if (n_whole) ce = cudaEventRecord(b->fork, b->prep);
+    // The whole circuits wait for nothing: they run beside each other and the
+    // kernel after them where these leave room on the SMs; they come first,
+    // the largest before the others, as their time is the latency of a
+    // circuit's gates. They are a chain of dependent launches and not
+    // branches of the graph: a branch takes one of the device's few hardware
+    // queues, and there it waits behind whatever another stream of the process
+    // has queued (a server's batches behind all passes of its largest
+    // requests: the requests of at most 20 qubits took 1.2 to 1.5 s at the
+    // median with branches, 0.14 s so; a batch beside six such streams 178 and 0.3 ms).
+    cudaError_t ce = cudaMemsetAsync(b->d_done, 0, sizeof(uint32_t) * (b->n + 2), b->prep);
+    double *const dn = reinterpret_cast<double *>(dd + ds_items + ds_parts + ds_img);
+    if (ce == cudaSuccess && b->n_dense_items) ce = cudaMemsetAsync(dn, 0, sizeof(double) * b->n_dense_parts, b->prep);
+    B.beside = false;
     for (int t = BATCH_WHOLE_QUBITS; t >= BATCH_MIN_QUBITS; t--) {
-        const int i = t - BATCH_MIN_QUBITS;
-        if (wholes[t].empty()) continue;
-        if (ce == cudaSuccess) ce = cudaStreamWaitEvent(b->side[i], b->fork, 0);
-        if (ce == cudaSuccess) ce = launch_batch_whole(t, B, d_whole[t], (uint32_t)wholes[t].size(), b->side[i]);
-        if (ce == cudaSuccess) ce = cudaEventRecord(b->join[i], b->side[i]);
+        if (ce != cudaSuccess || wholes[t].empty()) continue;
+        ce = launch_batch_whole(t, B, d_whole[t], (uint32_t)wholes[t].size(), b->prep);
+        B.beside = true;
     }
-    if (ce == cudaSuccess) ce = cudaMemsetAsync(b->d_done, 0, sizeof(uint32_t) * (b->n + 2), b->prep);
     if (ce == cudaSuccess && b->n_dense_items) {
-        double *dn = reinterpret_cast<double *>(dd + ds_items + ds_parts + ds_img);
-        ce = cudaMemsetAsync(dn, 0, sizeof(double) * b->n_dense_parts, b->prep);
-        if (ce == cudaSuccess)
-            ce = launch_dense6_batch(b->sv, reinterpret_cast<const DenseBatchPart *>(dd + ds_items),
-                                     reinterpret_cast<const DenseBatchItem *>(dd), b->n_dense_items,
-                                     dd + ds_items + ds_parts, b->d_done, b->d_done + b->n + 1, b->d_err, dn,
-                                     b->prep);
+        ce = launch_dense6_batch(b->sv, reinterpret_cast<const DenseBatchPart *>(dd + ds_items),
+                                 reinterpret_cast<const DenseBatchItem *>(dd), b->n_dense_items,
+                                 dd + ds_items + ds_parts, b->d_done, b->d_done + b->n + 1, b->d_err, dn, b->prep,
+                                 B.beside);
+        B.beside = false;
     }
     if (ce == cudaSuccess && B.n_items) ce = launch_batch(B, b->warps, n_ctas, b->prep);
-    for (int i = 0; i < sv_batch::SIDES; i++)
-        if (ce == cudaSuccess && !wholes[i + BATCH_MIN_QUBITS].empty())
-            ce = cudaStreamWaitEvent(b->prep, b->join[i], 0);
     cudaGraph_t g = nullptr;
     cudaError_t ee = cudaStreamEndCapture(b->prep, &g);
     if (ce != cudaSuccess || ee != cudaSuccess) {
@@ -643,7 +622,7 @@ sv_status sv_batch_destroy(sv_batch *b) {
         cudaStreamSynchronize(b->stream);   // the frees complete before the stream goes
         cudaStreamDestroy(b->stream);
     }
-    drop_streams(b);                        // idle: drop_program synchronised prep
+    cudaStreamDestroy(b->prep);             // idle: drop_program synchronised prep
     delete b;
     if (e != cudaSuccess) return bfail(SV_ERR_CUDA, std::string("pending batch work failed: ") + cudaGetErrorString(e));
     return SV_OK;

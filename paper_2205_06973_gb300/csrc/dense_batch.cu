@@ -41,6 +41,7 @@
 #include <cstdint>
 
 #include "dense.hpp"
+#include "batch.hpp"
 #include "dense_batch.hpp"
 #include "dense_common.cuh"
 
@@ -556,11 +557,13 @@ k_dense6_batch(float2 *__restrict__ svbase, const DenseBatchPart *__restrict__ p
         tc_fence_after();
         tmem_dealloc(tmem, TMEM_COLS);
     }
+    // done when the kernel before is, which may run beside this one
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
 }
 
 cudaError_t launch_dense6_batch(void *svbase, const DenseBatchPart *parts, const DenseBatchItem *items,
                                 uint32_t n_items, const void *r_imgs, uint32_t *done, uint32_t *head, int *err,
-                                double *dn, cudaStream_t st) {
+                                double *dn, cudaStream_t st, bool beside) {
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -572,9 +575,10 @@ cudaError_t launch_dense6_batch(void *svbase, const DenseBatchPart *parts, const
         return cudaErrorMisalignedAddress;
     unsigned grid = (unsigned)sms;
     if (n_items < grid) grid = n_items < 1 ? 1 : n_items;
-    k_dense6_batch<<<grid, THREADS, SMEM, st>>>(reinterpret_cast<float2 *>(svbase), parts, items, n_items,
-                                                reinterpret_cast<const uint8_t *>(r_imgs), done, head, err, dn);
-    return cudaGetLastError();
+    BatchConfig c(grid, THREADS, SMEM, st, beside);
+    e = cudaLaunchKernelEx(&c.cfg, k_dense6_batch, reinterpret_cast<float2 *>(svbase), parts, items, n_items,
+                           reinterpret_cast<const uint8_t *>(r_imgs), done, head, err, dn);
+    return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 }  // namespace hisv

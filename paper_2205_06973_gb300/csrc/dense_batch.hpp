@@ -46,9 +46,9 @@ constexpr int DENSE_BATCH_ERR_WORDS = 8;
 // items[n_items] over parts[]; r_imgs: one 64 KiB R image per part; done:
 // n circuit counters then the queue ticket, zeroed before the launch; dn:
 // one FP64 norm slot per pass, zeroed before the launch; err: the error
-// record (DENSE_BATCH_ERR_WORDS ints).
+// record (DENSE_BATCH_ERR_WORDS ints); beside: see BatchLaunch.
 cudaError_t launch_dense6_batch(void *svbase, const DenseBatchPart *parts, const DenseBatchItem *items,
                                 uint32_t n_items, const void *r_imgs, uint32_t *done, uint32_t *head, int *err,
-                                double *dn, cudaStream_t st);
+                                double *dn, cudaStream_t st, bool beside);
 
 }  // namespace hisv
