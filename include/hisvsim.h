@@ -262,7 +262,8 @@ sv_status sv_plan_destroy(sv_plan *p);
  * and scatters it back (Algorithm 1). The plan's qubit count must equal the
  * state's. Stream-ordered (SV_FLAG_SYNC waits). The first call for a given
  * precision and tile uploads the part program to device memory (owned by the
- * plan). States with n < 10 run the whole gate list in one launch. */
+ * plan). States with n < 10 run the whole gate list in one launch, which
+ * needs nothing of the plan afterwards. */
 sv_status sv_apply_parts(sv_state *s, sv_plan *p, uint32_t flags);
 
 /* -------------------------------------------------------------- measure ---

@@ -783,7 +783,6 @@ sv_status sv_plan_destroy(sv_plan *p) {
         dev_free(kv.second.d_windows, 0);
         dev_free(kv.second.d_aimg, 0);
         dev_free(kv.second.d_pimg, 0);
-        dev_free(kv.second.d_small, 0);
     }
     cudaSetDevice(cur);
     delete p;
@@ -855,53 +854,27 @@ static sv_status apply_gatewise(sv_state *s, sv_plan *p) {
     return SV_OK;
 }
 
-// A circuit on fewer than 10 qubits in one launch; the op records are
-// uploaded at the plan's first apply for the precision and device and kept in
-// the plan. Where that cannot be done now (no memory, or the stream is being
-// captured, which an upload with its wait would break) the circuit runs gate
-// by gate.
+// A circuit on fewer than 10 qubits in one launch (at most 640 ops; 384 in
+// complex128). The op records are made at the plan's first apply for the
+// precision and kept in the plan; the launch takes a copy.
 static sv_status apply_small(sv_state *s, sv_plan *p) {
     if (p->gates.empty()) return SV_OK;
     const bool fp64 = is_fp64(s);
-    const DevProgram *prog = nullptr;
-    {
+    const void *ops;
+    uint32_t n_ops;
+    auto made = [&](auto &v, auto list) {
+        using Real = decltype(list);
         std::lock_guard<std::recursive_mutex> lk(p->mu);
-        auto key = std::make_tuple(s->dev, fp64, 0, 0);   // tile 0: no part program has it
-        auto it = p->dev_progs.find(key);
-        if (it == p->dev_progs.end()) {
-            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-            cudaError_t e = cudaStreamIsCapturing(s->stream, &cap);
-            if (e != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-                cudaGetLastError();
-                return apply_gatewise(s, p);
-            }
-            std::vector<SmallOp<float>> f;
-            std::vector<SmallOp<double>> d;
-            if (fp64) d = small_ops<double>(p);
-            else f = small_ops<float>(p);
-            const void *src = fp64 ? static_cast<const void *>(d.data()) : f.data();
-            const size_t bytes = fp64 ? d.size() * sizeof(d[0]) : f.size() * sizeof(f[0]);
-            DevProgram dp;
-            dp.dev = s->dev;
-            dp.n_small = (uint32_t)(fp64 ? d.size() : f.size());
-            e = dev_alloc(&dp.d_small, bytes, s->stream);
-            if (e != cudaSuccess) {
-                cudaGetLastError();
-                return apply_gatewise(s, p);
-            }
-            e = cudaMemcpyAsync(dp.d_small, src, bytes, cudaMemcpyHostToDevice, s->stream);
-            // shared by every state that applies the plan, on any stream:
-            // complete before it is published
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-            if (e != cudaSuccess) {
-                dev_free(dp.d_small, s->stream);
-                return fail(SV_ERR_CUDA, std::string("program upload: ") + cudaGetErrorString(e));
-            }
-            it = p->dev_progs.emplace(key, dp).first;
+        if (v.empty()) {
+            v = small_ops<Real>(p);
+            v.resize(v.size() + small_most(fp64));   // launch_small copies whole records lists
         }
-        prog = &it->second;   // map nodes do not move
-    }
-    CUDA_TRY(launch_small(fp64, s->buf, s->n, prog->d_small, prog->n_small, s->stream));
+        ops = v.data();
+        n_ops = (uint32_t)(v.size() - small_most(fp64));
+    };
+    if (fp64) made(p->small64, double());
+    else made(p->small32, float());
+    CUDA_TRY(launch_small(fp64, s->buf, s->n, ops, n_ops, s->stream));
     return SV_OK;
 }
 

@@ -14,6 +14,7 @@
 #include "jit.hpp"
 #include "partition.hpp"
 #include "planner.hpp"
+#include "small.hpp"
 
 using hisv::GateRef;
 using hisv::Program;
@@ -37,8 +38,6 @@ struct DevProgram {
     std::vector<hisv::PartLaunch> parts;   // and its parts (launch arguments)
     uint8_t *d_aimg = nullptr;      // R images of the dense parts
     uint8_t *d_pimg = nullptr;      // R images of the dense pairs (two per pass)
-    void *d_small = nullptr;        // op records of a circuit on fewer than 10 qubits
-    uint32_t n_small = 0;
 };
 
 struct sv_state {
@@ -74,6 +73,8 @@ struct sv_plan {
     int k2 = 0;
     std::map<std::tuple<bool, int, int>, std::unique_ptr<Program>> host_progs;   // (fp64, t, mode)
     std::map<std::tuple<int, bool, int, int>, DevProgram> dev_progs;             // (dev, fp64, t, mode)
+    std::vector<hisv::SmallOp<float>> small32;    // op records of a circuit on fewer than 10 qubits
+    std::vector<hisv::SmallOp<double>> small64;
     std::vector<std::vector<double>> mats;                                 // gatewise matrices
     std::map<std::tuple<int, int, int>, std::unique_ptr<hisv::JitProgram>> jit_progs;   // (precision, t, mode)
     // the caches above are filled on first use; several host threads may

@@ -19,7 +19,7 @@ enum SmallKind : int32_t {
     SMALL_PERM           // new[x] = old[perm[n] ^ XOR of perm[b] over the set bits b of x] (CX, SWAP)
 };
 
-template <typename Real> struct SmallOp {
+template <typename Real> struct alignas(16) SmallOp {
     union {
         Real m[8];
         uint16_t perm[SMALL_MAX_QUBITS + 1];
@@ -27,7 +27,12 @@ template <typename Real> struct SmallOp {
     int32_t kind, q0, q1, pad;
 };
 
-// Apply n_ops ops (device memory, 16-byte aligned) to the n-qubit state.
+// Op records that one launch takes (30 KiB of kernel parameters).
+constexpr uint32_t small_most(bool fp64) { return fp64 ? 384u : 640u; }
+
+// Apply n_ops ops to the n-qubit state. ops (host memory) holds
+// small_most(fp64) records behind them that are never run; the launch takes
+// a copy.
 cudaError_t launch_small(bool fp64, void *sv, int n, const void *ops, uint32_t n_ops, cudaStream_t st);
 
 }  // namespace hisv
