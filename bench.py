@@ -102,7 +102,7 @@ KERNEL_SOURCES = {
     "k_dense6_pair": ("dense_pair.cu", "dense.hpp", "dense_common.cuh", "planner.cpp"),
     "k_part": ("part_kernel.cuh", "part_f32.cu", "part_f64.cu", "interp.cpp", "interp.hpp", "ops.cuh", "packed.cuh",
                "ops_core.cuh", "program.hpp", "planner.cpp"),
-    "hisv_part": ("jit.cpp", "jit_prelude.cuh", "ops_core.cuh", "program.hpp", "planner.cpp"),
+    "hisv_part": ("jit.cpp", "jit_prelude.cuh", "ops_core.cuh", "packed.cuh", "program.hpp", "planner.cpp"),
 }
 
 
@@ -550,14 +550,15 @@ def grid_section(n, gates, st, peak, fp32_peak=None):
         for k in (8, 10, 12):
             plan = api.Plan(gates, n, method, k)
             passes = plan.stats("c64")["passes"]
-            flops = plan.flops("c64")[0]
-            row = {"method": method, "k": k, "passes": passes, "executed_fp32_flops": flops}
+            row = {"method": method, "k": k, "passes": passes}
             for name, jit in (("interpreter", False), ("specialised", True)):
+                flops = plan.flops("c64", jit=jit)[0]
                 if jit:
                     row["compile_s"] = round(plan.specialise("c64"), 2)
                 ms = _timed(st, plan, jit=jit)
                 gbs = plan.stats("c64", jit=jit)["passes"] * 2 * st.nbytes / (ms / 1e3) / 1e9
-                row[name] = {"ms": round(ms, 2), "GBs": round(gbs, 1), "frac": round(gbs / peak, 4)}
+                row[name] = {"ms": round(ms, 2), "GBs": round(gbs, 1), "frac": round(gbs / peak, 4),
+                             "executed_fp32_flops": flops}
                 if fp32_peak:
                     fl = flops / (ms / 1e3)
                     row[name]["fp32_tflops"] = round(fl / 1e12, 2)
@@ -598,8 +599,8 @@ def c128_section(n, gates, peak, fp64_peak):
                                  ("beam", 10, True, "c128df"), ("beam", 8, True, "c128df"),
                                  ("dagp", 10, True, "c128df")):
         plan = api.Plan(gates, n, method, k, dfs_trials=16)
-        passes = plan.stats("c128", jit=jit)["passes"]
-        flops = plan.flops("c128")[0]
+        passes = plan.stats(prec, jit=jit)["passes"]
+        flops = plan.flops(prec, jit=jit)[0]
         cs = plan.specialise(prec) if jit else 0.0
         ms = _timed(st if prec == "c128" else sdf, plan, jit=jit, reps=1)
         gbs = passes * 2 * st.nbytes / (ms / 1e3) / 1e9

@@ -194,14 +194,17 @@ sv_status sv_plan_build(const sv_gate *gates, size_t n_gates, int n_qubits, sv_m
 /* Copy the partition out: part_of_gate[n_gates] (may be NULL) and the number
  * of parts. n_gates must equal the plan's gate count. */
 sv_status sv_plan_export(const sv_plan *p, uint32_t *part_of_gate, size_t n_gates, uint32_t *n_parts);
-/* Statistics of the compiled device program for a precision, tile and apply
- * flags (SV_FLAG_TC_DENSE changes the program): passes = parts run on the
- * GPU (without SV_FLAG_SPECIALISE a complex64 state of at most 13 qubits on
- * the default tile may run them in one launch; with it, the passes of the
- * specialised kernels, which cut parts whose tiles would have short runs and
- * join parts of two-qubit phases to others), phases = register phases of the
- * plan's gate-list parts, ops = their kernel ops, dense = parts run as fused unitaries on the tensor cores (any output
- * pointer may be NULL). Compiles on the host if needed; no device work. */
+/* Statistics of the device program that an apply with the precision, tile and
+ * flags runs: passes = parts run on the GPU, phases = register phases of its
+ * gate-list parts, ops = their kernel ops, dense = parts run as fused
+ * unitaries on the tensor cores (any output pointer may be NULL). With
+ * SV_FLAG_SPECIALISE that program may have other parts than the plan: those
+ * whose tiles would have short runs are cut, and parts of two-qubit phases
+ * join others. Two applies run another program than the one described: a
+ * complex64 state of at most 13 qubits on the default tile may take the
+ * plan's parts in one launch, and a double-float state is specialised
+ * without the flag too (describe it with the flag). Compiles on the host if
+ * needed, for the apply as well; no device work. */
 sv_status sv_plan_stats(sv_plan *p, sv_precision prec, int tile_qubits, uint32_t flags, uint32_t *passes,
                         uint32_t *phases, uint32_t *ops, uint32_t *dense);
 /* sv_plan_build_ml: multi-level partitioning (Sec. IV-B, "Multi-level
@@ -237,15 +240,17 @@ sv_status sv_plan_specialise(sv_plan *p, sv_precision prec, int tile_qubits, uin
 /* sv_plan_source: the generated CUDA source of gate-list part i (execution
  * order among the gate-list parts) of the plan's program for prec, tile and
  * flags, copied NUL-terminated into buf (cap bytes); *len receives the
- * source length. Host only. It is the plan's own part in the default shape; an
- * apply may cut and join parts (sv_plan_stats) and choose another tile. */
+ * source length. Host only. With SV_FLAG_SPECIALISE the program is the one
+ * that an apply runs (sv_plan_stats); without, the plan's own parts, on the
+ * default tile and register bits unless given. */
 sv_status sv_plan_source(sv_plan *p, sv_precision prec, int tile_qubits, uint32_t flags, uint32_t part, char *buf,
                          size_t cap, size_t *len);
 /* sv_plan_flops: the floating-point operations one apply of the plan
- * executes for the precision, tile and flags (host only): *alu_flops on the
+ * executes for the precision, tile and flags (host only; of the program that
+ * sv_plan_stats describes): *alu_flops on the
  * CUDA cores, counted per op of the compiled program as its arithmetic over
- * the amplitudes it touches (an FMA counts two; H 2, RX/RY 6, a fused 2x2
- * 14, a diagonal 6 on the amplitudes it scales; permutations and sign
+ * the amplitudes it touches (an FMA counts two; H 2, RX/RY 4, a fused 2x2
+ * 11, a diagonal 6 on the amplitudes it scales; permutations and sign
  * changes 0; gate by gate: 14 per one-qubit and 30 per two-qubit gate, the
  * general matrices of Sec. III-A), and *tensor_flops on the tensor cores
  * (1536 per amplitude per dense part: three split-BF16 products of the

@@ -55,10 +55,11 @@ class Plan:
                                     ctypes.byref(a), ctypes.byref(b), ctypes.byref(c), ctypes.byref(d)))
         return {"passes": a.value, "phases": b.value, "ops": c.value, "dense": d.value}
 
-    def flops(self, precision="c64", tile=0, tc=False, gatewise=False):
+    def flops(self, precision="c64", tile=0, tc=False, gatewise=False, jit=False):
         """(CUDA-core flops, tensor-core flops) of one apply (sv_plan_flops)."""
         a, b = ctypes.c_double(), ctypes.c_double()
-        flags = N.tc_flags(tc) | (N.SV_FLAG_GATEWISE if gatewise else 0)
+        flags = (N.tc_flags(tc) | (N.SV_FLAG_GATEWISE if gatewise else 0)
+                 | (N.SV_FLAG_SPECIALISE if jit else 0))
         N.check(N.lib.sv_plan_flops(self.h, N.PRECISIONS[precision], tile, flags,
                                     ctypes.byref(a), ctypes.byref(b)))
         return a.value, b.value
@@ -74,11 +75,12 @@ class Plan:
                                          1 if load else 0, ctypes.byref(s)))
         return s.value
 
-    def source(self, part, precision="c64", tile=0, tc=False, regbits=0):
-        """Generated CUDA source of gate-list part ``part``."""
+    def source(self, part, precision="c64", tile=0, tc=False, regbits=0, jit=False):
+        """Generated CUDA source of gate-list part ``part``; jit: of the
+        program that a specialised apply runs."""
         n = ctypes.c_size_t()
         args = (self.h, N.PRECISIONS[precision], tile,
-                N.tc_flags(tc) | N.SV_FLAG_REGBITS(regbits), part)
+                N.tc_flags(tc) | N.SV_FLAG_REGBITS(regbits) | (N.SV_FLAG_SPECIALISE if jit else 0), part)
         N.check(N.lib.sv_plan_source(*args, None, 0, ctypes.byref(n)))
         buf = ctypes.create_string_buffer(n.value + 1)
         N.check(N.lib.sv_plan_source(*args, buf, n.value + 1, ctypes.byref(n)))

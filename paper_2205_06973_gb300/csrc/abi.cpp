@@ -649,9 +649,10 @@ static int interp_mode(const sv_plan *p, bool fp64, uint32_t flags, int t_user, 
 // asks for the statistics first (on a thread that plans) has compiled it for
 // the apply; but the plan's own parts where the apply makes them one, and the
 // default shape for register bits that the interpreter does not take and for
-// double-float states.
+// double-float states (without SV_FLAG_SPECIALISE).
 static int stats_mode(const sv_plan *p, sv_precision prec, uint32_t flags, int t_user, int &t) {
     const bool fp64 = prec != SV_C64;
+    if (flags & SV_FLAG_SPECIALISE) return spec_mode(p, prec, flags, t_user, t);
     if (!((flags >> 8) & 0xFu) && prec != SV_C128DF) return interp_mode(p, fp64, flags, t_user, t, false);
     t = t_user ? t_user : default_tile(fp64, p->max_part);
     return dense_mode(flags, fp64) & ~kModeJit;
@@ -661,9 +662,8 @@ sv_status sv_plan_stats(sv_plan *p, sv_precision prec, int t, uint32_t flags, ui
                         uint32_t *ops, uint32_t *dense) {
     if (!p) return fail(SV_ERR_ARG, "plan is NULL");
     const bool fp64 = prec != SV_C64;
-    const int t_user = t;
     if (t != 0 && (t < part_tmin() || t > part_tmax(fp64))) return fail(SV_ERR_ARG, "tile_qubits out of range");
-    const int mode = stats_mode(p, prec, flags, t_user, t);
+    const int mode = stats_mode(p, prec, flags, t, t);
     if (p->method == SV_PART_NONE || p->n < part_tmin() || (flags & SV_FLAG_GATEWISE)) {
         if (passes) *passes = (uint32_t)p->gates.size();
         if (phases) *phases = 0;
@@ -675,13 +675,6 @@ sv_status sv_plan_stats(sv_plan *p, sv_precision prec, int t, uint32_t flags, ui
     sv_status st = get_host_program(p, fp64, t, mode, &prog);
     if (st != SV_OK) return st;
     if (passes) *passes = (uint32_t)prog->kind.size();
-    if (passes && (flags & SV_FLAG_SPECIALISE)) {   // the specialised kernels' passes
-        int ts = 0;
-        if ((spec_mode(p, prec, flags, t_user, ts) & kModeRefine) && p->max_part <= ts) {
-            std::vector<uint32_t> pog;
-            *passes = refine_parts(p->gates, p->n, p->pog, p->n_parts, fp64, ts, pog);
-        }
-    }
     if (phases) *phases = (uint32_t)prog->phases.size();
     if (ops) *ops = (uint32_t)prog->ops.size();
     if (dense) *dense = (uint32_t)(prog->dense.size() + prog->pairs.size());
@@ -733,9 +726,10 @@ sv_status sv_plan_source(sv_plan *p, sv_precision prec, int t, uint32_t flags, u
                          size_t *len) {
     if (!p) return fail(SV_ERR_ARG, "plan is NULL");
     const bool fp64 = prec != SV_C64;
-    if (t == 0) t = default_tile(fp64, p->max_part);
-    if (t < part_tmin() || t > part_tmax(fp64)) return fail(SV_ERR_ARG, "tile_qubits out of range");
-    const int mode = dense_mode(flags, fp64);
+    if (t != 0 && (t < part_tmin() || t > part_tmax(fp64))) return fail(SV_ERR_ARG, "tile_qubits out of range");
+    int mode = dense_mode(flags, fp64);
+    if (flags & SV_FLAG_SPECIALISE) mode = spec_mode(p, prec, flags, t, t);
+    else if (t == 0) t = default_tile(fp64, p->max_part);
     const Program *hp = nullptr;
     sv_status st = get_host_program(p, fp64, t, mode, &hp);
     if (st != SV_OK) return st;
@@ -764,7 +758,7 @@ sv_status sv_plan_flops(sv_plan *p, sv_precision prec, int t, uint32_t flags, do
         const Program *hp = nullptr;
         sv_status st = get_host_program(p, fp64, t, mode, &hp);
         if (st != SV_OK) return st;
-        program_flops(*hp, a, b);
+        program_flops(*hp, a, b, (mode & kModeJit) != 0);
     }
     const double N = std::ldexp(1.0, p->n);
     if (alu_flops) *alu_flops = a * N;

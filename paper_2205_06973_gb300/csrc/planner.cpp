@@ -1152,9 +1152,10 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
 // program's kernels execute (an FMA counts two; sign changes, permutations
 // and shared-memory moves count none): per op of a gate-list part, the
 // arithmetic of its template in ops_core.cuh over the amplitudes it touches,
-// plus the store factor; per dense part, the split-BF16 products (3 x 128
+// plus the store factor (gather: a run of OP_CPT on a register bit is one
+// product, as the specialised kernels apply it); per dense part, the split-BF16 products (3 x 128
 // real MACs per real output, 1536 per complex amplitude, tensor cores).
-void program_flops(const Program &prog, double &alu_per_amp, double &tensor_per_amp) {
+void program_flops(const Program &prog, double &alu_per_amp, double &tensor_per_amp, bool gather) {
     alu_per_amp = 0.0;
     tensor_per_amp = 0.0;
     const int NR = 1 << prog.R;
@@ -1166,14 +1167,24 @@ void program_flops(const Program &prog, double &alu_per_amp, double &tensor_per_
         const PartLaunch &L = prog.parts[prog.index[i]];
         for (uint32_t p = 0; p < L.n_phases; p++) {
             const Phase &ph = prog.phases[L.phase_begin + p];
+            uint32_t gathered = 0;   // register bits whose OP_CPT run is one product (specialised kernels)
             for (uint32_t k = 0; k < ph.op_count; k++) {
                 const Op &op = prog.ops[ph.op_begin + k];
+                switch (op.kind) {
+                case OP_H: case OP_RXS: case OP_RYS: case OP_U2S: case OP_X: case OP_Y: gathered &= ~(1u << op.a); break;
+                case OP_CX: case OP_CXT: gathered &= ~(1u << op.b); break;
+                default: break;
+                }
                 switch (op.kind) {
                 case OP_H: alu_per_amp += 2.0; break;                 // a + b, a - b per component pair
                 case OP_RXS: case OP_RYS: alu_per_amp += 4.0; break;  // one multiply-add per component
                 case OP_U2S: alu_per_amp += 11.0; break;              // x + u y (8), v x + w y (14) per pair
                 case OP_DIAG: case OP_TAPPLY: alu_per_amp += 6.0; break;   // complex product, all
-                case OP_P: case OP_CPT: alu_per_amp += 3.0; break;    // complex product on half
+                case OP_P: alu_per_amp += 3.0; break;                 // complex product on half
+                case OP_CPT:
+                    if (!gather || !((gathered >> op.a) & 1)) alu_per_amp += 3.0;
+                    gathered |= 1u << op.a;
+                    break;
                 case OP_CP: alu_per_amp += 1.5; break;                // complex product on a quarter
                 default: break;                                       // X, Y, Z, CX, CZ, SWAP, thread phases
                 }

@@ -70,7 +70,7 @@ bool compile_program(const std::vector<GateRef> &gates, int n, const std::vector
 
 // Floating-point operations per state amplitude that the program's kernels
 // execute: CUDA-core arithmetic (alu) and tensor-core products (tensor).
-void program_flops(const Program &prog, double &alu_per_amp, double &tensor_per_amp);
+void program_flops(const Program &prog, double &alu_per_amp, double &tensor_per_amp, bool gather);
 
 // Fused unitary of gates acting on the qubits qs[0..k) (local bit j <-> qs[j]):
 // U = G_last ... G_first as a 2^k x 2^k row-major interleaved complex matrix.
