@@ -223,7 +223,7 @@ def choose_plan(gates, n, candidates=PLAN_CANDIDATES):
         if len(cand) > 4 and n < cand[4]:
             continue
         plan = api.Plan(gates, n, method, min(k, n), dfs_trials=16)
-        e = estimate_s(n, plan.stats("c64", 0, tc=tc), tc, jit)
+        e = estimate_s(n, plan.stats("c64", 0, tc=tc, jit=jit), tc, jit)
         est.append({"method": method, "k": k, "tc": tc, "jit": jit, "est_s": e})
         if best is None or e < best[2]:
             if best is not None:
