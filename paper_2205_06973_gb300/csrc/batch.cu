@@ -215,64 +215,68 @@ k_batch_whole(float2 *__restrict__ svbase, const BatchWhole *__restrict__ circui
     pdl_wait();   // done when the kernel before is
 }
 
-// p[i] = |a_i|^2 over the concatenated states, 2^10 amplitudes per warp and
+// p[i] = |a_i|^2 over the concatenated states, 2^10 amplitudes per block and
 // iteration (the smallest circuit, and every circuit's offset is a multiple
 // of it), on the FP32 pipes as in k_probs_fast; partials (may be null)
 // receives each chunk's FP64 sum. One block per circuit with FP64 arithmetic
 // left a batch's largest circuits to single SMs: 2.83 ms for 160 circuits of
 // 10 to 20 qubits (28.5 M amplitudes), the time of one 20-qubit circuit;
-// 0.1 ms here.
+// 0.06 ms here, 0.12 with norms.
 constexpr int BPROB_CHUNK = 1 << BATCH_MIN_QUBITS;
 constexpr int BPROB_THREADS = 128;
-constexpr int BPROB_U = 4;   // 16-byte loads in flight per thread
-static_assert(BPROB_CHUNK / 2 % (2 * 32 * BPROB_U) == 0 && 2 * (2 * BPROB_U) <= PROB_SUM, "pairs of a warp's rounds");
+constexpr int BPROB_U = 4;   // 16-byte loads in flight per thread: a chunk in one round
+static_assert(BPROB_CHUNK == 2 * BPROB_THREADS * BPROB_U && 2 * BPROB_U <= PROB_SUM, "a chunk per block");
 
 __global__ void __launch_bounds__(BPROB_THREADS, 10)
 k_batch_probs(const float4 *__restrict__ sv, uint64_t n_chunks, float *__restrict__ out, bool pairs,
               double *__restrict__ partials) {
-    constexpr int WARPS = BPROB_THREADS / 32;
-    const uint32_t lane = threadIdx.x & 31;
-    for (uint64_t c = (uint64_t)blockIdx.x * WARPS + (threadIdx.x >> 5); c < n_chunks; c += (uint64_t)gridDim.x * WARPS) {
+    __shared__ double red[BPROB_THREADS / 32];
+    for (uint64_t c = blockIdx.x; c < n_chunks; c += gridDim.x) {
+        const uint64_t at = c * (BPROB_CHUNK / 2) + threadIdx.x;
+        float4 v[BPROB_U];
+#pragma unroll
+        for (int u = 0; u < BPROB_U; u++) v[u] = __ldcs(sv + at + BPROB_THREADS * u);
         NormSum sum;
         double acc = 0.0;
-        for (int r = 0; r < BPROB_CHUNK / 2; r += 32 * BPROB_U) {
-            const uint64_t at = c * (BPROB_CHUNK / 2) + r + lane;
-            float4 v[BPROB_U];
+        const bool ok = sum.fits<false>(v, acc);
 #pragma unroll
-            for (int u = 0; u < BPROB_U; u++) v[u] = __ldcs(sv + at + 32 * u);
-            const bool ok = sum.fits<false>(v, acc);
-#pragma unroll
-            for (int u = 0; u < BPROB_U; u++) {
-                float p, q;
-                if (ok) {
-                    const Squares a(make_float2(v[u].x, v[u].y)), b(make_float2(v[u].z, v[u].w));
-                    sum.add(a);
-                    sum.add(b);
-                    p = a.prob();
-                    q = b.prob();
-                } else {
-                    const double a = (double)v[u].x * v[u].x + (double)v[u].y * v[u].y;
-                    const double b = (double)v[u].z * v[u].z + (double)v[u].w * v[u].w;
-                    acc += a;
-                    acc += b;
-                    p = (float)a;
-                    q = (float)b;
-                }
-                if (out) {
-                    const uint64_t i = 2 * (at + 32 * u);
-                    if (pairs) *reinterpret_cast<float2 *>(out + i) = make_float2(p, q);
-                    else {
-                        out[i] = p;
-                        out[i + 1] = q;
-                    }
+        for (int u = 0; u < BPROB_U; u++) {
+            float p, q;
+            if (ok) {
+                const Squares a(make_float2(v[u].x, v[u].y)), b(make_float2(v[u].z, v[u].w));
+                sum.add(a);
+                sum.add(b);
+                p = a.prob();
+                q = b.prob();
+            } else {
+                const double a = (double)v[u].x * v[u].x + (double)v[u].y * v[u].y;
+                const double b = (double)v[u].z * v[u].z + (double)v[u].w * v[u].w;
+                acc += a;
+                acc += b;
+                p = (float)a;
+                q = (float)b;
+            }
+            if (out) {
+                const uint64_t i = 2 * (at + BPROB_THREADS * u);
+                if (pairs) *reinterpret_cast<float2 *>(out + i) = make_float2(p, q);
+                else {
+                    out[i] = p;
+                    out[i + 1] = q;
                 }
             }
-            if (partials && (r & (32 * BPROB_U))) acc += sum.take();   // every second round
         }
         if (!partials) continue;
+        acc += sum.take();
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) partials[c] = acc;
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double s = 0.0;
+            for (int w = 0; w < BPROB_THREADS / 32; w++) s += red[w];
+            partials[c] = s;
+        }
+        __syncthreads();
     }
 }
 
@@ -348,8 +352,7 @@ cudaError_t launch_batch_whole(int t, const BatchLaunch &B, const BatchWhole *ci
 cudaError_t launch_batch_probs(float2 *svbase, uint64_t total, const uint64_t *circ_off, const uint32_t *circ_n,
                                uint32_t n_circ, float *out, double *partials, double *norms, cudaStream_t st) {
     const uint64_t chunks = total / BPROB_CHUNK;
-    const uint64_t need = (chunks + BPROB_THREADS / 32 - 1) / (BPROB_THREADS / 32);
-    const uint64_t blocks = need < 152 * 10 ? need : 152 * 10;
+    const uint64_t blocks = chunks < 152 * 10 ? chunks : 152 * 10;
     if (out || norms) {
         k_batch_probs<<<(unsigned)blocks, BPROB_THREADS, 0, st>>>(reinterpret_cast<const float4 *>(svbase), chunks, out,
                                                         (reinterpret_cast<uintptr_t>(out) & 7) == 0,
