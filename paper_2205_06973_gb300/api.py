@@ -195,7 +195,7 @@ class State:
         return norm.value
 
     def summary(self):
-        """(norm, |a_0|^2, argmax_x |a_x|^2, max |a_x|^2) in FP64 without a
+        """(norm, |a_0|^2, argmax_x |a_x|^2, max |a_x|^2) to FP64's accuracy without a
         probability vector (sv_measure_summary; synchronises)."""
         nrm, p0, pm = ctypes.c_double(), ctypes.c_double(), ctypes.c_double()
         am = ctypes.c_uint64()

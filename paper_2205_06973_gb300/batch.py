@@ -85,7 +85,7 @@ class Batch:
 
     def probs(self, out=None, norms=True):
         """Probabilities of all states (one float32 device tensor, concatenated)
-        and the per-circuit norms (numpy, FP64 accumulation) if requested."""
+        and the per-circuit norms (numpy, to FP64's accuracy) if requested."""
         if out is None:
             out = torch.empty(self.total, dtype=torch.float32, device="cuda")
         nrm = np.zeros(self.n, dtype=np.float64) if norms else None

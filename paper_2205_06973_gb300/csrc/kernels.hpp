@@ -30,7 +30,7 @@ cudaError_t launch_part_f64(int t, int R, void *sv, const PartLaunch &L, const v
 cudaError_t launch_gate1(bool fp64, void *sv, int n, int q, const double *m, cudaStream_t st);
 cudaError_t launch_gate2(bool fp64, void *sv, int n, int q0, int q1, const double *m, cudaStream_t st);
 
-// p[x] = |a_x|^2 (float or double out, may be null) and FP64 block partial sums
+// p[x] = |a_x|^2 (float or double out, may be null) and block partial sums
 // of the norm reduced into *d_norm. partials has nblocks doubles, of which at
 // most nblocks are used. ticket: a zeroed device word, left zero, that lets
 // the last block add the partials up; null takes a second launch for it
@@ -39,7 +39,7 @@ cudaError_t launch_probs(bool fp64, const void *sv, int n, void *out, int out_fp
                          int nblocks, double *d_norm, cudaStream_t st, bool df, uint32_t *ticket);
 
 // Norm, |a_0|^2 and the largest |a_x|^2 with its index (ties to the smaller
-// index), FP64, without a probability vector: scratch holds 3 * nblocks
+// index), to FP64's accuracy, without a probability vector: scratch holds 3 * nblocks
 // doubles, out 4 (out[3] holds the index's bits); ticket as above, required.
 cudaError_t launch_summary(bool fp64, const void *sv, int n, double *scratch, int nblocks, double *out,
                            cudaStream_t st, bool df, uint32_t *ticket);

@@ -41,7 +41,7 @@ Admitted states stay on the device until their result is taken.
   ``k_large`` on the gate-list kernel.
 
 A request's result is a summary of its probability distribution (Sec. II-A):
-the norm (FP64 accumulation on the device), the probability of |0...0> and
+the norm (summed on the device to FP64's accuracy), the probability of |0...0> and
 the most likely basis state with its probability; large requests get it from
 a device reduction that writes no probability vector (sv_measure_summary),
 so the only device memory a request holds is its state. The full state can
